@@ -312,6 +312,7 @@ int sketchssm_step_mixed(sketchssm_ctx* ctx, const int32_t* phase, const void* q
     pu.write_sketch = 1;
     pu.write_state = 1;
     pu.n_dev = phase;
+    pu.late_wait = 1;
     rc = launch_update(ctx, pu, cs);
     if (rc != SKETCHSSM_OK) return rc;
     launched += ctx->last_launches;

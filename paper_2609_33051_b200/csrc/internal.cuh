@@ -78,6 +78,8 @@ struct Params {
     const int* head_rank; // optional [H]: sketch rank per head index (0: the head reads the full state); nullptr: R for every head
     const int* n_dev;     // optional [B]: per-sequence phase of a mixed step (>= 0: decode step at that ring fill; < 0: flush with
                           // -v - 1 buffered tokens); nullptr: n_before for every sequence
+    int late_wait;        // update (CUDA cores): wait for the predecessor in the stream (the decode kernel of the same mixed step)
+                          // at the end of the kernel instead of at its start
     int n_cap;            // update (CUDA cores) with per-sequence phases: ring rows the shared-memory layout has room for
     int sketch_bf16;      // U (and the fixed C) are stored as bfloat16
     float* erase;         // projected erase vectors f_s [B][H][L][R] (Eq. 44-45), or nullptr: c_t = C q~_t from the swept query

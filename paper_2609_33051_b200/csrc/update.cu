@@ -1,20 +1,31 @@
-// State-update (flush) kernel of the SketchSSM hot path (sm_100a), CUDA-core version.
+// State-update (flush) kernel of the SketchSSM hot path (sm_100a), CUDA-core version: every configuration, fp32 throughout.
 //
-// Every V-column of S is an independent K-vector recurrence under all three transitions: the erase
-// dot <k_s, S[:, j]> touches one column only.  A CTA owns a tile of VT = 64 columns of one (b, h)
-// state; a column lives in the registers of 4 threads (K/4 rows each), so the whole tile is read
-// from HBM once, replayed on chip, projected onto Omega for the sketch rows U[g, j] = <S[:, j], omega_g>
-// and onto q for the exact output, and written back once (Algorithm 1, flush step; Eq. 3 and Eq. 7).
+// Every V-column of S is an independent K-vector recurrence under all three transitions: the erase dot <k_s, S[:, j]>
+// touches one column only.  A CTA owns the whole state of a head and a warp 16 of its columns: eight lanes share four
+// columns, K/8 rows each, in registers.  The state is read once, replayed on chip, projected onto Omega for the sketch
+// rows U[g, j] = <S[:, j], omega_g> and onto q for the exact output, and written once (Algorithm 1, flush; Eq. 3, Eq. 7).
 //
-//   delta rule (GDN, KDA), token by token:  col <- D_s col;  e = beta_s (v_s[j] - <k_s, col>);  col += e k_s
-//   Mamba-2, closed form of Eq. 3:          col <- d col + sum_s (beta_s prod_{j>s} a_j) v_s[j] k_s
+//   Mamba-2, closed form of Eq. 3:   S <- d S + sum_s (beta_s prod_{j>s} a_j) k_s v_s^T
+//   delta rule (GDN, KDA), eight tokens at a time, with G_s = prod_{m<=s} g_m, Dn_s = prod_{m>s} g_m (within the eight):
+//     P_s = <G_s k_s, S_0>;  e_s = beta_s (v_s - P_s - sum_{j<s} A_sj e_j),  A_sj = sum_i k_s[i] k_j[i] prod_{j<m<=s} g_m[i];
+//     S <- G_8 S_0 + sum_s (Dn_s k_s) e_s^T
+//   which is the token-by-token recurrence with the eight erase dots taken from the same state: one decay of the state
+//   and one reduction over the rows for eight tokens.  No quotient of decay products is formed.
+//
+// What bounds it: fp32 issue and the shared-memory reads of the key rows (2 n + r + 1 multiply-adds per state element).
+// Four columns per lane: a 128-bit read of a key row feeds eight packed multiply-adds.  One column per lane and 64-column
+// tiles, as before, read four times as many key rows and multiplied the state by the decay at every token.
 #include "internal.cuh"
+#include "lanegroup.cuh"
 
 namespace sketchssm {
 
-constexpr int kParts = 4;               // threads per column; a CTA owns VT = 64 columns (80 when V = 80) of one head
+constexpr int kParts = 8;               // lanes that share a group of four columns
+constexpr int kTok = 8;                 // tokens replayed together
+constexpr int kPairs = 32;              // pairs (s, j < s) of kTok tokens, padded from 28
+constexpr int kScan = 1024;             // sequences whose phases are looked through at a time
 
-// shared-memory row of K floats split into kParts parts, each padded by 4 floats so that the four
+// shared-memory row of K floats split into kParts parts, each padded by 4 floats so that the eight
 // parts of a warp read from different banks with 128-bit loads
 template <int K>
 struct PaddedRow {
@@ -44,276 +55,653 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
 }
 
 struct UpdateSmem {
-    uint32_t k_off, g_off, v_off, beta_off, dec_off, q_off, om_off, total;
+    uint32_t kh_off, kt_off, g_off, gram_off, a_off, beta_off, pre_off, suf_off, v_off, e_off, q_off, om_off, list_off, bar_off;
+    uint32_t st_off, st_k, st_v, st_gate, st_g, st_tq, st_tk, st_tv, st_tg;      // stage (0 bytes without one)
+    uint32_t total;
 };
 
+// Omega rows are four floats further apart than a key row: the transposing fill writes consecutive ranks, which would
+// otherwise all fall into one bank.
 template <int K>
-__host__ __device__ inline UpdateSmem make_update_smem(int kind, int n_tot, int R4, int kVT) {
+__host__ __device__ constexpr int omega_stride() { return PaddedRow<K>::stride + 4; }
+
+template <int K>
+__host__ __device__ inline UpdateSmem make_update_smem(int kind, int n_tot, int R, int V, int L, int io, int mixed, int stage) {
     UpdateSmem u;
     const int ntok = n_tot > 0 ? n_tot : 1;
+    const int nb = (ntok + kTok - 1) / kTok;
+    const int R8 = (R + 7) & ~7;
+    const bool delta = kind != SKETCHSSM_MAMBA2, kda = kind == SKETCHSSM_KDA;
+    const uint32_t row = PaddedRow<K>::stride * 4;
     uint32_t off = 0;
-    u.k_off = off; off += (uint32_t)(ntok * PaddedRow<K>::stride * 4);
-    u.g_off = off; off += kind == SKETCHSSM_KDA ? (uint32_t)(ntok * PaddedRow<K>::stride * 4) : 0u;
-    u.v_off = off; off += (uint32_t)(ntok * kVT * 4);
-    u.beta_off = off; off += (uint32_t)(((ntok + 3) & ~3) * 4);
-    u.dec_off = off; off += (uint32_t)(((ntok + 3) & ~3) * 4);
-    u.q_off = off; off += (uint32_t)(PaddedRow<K>::stride * 4);
-    u.om_off = off; off += (uint32_t)(kParts * ((K / kParts) * R4 + 4) * 4);
+    u.kt_off = off; off += (uint32_t)(nb * kTok) * row;
+    u.kh_off = off; off += kda ? (uint32_t)(nb * kTok) * row : 0u;
+    u.g_off = off; off += kda ? (uint32_t)nb * row : 0u;
+    u.gram_off = off; off += delta ? (uint32_t)(nb * (K / 32) * kPairs * 4) : 0u;
+    u.a_off = off; off += delta ? (uint32_t)(nb * kPairs * 4) : 0u;
+    u.beta_off = off; off += (uint32_t)(nb * kTok * 4);
+    u.pre_off = off; off += (uint32_t)(nb * kTok * 4);
+    u.suf_off = off; off += kind == SKETCHSSM_GDN ? (uint32_t)(nb * kTok * 4) : 0u;
+    u.v_off = off; off += (uint32_t)(ntok * V * io);
+    u.e_off = off; off += (uint32_t)(V / 16) * (kTok * 16 * 4);
+    u.q_off = off; off += row;
+    u.om_off = off; off += (uint32_t)(R8 * omega_stride<K>() * 4);
+    u.list_off = off; off += mixed ? (uint32_t)((kScan + 32) * 4) : 0u;
+    u.bar_off = off; off += 16u;
+    off = (off + 127u) & ~127u;
+    u.st_off = u.st_k = u.st_v = u.st_gate = u.st_g = u.st_tq = u.st_tk = u.st_tv = u.st_tg = off;
+    if (stage) {
+        off += (uint32_t)(K * V * 4);
+        u.st_k = off; off += (uint32_t)(ntok * K * io);
+        u.st_v = off; off += (uint32_t)(ntok * V * io);
+        u.st_gate = off; off += (uint32_t)((kda ? 1 : 2) * L * 4);
+        u.st_g = off; off += kda ? (uint32_t)(ntok * K * io) : 0u;
+        u.st_tq = off; off += (uint32_t)(K * io);
+        u.st_tk = off; off += (uint32_t)(K * io);
+        u.st_tv = off; off += (uint32_t)(V * io);
+        u.st_tg = off; off += kda ? (uint32_t)(K * io) : 0u;
+    }
     u.total = off;
     return u;
 }
 
-template <int KIND, typename IO, int K, int kVT>
-__global__ void __launch_bounds__(kVT * kParts) update_kernel(const Params p) {
-    constexpr int kUpdThreads = kVT * kParts;
-    using PR = PaddedRow<K>;
-    constexpr int RP = PR::RP;
-    extern __shared__ __align__(128) unsigned char smem[];
-
-    const int V = p.dv;
-    const int R = p.R, H = p.H;
-    const int R4 = (R + 3) & ~3;
-    const int vtiles = V / kVT;
-    const int bh = blockIdx.x / vtiles;
-    const int v0 = (blockIdx.x % vtiles) * kVT;
-    const int b = bh / H, h = bh % H;
-    // ring fill: the call's n_before, or with per-sequence phases the sequence's own (a sequence whose phase says
-    // "decode step" is left alone by this kernel)
-    int n_ring = p.n_before;
-    if (p.n_dev != nullptr) {
-        const int ph = p.n_dev[b];
-        if (ph >= 0) return;
-        n_ring = -ph - 1;
-    }
-    const int n_tot = n_ring + (p.has_token ? 1 : 0);
-
-    const UpdateSmem us = make_update_smem<K>(KIND, p.n_dev != nullptr ? p.n_cap : n_tot, R4, kVT);
-    float* sK = reinterpret_cast<float*>(smem + us.k_off);
-    float* sG = reinterpret_cast<float*>(smem + us.g_off);
-    float* sV = reinterpret_cast<float*>(smem + us.v_off);
-    float* sBeta = reinterpret_cast<float*>(smem + us.beta_off);
-    float* sDec = reinterpret_cast<float*>(smem + us.dec_off);
-    float* sQ = reinterpret_cast<float*>(smem + us.q_off);
-    float* sOm = reinterpret_cast<float*>(smem + us.om_off);
-
-    const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
-    const int part = lane >> 3;                    // 0..3: which quarter of the rows
-    const int j = v0 + warp * 8 + (lane & 7);      // this thread's column
-    const int jl = j - v0;
-
-    // ---- state tile -> registers (issued first: the long-latency stream) ----
-    float col[RP];
-    const float* Sg = p.state + (size_t)bh * K * V + (size_t)(part * RP) * V + j;
+// Dot products of this lane's rows of four columns with four rows of shared memory: vals[4 t + c].
+template <int RP>
+__device__ __forceinline__ void dot4(const f32x2 (&c2)[4][RP / 2], const float* row, int stride, float* vals) {
+    f32x2 acc[4][4];
 #pragma unroll
-    for (int ii = 0; ii < RP; ++ii) col[ii] = Sg[(size_t)ii * V];
-
-    // ---- ring + current token -> shared memory (fp32) ----
-    const unsigned char* rh = p.ring + (size_t)bh * p.rl.head_bytes;
-    const IO* rk = reinterpret_cast<const IO*>(rh);
-    const IO* rv = reinterpret_cast<const IO*>(rh + p.rl.v_off);
-    const float* rbeta = reinterpret_cast<const float*>(rh + p.rl.beta_off);
-    for (int idx = tid; idx < n_tot * K; idx += kUpdThreads) {
-        const int s = idx / K, i = idx % K;
-        float kv, gv = 1.f;
-        if (s < n_ring) {
-            kv = static_cast<float>(rk[(size_t)s * K + i]);
-            if constexpr (KIND == SKETCHSSM_KDA)
-                gv = static_cast<float>(reinterpret_cast<const IO*>(rh + p.rl.decay_off)[(size_t)s * K + i]);
-        } else {
-            kv = static_cast<float>(reinterpret_cast<const IO*>(p.k)[(size_t)bh * K + i]);
-            if constexpr (KIND == SKETCHSSM_KDA)
-                gv = static_cast<float>(reinterpret_cast<const IO*>(p.decay)[(size_t)bh * K + i]);
-        }
-        sK[s * PR::stride + PR::at(i)] = kv;
-        if constexpr (KIND == SKETCHSSM_KDA) sG[s * PR::stride + PR::at(i)] = gv;
-    }
-    for (int idx = tid; idx < n_tot * kVT; idx += kUpdThreads) {
-        const int s = idx / kVT, c = idx % kVT;
-        sV[idx] = s < n_ring ? static_cast<float>(rv[(size_t)s * V + v0 + c])
-                             : static_cast<float>(reinterpret_cast<const IO*>(p.v)[(size_t)bh * V + v0 + c]);
-    }
-    if (tid < n_tot) {
-        const int s = tid;
-        sBeta[s] = s < n_ring ? rbeta[s] : p.beta[bh];
-        if constexpr (KIND != SKETCHSSM_KDA) {
-            sDec[s] = s < n_ring ? reinterpret_cast<const float*>(rh + p.rl.decay_off)[s]
-                                 : reinterpret_cast<const float*>(p.decay)[bh];
-        }
-    }
-    if (p.q != nullptr) {
-        for (int i = tid; i < K; i += kUpdThreads)
-            sQ[PR::at(i)] = static_cast<float>(reinterpret_cast<const IO*>(p.q)[(size_t)bh * K + i]);
-    }
-    if (p.write_sketch) {
-        const float* og = p.omega + (size_t)h * K * R;
-        for (int idx = tid; idx < K * R4; idx += kUpdThreads) {
-            const int i = idx / R4, g = idx % R4;
-            sOm[(i / RP) * (RP * R4 + 4) + (i % RP) * R4 + g] = g < R ? og[(size_t)i * R + g] : 0.f;
-        }
-    }
-    __syncthreads();
-
-    if constexpr (KIND == SKETCHSSM_MAMBA2) {
-        // sBeta[s] <- beta_s * prod_{j>s} a_j ;  total decay d = prod_j a_j
-        __shared__ float s_total;
-        if (tid == 0) {
-            float suf = 1.f;
-            for (int s = n_tot - 1; s >= 0; --s) {
-                sBeta[s] *= suf;
-                suf *= sDec[s];
+    for (int i4 = 0; i4 < RP / 4; ++i4) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const float4 kq = *reinterpret_cast<const float4*>(row + t * stride + 4 * i4);
+            const f32x2 k01 = pack2(kq.x, kq.y), k23 = pack2(kq.z, kq.w);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                acc[t][c] = i4 == 0 ? mul2(k01, c2[c][0]) : fma2(k01, c2[c][2 * i4], acc[t][c]);
+                acc[t][c] = fma2(k23, c2[c][2 * i4 + 1], acc[t][c]);
             }
-            s_total = suf;
-        }
-        __syncthreads();
-        if (n_tot > 0) {
-            const float d = s_total;
-            f32x2 c2[RP / 2];
-#pragma unroll
-            for (int i2 = 0; i2 < RP / 2; ++i2) c2[i2] = pack2(col[2 * i2] * d, col[2 * i2 + 1] * d);
-            for (int s = 0; s < n_tot; ++s) {
-                const float w = sBeta[s] * sV[s * kVT + jl];
-                const f32x2 w2 = pack2(w, w);
-                const float4* kp = reinterpret_cast<const float4*>(sK + s * PR::stride + part * (RP + 4));
-#pragma unroll
-                for (int i4 = 0; i4 < RP / 4; ++i4) {
-                    const float4 kq = kp[i4];
-                    c2[2 * i4] = fma2(pack2(kq.x, kq.y), w2, c2[2 * i4]);
-                    c2[2 * i4 + 1] = fma2(pack2(kq.z, kq.w), w2, c2[2 * i4 + 1]);
-                }
-            }
-#pragma unroll
-            for (int i2 = 0; i2 < RP / 2; ++i2) unpack2(c2[i2], col[2 * i2], col[2 * i2 + 1]);
-        }
-    } else {
-        f32x2 c2[RP / 2];
-#pragma unroll
-        for (int i2 = 0; i2 < RP / 2; ++i2) c2[i2] = pack2(col[2 * i2], col[2 * i2 + 1]);
-        for (int s = 0; s < n_tot; ++s) {
-            const float4* kp = reinterpret_cast<const float4*>(sK + s * PR::stride + part * (RP + 4));
-            f32x2 k2[RP / 2];
-#pragma unroll
-            for (int i4 = 0; i4 < RP / 4; ++i4) {
-                const float4 kq = kp[i4];
-                k2[2 * i4] = pack2(kq.x, kq.y);
-                k2[2 * i4 + 1] = pack2(kq.z, kq.w);
-            }
-            f32x2 dot01 = pack2(0.f, 0.f), dot23 = dot01;
-            if constexpr (KIND == SKETCHSSM_GDN) {
-                const float a = sDec[s];
-                const f32x2 a2 = pack2(a, a);
-#pragma unroll
-                for (int i4 = 0; i4 < RP / 4; ++i4) {
-                    c2[2 * i4] = mul2(c2[2 * i4], a2);
-                    c2[2 * i4 + 1] = mul2(c2[2 * i4 + 1], a2);
-                    dot01 = fma2(k2[2 * i4], c2[2 * i4], dot01);
-                    dot23 = fma2(k2[2 * i4 + 1], c2[2 * i4 + 1], dot23);
-                }
-            } else {
-                const float4* gp = reinterpret_cast<const float4*>(sG + s * PR::stride + part * (RP + 4));
-#pragma unroll
-                for (int i4 = 0; i4 < RP / 4; ++i4) {
-                    const float4 gq = gp[i4];
-                    c2[2 * i4] = mul2(c2[2 * i4], pack2(gq.x, gq.y));
-                    c2[2 * i4 + 1] = mul2(c2[2 * i4 + 1], pack2(gq.z, gq.w));
-                    dot01 = fma2(k2[2 * i4], c2[2 * i4], dot01);
-                    dot23 = fma2(k2[2 * i4 + 1], c2[2 * i4 + 1], dot23);
-                }
-            }
-            float d0, d1, d2, d3;
-            unpack2(dot01, d0, d1);
-            unpack2(dot23, d2, d3);
-            float dot = (d0 + d2) + (d1 + d3);
-            dot += __shfl_xor_sync(0xffffffffu, dot, 8);
-            dot += __shfl_xor_sync(0xffffffffu, dot, 16);
-            const float e = sBeta[s] * (sV[s * kVT + jl] - dot);
-            const f32x2 e2 = pack2(e, e);
-#pragma unroll
-            for (int i2 = 0; i2 < RP / 2; ++i2) c2[i2] = fma2(k2[i2], e2, c2[i2]);
-        }
-#pragma unroll
-        for (int i2 = 0; i2 < RP / 2; ++i2) unpack2(c2[i2], col[2 * i2], col[2 * i2 + 1]);
-    }
-
-    // ---- write the updated tile back ----
-    if (p.write_state && n_tot > 0) {
-        float* So = p.state + (size_t)bh * K * V + (size_t)(part * RP) * V + j;
-#pragma unroll
-        for (int ii = 0; ii < RP; ++ii) So[(size_t)ii * V] = col[ii];
-    }
-
-    // ---- exact output o[j] = <S_new[:, j], q> ----
-    if (p.out != nullptr) {
-        const float4* qp = reinterpret_cast<const float4*>(sQ + part * (RP + 4));
-        float acc = 0.f;
-#pragma unroll
-        for (int i4 = 0; i4 < RP / 4; ++i4) {
-            const float4 qq = qp[i4];
-            acc = fmaf(qq.x, col[4 * i4 + 0], acc);
-            acc = fmaf(qq.y, col[4 * i4 + 1], acc);
-            acc = fmaf(qq.z, col[4 * i4 + 2], acc);
-            acc = fmaf(qq.w, col[4 * i4 + 3], acc);
-        }
-        acc += __shfl_xor_sync(0xffffffffu, acc, 8);
-        acc += __shfl_xor_sync(0xffffffffu, acc, 16);
-        if (part == 0) {
-            if (p.out_bf16) reinterpret_cast<__nv_bfloat16*>(p.out)[(size_t)bh * V + j] = __float2bfloat16_rn(acc);
-            else reinterpret_cast<float*>(p.out)[(size_t)bh * V + j] = acc;
         }
     }
-
-    // ---- sketch rows U[g, j] = <S_new[:, j], omega_g>, 4 ranks at a time ----
-    if (p.write_sketch) {
-        const size_t ug = (size_t)bh * R * V + j;
-        for (int g0 = 0; g0 < R4; g0 += 4) {
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-            const float* op = sOm + (size_t)part * (RP * R4 + 4) + g0;
 #pragma unroll
-            for (int ii = 0; ii < RP; ++ii) {
-                const float4 w = *reinterpret_cast<const float4*>(op + ii * R4);
-                a0 = fmaf(w.x, col[ii], a0);
-                a1 = fmaf(w.y, col[ii], a1);
-                a2 = fmaf(w.z, col[ii], a2);
-                a3 = fmaf(w.w, col[ii], a3);
-            }
-            a0 += __shfl_xor_sync(0xffffffffu, a0, 8);  a0 += __shfl_xor_sync(0xffffffffu, a0, 16);
-            a1 += __shfl_xor_sync(0xffffffffu, a1, 8);  a1 += __shfl_xor_sync(0xffffffffu, a1, 16);
-            a2 += __shfl_xor_sync(0xffffffffu, a2, 8);  a2 += __shfl_xor_sync(0xffffffffu, a2, 16);
-            a3 += __shfl_xor_sync(0xffffffffu, a3, 8);  a3 += __shfl_xor_sync(0xffffffffu, a3, 16);
-            // part p stores rank g0 + p
-            const float mine = part == 0 ? a0 : part == 1 ? a1 : part == 2 ? a2 : a3;
-            if (g0 + part < R) store_sketch(p, ug + (size_t)(g0 + part) * V, mine);
+    for (int t = 0; t < 4; ++t) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float a, b;
+            unpack2(acc[t][c], a, b);
+            vals[4 * t + c] = a + b;
         }
     }
 }
 
-template <int KIND, typename IO, int K, int kVT>
+// Sums over the eight parts (lane bits 2..4): part p ends up with the four columns of row p in v[0..3].
+__device__ __forceinline__ void reduce_parts(float (&v)[32], int lane) {
+#pragma unroll
+    for (int lvl = 0; lvl < 3; ++lvl) {
+        const int o = 16 >> lvl, half = 16 >> lvl;
+        const bool upper = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            if (i < half) {
+                const float send = upper ? v[i] : v[i + half];
+                const float keep = upper ? v[i + half] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+    }
+}
+
+// Resident CTAs that the register file is divided for: 128 registers a thread hold 64 of the state, the 32 accumulators
+// of four dot products and the key rows in flight.
+template <int V>
+__host__ __device__ constexpr int update_ctas() { return V == 128 ? 2 : V == 80 ? 3 : 4; }
+
+template <int KIND, typename IO, int K, int V>
+__global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const Params p) {
+    constexpr int T = 2 * V;                        // V / 16 warps
+    using PR = PaddedRow<K>;
+    constexpr int RP = PR::RP, KS = PR::stride, OS = omega_stride<K>();
+    constexpr bool DELTA = KIND != SKETCHSSM_MAMBA2, KDA = KIND == SKETCHSSM_KDA;
+    extern __shared__ __align__(128) unsigned char smem[];
+
+    const int R = p.R, H = p.H, B = p.B;
+    const int R8 = (R + 7) & ~7;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int part = lane >> 2;                     // which rows: part * RP ..
+    const int j0 = warp * 16 + (lane & 3) * 4;      // first of this lane's four columns
+    const bool mixed = p.n_dev != nullptr;
+
+    // With per-sequence phases the flush may run beside the decode kernel that was launched just before it (each leaves
+    // the other's sequences alone, and that kernel let its dependents start only after its own predecessor was done), so
+    // it waits at its end instead; the launcher asks for it.
+    if (!p.late_wait) grid_dep_wait();
+    grid_dep_launch_dependents();
+
+    const bool staged = p.stages != 0;
+    const UpdateSmem us = make_update_smem<K>(KIND, mixed ? p.n_cap : p.n_before + (p.has_token ? 1 : 0), R, V, p.L,
+                                              (int)sizeof(IO), mixed, staged);
+    float* sKt = reinterpret_cast<float*>(smem + us.kt_off);
+    float* sKh = reinterpret_cast<float*>(smem + us.kh_off);
+    float* sG = reinterpret_cast<float*>(smem + us.g_off);
+    float* sGram = reinterpret_cast<float*>(smem + us.gram_off);
+    float* sA = reinterpret_cast<float*>(smem + us.a_off);
+    float* sBeta = reinterpret_cast<float*>(smem + us.beta_off);
+    float* sPre = reinterpret_cast<float*>(smem + us.pre_off);      // GDN: decay up to a token of its eight; Mamba-2: [0] the total
+    float* sSuf = reinterpret_cast<float*>(smem + us.suf_off);      // GDN: decay behind it
+    IO* sV = reinterpret_cast<IO*>(smem + us.v_off);
+    float* sE = reinterpret_cast<float*>(smem + us.e_off) + warp * (kTok * 16);
+    float* sQ = reinterpret_cast<float*>(smem + us.q_off);
+    float* sOm = reinterpret_cast<float*>(smem + us.om_off);
+    int* sList = reinterpret_cast<int*>(smem + us.list_off);
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + us.bar_off);
+    float* sTok = reinterpret_cast<float*>(smem + us.bar_off + 8);  // the current token's beta and scalar decay (staged)
+
+    // One head ahead, by bulk copies into a stage: the state, the buffered tokens and the current token's rows.  A CTA holds
+    // one head in registers, and two to four CTAs per SM do not cover the latency of memory between two heads by
+    // themselves.  The token's scalar gates travel through the registers of the thread that issues the copies.
+    int h_staged = -1;                              // head index whose Omega is in shared memory
+    uint32_t parity = 0;
+    bool failed = false;
+    float next_beta = 0.f, next_decay = 1.f;
+    auto request = [&](int b, int h, int n_ring) {      // thread 0
+        const size_t bh = (size_t)b * H + h;
+        const unsigned char* rh = p.ring + bh * p.rl.head_bytes;
+        constexpr uint32_t kRow = (uint32_t)(K * sizeof(IO)), vRow = (uint32_t)(V * sizeof(IO));
+        const uint32_t gates = (uint32_t)((KDA ? 1 : 2) * p.L * 4);
+        uint32_t bytes = (uint32_t)(K * V * 4);
+        if (n_ring > 0) bytes += (uint32_t)n_ring * ((KDA ? 2 : 1) * kRow + vRow) + gates;
+        if (p.has_token) bytes += (KDA ? 2 : 1) * kRow + vRow;
+        if (p.q != nullptr) bytes += kRow;
+        mbar_expect_tx(bar, bytes);
+        bulk_g2s(smem + us.st_off, p.state + bh * (size_t)(K * V), (uint32_t)(K * V * 4), bar);
+        if (n_ring > 0) {
+            bulk_g2s(smem + us.st_k, rh, (uint32_t)n_ring * kRow, bar);
+            bulk_g2s(smem + us.st_v, rh + p.rl.v_off, (uint32_t)n_ring * vRow, bar);
+            bulk_g2s(smem + us.st_gate, rh + p.rl.beta_off, gates, bar);
+            if constexpr (KDA) bulk_g2s(smem + us.st_g, rh + p.rl.decay_off, (uint32_t)n_ring * kRow, bar);
+        }
+        if (p.has_token) {
+            bulk_g2s(smem + us.st_tk, reinterpret_cast<const IO*>(p.k) + bh * K, kRow, bar);
+            bulk_g2s(smem + us.st_tv, reinterpret_cast<const IO*>(p.v) + bh * V, vRow, bar);
+            if constexpr (KDA) bulk_g2s(smem + us.st_tg, reinterpret_cast<const IO*>(p.decay) + bh * K, kRow, bar);
+            next_beta = p.beta[bh];
+            if constexpr (!KDA) next_decay = reinterpret_cast<const float*>(p.decay)[bh];
+        }
+        if (p.q != nullptr) bulk_g2s(smem + us.st_tq, reinterpret_cast<const IO*>(p.q) + bh * K, kRow, bar);
+    };
+
+    // n_next: ring fill of the CTA's next head (b_next, h_next); negative if there is none
+    auto replay = [&](int b, int h, int n_ring, int b_next, int h_next, int n_next) {
+        const size_t bh = (size_t)b * H + h;
+        const int n_tot = n_ring + (p.has_token ? 1 : 0);
+        const int nb = (n_tot + kTok - 1) / kTok;
+
+        // ---- state -> registers ----
+        float4 raw[RP];
+        const unsigned char* rh = p.ring + bh * p.rl.head_bytes;
+        const IO* rk = reinterpret_cast<const IO*>(rh);
+        const IO* rv = reinterpret_cast<const IO*>(rh + p.rl.v_off);
+        const float* rbeta = reinterpret_cast<const float*>(rh + p.rl.beta_off);
+        const float* rdec = reinterpret_cast<const float*>(rh + p.rl.decay_off);
+        const IO* tk = reinterpret_cast<const IO*>(p.k) + bh * K;
+        const IO* tv = reinterpret_cast<const IO*>(p.v) + bh * V;
+        const IO* tq = reinterpret_cast<const IO*>(p.q) + bh * K;
+        const IO* tg = reinterpret_cast<const IO*>(p.decay) + bh * K;            // KDA
+        const float* tbeta = p.beta + bh;
+        const float* tdec = reinterpret_cast<const float*>(p.decay) + bh;        // scalar decays
+        if (staged) {
+            rk = reinterpret_cast<const IO*>(smem + us.st_k);
+            rv = reinterpret_cast<const IO*>(smem + us.st_v);
+            rbeta = reinterpret_cast<const float*>(smem + us.st_gate);
+            rdec = KDA ? reinterpret_cast<const float*>(smem + us.st_g) : rbeta + p.L;
+            tk = reinterpret_cast<const IO*>(smem + us.st_tk);
+            tv = reinterpret_cast<const IO*>(smem + us.st_tv);
+            tq = reinterpret_cast<const IO*>(smem + us.st_tq);
+            tg = reinterpret_cast<const IO*>(smem + us.st_tg);
+            tbeta = sTok;
+            tdec = sTok + 1;
+            failed = !mbar_wait_bounded(bar, parity);
+            if (failed) mbar_wait_bounded(bar, parity, 1u << 14);    // a last chance for copies in flight before the CTA leaves
+            parity ^= 1u;
+            const float* Ss = reinterpret_cast<const float*>(smem + us.st_off) + (part * RP) * V + j0;
+#pragma unroll
+            for (int i = 0; i < RP; ++i) raw[i] = *reinterpret_cast<const float4*>(Ss + i * V);
+        } else {
+            const float* Sg = p.state + bh * (size_t)(K * V) + (size_t)(part * RP) * V + j0;
+#pragma unroll
+            for (int i = 0; i < RP; ++i) raw[i] = *reinterpret_cast<const float4*>(Sg + (size_t)i * V);
+        }
+
+        // ---- ring + current token -> shared memory (fp32) ----
+        if constexpr (DELTA) {
+            // a thread per (eight tokens, channel)
+            for (int idx = tid; idx < nb * K; idx += T) {
+                const int blk = idx / K, i = idx % K;
+                float k[kTok], g[kTok];
+#pragma unroll
+                for (int s = 0; s < kTok; ++s) {
+                    const int t = blk * kTok + s;
+                    k[s] = 0.f;
+                    g[s] = 1.f;
+                    if (t < n_ring) {
+                        k[s] = static_cast<float>(rk[(size_t)t * K + i]);
+                        g[s] = KDA ? static_cast<float>(reinterpret_cast<const IO*>(rdec)[(size_t)t * K + i]) : rdec[t];
+                    } else if (t < n_tot) {
+                        k[s] = static_cast<float>(tk[i]);
+                        g[s] = KDA ? static_cast<float>(tg[i]) : *tdec;
+                    }
+                }
+                const int at = blk * kTok * KS + PR::at(i);
+                float pre = 1.f, suf = 1.f;
+                if constexpr (KDA) {
+#pragma unroll
+                    for (int s = 0; s < kTok; ++s) {
+                        pre *= g[s];
+                        sKh[at + s * KS] = pre * k[s];
+                    }
+                    sG[blk * KS + PR::at(i)] = pre;
+#pragma unroll
+                    for (int s = kTok - 1; s >= 0; --s) {
+                        sKt[at + s * KS] = suf * k[s];
+                        suf *= g[s];
+                    }
+                } else {
+#pragma unroll
+                    for (int s = 0; s < kTok; ++s) sKt[at + s * KS] = k[s];
+                    if (i == 0) {                // scalar decays are applied to the dot products and the e instead
+#pragma unroll
+                        for (int s = 0; s < kTok; ++s) {
+                            pre *= g[s];
+                            sPre[blk * kTok + s] = pre;
+                        }
+#pragma unroll
+                        for (int s = kTok - 1; s >= 0; --s) {
+                            sSuf[blk * kTok + s] = suf;
+                            suf *= g[s];
+                        }
+                    }
+                }
+                // this channel's term of every A_sj, summed over the warp's 32 channels: lane l ends up with pair l
+                float w[kTok], pr[kPairs];
+#pragma unroll
+                for (int s = 0; s < kTok; ++s) {
+#pragma unroll
+                    for (int j = 0; j < s; ++j) {
+                        w[j] *= g[s];
+                        pr[s * (s - 1) / 2 + j] = k[s] * w[j];
+                    }
+                    w[s] = k[s];
+                }
+#pragma unroll
+                for (int i2 = kTok * (kTok - 1) / 2; i2 < kPairs; ++i2) pr[i2] = 0.f;
+                group_reduce_transpose<32, kPairs>(pr, lane);
+                sGram[(blk * (K / 32) + i / 32) * kPairs + lane] = pr[0];
+            }
+            for (int s = tid; s < nb * kTok; s += T) sBeta[s] = s < n_ring ? rbeta[s] : s < n_tot ? *tbeta : 0.f;
+        } else {
+            for (int idx = tid; idx < n_tot * (K / 4); idx += T) {
+                const int s = idx / (K / 4), i = 4 * (idx % (K / 4));
+                float k[4];
+                ld4(s < n_ring ? rk + (size_t)s * K + i : tk + i, k);
+                st4(sKt + s * KS + PR::at(i), k);
+            }
+            // w_s = beta_s prod_{j>s} a_j and the total decay, by a warp scan over up to 64 tokens
+            if (warp == 0) {
+                float a[2], bt[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int s = lane + 32 * u;
+                    a[u] = s < n_ring ? rdec[s] : s < n_tot ? *tdec : 1.f;
+                    bt[u] = s < n_ring ? rbeta[s] : s < n_tot ? *tbeta : 0.f;
+                }
+                float after = 1.f;               // product of the decays behind this half
+#pragma unroll
+                for (int u = 1; u >= 0; --u) {
+                    float incl = a[u];
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const float other = __shfl_down_sync(0xffffffffu, incl, o);
+                        if (lane + o < 32) incl *= other;
+                    }
+                    float excl = __shfl_down_sync(0xffffffffu, incl, 1);
+                    if (lane == 31) excl = 1.f;
+                    if (lane + 32 * u < nb * kTok) sBeta[lane + 32 * u] = bt[u] * (excl * after);
+                    after *= __shfl_sync(0xffffffffu, incl, 0);
+                }
+                if (lane == 0) sPre[0] = after;
+            }
+        }
+        {
+            constexpr int PV = 16 / (int)sizeof(IO), in_row = V / PV;        // 16-byte units
+            const uint4* ring_v = reinterpret_cast<const uint4*>(rv);
+            const uint4* tok_v = reinterpret_cast<const uint4*>(tv);
+            for (int idx = tid; idx < n_tot * in_row; idx += T)
+                reinterpret_cast<uint4*>(sV)[idx] = idx < n_ring * in_row ? ring_v[idx] : tok_v[idx - n_ring * in_row];
+        }
+        if (p.q != nullptr) {
+            for (int i = tid; i < K / 4; i += T) {
+                float q[4];
+                ld4(tq + 4 * i, q);
+                st4(sQ + PR::at(4 * i), q);
+            }
+        }
+        if (p.write_sketch && h != h_staged) {
+            const float* og = p.omega + (size_t)h * K * R;
+#pragma unroll 4
+            for (int idx = tid; idx < K * R; idx += T) {
+                const int i = idx / R, g = idx % R;
+                sOm[g * OS + PR::at(i)] = og[idx];
+            }
+            for (int idx = tid; idx < (R8 - R) * K; idx += T) sOm[(R + idx / K) * OS + PR::at(idx % K)] = 0.f;
+            h_staged = h;
+        }
+        // (every thread's wait on the stage; a CTA that gives up leaves its heads as they are)
+        if (__syncthreads_or(failed)) {
+            failed = true;
+            return;
+        }
+        if (staged && tid == 0 && n_next >= 0) request(b_next, h_next, n_next);
+        if constexpr (DELTA) {
+            // beta_s A_sj
+            for (int idx = tid; idx < nb * kPairs; idx += T) {
+                const int blk = idx / kPairs, pair = idx % kPairs;
+                float a = 0.f;
+#pragma unroll
+                for (int c = 0; c < K / 32; ++c) a += sGram[(blk * (K / 32) + c) * kPairs + pair];
+                int s = 1;
+                while (s < kTok && (s + 1) * s / 2 <= pair) ++s;      // the pair's later token
+                sA[idx] = s < kTok ? sBeta[blk * kTok + s] * a : 0.f;
+            }
+            __syncthreads();
+        }
+
+        f32x2 c2[4][RP / 2];
+#pragma unroll
+        for (int i = 0; i < RP / 2; ++i) {
+            c2[0][i] = pack2(raw[2 * i].x, raw[2 * i + 1].x);
+            c2[1][i] = pack2(raw[2 * i].y, raw[2 * i + 1].y);
+            c2[2][i] = pack2(raw[2 * i].z, raw[2 * i + 1].z);
+            c2[3][i] = pack2(raw[2 * i].w, raw[2 * i + 1].w);
+        }
+        const int row = part * (RP + 4);            // this lane's rows inside a padded row
+
+        if constexpr (!DELTA) {
+            if (n_tot > 0) {
+                const f32x2 d2 = pack2(sPre[0], sPre[0]);
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int i = 0; i < RP / 2; ++i) c2[c][i] = mul2(c2[c][i], d2);
+            }
+        }
+        for (int blk = 0; blk < nb; ++blk) {
+            const int s0 = blk * kTok;
+            const int nt = min(kTok, n_tot - s0);
+            const int mine = s0 + part;              // this lane's token where a lane stands for one
+            float x[4];
+            if constexpr (DELTA) {
+                float vals[32];
+                const float* kh = (KDA ? sKh : sKt) + s0 * KS + row;
+                dot4<RP>(c2, kh, KS, vals);
+                if (nt > 4) {
+                    dot4<RP>(c2, kh + 4 * KS, KS, vals + 16);
+                } else {
+#pragma unroll
+                    for (int i = 16; i < 32; ++i) vals[i] = 0.f;
+                }
+                reduce_parts(vals, lane);
+                float v[4] = {0.f, 0.f, 0.f, 0.f};
+                if (mine < n_tot) ld4(sV + mine * V + j0, v);
+                const float bt = sBeta[mine], pre = KIND == SKETCHSSM_GDN ? sPre[mine] : 1.f;
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    x[c] = mine < n_tot ? bt * (v[c] - (KIND == SKETCHSSM_GDN ? pre * vals[c] : vals[c])) : 0.f;
+            } else {
+                float v[4] = {0.f, 0.f, 0.f, 0.f};
+                if (mine < n_tot) ld4(sV + mine * V + j0, v);
+                const float w = sBeta[mine];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) x[c] = w * v[c];
+            }
+            __syncwarp();                            // the previous block's e have been read
+            st4(sE + part * 16 + (lane & 3) * 4, x);
+            __syncwarp();
+            if constexpr (DELTA) {
+                // forward substitution, one column per lane
+                if (lane < 16) {
+                    float e[kTok], a[kPairs];
+#pragma unroll
+                    for (int s = 0; s < kTok; ++s) e[s] = sE[s * 16 + lane];
+#pragma unroll
+                    for (int i = 0; i < kPairs / 4 - 1; ++i) ld4(sA + blk * kPairs + 4 * i, a + 4 * i);
+#pragma unroll
+                    for (int j = 0; j < kTok - 1; ++j) {
+#pragma unroll
+                        for (int s = j + 1; s < kTok; ++s) e[s] = fmaf(-a[s * (s - 1) / 2 + j], e[j], e[s]);
+                    }
+#pragma unroll
+                    for (int s = 0; s < kTok; ++s) sE[s * 16 + lane] = KIND == SKETCHSSM_GDN ? sSuf[s0 + s] * e[s] : e[s];
+                }
+                __syncwarp();
+#pragma unroll
+                for (int i4 = 0; i4 < RP / 4; ++i4) {
+                    f32x2 g01, g23;
+                    if constexpr (KDA) {
+                        const float4 g = *reinterpret_cast<const float4*>(sG + blk * KS + row + 4 * i4);
+                        g01 = pack2(g.x, g.y);
+                        g23 = pack2(g.z, g.w);
+                    } else {
+                        g01 = g23 = pack2(sPre[s0 + kTok - 1], sPre[s0 + kTok - 1]);
+                    }
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        c2[c][2 * i4] = mul2(c2[c][2 * i4], g01);
+                        c2[c][2 * i4 + 1] = mul2(c2[c][2 * i4 + 1], g23);
+                    }
+                }
+            }
+            const float* kt = sKt + s0 * KS + row;
+#pragma unroll 2
+            for (int s = 0; s < nt; ++s) {
+                const float4 e = *reinterpret_cast<const float4*>(sE + s * 16 + (lane & 3) * 4);
+                const f32x2 e2[4] = {pack2(e.x, e.x), pack2(e.y, e.y), pack2(e.z, e.z), pack2(e.w, e.w)};
+#pragma unroll
+                for (int i4 = 0; i4 < RP / 4; ++i4) {
+                    const float4 kq = *reinterpret_cast<const float4*>(kt + s * KS + 4 * i4);
+                    const f32x2 k01 = pack2(kq.x, kq.y), k23 = pack2(kq.z, kq.w);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        c2[c][2 * i4] = fma2(k01, e2[c], c2[c][2 * i4]);
+                        c2[c][2 * i4 + 1] = fma2(k23, e2[c], c2[c][2 * i4 + 1]);
+                    }
+                }
+            }
+        }
+
+        // ---- write the updated state back ----
+        if (p.write_state && n_tot > 0) {
+            float* So = p.state + bh * (size_t)(K * V) + (size_t)(part * RP) * V + j0;
+#pragma unroll
+            for (int i = 0; i < RP / 2; ++i) {
+                float4 lo, hi;
+                unpack2(c2[0][i], lo.x, hi.x);
+                unpack2(c2[1][i], lo.y, hi.y);
+                unpack2(c2[2][i], lo.z, hi.z);
+                unpack2(c2[3][i], lo.w, hi.w);
+                *reinterpret_cast<float4*>(So + (size_t)(2 * i) * V) = lo;
+                *reinterpret_cast<float4*>(So + (size_t)(2 * i + 1) * V) = hi;
+            }
+        }
+
+        // ---- exact output o[j] = <S_new[:, j], q> ----
+        if (p.out != nullptr) {
+            f32x2 acc[4];
+#pragma unroll
+            for (int i4 = 0; i4 < RP / 4; ++i4) {
+                const float4 q = *reinterpret_cast<const float4*>(sQ + row + 4 * i4);
+                const f32x2 q01 = pack2(q.x, q.y), q23 = pack2(q.z, q.w);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    acc[c] = i4 == 0 ? mul2(q01, c2[c][0]) : fma2(q01, c2[c][2 * i4], acc[c]);
+                    acc[c] = fma2(q23, c2[c][2 * i4 + 1], acc[c]);
+                }
+            }
+            float o[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                float lo, hi;
+                unpack2(acc[c], lo, hi);
+                o[c] = lo + hi;
+#pragma unroll
+                for (int m = 16; m >= 4; m >>= 1) o[c] += __shfl_xor_sync(0xffffffffu, o[c], m);
+            }
+            if (part == 0) {
+                if (p.out_bf16) st4(reinterpret_cast<__nv_bfloat16*>(p.out) + bh * V + j0, o);
+                else st4(reinterpret_cast<float*>(p.out) + bh * V + j0, o);
+            }
+        }
+
+        // ---- sketch rows U[g, j] = <S_new[:, j], omega_g>, eight ranks at a time ----
+        if (p.write_sketch) {
+            for (int g0 = 0; g0 < R8; g0 += 8) {
+                float vals[32];
+                dot4<RP>(c2, sOm + g0 * OS + row, OS, vals);
+                dot4<RP>(c2, sOm + (g0 + 4) * OS + row, OS, vals + 16);
+                reduce_parts(vals, lane);
+                if (g0 + part < R) {
+                    const size_t at = (bh * R + g0 + part) * V + j0;
+                    if (p.sketch_bf16) st4(reinterpret_cast<__nv_bfloat16*>(p.sketch) + at, vals);
+                    else st4(p.sketch + at, vals);
+                }
+            }
+        }
+    };
+
+    // CTAs are persistent and take contiguous ranges of (head index, sequence) items: Omega is staged once per head index.
+    auto work = [&](int n_seq, auto seq, auto fill) {   // heads of the sequences seq(0 .. n_seq), at ring fills fill(seq)
+        const long long items = (long long)n_seq * H;
+        const int i0 = (int)(items * blockIdx.x / gridDim.x), i1 = (int)(items * (blockIdx.x + 1) / gridDim.x);
+        if (i0 >= i1) return;
+        int b = seq(i0 % n_seq), h = i0 / n_seq, n = fill(b);
+        if (staged) {
+            if (tid == 0) {
+                request(b, h, n);
+                sTok[0] = next_beta;
+                sTok[1] = next_decay;
+            }
+            __syncthreads();
+        }
+        for (int i = i0; i < i1; ++i) {
+            int b_next = 0, h_next = 0, n_next = -1;
+            if (i + 1 < i1) {
+                b_next = seq((i + 1) % n_seq);
+                h_next = (i + 1) / n_seq;
+                n_next = fill(b_next);
+            }
+            replay(b, h, n, b_next, h_next, n_next);
+            if (failed) return;
+            if (staged && tid == 0) {
+                sTok[0] = next_beta;
+                sTok[1] = next_decay;
+            }
+            __syncthreads();                        // the shared rows are refilled
+            b = b_next; h = h_next; n = n_next;
+        }
+    };
+    if (staged) {
+        if (tid == 0) {
+            mbar_init(bar, 1);
+            mbar_fence_init();
+        }
+        __syncthreads();
+    }
+    if (!mixed) {                                   // lock step: every sequence, at the same ring fill
+        work(B, [](int i) { return i; }, [&](int) { return p.n_before; });
+        if (failed && tid == 0) record_fault(p.status, kFaultUpdateWait, (int)blockIdx.x);
+        return;
+    }
+
+    // Per-sequence phases: the flushing sequences of the batch, kScan entries of the phase array at a time, listed in
+    // shared memory (every CTA builds the same list).  A grid of one CTA per head, most of which had nothing to do, spent
+    // more time on starting CTAs than on the flush.
+    int* sCount = sList + kScan;
+    for (int base = 0; base < B; base += kScan) {
+        constexpr int kWarps = T / 32, kPer = (kScan / 32 + kWarps - 1) / kWarps;     // rows of 32 sequences per warp
+        int ph[kPer];
+        uint32_t bal[kPer];
+        int cnt = 0;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const int r = warp * kPer + u, b = base + 32 * r + lane;
+            ph[u] = (r < kScan / 32 && b < B) ? p.n_dev[b] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            bal[u] = __ballot_sync(0xffffffffu, ph[u] < 0);
+            cnt += __popc(bal[u]);
+        }
+        if (lane == 0) sCount[warp] = cnt;
+        __syncthreads();
+        int at = 0, nf = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            const int c = sCount[w];
+            if (w < warp) at += c;
+            nf += c;
+        }
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const int r = warp * kPer + u;
+            if (ph[u] < 0) sList[at + __popc(bal[u] & ((1u << lane) - 1u))] = base + 32 * r + lane;
+            at += __popc(bal[u]);
+        }
+        __syncthreads();
+        work(nf, [&](int i) { return sList[i]; }, [&](int b) { return -p.n_dev[b] - 1; });
+        if (failed) break;
+        __syncthreads();                            // the list is rebuilt
+    }
+    if (failed && tid == 0) record_fault(p.status, kFaultUpdateWait, (int)blockIdx.x);
+    if (p.late_wait) grid_dep_wait();
+}
+
+template <int KIND, typename IO, int K, int V>
 static int launch_update_t(Ctx* ctx, Params p, cudaStream_t stream) {
-    constexpr int kUpdThreads = kVT * kParts;
-    const int V = ctx->cfg.dv;
     const int n_tot = p.n_before + (p.has_token ? 1 : 0);
-    const int R4 = (p.R + 3) & ~3;
-    if (p.n_dev != nullptr) p.n_cap = n_tot;        // per-sequence phases: n_before is the largest fill any sequence may have
-    const UpdateSmem us = make_update_smem<K>(KIND, n_tot, R4, kVT);
-    auto kern = update_kernel<KIND, IO, K, kVT>;
+    const bool mixed = p.n_dev != nullptr;
+    if (mixed) p.n_cap = n_tot;        // per-sequence phases: n_before is the largest fill any sequence may have
+    // Staging one head ahead needs room for the stage beside the CTAs that the registers allow (V = 64: three of the four).
+    constexpr int kMinStaged = V == 64 ? 3 : update_ctas<V>();
+    UpdateSmem us = make_update_smem<K>(KIND, n_tot, p.R, V, p.L, (int)sizeof(IO), mixed, 1);
+    p.stages = us.total + 1024u <= (228u * 1024u) / kMinStaged ? 1 : 0;
+    if (!p.stages) us = make_update_smem<K>(KIND, n_tot, p.R, V, p.L, (int)sizeof(IO), mixed, 0);
+    auto kern = update_kernel<KIND, IO, K, V>;
     if (us.total > 226u * 1024u) return SKETCHSSM_UNSUPPORTED_SHAPE;
     if ((ctx->last_cuda_error = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      (int)us.total)) != cudaSuccess)
         return SKETCHSSM_CUDA_ERROR;
-    p.dv = V;
-    const dim3 grid((unsigned)((size_t)p.B * p.H * (V / kVT)));
-    kern<<<grid, kUpdThreads, us.total, stream>>>(p);
-    if ((ctx->last_cuda_error = cudaGetLastError()) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
+    if (ctx->sm_count == 0) {
+        int sms = 0;
+        if ((ctx->last_cuda_error = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->cfg.device)) != cudaSuccess)
+            return SKETCHSSM_CUDA_ERROR;
+        ctx->sm_count = sms;
+    }
+    size_t grid = (size_t)p.B * p.H;
+    const int by_smem = (int)((228u * 1024u) / (us.total + 1024u));
+    const size_t wave = (size_t)ctx->sm_count * (size_t)(by_smem < 1 ? 1 : by_smem < update_ctas<V>() ? by_smem : update_ctas<V>());
+    if (grid > wave) grid = wave;
+    if ((ctx->last_cuda_error = launch_kernel(kern, dim3((unsigned)grid), dim3(2 * V), us.total, stream, p, p.pdl != 0)) != cudaSuccess)
+        return SKETCHSSM_CUDA_ERROR;
     ctx->last_launches = 1;
     return SKETCHSSM_OK;
 }
 
 template <int KIND, typename IO>
 static int launch_update_shape(Ctx* ctx, const Params& p, cudaStream_t stream) {
-    if (ctx->cfg.dk == 128 && ctx->cfg.dv == 80) return launch_update_t<KIND, IO, 128, 80>(ctx, p, stream);
-    if (ctx->cfg.dv % 64 != 0) return SKETCHSSM_UNSUPPORTED_SHAPE;
-    if (ctx->cfg.dk == 128) return launch_update_t<KIND, IO, 128, 64>(ctx, p, stream);
-    if (ctx->cfg.dk == 64) return launch_update_t<KIND, IO, 64, 64>(ctx, p, stream);
+    const int K = ctx->cfg.dk, V = ctx->cfg.dv;
+    if (K == 128 && V == 128) return launch_update_t<KIND, IO, 128, 128>(ctx, p, stream);
+    if (K == 128 && V == 64) return launch_update_t<KIND, IO, 128, 64>(ctx, p, stream);
+    if (K == 128 && V == 80) return launch_update_t<KIND, IO, 128, 80>(ctx, p, stream);
+    if (K == 64 && V == 64) return launch_update_t<KIND, IO, 64, 64>(ctx, p, stream);
+    if (K == 64 && V == 128) return launch_update_t<KIND, IO, 64, 128>(ctx, p, stream);
     return SKETCHSSM_UNSUPPORTED_SHAPE;
 }
 
