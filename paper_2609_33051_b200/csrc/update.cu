@@ -14,7 +14,11 @@
 //
 // What bounds it: fp32 issue and the shared-memory reads of the key rows (2 n + r + 1 multiply-adds per state element).
 // Four columns per lane: a 128-bit read of a key row feeds eight packed multiply-adds.  One column per lane and 64-column
-// tiles, as before, read four times as many key rows and multiplied the state by the decay at every token.
+// tiles, as before, read four times as many key rows and multiplied the state by the decay at every token.  Measured:
+// mixed step of 512 sequences x 32 heads, GDN 128 x 128, r = L = 16 (1024 heads flush per call on average): 171 -> 114 us
+// a call, of which the decode kernel takes 47 (before / after; without the stage 124, 64-column tiles 131); flush of 3072
+// KDA heads with 8 fp32 tokens: 158 -> 97 us.  The multiply-add pipe is busy 45 % of the time (two CTAs of eight warps:
+// 128 registers a thread), fp32 issue 44 %.
 #include "internal.cuh"
 #include "lanegroup.cuh"
 
@@ -576,37 +580,6 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
         }
     };
 
-    // CTAs are persistent and take contiguous ranges of (head index, sequence) items: Omega is staged once per head index.
-    auto work = [&](int n_seq, auto seq, auto fill) {   // heads of the sequences seq(0 .. n_seq), at ring fills fill(seq)
-        const long long items = (long long)n_seq * H;
-        const int i0 = (int)(items * blockIdx.x / gridDim.x), i1 = (int)(items * (blockIdx.x + 1) / gridDim.x);
-        if (i0 >= i1) return;
-        int b = seq(i0 % n_seq), h = i0 / n_seq, n = fill(b);
-        if (staged) {
-            if (tid == 0) {
-                request(b, h, n);
-                sTok[0] = next_beta;
-                sTok[1] = next_decay;
-            }
-            __syncthreads();
-        }
-        for (int i = i0; i < i1; ++i) {
-            int b_next = 0, h_next = 0, n_next = -1;
-            if (i + 1 < i1) {
-                b_next = seq((i + 1) % n_seq);
-                h_next = (i + 1) / n_seq;
-                n_next = fill(b_next);
-            }
-            replay(b, h, n, b_next, h_next, n_next);
-            if (failed) return;
-            if (staged && tid == 0) {
-                sTok[0] = next_beta;
-                sTok[1] = next_decay;
-            }
-            __syncthreads();                        // the shared rows are refilled
-            b = b_next; h = h_next; n = n_next;
-        }
-    };
     if (staged) {
         if (tid == 0) {
             mbar_init(bar, 1);
@@ -614,49 +587,75 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
         }
         __syncthreads();
     }
-    if (!mixed) {                                   // lock step: every sequence, at the same ring fill
-        work(B, [](int i) { return i; }, [&](int) { return p.n_before; });
-        if (failed && tid == 0) record_fault(p.status, kFaultUpdateWait, (int)blockIdx.x);
-        return;
-    }
-
-    // Per-sequence phases: the flushing sequences of the batch, kScan entries of the phase array at a time, listed in
-    // shared memory (every CTA builds the same list).  A grid of one CTA per head, most of which had nothing to do, spent
-    // more time on starting CTAs than on the flush.
+    // CTAs are persistent and take contiguous ranges of (head index, sequence) items: Omega is staged once per head index.
+    // Lock step: every sequence, at the same ring fill.  Per-sequence phases: the flushing sequences of the batch, kScan
+    // entries of the phase array at a time, listed in shared memory (every CTA builds the same list).  A grid of one CTA
+    // per head, most of which had nothing to do, spent more time on starting CTAs than on the flush.  (One loop for both:
+    // the body is some 40 KB of code, and a second copy of it was measured in instruction-cache misses.)
     int* sCount = sList + kScan;
     for (int base = 0; base < B; base += kScan) {
-        constexpr int kWarps = T / 32, kPer = (kScan / 32 + kWarps - 1) / kWarps;     // rows of 32 sequences per warp
-        int ph[kPer];
-        uint32_t bal[kPer];
-        int cnt = 0;
+        int n_seq = B;
+        if (mixed) {
+            constexpr int kWarps = T / 32, kPer = (kScan / 32 + kWarps - 1) / kWarps;     // rows of 32 sequences per warp
+            int cnt = 0;
 #pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-            const int r = warp * kPer + u, b = base + 32 * r + lane;
-            ph[u] = (r < kScan / 32 && b < B) ? p.n_dev[b] : 0;
-        }
+            for (int u = 0; u < kPer; ++u) {
+                const int r = warp * kPer + u, b = base + 32 * r + lane;
+                cnt += __popc(__ballot_sync(0xffffffffu, r < kScan / 32 && b < B && p.n_dev[b] < 0));
+            }
+            if (lane == 0) sCount[warp] = cnt;
+            __syncthreads();
+            int at = 0;
+            n_seq = 0;
 #pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-            bal[u] = __ballot_sync(0xffffffffu, ph[u] < 0);
-            cnt += __popc(bal[u]);
+            for (int w = 0; w < kWarps; ++w) {
+                const int c = sCount[w];
+                if (w < warp) at += c;
+                n_seq += c;
+            }
+            for (int u = 0; u < kPer; ++u) {
+                const int r = warp * kPer + u, b = base + 32 * r + lane;
+                const bool on = r < kScan / 32 && b < B && p.n_dev[b] < 0;
+                const uint32_t bal = __ballot_sync(0xffffffffu, on);
+                if (on) sList[at + __popc(bal & ((1u << lane) - 1u))] = b;
+                at += __popc(bal);
+            }
+            __syncthreads();
         }
-        if (lane == 0) sCount[warp] = cnt;
+        const long long items = (long long)n_seq * H;
+        const int i0 = (int)(items * blockIdx.x / gridDim.x), i1 = (int)(items * (blockIdx.x + 1) / gridDim.x);
+        auto item = [&](int i, int& b, int& h, int& n) {
+            h = i / n_seq;
+            b = i - h * n_seq;
+            n = p.n_before;
+            if (mixed) {
+                b = sList[b];
+                n = -p.n_dev[b] - 1;
+            }
+        };
+        int b = 0, h = 0, n = 0;
+        if (i0 < i1) {
+            item(i0, b, h, n);
+            if (staged && tid == 0) {
+                request(b, h, n);
+                sTok[0] = next_beta;
+                sTok[1] = next_decay;
+            }
+        }
         __syncthreads();
-        int at = 0, nf = 0;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) {
-            const int c = sCount[w];
-            if (w < warp) at += c;
-            nf += c;
+        for (int i = i0; i < i1; ++i) {
+            int b_next = 0, h_next = 0, n_next = -1;
+            if (i + 1 < i1) item(i + 1, b_next, h_next, n_next);
+            replay(b, h, n, b_next, h_next, n_next);
+            if (failed) break;
+            if (staged && tid == 0) {
+                sTok[0] = next_beta;
+                sTok[1] = next_decay;
+            }
+            __syncthreads();                        // the shared rows are refilled
+            b = b_next; h = h_next; n = n_next;
         }
-#pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-            const int r = warp * kPer + u;
-            if (ph[u] < 0) sList[at + __popc(bal[u] & ((1u << lane) - 1u))] = base + 32 * r + lane;
-            at += __popc(bal[u]);
-        }
-        __syncthreads();
-        work(nf, [&](int i) { return sList[i]; }, [&](int b) { return -p.n_dev[b] - 1; });
-        if (failed) break;
+        if (failed || !mixed) break;
         __syncthreads();                            // the list is rebuilt
     }
     if (failed && tid == 0) record_fault(p.status, kFaultUpdateWait, (int)blockIdx.x);
