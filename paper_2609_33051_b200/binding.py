@@ -100,8 +100,8 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     return lib
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()       # (the declared argument types make the C pointer of it)
 
 
 class SketchSSM:
@@ -181,9 +181,10 @@ class SketchSSM:
             raise SketchSSMError(fn, rc, text)
 
     @staticmethod
-    def _stream(stream) -> ctypes.c_void_p:
-        s = torch.cuda.current_stream() if stream is None else stream
-        return ctypes.c_void_p(s.cuda_stream)
+    def _stream(stream) -> int:
+        """The stream's handle; None: the current stream of the current device (read without building a Stream object,
+        which costs as much as the rest of a call's marshalling)."""
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
 
     def new_output(self) -> torch.Tensor:
         return torch.empty(self.B, self.H, self.V, dtype=TORCH_DTYPE[self.out], device=self.device)
@@ -205,13 +206,15 @@ class SketchSSM:
                      flags: int = 0, stream=None):
         rc = self.lib.sketchssm_state_update(self._ctx, n_before, _ptr(q), _ptr(k), _ptr(v), _ptr(beta),
                                              _ptr(decay), _ptr(out), flags, self._stream(stream))
-        self._check("sketchssm_state_update", rc)
+        if rc:
+            self._check("sketchssm_state_update", rc)
         return out
 
     def decode_step(self, n_before: int, q, k, v, beta, decay, out, flags: int = 0, stream=None):
         rc = self.lib.sketchssm_decode_step(self._ctx, n_before, _ptr(q), _ptr(k), _ptr(v), _ptr(beta),
                                             _ptr(decay), _ptr(out), flags, self._stream(stream))
-        self._check("sketchssm_decode_step", rc)
+        if rc:
+            self._check("sketchssm_decode_step", rc)
         return out
 
     def decode_step_static(self, n_before: int, q, k, v, beta, decay, out, flags: int = 0, stream=None):
@@ -219,7 +222,8 @@ class SketchSSM:
         scratch; its kernel-to-kernel hand-off uses the library's fixed 4 MiB device array."""
         rc = self.lib.sketchssm_decode_step_static(self._ctx, n_before, _ptr(q), _ptr(k), _ptr(v), _ptr(beta),
                                                    _ptr(decay), _ptr(out), flags, self._stream(stream))
-        self._check("sketchssm_decode_step_static", rc)
+        if rc:
+            self._check("sketchssm_decode_step_static", rc)
         return out
 
     def step_mixed(self, phase: torch.Tensor, q, k, v, beta, decay, out, stream=None):
@@ -228,13 +232,15 @@ class SketchSSM:
         assert phase.dtype == torch.int32 and phase.is_cuda and phase.numel() == self.B
         rc = self.lib.sketchssm_step_mixed(self._ctx, _ptr(phase), _ptr(q), _ptr(k), _ptr(v), _ptr(beta), _ptr(decay),
                                            _ptr(out), 0, self._stream(stream))
-        self._check("sketchssm_step_mixed", rc)
+        if rc:
+            self._check("sketchssm_step_mixed", rc)
         return out
 
     def full_read_decode(self, n_before: int, q, k, v, beta, decay, out, flags: int = 0, stream=None):
         rc = self.lib.sketchssm_full_read_decode(self._ctx, n_before, _ptr(q), _ptr(k), _ptr(v), _ptr(beta),
                                                  _ptr(decay), _ptr(out), flags, self._stream(stream))
-        self._check("sketchssm_full_read_decode", rc)
+        if rc:
+            self._check("sketchssm_full_read_decode", rc)
         return out
 
     def new_token_buffers(self, pinned_host: bool = False):
@@ -255,7 +261,8 @@ class SketchSSM:
         rc = self.lib.sketchssm_step_host(self._ctx, op, n_before, _ptr(host["q"]), _ptr(host["k"]), _ptr(host["v"]),
                                           _ptr(host["beta"]), _ptr(host["decay"]), _ptr(host["out"]),
                                           ctypes.byref(st), flags, self._stream(stream))
-        self._check("sketchssm_step_host", rc)
+        if rc:
+            self._check("sketchssm_step_host", rc)
         return host["out"]
 
     def selftest_wait_timeout(self, poll_limit: int = 2048, where: int = 99, stream=None):

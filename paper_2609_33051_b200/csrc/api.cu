@@ -194,6 +194,8 @@ int sketchssm_create(const sketchssm_config* cfg, sketchssm_ctx** out) {
     c->last_launches = 0;
     c->sketch_fresh = true;
     c->last_cuda_error = cudaSuccess;
+    for (const void*& k : c->unlocked) k = nullptr;
+    c->unlocked_next = 0;
     c->tune_batches_per_cta = 0;
     c->tune_stages = 0;
     c->tune_warps_per_cta = 0;

@@ -622,13 +622,8 @@ static int launch_coef_kv(Ctx* ctx, const Params& p, cudaStream_t stream) {
     const int m = exact ? p.R : (p.R < p.pivots ? p.R : p.pivots);
     const CoefSmem sm = make_coef_smem(K, V, p.R, m);
     auto kern = exact ? coef_map_kernel<K, V, 1, 4> : (m <= 4 ? coef_map_kernel<K, V, 0, 4> : coef_map_kernel<K, V, 0, 8>);
-    if (sm.total > 48u * 1024u) {
-        if ((ctx->last_cuda_error = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm.total)) != cudaSuccess)
-            return SKETCHSSM_CUDA_ERROR;
-    }
     // (shared memory carved out for as many CTAs per SM as the registers allow; the kernel makes little use of L1)
-    if ((ctx->last_cuda_error = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
-        return SKETCHSSM_CUDA_ERROR;
+    if ((ctx->last_cuda_error = unlock_smem(ctx, kern, true)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     const size_t heads = (size_t)p.B * p.H;
     kern<<<dim3((unsigned)heads), dim3(kCoefThreads), sm.total, stream>>>(p);
     if ((ctx->last_cuda_error = cudaGetLastError()) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;

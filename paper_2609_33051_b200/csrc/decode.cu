@@ -725,9 +725,7 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
     }
     if (best_nw == 0) return SKETCHSSM_UNSUPPORTED_SHAPE;
     const DecodeSmem d = make_decode_smem(K, p.R, best_nw, p.full_read, p.coef_per_seq, sl.total);
-    if ((ctx->last_cuda_error = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)d.total)) != cudaSuccess)
-        return SKETCHSSM_CUDA_ERROR;
+    if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     long long grid = (long long)ctx->sm_count * best_ctas;
     const long long total = (long long)p.B * p.H;
     if (p.batches_per_cta > 0) grid = (total + p.batches_per_cta - 1) / p.batches_per_cta;   // explicit items per CTA

@@ -430,9 +430,7 @@ static int launch_weights_t(Ctx* ctx, Params p, cudaStream_t stream) {
     p.stages = best_st;
     const WSmem d = make_wsmem(K, RP, best_nw * HPW, best_st, p.full_read, sl.total);
     auto kern = decode_weights_kernel<KIND, IO, K, LPH, RP>;
-    if ((ctx->last_cuda_error = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)d.total)) != cudaSuccess)
-        return SKETCHSSM_CUDA_ERROR;
+    if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     long long grid = (long long)ctx->sm_count * best_ctas;
     const long long total = (long long)p.B * p.H;
     const long long min_items = (long long)best_nw * HPW;

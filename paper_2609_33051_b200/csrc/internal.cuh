@@ -33,6 +33,11 @@ struct Ctx {
     int last_launches;
     bool sketch_fresh;  // the last hot-path call on this context was a state update that wrote the sketch (or none was made yet)
     cudaError_t last_cuda_error;  // of the most recent failing runtime call
+    // Kernels whose dynamic shared memory this context has already had unlocked: a kernel needs that once per device, and
+    // asking again at every launch cost the host a good part of a launch.
+    static constexpr int kUnlockSlots = 16;
+    const void* unlocked[kUnlockSlots];
+    int unlocked_next;
 };
 
 // Arguments common to the three kernels.
@@ -108,6 +113,26 @@ int launch_update_tc_ws_kda(Ctx* ctx, const Params& p, cudaStream_t stream); // 
 // device helpers
 // ---------------------------------------------------------------------------------------------
 #ifdef __CUDACC__
+
+// Allow a kernel all the dynamic shared memory the device has (always the same amount, so that contexts that launch the
+// same kernel with different sizes do not undo each other's), and optionally ask for the largest carveout.
+template <typename Kern>
+inline cudaError_t unlock_smem(Ctx* ctx, Kern kernel, bool max_carveout = false) {
+    const void* kern = reinterpret_cast<const void*>(kernel);
+    for (const void* k : ctx->unlocked)
+        if (k == kern) return cudaSuccess;
+    cudaFuncAttributes fa;
+    int optin = 0;
+    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->cfg.device);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+    if (e == cudaSuccess && max_carveout)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    ctx->unlocked[ctx->unlocked_next] = kern;
+    ctx->unlocked_next = (ctx->unlocked_next + 1) % Ctx::kUnlockSlots;
+    return cudaSuccess;
+}
 
 // Launch with (or without) the programmatic-stream-serialization attribute.
 template <typename Kern>

@@ -674,9 +674,7 @@ static int launch_update_t(Ctx* ctx, Params p, cudaStream_t stream) {
     if (!p.stages) us = make_update_smem<K>(KIND, n_tot, p.R, V, p.L, (int)sizeof(IO), mixed, 0);
     auto kern = update_kernel<KIND, IO, K, V>;
     if (us.total > 226u * 1024u) return SKETCHSSM_UNSUPPORTED_SHAPE;
-    if ((ctx->last_cuda_error = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)us.total)) != cudaSuccess)
-        return SKETCHSSM_CUDA_ERROR;
+    if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     if (ctx->sm_count == 0) {
         int sms = 0;
         if ((ctx->last_cuda_error = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->cfg.device)) != cudaSuccess)

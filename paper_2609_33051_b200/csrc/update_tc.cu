@@ -418,9 +418,7 @@ int launch_update_tc(Ctx* ctx, const Params& p_in, cudaStream_t stream) {
     long long grid = (long long)ctx->sm_count * ctas;
     if (grid > n_tiles) grid = n_tiles;
     auto kern = c.dv == 128 ? update_tc_mamba2_kernel<128> : update_tc_mamba2_kernel<64>;
-    if ((ctx->last_cuda_error = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)sm.total)) != cudaSuccess)
-        return SKETCHSSM_CUDA_ERROR;
+    if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     if ((ctx->last_cuda_error = launch_kernel(kern, dim3((unsigned)grid), dim3(kTcThreads), sm.total, stream, p, p.pdl != 0)) != cudaSuccess)
         return SKETCHSSM_CUDA_ERROR;
     ctx->last_launches = 1;

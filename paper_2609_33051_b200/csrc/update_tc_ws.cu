@@ -808,9 +808,7 @@ int launch_update_tc_ws(Ctx* ctx, const Params& p_in, cudaStream_t stream) {
     if (grid > n_tiles) grid = n_tiles;
     auto kern = NP > 32 ? (c.dv == 128 ? update_tc_ws_mamba2_kernel<128, true> : update_tc_ws_mamba2_kernel<64, true>)
                         : (c.dv == 128 ? update_tc_ws_mamba2_kernel<128, false> : update_tc_ws_mamba2_kernel<64, false>);
-    if ((ctx->last_cuda_error = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)sm.total)) != cudaSuccess)
-        return SKETCHSSM_CUDA_ERROR;
+    if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     if ((ctx->last_cuda_error = launch_kernel(kern, dim3((unsigned)grid), dim3(kWsThreads), sm.total, stream, p, p.pdl != 0)) != cudaSuccess)
         return SKETCHSSM_CUDA_ERROR;
     ctx->last_launches = 1;

@@ -1030,9 +1030,7 @@ static int launch_kda_pass(Ctx* ctx, const Params& p_in, cudaStream_t stream) {
     long long grid = (long long)ctx->sm_count;
     if (grid > n_tiles) grid = n_tiles;
     auto kern = update_tc_ws_kda_kernel;
-    if ((ctx->last_cuda_error = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)sm.total)) != cudaSuccess)
-        return SKETCHSSM_CUDA_ERROR;
+    if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     if ((ctx->last_cuda_error = launch_kernel(kern, dim3((unsigned)grid), dim3(kKThreads), sm.total, stream, p, p.pdl != 0)) != cudaSuccess)
         return SKETCHSSM_CUDA_ERROR;
     return SKETCHSSM_OK;
