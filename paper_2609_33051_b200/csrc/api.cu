@@ -95,6 +95,16 @@ int decode_params(sketchssm_ctx* ctx, int full_read, int n_before, const void* q
     return SKETCHSSM_OK;
 }
 
+int launch_decode(Ctx* ctx, const Params& p, cudaStream_t stream) {
+    const bool bf = ctx->cfg.io_dtype == SKETCHSSM_BF16;
+    switch (ctx->cfg.kind) {
+        case SKETCHSSM_MAMBA2: return bf ? launch_decode_group<0, 1>(ctx, p, stream) : launch_decode_group<0, 0>(ctx, p, stream);
+        case SKETCHSSM_GDN: return bf ? launch_decode_group<1, 1>(ctx, p, stream) : launch_decode_group<1, 0>(ctx, p, stream);
+        case SKETCHSSM_KDA: return bf ? launch_decode_group<2, 1>(ctx, p, stream) : launch_decode_group<2, 0>(ctx, p, stream);
+    }
+    return SKETCHSSM_INVALID_ARG;
+}
+
 // The flush kernel for this configuration: the warp-specialised tensor-core kernels where their shape limits allow,
 // the single-group tensor-core kernel for Mamba-2 ranks above 32, CUDA cores otherwise.
 int dispatch_update(sketchssm_ctx* ctx, const Params& p, cudaStream_t cs) {

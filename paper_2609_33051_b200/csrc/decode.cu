@@ -28,7 +28,7 @@ namespace {
 #define DEC_WAIT(bar, parity) mbar_wait_bounded(bar, parity)
 // parity of the sketch barrier's phase for the current head: with one rank for all heads both barriers advance together
 // (the ring barrier's parity has already been flipped when the sketch is waited for)
-#define PARB (GEN ? parB : (parA ^ 1u))
+#define PARB (ANY ? parB : (parA ^ 1u))
 
 struct StageLayout {
     uint32_t u_off, u_bytes;        // sketch U (sketch mode only)
@@ -89,13 +89,22 @@ __host__ __device__ inline DecodeSmem make_decode_smem(int K, int R, int nwarps,
 }  // namespace
 
 // RT: the sketch rank as a compile-time constant (loops over ranks unroll fully), or 0 for any rank.
-// GEN: 0 = one ring fill and one rank for every head of the launch (copy sizes are per-lane constants);
-//      1 = per-sequence phases and / or a per-head rank table (sizes follow the head);
-//      2 = 1 with the coefficient vector formed from projected erase vectors (delta-rule kinds).
-// UB: the sketch rows and the fixed coefficient map are stored as bfloat16 (a compile-time fact for the lean
-//     instantiation; the general ones read the flag of the launch).
-template <int KIND, typename IO, int K, int V, int RT, int GEN, bool UB = false>
-__global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 3 : 4) decode_kernel(const Params p) {
+// F: what the launch needs beyond one ring fill, one rank and one fp32 map for all heads, as compile-time facts:
+//   kSeq  per-sequence phases (sizes follow the sequence)        kPS  a coefficient map per (batch, head)
+//   kER   c_t from projected erase vectors (delta-rule kinds)    kUB  sketch and map stored as bfloat16
+//   kFull every head reads the full state (no sketch rows, no map)
+//   kAny  general: per-head ranks (rank 0: that head reads the full state), and kSeq / kPS / kUB as the launch says (kER
+//         stays a compile-time fact).
+// Every flag that is decided inside the loops over heads, ranks or slots costs the launches that do not use it: with the
+// full-read branch and the run-time flags out of the lean instantiations none of them spills, and the launches that had
+// to run the general one take (general -> own, r = L = 16, bfloat16 I/O): state-dependent bfloat16 map, Mamba-2 64-head
+// batch of 256, 33 -> 31 us; the same with erase vectors, GDN 32-head batch of 512, 53 -> 45 us; mixed step of that layer
+// 48 -> 46 us; V = 80 layer of 37 x 24 heads with two dense heads (prefetch below) 13 -> 10 us.
+constexpr int kSeq = 1, kPS = 2, kER = 4, kUB = 8, kAny = 16, kFull = 32;
+
+template <int KIND, typename IO, int K, int V, int RT, int F>
+__global__ void __launch_bounds__(256, ((F & ~(kUB | kFull)) || KIND != SKETCHSSM_MAMBA2) ? 3 : 4) decode_kernel(const Params p) {
+    constexpr bool ANY = (F & kAny) != 0, DYN = ANY || (F & kSeq) != 0, FULL = (F & kFull) != 0;
     constexpr int EK = K / 32;
     constexpr int EV = V % 32 == 0 ? V / 32 : 4;        // value elements per lane ...
     constexpr int VL = V / EV;                          // ... on the first VL lanes (all 32, or 20 for V = 80)
@@ -109,16 +118,16 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
     const int L = p.L, H = p.H, B = p.B;
     const int n_cap = p.n_before;                       // ring rows the stage has room for (per-sequence phases: the largest fill)
     const bool vlane = VL == 32 || lane < VL;           // this lane holds value elements
-    const bool per_seq = GEN && p.coef_per_seq;         // the head's own coefficient map travels with its sketch rows
-    const bool u_bf16 = UB || (GEN && p.sketch_bf16);   // sketch rows (and the fixed coefficient map) stored as bfloat16
+    const bool per_seq = ANY ? p.coef_per_seq != 0 : (F & kPS) != 0;   // the head's own coefficient map travels with its sketch rows
+    const bool u_bf16 = ANY ? p.sketch_bf16 != 0 : (F & kUB) != 0;     // sketch rows (and the coefficient map) stored as bfloat16
     const int su = u_bf16 ? 2 : 4;
     const int RP = (R + 7) & ~7;
     // c_t from the projected erase vectors of the buffered tokens instead of the swept query (delta-rule kinds)
-    constexpr bool ER = GEN == 2;
-    const bool er = ER && !p.full_read;
+    constexpr bool ER = (F & kER) != 0;
+    constexpr bool er = ER;
 
-    const StageLayout sl = make_stage_layout(KIND, (int)sizeof(IO), K, V, R, L, n_cap, p.full_read, per_seq, su, er);
-    const DecodeSmem ds = make_decode_smem(K, R, nwarps, p.full_read, per_seq, sl.total);
+    const StageLayout sl = make_stage_layout(KIND, (int)sizeof(IO), K, V, R, L, n_cap, FULL, per_seq, su, er);
+    const DecodeSmem ds = make_decode_smem(K, R, nwarps, FULL, per_seq, sl.total);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + ds.bar_off) + warp * 2;
     float* sX = reinterpret_cast<float*>(smem + ds.scratch_off + (size_t)warp * ds.scratch_stride);   // c or q~
     float* sP = sX + K;                                                                               // dot products
@@ -138,7 +147,7 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
     }
     // coefficient maps of the (at most two) head indices of this range, rows padded with zeros.  C is a constant of
     // the layer (never written by these kernels), so it may be staged before the predecessor in the stream is done.
-    if (!p.full_read && !per_seq && item1 > item0) {
+    if (!FULL && !per_seq && item1 > item0) {
         const int nslots = h_last > h_first ? 2 : 1;
         for (int s = 0; s < nslots; ++s) {
             float4* dst = reinterpret_cast<float4*>(smem + (size_t)s * ds.coef_slot_bytes);
@@ -191,16 +200,16 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
     const uint32_t rowA = (uint32_t)((K + V) * sizeof(IO)) + (KIND == SKETCHSSM_KDA ? (uint32_t)(K * sizeof(IO)) : 0u);
     const uint32_t gateA = (uint32_t)((KIND == SKETCHSSM_KDA ? 1 : 2) * L * 4);
     const uint32_t rowB = (uint32_t)(V * su) + (per_seq ? (uint32_t)(K * su) : 0u);
-    const int r_uni = p.full_read ? 0 : R;          // GEN = 0: the rank of every head
-    // GEN = 0: the size of this lane's copy and the two transaction totals are constants of the launch
+    const int r_uni = FULL ? 0 : R;          // the rank of every head (without kAny)
+    // one ring fill for all heads: the size of this lane's copy and the two transaction totals are constants of the launch
     const uint32_t cp_fixed = cp_mode == 0 ? cp_unit : cp_mode == 1 ? cp_unit * (uint32_t)n_cap
                             : cp_mode == 2 ? (n_cap > 0 ? cp_unit : 0u) : cp_unit * (uint32_t)r_uni;
     const uint32_t txA_fixed = tokA + (uint32_t)n_cap * rowA + (n_cap > 0 ? gateA : 0u);
-    const uint32_t txB_fixed = (uint32_t)r_uni * rowB;
+    const uint32_t txB_fixed = (uint32_t)r_uni * rowB + (er ? (uint32_t)(n_cap * R * su) : 0u);
     uint64_t* barA = &bars[0];
     uint64_t* barB = &bars[1];
     auto issue_a = [&](size_t bh, int n_it) {      // whole warp; n_it: ring fill of the head
-        if constexpr (GEN) {
+        if constexpr (DYN) {
             if (lane == 0) mbar_expect_tx(barA, tokA + (uint32_t)n_it * rowA + (n_it > 0 ? gateA : 0u));
             __syncwarp();
             const uint32_t bytes = cp_mode == 0 ? cp_unit : cp_mode == 1 ? cp_unit * (uint32_t)n_it : (n_it > 0 ? cp_unit : 0u);
@@ -213,7 +222,7 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
     };
     // whole warp; r_it: sketch rank of the head (0: nothing to fetch), n_it: its ring fill (rows of erase vectors)
     auto issue_b = [&](size_t bh, int r_it, int n_it) {
-        if constexpr (GEN) {
+        if constexpr (DYN) {
             const uint32_t fbytes = er ? (uint32_t)n_it * (uint32_t)(R * su) : 0u;
             if (lane == 8 && r_it > 0) mbar_expect_tx(barB, (uint32_t)r_it * rowB + fbytes);
             __syncwarp();
@@ -223,7 +232,7 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
         } else {
             if (lane == 8 && txB_fixed) mbar_expect_tx(barB, txB_fixed);
             __syncwarp();
-            if ((lane == 8 || lane == 9) && cp_fixed) bulk_g2s(my_stage + cp_dst, cp_base + bh * cp_stride, cp_fixed, barB);
+            if ((lane == 8 || lane == 9 || (ER && lane == 10)) && cp_fixed) bulk_g2s(my_stage + cp_dst, cp_base + bh * cp_stride, cp_fixed, barB);
         }
     };
 
@@ -246,8 +255,7 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
     // Per-head sketch rank: the configured rank, or the caller's table (0 = this head reads the full state instead).
     // The table is a layer constant like C, so it may be read before the predecessor in the stream is done.
     auto rank_of = [&](int hh) -> int {
-        if constexpr (!GEN) return r_uni;
-        if (p.full_read) return 0;
+        if constexpr (!ANY) return r_uni;
         if (p.head_rank == nullptr) return R;
         const int r = p.head_rank[hh];
         return r < 0 ? 0 : (r > R ? R : r);
@@ -255,7 +263,7 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
     // Per-sequence ring fill: the call's n_before, or the caller's per-sequence phase (negative: the sequence takes the
     // flush step in this call and is skipped here).
     auto fill_of = [&](int bb) -> int {
-        if constexpr (!GEN) return n_cap;
+        if constexpr (!DYN) return n_cap;
         return p.n_dev == nullptr ? n_cap : p.n_dev[bb];
     };
 
@@ -284,7 +292,7 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
     if (item < item1) {
         const size_t bh0 = (size_t)b * H + h;
         n = fill_of(b);
-        if (!GEN || n >= 0) {
+        if (!DYN || n >= 0) {
             issue_a(bh0, n);
             if (!early_u) issue_b(bh0, rk, n);
             scalar_gates(bh0, bt_next, dsc_next);
@@ -296,7 +304,8 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
     uint32_t parA = 0, parB = 0;     // phase parities of the two barriers (a phase passes only for heads that issued copies)
 
     while (item < item1) {
-        if constexpr (!GEN) { n = n_cap; n_next = n_cap; rk = r_uni; rk_next = r_uni; }      // launch constants
+        if constexpr (!DYN) { n = n_cap; n_next = n_cap; }      // launch constants
+        if constexpr (!ANY) { rk = r_uni; rk_next = r_uni; }
         const size_t bh = (size_t)b * H + h;
         const int item_next = claim();
         const bool has_next = item_next < item1;
@@ -305,25 +314,31 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
             rk_next = rank_of(hn);
             n_next = fill_of(bn);
         }
-        const bool go_next = has_next && (!GEN || n_next >= 0);          // the next head takes a decode step in this call
+        const bool go_next = has_next && (!DYN || n_next >= 0);          // the next head takes a decode step in this call
         const size_t bh_next = (size_t)bn * H + hn;
         const float bt = bt_next, dsc = dsc_next;
         if (go_next) scalar_gates(bh_next, bt_next, dsc_next);
 
-        if constexpr (GEN) {
+        if constexpr (DYN) {
             if (n < 0) {             // this sequence takes the flush step in this call: nothing to do here
                 if (go_next) { issue_a(bh_next, n_next); issue_b(bh_next, rk_next, n_next); }
                 item = item_next; h = hn; b = bn; n = n_next; rk = rk_next;
                 continue;
             }
         }
-        const bool full = rk == 0;   // exact read of the whole state for this head
+        const bool full = ANY ? rk == 0 : FULL;   // exact read of the whole state for this head
         const bool er_h = er && !full;       // this head forms c_t from projected erase vectors
+        // A dense-fallback head among sketched ones takes its rows through registers, a few at a time, and would finish long
+        // after the others: the rows after those are asked into L2 (the first ones during the sweep, kAhead rows ahead: at
+        // most 57 MB over all resident warps, within the 126 MB of L2).  Where every head reads its state the bytes in
+        // flight suffice without that, and the requests cost time (window of fp32 KDA full reads, 3072 heads: 440 -> 479 us).
+        constexpr int kAhead = 32;
+        if (ANY && full && lane == 0) prefetch_l2(p.state + bh * (size_t)K * V, (uint32_t)(kAhead * V * 4));
 
         if (__any_sync(0xffffffffu, !DEC_WAIT(barA, parA))) {
-            if (lane == 0) record_fault(p.status, p.full_read ? kFaultFullReadWait : kFaultDecodeWait, (int)blockIdx.x);
+            if (lane == 0) record_fault(p.status, FULL ? kFaultFullReadWait : kFaultDecodeWait, (int)blockIdx.x);
             pendA = (int)parA;
-            pendB = full ? -1 : (int)(GEN ? parB : parA);
+            pendB = full ? -1 : (int)(ANY ? parB : parA);
             break;
         }
         parA ^= 1u;
@@ -479,7 +494,7 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
                         const int s = sb - (lane >> 2);
                         float sc = 1.f;
                         if constexpr (KIND == SKETCHSSM_GDN) sc = __shfl_sync(0xffffffffu, dl_lane, s < 0 ? 0 : s);
-                        if ((lane & 3) == 0 && s >= 0) { sP[s] = pq[0] * sc; sP[32 + s] = pk[0] * sc; }
+                        if ((lane & 3) == 0 && s >= 0) *reinterpret_cast<float2*>(sP + 2 * s) = make_float2(pq[0] * sc, pk[0] * sc);
                     }
                     __syncwarp();
                 }
@@ -536,7 +551,7 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
                     break;
                 }
             }
-            const bool c16 = GEN && per_seq && u_bf16;       // the head's own map travels as bfloat16 (the shared map was widened when staged)
+            const bool c16 = per_seq && u_bf16;       // the head's own map travels as bfloat16 (the shared map was widened when staged)
             const int rp_it = RT ? ((RT + 7) & ~7) : ((rk + 7) & ~7);
             bool both = false;       // erase mode: C (d_[t] * q_t) and C (d_[t] * k_t) in one pass over the rows of C
             if constexpr (ER) both = er_h;
@@ -587,7 +602,7 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
                     break;
                 }
             }
-            if constexpr (GEN) parB ^= 1u;
+            if constexpr (ANY) parB ^= 1u;
             if constexpr (ER) {
                 if (er_h) {
                     // f_t = beta_t [C (d_[t] * k_t) - sum_{s<t} f_s <l_s(t), k_t>]  (Eq. 45), stored for the later steps;
@@ -595,20 +610,32 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
                     // (with bfloat16 storage the vectors are rounded once, where they are stored; this step uses the rounded f_t too)
                     const float* sF = reinterpret_cast<const float*>(sb + sl.f_off);
                     const __nv_bfloat16* sF16 = reinterpret_cast<const __nv_bfloat16*>(sb + sl.f_off);
-                    for (int g = lane; g < rk; g += 32) {
-                        float fq = sX[g], fk = sX[rp_it + g];
-                        for (int s = 0; s < n; ++s) {
-                            const float f = u_bf16 ? __bfloat162float(sF16[s * R + g]) : sF[s * R + g];
-                            fq = fmaf(-f, sP[s], fq);
-                            fk = fmaf(-f, sP[32 + s], fk);
+                    // Up to 16 coefficients: the two halves of the warp take every other slot.
+                    const bool two = (RT ? RT : rk) <= 16;
+                    const int s_first = two ? lane >> 4 : 0, s_step = two ? 2 : 1;
+                    for (int g = two ? lane & 15 : lane; g < (two ? 16 : rk); g += 32) {
+                        const bool on = g < rk;
+                        float fq = 0.f, fk = 0.f;
+#pragma unroll 4
+                        for (int s = s_first; s < n; s += s_step) {
+                            const float f = u_bf16 ? __bfloat162float(sF16[s * R + (on ? g : 0)]) : sF[s * R + (on ? g : 0)];
+                            const float2 l = *reinterpret_cast<const float2*>(sP + 2 * s);
+                            fq = fmaf(f, l.x, fq);
+                            fk = fmaf(f, l.y, fk);
                         }
-                        float f_t = bt * fk;
-                        if (u_bf16) f_t = __bfloat162float(__float2bfloat16_rn(f_t));
-                        sX[g] = fmaf(-f_t, kq_t, fq);
-                        if (p.append) {
-                            const size_t idx = (bh * L + n) * (size_t)R + g;
-                            if (u_bf16) reinterpret_cast<__nv_bfloat16*>(p.erase)[idx] = __float2bfloat16_rn(f_t);
-                            else p.erase[idx] = f_t;
+                        if (two) {
+                            fq += __shfl_xor_sync(0xffffffffu, fq, 16);
+                            fk += __shfl_xor_sync(0xffffffffu, fk, 16);
+                        }
+                        if (on && (!two || lane < 16)) {
+                            float f_t = bt * (sX[rp_it + g] - fk);
+                            if (u_bf16) f_t = __bfloat162float(__float2bfloat16_rn(f_t));
+                            sX[g] = fmaf(-f_t, kq_t, sX[g] - fq);
+                            if (p.append) {
+                                const size_t idx = (bh * L + n) * (size_t)R + g;
+                                if (u_bf16) reinterpret_cast<__nv_bfloat16*>(p.erase)[idx] = __float2bfloat16_rn(f_t);
+                                else p.erase[idx] = f_t;
+                            }
                         }
                     }
                     __syncwarp();
@@ -634,8 +661,10 @@ __global__ void __launch_bounds__(256, (GEN >= 1 || KIND != SKETCHSSM_MAMBA2) ? 
             __syncwarp();
             if (vlane) {
                 const float* Sg = p.state + bh * (size_t)K * V + lane * EV;
-                constexpr int RB = 8;
+                constexpr int RB = 32 / EV;              // rows in flight: 32 registers
                 for (int i0 = 0; i0 < K; i0 += RB) {
+                    if (ANY && lane == 0 && i0 + kAhead < K)
+                        prefetch_l2(p.state + (bh * K + i0 + kAhead) * V, (uint32_t)(RB * V * 4));
                     float rows[RB][EV];
 #pragma unroll
                     for (int r = 0; r < RB; ++r) load_io<EV>(Sg, (i0 + r) * V, rows[r]);
@@ -688,24 +717,46 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
     // warps per CTA / CTAs per SM: as many resident warps per SM as shared memory allows (capped), preferring
     // fewer, larger CTAs
     const int cap = p.max_warps_per_sm > 0 ? p.max_warps_per_sm : 32;
-    // bfloat16 storage with nothing else that needs the general kernel: the lean rank-16 instantiation reads it too
-    const bool lean_bf16 = p.sketch_bf16 && p.R == 16 && !p.full_read && p.head_rank == nullptr && p.n_dev == nullptr &&
-                           !p.coef_per_seq && !erase;
-    const bool gen = p.head_rank != nullptr || p.n_dev != nullptr || p.coef_per_seq || (p.sketch_bf16 && !lean_bf16) || erase;
-    const bool fixed16 = p.R == 16 && !gen;     // the unrolled rank-16 instantiation needs one rank for all heads
-    auto kern = gen ? decode_kernel<KIND, IO, K, V, 0, 1> : fixed16 ? decode_kernel<KIND, IO, K, V, 16, 0> : decode_kernel<KIND, IO, K, V, 0, 0>;
-    // rank 32 unrolled as well (state rows of 128 only: every instantiation costs build time; rank 8 measured no gain)
-    bool fixed32 = false;
-    if constexpr (K == 128) {
-        if (!gen && p.R == 32) { kern = decode_kernel<KIND, IO, K, V, 32, 0>; fixed32 = true; }
+    // What the launch needs, and the instantiation for it: rank 16 (32 rows of 128 as well) unrolled; the combinations of a
+    // deployment with rank 16, 128 state rows and bfloat16 I/O (mixed steps, the state-dependent map in either storage, the
+    // erase vectors) as instantiations of their own; everything else general.  (Every instantiation costs build time;
+    // rank 8 unrolled measured no gain.)
+    const int need = p.full_read ? kFull
+                                 : (p.n_dev != nullptr ? kSeq : 0) | (p.coef_per_seq ? kPS : 0) | (erase ? kER : 0) |
+                                       (p.sketch_bf16 ? kUB : 0) | (p.head_rank != nullptr ? kAny : 0);
+    auto kern = decode_kernel<KIND, IO, K, V, 0, kAny>;
+    int variant = 0;
+    if (need == 0) {
+        kern = p.R == 16 ? decode_kernel<KIND, IO, K, V, 16, 0> : decode_kernel<KIND, IO, K, V, 0, 0>;
+        variant = p.R == 16 ? 1 : 2;
+        if constexpr (K == 128) {
+            if (p.R == 32) { kern = decode_kernel<KIND, IO, K, V, 32, 0>; variant = 3; }
+        }
+    } else if (need == kFull) {
+        kern = decode_kernel<KIND, IO, K, V, 0, kFull>;
+        variant = 12;
+    } else if (need == kUB && p.R == 16) {
+        kern = decode_kernel<KIND, IO, K, V, 16, kUB>;
+        variant = 4;
     }
-    if (lean_bf16) kern = decode_kernel<KIND, IO, K, V, 16, 0, true>;
     if constexpr (KIND != SKETCHSSM_MAMBA2) {
-        if (erase) kern = decode_kernel<KIND, IO, K, V, 0, 2>;
+        if (erase) { kern = decode_kernel<KIND, IO, K, V, 0, kAny | kER>; variant = 5; }
     }
-    // registers per thread of the two instantiations (queried once): they bound the resident warps like shared memory does
-    static int regs_per_thread[6] = {0, 0, 0, 0, 0, 0};
-    int& regs = regs_per_thread[fixed32 ? 5 : lean_bf16 ? 4 : erase ? 3 : gen ? 2 : fixed16 ? 1 : 0];
+    if constexpr (K == 128 && V != 80 && sizeof(IO) == 2) {
+        if (p.R == 16) {        // (a full read has its own)
+            if (need == kSeq) { kern = decode_kernel<KIND, IO, K, V, 16, kSeq>; variant = 6; }
+            if (need == kPS) { kern = decode_kernel<KIND, IO, K, V, 16, kPS>; variant = 7; }
+            if (need == (kPS | kUB)) { kern = decode_kernel<KIND, IO, K, V, 16, kPS | kUB>; variant = 8; }
+            if (need == (kSeq | kPS | kUB)) { kern = decode_kernel<KIND, IO, K, V, 16, kSeq | kPS | kUB>; variant = 9; }
+            if constexpr (KIND != SKETCHSSM_MAMBA2) {
+                if (need == kER) { kern = decode_kernel<KIND, IO, K, V, 16, kER>; variant = 10; }
+                if (need == (kER | kPS | kUB)) { kern = decode_kernel<KIND, IO, K, V, 16, kER | kPS | kUB>; variant = 11; }
+            }
+        }
+    }
+    // registers per thread of the instantiation (queried once): they bound the resident warps like shared memory does
+    static int regs_per_thread[13] = {0};
+    int& regs = regs_per_thread[variant];
     if (regs == 0) {
         cudaFuncAttributes fa;
         if ((ctx->last_cuda_error = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
@@ -749,19 +800,14 @@ static int launch_decode_shape(Ctx* ctx, const Params& p, cudaStream_t stream) {
     return SKETCHSSM_UNSUPPORTED_SHAPE;
 }
 
-template <int KIND>
-static int launch_decode_io(Ctx* ctx, const Params& p, cudaStream_t stream) {
-    if (ctx->cfg.io_dtype == SKETCHSSM_BF16) return launch_decode_shape<KIND, __nv_bfloat16>(ctx, p, stream);
-    return launch_decode_shape<KIND, float>(ctx, p, stream);
+// one translation unit per (recurrence kind, I/O type), so that they compile side by side
+#if SKETCHSSM_GROUP_IO
+using GroupIO = __nv_bfloat16;
+#else
+using GroupIO = float;
+#endif
+template <>
+int launch_decode_group<SKETCHSSM_GROUP_KIND, SKETCHSSM_GROUP_IO>(Ctx* ctx, const Params& p, cudaStream_t stream) {
+    return launch_decode_shape<SKETCHSSM_GROUP_KIND, GroupIO>(ctx, p, stream);
 }
-
-int launch_decode(Ctx* ctx, const Params& p, cudaStream_t stream) {
-    switch (ctx->cfg.kind) {
-        case SKETCHSSM_MAMBA2: return launch_decode_io<SKETCHSSM_MAMBA2>(ctx, p, stream);
-        case SKETCHSSM_GDN: return launch_decode_io<SKETCHSSM_GDN>(ctx, p, stream);
-        case SKETCHSSM_KDA: return launch_decode_io<SKETCHSSM_KDA>(ctx, p, stream);
-    }
-    return SKETCHSSM_INVALID_ARG;
-}
-
 }  // namespace sketchssm

@@ -91,7 +91,9 @@ struct Params {
     int tok_base;         // update (GDN tensor-core kernel): first ring row of this pass when a flush is replayed in blocks of 16 tokens
 };
 
-int launch_decode(Ctx* ctx, const Params& p, cudaStream_t stream);        // one warp per head
+// decode, one warp per head: one entry per (kind, I/O type)
+template <int KIND, int BF16>
+int launch_decode_group(Ctx* ctx, const Params& p, cudaStream_t stream);
 // two-kernel decode with the weight hand-off in the library's static device array
 int launch_decode_static(Ctx* ctx, const Params& p, cudaStream_t stream);
 // decode as two kernels (weights, then output rows), one entry per (kind, I/O type)
