@@ -20,8 +20,8 @@
 // ||S||_F^2 rides along.  One warp then builds and inverts the p x p system in registers while the others prepare two
 // small per-rank tables, and thread k forms column k of C in two passes over the ranks with its row of Omega in
 // registers (stores coalesced across the CTA).  The single-warp stages rotate over the warps from CTA to CTA.
-// Exact form: thread k streams row k of S against all G sketch rows, Cholesky by one warp, one pair of triangular
-// solves per thread.  The kernel runs after the flush kernel of the same call and re-reads S_new and U from memory:
+// Exact form: ridge_map_kernel below for up to 32 ranks; above (and with fp32 inputs) thread k streams row k of S against
+// all G sketch rows, Cholesky by one warp, one pair of triangular solves per thread.  The kernel runs after the flush kernel of the same call and re-reads S_new and U from memory:
 // the map needs the complete sketch before it can contract the state with it.
 #include "internal.cuh"
 #include "lanegroup.cuh"
@@ -616,9 +616,221 @@ __global__ void __launch_bounds__(kCoefThreads) coef_map_kernel(const Params p) 
     }
 }
 
+// The exact ridge form for up to GT ranks (8, 16, 24 or 32), rows beyond the head's rank zero: A = U U^T + lam mu I, Y = S U^T and
+// C = A^{-1} Y^T, everything in fp32.  A thread per column of C (K threads); Y as a register-tiled product: two rows of S and
+// half of the ranks per thread, S through shared memory CW columns at a time (read whole lines, the next columns in
+// registers meanwhile), packed pairs of columns; A factored by one warp with a row per lane; both substitutions in
+// registers.  The one-warp factorisation and the two substitutions are chains; 80 registers (up to 16 ranks) leave six
+// CTAs per SM to cover them.  Maps of 16384 Mamba-2 heads of rank 16 (K = 128, V = 64): 300 us; a thread per state row
+// reading its own row, with factor and right-hand sides in shared memory, took 650; 32 columns at a time with 128
+// registers (four CTAs) and IEEE square roots and divisions 340.  Ranks rounded up to 16 and 32 only: 0.9 x the former
+// kernel's speed at ranks 8 and 24.
+template <int K, int V, int GT>
+struct RidgeSmem {
+    static constexpr int CW = 16;                        // columns of S staged at a time
+    static constexpr int SP = CW + 4, UP = V + 4, YP = GT + 4;   // row pitches (floats): 128-bit accesses of eight rows hit all banks
+    static constexpr int kStage = K * SP > K * YP ? K * SP : K * YP;   // S columns, then Y
+    static constexpr int u = 0, st = u + GT * UP, l = st + kStage, lt = l + GT * YP, inv = lt + GT * YP, red = inv + GT, total = red + 8;
+};
+
+template <int K, int V, int GT>
+__global__ void __launch_bounds__(K, (GT <= 16 ? 6 : 4) * (128 / K)) ridge_map_kernel(const Params p) {
+    using SM = RidgeSmem<K, V, GT>;
+    constexpr int CW = SM::CW, SP = SM::SP, UP = SM::UP, YP = SM::YP, NW = K / 32;
+    extern __shared__ __align__(16) float sm[];
+    float *sU = sm + SM::u, *sS = sm + SM::st, *sY = sm + SM::st, *sL = sm + SM::l, *sLT = sm + SM::lt, *sInv = sm + SM::inv,
+          *sRed = sm + SM::red;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const size_t bh = (size_t)gridDim.x - 1 - blockIdx.x;      // descending, as above
+    const int h = (int)(bh % (size_t)p.H);
+    int G = p.R;
+    if (p.head_rank != nullptr) {
+        const int r = p.head_rank[h];
+        G = r < 0 ? 0 : (r > p.R ? p.R : r);
+    }
+    if (G == 0) return;
+    if (p.n_dev != nullptr && p.n_dev[bh / (size_t)p.H] >= 0) return;
+    const int RS = p.R;
+    const bool bf = p.sketch_bf16 != 0;
+    const float* Sg = p.state + bh * (size_t)K * V;
+
+    // the first CW columns of S on their way; thread t loads 16-byte units t, t + K, ...
+    constexpr int UN = CW / 4;                                 // units per row = units per thread
+    float4 nxt[UN];
+    auto fetch = [&](int c) {
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+            const int idx = tid + u * K, r = idx / UN, q = idx % UN;
+            nxt[u] = *reinterpret_cast<const float4*>(Sg + (size_t)r * V + c * CW + 4 * q);
+        }
+    };
+    fetch(0);
+    for (int i = tid; i < GT * (V / 4); i += K) {
+        const int g = i / (V / 4), c = i % (V / 4);
+        float x[4] = {0.f, 0.f, 0.f, 0.f};
+        if (g < G) {
+            const size_t at = (bh * RS + g) * V + 4 * c;
+            if (bf) ld4(reinterpret_cast<const __nv_bfloat16*>(p.sketch) + at, x);
+            else ld4(p.sketch + at, x);
+        }
+        st4(sU + g * UP + 4 * c, x);
+    }
+
+    // ---- Y[k][g] = <S[k,:], U_g>: rows k0 and k0 + K/2, ranks half * GH .. + GH - 1 ----
+    constexpr int GH = GT / 2;
+    const int k0 = tid % (K / 2), half = tid / (K / 2);
+    float ss = 0.f;
+    f32x2 acc[2][GH];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int j = 0; j < GH; ++j) acc[r][j] = pack2(0.f, 0.f);
+#pragma unroll 1
+    for (int c = 0; c < V / CW; ++c) {
+        if (c > 0) __syncthreads();
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+            const int idx = tid + u * K, r = idx / UN, q = idx % UN;
+            const float4 x = nxt[u];
+            ss = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, ss))));
+            *reinterpret_cast<float4*>(sS + r * SP + 4 * q) = x;
+        }
+        __syncthreads();
+        if (c + 1 < V / CW) fetch(c + 1);
+#pragma unroll
+        for (int q = 0; q < UN; ++q) {
+            const float4 a = *reinterpret_cast<const float4*>(sS + k0 * SP + 4 * q);
+            const float4 b = *reinterpret_cast<const float4*>(sS + (k0 + K / 2) * SP + 4 * q);
+            const f32x2 a01 = pack2(a.x, a.y), a23 = pack2(a.z, a.w), b01 = pack2(b.x, b.y), b23 = pack2(b.z, b.w);
+#pragma unroll
+            for (int j = 0; j < GH; ++j) {
+                const float4 w = *reinterpret_cast<const float4*>(sU + (half * GH + j) * UP + c * CW + 4 * q);
+                const f32x2 w01 = pack2(w.x, w.y), w23 = pack2(w.z, w.w);
+                acc[0][j] = fma2(a23, w23, fma2(a01, w01, acc[0][j]));
+                acc[1][j] = fma2(b23, w23, fma2(b01, w01, acc[1][j]));
+            }
+        }
+    }
+    // Gram matrix, lower triangle
+    for (int i = tid; i < GT * GT; i += K) {
+        const int g = i / GT, j = i % GT;
+        if (j <= g) {
+            f32x2 a = pack2(0.f, 0.f), b = a;
+#pragma unroll 4
+            for (int v = 0; v < V; v += 4) {
+                const float4 x = *reinterpret_cast<const float4*>(sU + g * UP + v), y = *reinterpret_cast<const float4*>(sU + j * UP + v);
+                a = fma2(pack2(x.x, x.y), pack2(y.x, y.y), a);
+                b = fma2(pack2(x.z, x.w), pack2(y.z, y.w), b);
+            }
+            float a0, a1, b0, b1;
+            unpack2(a, a0, a1);
+            unpack2(b, b0, b1);
+            sL[g * YP + j] = (a0 + a1) + (b0 + b1);
+        }
+    }
+    ss = warp_sum(ss);
+    if (lane == 0) sRed[warp] = ss;
+    __syncthreads();                       // the staged columns have been read, the Gram matrix and the norm are complete
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int j4 = 0; j4 < GH; j4 += 4) {
+            float y[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float lo, hi;
+                unpack2(acc[r][j4 + j], lo, hi);
+                y[j] = lo + hi;
+            }
+            st4(sY + (k0 + r * (K / 2)) * YP + half * GH + j4, y);
+        }
+    if (warp == 0) {
+        // Cholesky factor, a row per lane
+        float s2 = 0.f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) s2 += sRed[w];
+        const float mu = s2 > 0.f ? s2 / (float)K : 1.f;
+        const int r = lane < GT ? lane : GT - 1;
+        float a[GT];
+#pragma unroll
+        for (int j = 0; j < GT; ++j) a[j] = j <= r ? sL[r * YP + j] : 0.f;
+#pragma unroll
+        for (int j = 0; j < GT; ++j)
+            if (j == r) a[j] += p.ridge_lambda * mu;
+#pragma unroll
+        for (int c = 0; c < GT; ++c) {
+            // 1 / sqrt by one Newton step on the approximation: the chain over the columns is what this stage takes
+            const float x = fmaxf(__shfl_sync(0xffffffffu, a[c], c), 1e-30f);
+            float inv = rsqrtf(x);
+            inv = fmaf(0.5f * inv, fmaf(-x * inv, inv, 1.f), inv);
+            a[c] = r == c ? x * inv : a[c] * inv;
+            if (lane == c) sInv[c] = inv;
+#pragma unroll
+            for (int j = c + 1; j < GT; ++j) a[j] = fmaf(-a[c], __shfl_sync(0xffffffffu, a[c], j), a[j]);
+        }
+        if (lane < GT) {
+#pragma unroll
+            for (int j = 0; j < GT; ++j) {
+                sL[r * YP + j] = a[j];
+                sLT[j * YP + r] = a[j];
+            }
+        }
+    }
+    __syncthreads();
+    // ---- column k of C: L L^T c = Y[k][:] ----
+    float y[GT];
+#pragma unroll
+    for (int g = 0; g < GT; g += 4) ld4(sY + tid * YP + g, y + g);
+#pragma unroll
+    for (int g = 0; g < GT; ++g) {
+#pragma unroll
+        for (int j4 = 0; j4 < (g + 3) / 4; ++j4) {
+            const float4 l = *reinterpret_cast<const float4*>(sL + g * YP + 4 * j4);
+            if (4 * j4 + 0 < g) y[g] = fmaf(-l.x, y[4 * j4 + 0], y[g]);
+            if (4 * j4 + 1 < g) y[g] = fmaf(-l.y, y[4 * j4 + 1], y[g]);
+            if (4 * j4 + 2 < g) y[g] = fmaf(-l.z, y[4 * j4 + 2], y[g]);
+            if (4 * j4 + 3 < g) y[g] = fmaf(-l.w, y[4 * j4 + 3], y[g]);
+        }
+        y[g] *= sInv[g];
+    }
+    float* Cg = const_cast<float*>(p.coef) + bh * (size_t)RS * K + tid;
+    __nv_bfloat16* Cg16 = reinterpret_cast<__nv_bfloat16*>(const_cast<float*>(p.coef)) + bh * (size_t)RS * K + tid;
+#pragma unroll
+    for (int g = GT - 1; g >= 0; --g) {
+#pragma unroll
+        for (int j4 = (g + 1) / 4; j4 < GT / 4; ++j4) {
+            const float4 l = *reinterpret_cast<const float4*>(sLT + g * YP + 4 * j4);
+            if (4 * j4 + 0 > g) y[g] = fmaf(-l.x, y[4 * j4 + 0], y[g]);
+            if (4 * j4 + 1 > g) y[g] = fmaf(-l.y, y[4 * j4 + 1], y[g]);
+            if (4 * j4 + 2 > g) y[g] = fmaf(-l.z, y[4 * j4 + 2], y[g]);
+            if (4 * j4 + 3 > g) y[g] = fmaf(-l.w, y[4 * j4 + 3], y[g]);
+        }
+        y[g] *= sInv[g];
+        if (g < G) {
+            if (bf) Cg16[(size_t)g * K] = __float2bfloat16_rn(y[g]);
+            else Cg[(size_t)g * K] = y[g];
+        }
+    }
+}
+
+template <int K, int V, int GT>
+static int launch_ridge(Ctx* ctx, const Params& p, cudaStream_t stream) {
+    auto kern = ridge_map_kernel<K, V, GT>;
+    if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
+    kern<<<dim3((unsigned)((size_t)p.B * p.H)), dim3(K), RidgeSmem<K, V, GT>::total * 4, stream>>>(p);
+    if ((ctx->last_cuda_error = cudaGetLastError()) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
+    ctx->last_launches += 1;
+    return SKETCHSSM_OK;
+}
+
 template <int K, int V>
 static int launch_coef_kv(Ctx* ctx, const Params& p, cudaStream_t stream) {
     const bool exact = p.pivots <= 0;
+    // (fp32 inputs keep the kernel with the summation order they had: their results are held to 1e-5, and two orders of the
+    // same system differ by more, 1.4e-5, through its condition number)
+    if (exact && p.R <= 32 && ctx->cfg.io_dtype == SKETCHSSM_BF16)
+        return p.R <= 8 ? launch_ridge<K, V, 8>(ctx, p, stream) : p.R <= 16 ? launch_ridge<K, V, 16>(ctx, p, stream)
+             : p.R <= 24 ? launch_ridge<K, V, 24>(ctx, p, stream) : launch_ridge<K, V, 32>(ctx, p, stream);
     const int m = exact ? p.R : (p.R < p.pivots ? p.R : p.pivots);
     const CoefSmem sm = make_coef_smem(K, V, p.R, m);
     auto kern = exact ? coef_map_kernel<K, V, 1, 4> : (m <= 4 ? coef_map_kernel<K, V, 0, 4> : coef_map_kernel<K, V, 0, 8>);

@@ -26,6 +26,25 @@ __device__ __forceinline__ void st4(__nv_bfloat16* p, const float* s) {
     *reinterpret_cast<uint2*>(p) = t;
 }
 
+// Packed pairs of fp32 (sm_100: one instruction for two independent IEEE operations), for loops bound by instruction issue.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 r, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // A lane j of a group owns the element chunks {4 (j + LPH m) .. +3 : m = 0 .. E/4-1} of a row.
 template <int E, int LPH, typename T>
 __device__ __forceinline__ void load_row(const T* row, int j, float (&d)[E]) {

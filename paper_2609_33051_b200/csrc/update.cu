@@ -38,26 +38,6 @@ struct PaddedRow {
     __host__ __device__ static constexpr int at(int i) { return i + 4 * (i / RP); }
 };
 
-// Packed pairs of fp32 (sm_100: one instruction for two independent IEEE operations): the replay loops are bound by
-// instruction issue, and a column's rows are independent.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 r, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r)); }
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-    f32x2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 struct UpdateSmem {
     uint32_t kh_off, kt_off, g_off, gram_off, a_off, beta_off, pre_off, suf_off, v_off, e_off, q_off, om_off, list_off, bar_off;
     uint32_t st_off, st_k, st_v, st_gate, st_g, st_tq, st_tk, st_tv, st_tg;      // stage (0 bytes without one)
