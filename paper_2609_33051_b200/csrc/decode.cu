@@ -102,8 +102,14 @@ __host__ __device__ inline DecodeSmem make_decode_smem(int K, int R, int nwarps,
 // 48 -> 46 us; V = 80 layer of 37 x 24 heads with two dense heads (prefetch below) 13 -> 10 us.
 constexpr int kSeq = 1, kPS = 2, kER = 4, kUB = 8, kAny = 16, kFull = 32;
 
+// Warps of the largest CTA; two such CTAs per SM set the register budget: 64 registers for the lean Mamba-2 kernels (32
+// warps), 80 for the others (24 warps).
+__host__ __device__ constexpr int decode_max_warps(int kind, int F) {
+    return (F & ~(kUB | kFull)) != 0 || kind != SKETCHSSM_MAMBA2 ? 12 : 16;
+}
+
 template <int KIND, typename IO, int K, int V, int RT, int F>
-__global__ void __launch_bounds__(256, ((F & ~(kUB | kFull)) || KIND != SKETCHSSM_MAMBA2) ? 3 : 4) decode_kernel(const Params p) {
+__global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kernel(const Params p) {
     constexpr bool ANY = (F & kAny) != 0, DYN = ANY || (F & kSeq) != 0, FULL = (F & kFull) != 0;
     constexpr int EK = K / 32;
     constexpr int EV = V % 32 == 0 ? V / 32 : 4;        // value elements per lane ...
@@ -764,7 +770,12 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
     }
     const int reg_warps = 65536 / (regs * 32);          // warps the register file holds
     int best_nw = 0, best_ctas = 1, best_warps = 0;
-    for (int nw = 8; nw >= 1; --nw) {
+    // (eight warps and fewer first: larger CTAs only where they hold more warps per SM than any number of smaller ones, the
+    // staged coefficient maps being shared by more of them.  Windows, CTAs of at most 8 -> 16 (12) warps: Mamba-2 layer of
+    // batch 256 624 -> 605 us, 2048 4458 -> 4385, rank 32 with L = 64 4750 -> 4677, state-dependent bfloat16 map 917 -> 890)
+    const int max_nw = decode_max_warps(KIND, need);
+    for (int i = 0; i < max_nw; ++i) {
+        const int nw = i < 8 ? 8 - i : i + 1;
         if (p.warps_per_cta && nw != p.warps_per_cta) continue;
         const DecodeSmem d = make_decode_smem(K, p.R, nw, p.full_read, p.coef_per_seq, sl.total);
         if (d.total > smem_budget) continue;
