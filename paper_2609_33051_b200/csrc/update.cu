@@ -26,6 +26,13 @@ namespace sketchssm {
 
 constexpr int kParts = 8;               // lanes that share a group of four columns
 constexpr int kTok = 8;                 // tokens replayed together
+// Tokens whose key rows are in shared memory at a time.  All rows of a long window at once left room for one CTA per SM or
+// for no stage; every further chunk costs two block barriers.  Flush of 8192 heads in us, 16 / 32 at a time: KDA (two rows
+// per token) V = 64, L = 32 479 / 652; K = V = 64, L = 64 GDN 396 / 422, Mamba-2 196 / 204; GDN V = 80, L = 64, r = 32 1137 /
+// 1229; GDN V = 128, L = 32, r = 32 (no stage either way) 1027 / 969; Mamba-2 V = 64, L = 64 415 / 396.
+__host__ __device__ constexpr int update_chunk(int kind, int K, int V) {
+    return kind == SKETCHSSM_KDA || K == 64 || (kind == SKETCHSSM_GDN && V == 80) ? 16 : 32;
+}
 constexpr int kPairs = 32;              // pairs (s, j < s) of kTok tokens, padded from 28
 constexpr int kScan = 1024;             // sequences whose phases are looked through at a time
 
@@ -52,8 +59,9 @@ __host__ __device__ constexpr int omega_stride() { return PaddedRow<K>::stride +
 template <int K>
 __host__ __device__ inline UpdateSmem make_update_smem(int kind, int n_tot, int R, int V, int L, int io, int mixed, int stage) {
     UpdateSmem u;
-    const int ntok = n_tot > 0 ? n_tot : 1;
-    const int nb = (ntok + kTok - 1) / kTok;
+    const int ntok = n_tot > 0 ? n_tot : 1;                        // in the stage, and the tokens' weights
+    const int nchunk = ntok < update_chunk(kind, K, V) ? ntok : update_chunk(kind, K, V);              // key rows, values and pair sums
+    const int nb = (nchunk + kTok - 1) / kTok;
     const int R8 = (R + 7) & ~7;
     const bool delta = kind != SKETCHSSM_MAMBA2, kda = kind == SKETCHSSM_KDA;
     const uint32_t row = PaddedRow<K>::stride * 4;
@@ -63,10 +71,10 @@ __host__ __device__ inline UpdateSmem make_update_smem(int kind, int n_tot, int 
     u.g_off = off; off += kda ? (uint32_t)nb * row : 0u;
     u.gram_off = off; off += delta ? (uint32_t)(nb * (K / 32) * kPairs * 4) : 0u;
     u.a_off = off; off += delta ? (uint32_t)(nb * kPairs * 4) : 0u;
-    u.beta_off = off; off += (uint32_t)(nb * kTok * 4);
+    u.beta_off = off; off += (uint32_t)(((ntok + kTok - 1) / kTok) * kTok * 4);
     u.pre_off = off; off += (uint32_t)(nb * kTok * 4);
     u.suf_off = off; off += kind == SKETCHSSM_GDN ? (uint32_t)(nb * kTok * 4) : 0u;
-    u.v_off = off; off += (uint32_t)(ntok * V * io);
+    u.v_off = off; off += (uint32_t)(nchunk * V * io);
     u.e_off = off; off += (uint32_t)(V / 16) * (kTok * 16 * 4);
     u.q_off = off; off += row;
     u.om_off = off; off += (uint32_t)(R8 * omega_stride<K>() * 4);
@@ -145,6 +153,7 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
     using PR = PaddedRow<K>;
     constexpr int RP = PR::RP, KS = PR::stride, OS = omega_stride<K>();
     constexpr bool DELTA = KIND != SKETCHSSM_MAMBA2, KDA = KIND == SKETCHSSM_KDA;
+    constexpr int kChunk = update_chunk(KIND, K, V);
     extern __shared__ __align__(128) unsigned char smem[];
 
     const int R = p.R, H = p.H, B = p.B;
@@ -217,7 +226,6 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
     auto replay = [&](int b, int h, int n_ring, int b_next, int h_next, int n_next) {
         const size_t bh = (size_t)b * H + h;
         const int n_tot = n_ring + (p.has_token ? 1 : 0);
-        const int nb = (n_tot + kTok - 1) / kTok;
 
         // ---- state -> registers ----
         float4 raw[RP];
@@ -255,7 +263,22 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
             for (int i = 0; i < RP; ++i) raw[i] = *reinterpret_cast<const float4*>(Sg + (size_t)i * V);
         }
 
-        // ---- ring + current token -> shared memory (fp32) ----
+        f32x2 c2[4][RP / 2];
+#pragma unroll
+        for (int i = 0; i < RP / 2; ++i) {
+            c2[0][i] = pack2(raw[2 * i].x, raw[2 * i + 1].x);
+            c2[1][i] = pack2(raw[2 * i].y, raw[2 * i + 1].y);
+            c2[2][i] = pack2(raw[2 * i].z, raw[2 * i + 1].z);
+            c2[3][i] = pack2(raw[2 * i].w, raw[2 * i + 1].w);
+        }
+        const int row = part * (RP + 4);            // this lane's rows inside a padded row
+
+        // kChunk tokens at a time: their rows -> shared memory (fp32), then the replay
+#pragma unroll 1
+        for (int c0 = 0; c0 == 0 || c0 < n_tot; c0 += kChunk) {
+        const int n_here = min(n_tot - c0, kChunk), nb = (n_here + kTok - 1) / kTok;
+        const bool last = c0 + kChunk >= n_tot;
+        if (c0 > 0) __syncthreads();                 // the previous tokens' rows have been read
         if constexpr (DELTA) {
             // a thread per (eight tokens, channel)
             for (int idx = tid; idx < nb * K; idx += T) {
@@ -263,7 +286,7 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
                 float k[kTok], g[kTok];
 #pragma unroll
                 for (int s = 0; s < kTok; ++s) {
-                    const int t = blk * kTok + s;
+                    const int t = c0 + blk * kTok + s;
                     k[s] = 0.f;
                     g[s] = 1.f;
                     if (t < n_ring) {
@@ -320,16 +343,16 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
                 group_reduce_transpose<32, kPairs>(pr, lane);
                 sGram[(blk * (K / 32) + i / 32) * kPairs + lane] = pr[0];
             }
-            for (int s = tid; s < nb * kTok; s += T) sBeta[s] = s < n_ring ? rbeta[s] : s < n_tot ? *tbeta : 0.f;
+            for (int s = tid; s < nb * kTok; s += T) sBeta[s] = c0 + s < n_ring ? rbeta[c0 + s] : c0 + s < n_tot ? *tbeta : 0.f;
         } else {
-            for (int idx = tid; idx < n_tot * (K / 4); idx += T) {
+            for (int idx = tid; idx < n_here * (K / 4); idx += T) {
                 const int s = idx / (K / 4), i = 4 * (idx % (K / 4));
                 float k[4];
-                ld4(s < n_ring ? rk + (size_t)s * K + i : tk + i, k);
+                ld4(c0 + s < n_ring ? rk + (size_t)(c0 + s) * K + i : tk + i, k);
                 st4(sKt + s * KS + PR::at(i), k);
             }
             // w_s = beta_s prod_{j>s} a_j and the total decay, by a warp scan over up to 64 tokens
-            if (warp == 0) {
+            if (warp == 0 && c0 == 0) {
                 float a[2], bt[2];
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
@@ -348,7 +371,7 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
                     }
                     float excl = __shfl_down_sync(0xffffffffu, incl, 1);
                     if (lane == 31) excl = 1.f;
-                    if (lane + 32 * u < nb * kTok) sBeta[lane + 32 * u] = bt[u] * (excl * after);
+                    if (lane + 32 * u < n_tot) sBeta[lane + 32 * u] = bt[u] * (excl * after);
                     after *= __shfl_sync(0xffffffffu, incl, 0);
                 }
                 if (lane == 0) sPre[0] = after;
@@ -358,10 +381,12 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
             constexpr int PV = 16 / (int)sizeof(IO), in_row = V / PV;        // 16-byte units
             const uint4* ring_v = reinterpret_cast<const uint4*>(rv);
             const uint4* tok_v = reinterpret_cast<const uint4*>(tv);
-            for (int idx = tid; idx < n_tot * in_row; idx += T)
-                reinterpret_cast<uint4*>(sV)[idx] = idx < n_ring * in_row ? ring_v[idx] : tok_v[idx - n_ring * in_row];
+            for (int idx = tid; idx < n_here * in_row; idx += T) {
+                const int at = c0 * in_row + idx;
+                reinterpret_cast<uint4*>(sV)[idx] = at < n_ring * in_row ? ring_v[at] : tok_v[at - n_ring * in_row];
+            }
         }
-        if (p.q != nullptr) {
+        if (p.q != nullptr && c0 == 0) {
             for (int i = tid; i < K / 4; i += T) {
                 float q[4];
                 ld4(tq + 4 * i, q);
@@ -383,7 +408,7 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
             failed = true;
             return;
         }
-        if (staged && tid == 0 && n_next >= 0) request(b_next, h_next, n_next);
+        if (staged && last && tid == 0 && n_next >= 0) request(b_next, h_next, n_next);
         if constexpr (DELTA) {
             // beta_s A_sj
             for (int idx = tid; idx < nb * kPairs; idx += T) {
@@ -398,18 +423,8 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
             __syncthreads();
         }
 
-        f32x2 c2[4][RP / 2];
-#pragma unroll
-        for (int i = 0; i < RP / 2; ++i) {
-            c2[0][i] = pack2(raw[2 * i].x, raw[2 * i + 1].x);
-            c2[1][i] = pack2(raw[2 * i].y, raw[2 * i + 1].y);
-            c2[2][i] = pack2(raw[2 * i].z, raw[2 * i + 1].z);
-            c2[3][i] = pack2(raw[2 * i].w, raw[2 * i + 1].w);
-        }
-        const int row = part * (RP + 4);            // this lane's rows inside a padded row
-
         if constexpr (!DELTA) {
-            if (n_tot > 0) {
+            if (n_tot > 0 && c0 == 0) {
                 const f32x2 d2 = pack2(sPre[0], sPre[0]);
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
@@ -419,7 +434,7 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
         }
         for (int blk = 0; blk < nb; ++blk) {
             const int s0 = blk * kTok;
-            const int nt = min(kTok, n_tot - s0);
+            const int nt = min(kTok, n_here - s0);
             const int mine = s0 + part;              // this lane's token where a lane stands for one
             float x[4];
             if constexpr (DELTA) {
@@ -434,15 +449,15 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
                 }
                 reduce_parts(vals, lane);
                 float v[4] = {0.f, 0.f, 0.f, 0.f};
-                if (mine < n_tot) ld4(sV + mine * V + j0, v);
+                if (mine < n_here) ld4(sV + mine * V + j0, v);
                 const float bt = sBeta[mine], pre = KIND == SKETCHSSM_GDN ? sPre[mine] : 1.f;
 #pragma unroll
                 for (int c = 0; c < 4; ++c)
-                    x[c] = mine < n_tot ? bt * (v[c] - (KIND == SKETCHSSM_GDN ? pre * vals[c] : vals[c])) : 0.f;
+                    x[c] = mine < n_here ? bt * (v[c] - (KIND == SKETCHSSM_GDN ? pre * vals[c] : vals[c])) : 0.f;
             } else {
                 float v[4] = {0.f, 0.f, 0.f, 0.f};
-                if (mine < n_tot) ld4(sV + mine * V + j0, v);
-                const float w = sBeta[mine];
+                if (mine < n_here) ld4(sV + mine * V + j0, v);
+                const float w = mine < n_here ? sBeta[c0 + mine] : 0.f;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) x[c] = w * v[c];
             }
@@ -499,6 +514,8 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
                     }
                 }
             }
+        }
+
         }
 
         // ---- write the updated state back ----
@@ -647,10 +664,10 @@ static int launch_update_t(Ctx* ctx, Params p, cudaStream_t stream) {
     const int n_tot = p.n_before + (p.has_token ? 1 : 0);
     const bool mixed = p.n_dev != nullptr;
     if (mixed) p.n_cap = n_tot;        // per-sequence phases: n_before is the largest fill any sequence may have
-    // Staging one head ahead needs room for the stage beside the CTAs that the registers allow (V = 64: three of the four).
-    constexpr int kMinStaged = V == 64 ? 3 : update_ctas<V>();
+    // Staging one head ahead wherever two CTAs per SM fit with the stage, even if more would fit without: flush of 8192 KDA
+    // heads with V = 64, L = 16 304 us against 326 (GDN, where three fit, 271 against 317; V = 80 345 against 408).
     UpdateSmem us = make_update_smem<K>(KIND, n_tot, p.R, V, p.L, (int)sizeof(IO), mixed, 1);
-    p.stages = us.total + 1024u <= (228u * 1024u) / kMinStaged ? 1 : 0;
+    p.stages = us.total + 1024u <= (228u * 1024u) / 2u ? 1 : 0;
     if (!p.stages) us = make_update_smem<K>(KIND, n_tot, p.R, V, p.L, (int)sizeof(IO), mixed, 0);
     auto kern = update_kernel<KIND, IO, K, V>;
     if (us.total > 226u * 1024u) return SKETCHSSM_UNSUPPORTED_SHAPE;

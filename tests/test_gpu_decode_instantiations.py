@@ -1,0 +1,50 @@
+"""The decode kernel's instantiations for rank 16 with 128 state rows and bfloat16 I/O (mixed steps, state-dependent maps, erase
+vectors) against its general one, which a rank table that gives every head the full rank selects: same inputs, two windows.
+
+Bar: both sum at most L + rank + K products in fp32 in different orders, 2e-5 of the largest output; with bfloat16 storage an
+erase vector or an element of the next window's sketch may round to the other side, 2^-8 of it."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_33051_b200 import synth
+from tests import harness
+from tests.test_gpu_parity import make_layer
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("kind", synth.KINDS)
+@pytest.mark.parametrize("V", [64, 128])
+@pytest.mark.parametrize("coef,sketch,erase,mixed", [(None, "f32", False, True), ("pivot", "f32", False, False), ("pivot", "bf16", False, False),
+                                                     ("pivot", "bf16", False, True), (None, "f32", True, False), ("pivot", "bf16", True, False)])
+def test_specialised_and_general_decode_agree(kind, V, coef, sketch, erase, mixed):
+    if erase and kind == "mamba2":
+        pytest.skip("no erase term")
+    w = synth.Workload("t", kind, 21, 3, 128, V, 16, 8, 0, "bf16", 401, basis="qr")
+    outs = []
+    fill = np.arange(w.batch) % w.buf_len if mixed else np.zeros(w.batch, np.int64)
+    for table in (False, True):
+        m, *_rest, dev = make_layer(w, coef=coef, sketch=sketch, erase=erase)
+        if table:
+            m.head_rank = torch.full((w.heads,), 16, dtype=torch.int32, device=dev)
+            m.bind()
+        m.state_update(0)
+        got, o = [], m.new_output()
+        n = np.zeros(w.batch, np.int64)
+        for t in range(2 * w.buf_len):
+            tt = harness.token_tensors(w, synth.step_inputs(w, 0, t), dev)
+            args = (tt["q"], tt["k"], tt["v"], tt["beta"], tt["decay"], o)
+            if mixed:
+                flush = (n == w.buf_len - 1) | ((n == fill) & (t < w.buf_len))
+                m.step_mixed(torch.from_numpy(np.where(flush, -n - 1, n).astype(np.int32)).to(dev), *args)
+                n = np.where(flush, 0, n + 1)
+            elif t % w.buf_len < w.buf_len - 1:
+                m.decode_step(t % w.buf_len, *args)
+            else:
+                m.state_update(t % w.buf_len, *args)
+            got.append(o.cpu().numpy().copy())
+        m.check_status()
+        outs.append(np.stack(got))
+    assert np.all(np.isfinite(outs[0]))
+    assert harness.rel_err(outs[0], outs[1].astype(np.float64)) <= (2.0 ** -8 if sketch == "bf16" else 2e-5)
