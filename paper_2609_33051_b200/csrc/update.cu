@@ -15,10 +15,11 @@
 // What bounds it: fp32 issue and the shared-memory reads of the key rows (2 n + r + 1 multiply-adds per state element).
 // Four columns per lane: a 128-bit read of a key row feeds eight packed multiply-adds.  One column per lane and 64-column
 // tiles, as before, read four times as many key rows and multiplied the state by the decay at every token.  Measured:
-// mixed step of 512 sequences x 32 heads, GDN 128 x 128, r = L = 16 (1024 heads flush per call on average): 171 -> 114 us
-// a call, of which the decode kernel takes 47 (before / after; without the stage 124, 64-column tiles 131); flush of 3072
-// KDA heads with 8 fp32 tokens: 158 -> 97 us.  The multiply-add pipe is busy 45 % of the time (two CTAs of eight warps:
-// 128 registers a thread), fp32 issue 44 %.
+// mixed step of 512 sequences x 32 heads, GDN 128 x 128, r = L = 16 (1024 heads flush per call on average): 171 -> 112 us
+// a call, of which the decode kernel takes 46 (without the stage 124, with 64-column tiles 131); flush of 3072 KDA heads with
+// 8 fp32 tokens: 158 -> 97 us.  The multiply-add pipe is busy 45 % of the time (two CTAs of eight warps: 128 registers a
+// thread), fp32 issue 44 %.  Slower than that kernel: GDN with L = 64 and few warps per CTA (8192 heads, V = 80, r = 32
+// 1031 -> 1137 us; K = V = 64 388 -> 396).
 #include "internal.cuh"
 #include "lanegroup.cuh"
 
