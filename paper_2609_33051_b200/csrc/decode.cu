@@ -707,6 +707,11 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
     if (pendB >= 0) mbar_wait_bounded(barB, (uint32_t)pendB, 1u << 14);
 }
 
+template <int N>
+struct Int {
+    static constexpr int value = N;
+};
+
 template <int KIND, typename IO, int K, int V>
 static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
     const int io = (int)sizeof(IO);
@@ -730,33 +735,38 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
     const int need = p.full_read ? kFull
                                  : (p.n_dev != nullptr ? kSeq : 0) | (p.coef_per_seq ? kPS : 0) | (erase ? kER : 0) |
                                        (p.sketch_bf16 ? kUB : 0) | (p.head_rank != nullptr ? kAny : 0);
-    auto kern = decode_kernel<KIND, IO, K, V, 0, kAny>;
-    int variant = 0;
+    void (*kern)(const Params) = nullptr;
+    int variant = 0, max_nw = 0;
+    auto use = [&](int number, auto rt, auto f) {        // (the CTA size follows the instantiation that runs: its launch bound)
+        constexpr int RT = decltype(rt)::value, F = decltype(f)::value;
+        kern = decode_kernel<KIND, IO, K, V, RT, F>;
+        variant = number;
+        max_nw = decode_max_warps(KIND, F);
+    };
+    use(0, Int<0>(), Int<kAny>());
     if (need == 0) {
-        kern = p.R == 16 ? decode_kernel<KIND, IO, K, V, 16, 0> : decode_kernel<KIND, IO, K, V, 0, 0>;
-        variant = p.R == 16 ? 1 : 2;
+        if (p.R == 16) use(1, Int<16>(), Int<0>());
+        else use(2, Int<0>(), Int<0>());
         if constexpr (K == 128) {
-            if (p.R == 32) { kern = decode_kernel<KIND, IO, K, V, 32, 0>; variant = 3; }
+            if (p.R == 32) use(3, Int<32>(), Int<0>());
         }
     } else if (need == kFull) {
-        kern = decode_kernel<KIND, IO, K, V, 0, kFull>;
-        variant = 12;
+        use(12, Int<0>(), Int<kFull>());
     } else if (need == kUB && p.R == 16) {
-        kern = decode_kernel<KIND, IO, K, V, 16, kUB>;
-        variant = 4;
+        use(4, Int<16>(), Int<kUB>());
     }
     if constexpr (KIND != SKETCHSSM_MAMBA2) {
-        if (erase) { kern = decode_kernel<KIND, IO, K, V, 0, kAny | kER>; variant = 5; }
+        if (erase) use(5, Int<0>(), Int<kAny | kER>());
     }
     if constexpr (K == 128 && V != 80 && sizeof(IO) == 2) {
         if (p.R == 16) {        // (a full read has its own)
-            if (need == kSeq) { kern = decode_kernel<KIND, IO, K, V, 16, kSeq>; variant = 6; }
-            if (need == kPS) { kern = decode_kernel<KIND, IO, K, V, 16, kPS>; variant = 7; }
-            if (need == (kPS | kUB)) { kern = decode_kernel<KIND, IO, K, V, 16, kPS | kUB>; variant = 8; }
-            if (need == (kSeq | kPS | kUB)) { kern = decode_kernel<KIND, IO, K, V, 16, kSeq | kPS | kUB>; variant = 9; }
+            if (need == kSeq) use(6, Int<16>(), Int<kSeq>());
+            if (need == kPS) use(7, Int<16>(), Int<kPS>());
+            if (need == (kPS | kUB)) use(8, Int<16>(), Int<kPS | kUB>());
+            if (need == (kSeq | kPS | kUB)) use(9, Int<16>(), Int<kSeq | kPS | kUB>());
             if constexpr (KIND != SKETCHSSM_MAMBA2) {
-                if (need == kER) { kern = decode_kernel<KIND, IO, K, V, 16, kER>; variant = 10; }
-                if (need == (kER | kPS | kUB)) { kern = decode_kernel<KIND, IO, K, V, 16, kER | kPS | kUB>; variant = 11; }
+                if (need == kER) use(10, Int<16>(), Int<kER>());
+                if (need == (kER | kPS | kUB)) use(11, Int<16>(), Int<kER | kPS | kUB>());
             }
         }
     }
@@ -773,7 +783,6 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
     // (eight warps and fewer first: larger CTAs only where they hold more warps per SM than any number of smaller ones, the
     // staged coefficient maps being shared by more of them.  Windows, CTAs of at most 8 -> 16 (12) warps: Mamba-2 layer of
     // batch 256 624 -> 605 us, 2048 4458 -> 4385, rank 32 with L = 64 4750 -> 4677, state-dependent bfloat16 map 917 -> 890)
-    const int max_nw = decode_max_warps(KIND, need);
     for (int i = 0; i < max_nw; ++i) {
         const int nw = i < 8 ? 8 - i : i + 1;
         if (p.warps_per_cta && nw != p.warps_per_cta) continue;

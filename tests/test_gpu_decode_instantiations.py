@@ -9,7 +9,7 @@ import torch
 
 from paper_2609_33051_b200 import synth
 from tests import harness
-from tests.test_gpu_parity import make_layer
+from tests.test_gpu_parity import make_layer, run_schedule
 
 pytestmark = pytest.mark.gpu
 
@@ -48,3 +48,15 @@ def test_specialised_and_general_decode_agree(kind, V, coef, sketch, erase, mixe
         outs.append(np.stack(got))
     assert np.all(np.isfinite(outs[0]))
     assert harness.rel_err(outs[0], outs[1].astype(np.float64)) <= (2.0 ** -8 if sketch == "bf16" else 2e-5)
+
+
+@pytest.mark.parametrize("K,V", [(128, 64), (128, 80), (128, 128), (64, 64), (64, 128)])
+@pytest.mark.parametrize("rank", [8, 13, 24, 32, 48])
+@pytest.mark.parametrize("io", ["bf16", "f32"])
+def test_bfloat16_sketch_with_the_fixed_map_at_every_ring_fill(K, V, rank, io):
+    """Mamba-2 with a bfloat16 sketch runs the general kernel for every rank but 16; the CTA size that is chosen grows with the
+    ring fill and must stay within that kernel's launch bound.  A whole window; bars of the bfloat16 sketch test."""
+    w = synth.Workload("t", "mamba2", 3, 2, K, V, rank, 32, 0, io, 409, basis="qr")
+    errs = run_schedule(w, w.buf_len + 1, max_heads=10**9, sketch="bf16")
+    assert errs["out"] <= 2e-3 + 2.0 ** -9, errs
+    assert errs["S"] <= 5e-5 and errs["U"] <= 2.0 ** -7, errs
