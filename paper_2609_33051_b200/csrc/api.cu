@@ -108,7 +108,7 @@ int launch_decode(Ctx* ctx, const Params& p, cudaStream_t stream) {
 // The flush kernel for this configuration: the warp-specialised tensor-core kernels where their shape limits allow,
 // the single-group tensor-core kernel for Mamba-2 ranks above 32, CUDA cores otherwise.
 int dispatch_update(sketchssm_ctx* ctx, const Params& p, cudaStream_t cs) {
-    if (p.update_impl != 1) {
+    if (p.update_impl != 1 && p.update_impl < 4) {
         int rc;
         if (p.update_impl != 3) {
             rc = launch_update_tc_ws(ctx, p, cs);

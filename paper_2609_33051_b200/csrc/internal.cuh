@@ -73,7 +73,8 @@ struct Params {
     int warps_per_cta;   // decode: 0 = library default
     int max_warps_per_sm; // decode weights kernel: cap on resident warps per SM (0 = default)
     int update_impl;      // 0: warp-specialised tensor-core kernels where their shape limits allow, CUDA cores otherwise;
-                          // 1: CUDA cores only; 3: single-group tensor-core kernel for Mamba-2, CUDA cores otherwise
+                          // 1: CUDA cores only; 3: single-group tensor-core kernel for Mamba-2, CUDA cores otherwise;
+                          // 4, 5: as 1, the block or (delta rule) the column kernel at every size
     int pdl;              // launch the default decode and the tensor-core update with programmatic dependent launch
     int early_sketch;     // decode: the first head's sketch rows may be requested before the predecessor in the stream is
                           // waited for (no kernel that may still be running writes the sketch)
@@ -104,6 +105,7 @@ int launch_decode_split_gdn_bf16(Ctx* ctx, const Params& p, cudaStream_t stream)
 int launch_decode_split_kda_f32(Ctx* ctx, const Params& p, cudaStream_t stream);
 int launch_decode_split_kda_bf16(Ctx* ctx, const Params& p, cudaStream_t stream);
 int launch_update(Ctx* ctx, const Params& p, cudaStream_t stream);       // CUDA cores, every configuration
+int launch_update_cols(Ctx* ctx, const Params& p, cudaStream_t stream);  // CUDA cores, delta-rule kinds, a thread per quarter column (launch_update chooses)
 int launch_coef_map(Ctx* ctx, const Params& p, cudaStream_t stream);     // state-dependent coefficient maps from S_new and U (after a flush)
 int launch_wait_probe(Ctx* ctx, int poll_limit, int where, cudaStream_t stream);   // self-test: a bounded wait that runs out
 int launch_update_tc(Ctx* ctx, const Params& p, cudaStream_t stream);    // tcgen05 tensor cores, Mamba-2; UNSUPPORTED_SHAPE outside its domain

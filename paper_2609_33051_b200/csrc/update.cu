@@ -18,8 +18,7 @@
 // mixed step of 512 sequences x 32 heads, GDN 128 x 128, r = L = 16 (1024 heads flush per call on average): 171 -> 112 us
 // a call, of which the decode kernel takes 46 (without the stage 124, with 64-column tiles 131); flush of 3072 KDA heads with
 // 8 fp32 tokens: 158 -> 97 us.  The multiply-add pipe is busy 45 % of the time (two CTAs of eight warps: 128 registers a
-// thread), fp32 issue 44 %.  Slower than that kernel: GDN with L = 64 and few warps per CTA (8192 heads, V = 80, r = 32
-// 1031 -> 1137 us; K = V = 64 388 -> 396).
+// thread), fp32 issue 44 %.  Few heads and long GDN windows run update_cols.cu (update_cols_better below).
 #include "internal.cuh"
 #include "lanegroup.cuh"
 
@@ -30,7 +29,9 @@ constexpr int kTok = 8;                 // tokens replayed together
 // Tokens whose key rows are in shared memory at a time.  All rows of a long window at once left room for one CTA per SM or
 // for no stage; every further chunk costs two block barriers.  Flush of 8192 heads in us, 16 / 32 at a time: KDA (two rows
 // per token) V = 64, L = 32 479 / 652; K = V = 64, L = 64 GDN 396 / 422, Mamba-2 196 / 204; GDN V = 80, L = 64, r = 32 1137 /
-// 1229; GDN V = 128, L = 32, r = 32 (no stage either way) 1027 / 969; Mamba-2 V = 64, L = 64 415 / 396.
+// 1229; GDN V = 128, L = 32, r = 32 (no stage either way) 1027 / 969; Mamba-2 V = 64, L = 64 415 / 396.  Chosen
+// by how many CTAs fit instead, GDN gained up to 20 % where the column kernel is faster still, and Mamba-2 with V <= 80 lost (444
+// heads of V = 80, 32 fp32 tokens 25 -> 37 us).
 __host__ __device__ constexpr int update_chunk(int kind, int K, int V) {
     return kind == SKETCHSSM_KDA || K == 64 || (kind == SKETCHSSM_GDN && V == 80) ? 16 : 32;
 }
@@ -660,28 +661,55 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
     if (p.late_wait) grid_dep_wait();
 }
 
+// Where the column kernel (update_cols.cu) is the faster one; delta-rule kinds.  Of this kernel's gains over it the one
+// reduction per eight tokens is small for GDN, whose decay is one multiplication, and the projections do not pay for a replay
+// of many tokens; and a head's time is longer, so it loses where all CTAs wait for the last of few.  Time of this kernel over
+// that of the other, r = 8 to 32, both I/O types, 148 SMs:
+//   at most one tile of 64 columns (V = 80: 80) per SM            1.0 - 1.6   (two tiles per SM: 0.6 - 1.1)
+//   GDN, more than 32 tokens, not 128 x 128                       1.0 - 1.2   (8192 heads; 128 x 128 0.75 - 1.0)
+//   GDN, 17 to 32 tokens, K = 128, V <= 80                        0.95 - 1.1  (8192 heads; K = 64 0.8 - 1.0, up to 16 tokens 0.75 - 0.95)
+//   GDN, one to one and a half rounds of resident CTAs            0.95 - 1.5, median 1.15  (two full rounds 0.86)
+//   KDA, the same, V = 64 or K = 64                               0.95 - 1.4, median 1.07  (two full rounds 0.77)
+// Ranks above 32 outweigh the replay again, unless there is no room for the stage (bfloat16 rows read from global memory:
+// 64 tokens, r = 64, V = 80 1520 us against 1256).  Per-sequence phases: how many sequences flush is not known here, so only
+// the first line counts.
+static bool update_cols_better(const Ctx* ctx, const Params& p, int n_tot, size_t wave) {
+    const size_t heads = (size_t)p.B * p.H;
+    if (heads * (p.dv == 128 ? 2 : 1) <= (size_t)ctx->sm_count) return true;
+    if (p.n_dev != nullptr) return false;
+    const bool kda = ctx->cfg.kind == SKETCHSSM_KDA;
+    if (heads > wave && 2 * heads <= 3 * wave && (!kda || p.dv == 64 || p.dk == 64)) return true;
+    if (kda || (p.R > 32 && (p.stages || ctx->cfg.io_dtype != SKETCHSSM_BF16))) return false;
+    return p.dk == 128 && p.dv == 128 ? false : n_tot > (p.dk == 128 ? 16 : 32);
+}
+
 template <int KIND, typename IO, int K, int V>
 static int launch_update_t(Ctx* ctx, Params p, cudaStream_t stream) {
     const int n_tot = p.n_before + (p.has_token ? 1 : 0);
     const bool mixed = p.n_dev != nullptr;
     if (mixed) p.n_cap = n_tot;        // per-sequence phases: n_before is the largest fill any sequence may have
-    // Staging one head ahead wherever two CTAs per SM fit with the stage, even if more would fit without: flush of 8192 KDA
-    // heads with V = 64, L = 16 304 us against 326 (GDN, where three fit, 271 against 317; V = 80 345 against 408).
-    UpdateSmem us = make_update_smem<K>(KIND, n_tot, p.R, V, p.L, (int)sizeof(IO), mixed, 1);
-    p.stages = us.total + 1024u <= (228u * 1024u) / 2u ? 1 : 0;
-    if (!p.stages) us = make_update_smem<K>(KIND, n_tot, p.R, V, p.L, (int)sizeof(IO), mixed, 0);
-    auto kern = update_kernel<KIND, IO, K, V>;
-    if (us.total > 226u * 1024u) return SKETCHSSM_UNSUPPORTED_SHAPE;
-    if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     if (ctx->sm_count == 0) {
         int sms = 0;
         if ((ctx->last_cuda_error = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->cfg.device)) != cudaSuccess)
             return SKETCHSSM_CUDA_ERROR;
         ctx->sm_count = sms;
     }
+    // Staging one head ahead wherever two CTAs per SM fit with the stage, even if more would fit without: flush of 8192 KDA
+    // heads with V = 64, L = 16 304 us against 326 (GDN, where three fit, 271 against 317; V = 80 345 against 408).
+    UpdateSmem us = make_update_smem<K>(KIND, n_tot, p.R, V, p.L, (int)sizeof(IO), mixed, 1);
+    p.stages = us.total + 1024u <= (228u * 1024u) / 2u ? 1 : 0;
+    if (!p.stages) us = make_update_smem<K>(KIND, n_tot, p.R, V, p.L, (int)sizeof(IO), mixed, 0);
+    if (us.total > 226u * 1024u) return SKETCHSSM_UNSUPPORTED_SHAPE;
+    int by_smem = (int)((228u * 1024u) / (us.total + 1024u));
+    by_smem = by_smem < 1 ? 1 : by_smem < update_ctas<V>() ? by_smem : update_ctas<V>();
+    const size_t wave = (size_t)ctx->sm_count * (size_t)by_smem;
+    if (KIND != SKETCHSSM_MAMBA2 && p.update_impl != 4 && (p.update_impl == 5 || update_cols_better(ctx, p, n_tot, wave))) {
+        const int rc = launch_update_cols(ctx, p, stream);
+        if (rc != SKETCHSSM_UNSUPPORTED_SHAPE) return rc;
+    }
+    auto kern = update_kernel<KIND, IO, K, V>;
+    if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     size_t grid = (size_t)p.B * p.H;
-    const int by_smem = (int)((228u * 1024u) / (us.total + 1024u));
-    const size_t wave = (size_t)ctx->sm_count * (size_t)(by_smem < 1 ? 1 : by_smem < update_ctas<V>() ? by_smem : update_ctas<V>());
     if (grid > wave) grid = wave;
     if ((ctx->last_cuda_error = launch_kernel(kern, dim3((unsigned)grid), dim3(2 * V), us.total, stream, p, p.pdl != 0)) != cudaSuccess)
         return SKETCHSSM_CUDA_ERROR;

@@ -98,3 +98,61 @@ def test_mixed_step_over_many_sequences(kind):
     assert harness.rel_err(m.state.cpu().numpy(), S) <= BAR
     U = orc.sketch_of(S, np.broadcast_to(Om64, (w.batch,) + Om64.shape))
     assert harness.rel_err(m.sketch.cpu().numpy().transpose(0, 1, 3, 2), U) <= BAR
+
+
+@pytest.mark.parametrize("impl", [4, 5], ids=["eight_tokens", "columns"])
+@pytest.mark.parametrize("kind", ["gdn", "kda"])
+@pytest.mark.parametrize("K,V,rank,L,io", [(128, 128, 16, 20, "bf16"), (128, 64, 13, 20, "f32"), (128, 80, 5, 20, "bf16"),
+                                           (64, 128, 32, 20, "f32"), (64, 64, 8, 20, "bf16"), (128, 128, 64, 64, "f32"), (128, 80, 16, 64, "bf16")])
+def test_both_delta_rule_kernels(kind, K, V, rank, L, io, impl):
+    """The kernel that replays eight tokens together and the one that replays them singly, whichever the sizes would select."""
+    w = synth.Workload("t", kind, 3, 2, K, V, rank, L, 0, io, 229, basis="qr")
+    m, S0, Om, _C, _ = make_layer(w)
+    m.tune("update_impl", impl)
+    for n, token in [(0, False), (0, True), (3, True), (4, True), (7, True), (8, False), (8, True), (16, True), (L - 1, True), (L, False)]:
+        _flush(m, w, S0, Om, n, token)
+
+
+@pytest.mark.parametrize("kind,B,H,K,V,L", [("gdn", 37, 2, 128, 128, 8), ("gdn", 75, 2, 128, 128, 8), ("gdn", 37, 4, 128, 80, 8), ("gdn", 150, 1, 128, 64, 20),
+                                            ("gdn", 300, 2, 64, 64, 36), ("gdn", 89, 5, 128, 128, 8), ("kda", 37, 4, 64, 64, 8), ("kda", 30, 5, 64, 64, 8)])
+def test_either_side_of_the_rule_between_them(kind, B, H, K, V, L):
+    w = synth.Workload("t", kind, B, H, K, V, 8, L, 0, "f32", 233, basis="qr")
+    m, S0, Om, _C, _ = make_layer(w)
+    _flush(m, w, S0, Om, L - 1, True)
+
+
+@pytest.mark.parametrize("impl", [4, 5], ids=["eight_tokens", "columns"])
+@pytest.mark.parametrize("kind", synth.KINDS)
+@pytest.mark.parametrize("K,V,L,io", [(64, 64, 20, "f32"), (128, 128, 64, "f32"), (128, 80, 36, "bf16")])
+def test_mixed_step_with_fills_around_the_chunks(kind, K, V, L, io, impl):
+    """Windows of more tokens than a chunk: sequences flush and decode at fills on both sides of 16 and 32 in one call."""
+    fills = [n for n in (0, 6, 7, 8, 14, 15, 16, 17, 18, 30, 31, 32, 33, 47, 48, 62, 63) if n < L]
+    w = synth.Workload("t", kind, 2 * len(fills), 2, K, V, 8, L, 0, io, 239, basis="qr")
+    m, S0, Om, C, dev = make_layer(w)
+    m.tune("update_impl", impl)
+    m.state_update(0)
+    fill, flush = np.repeat(fills, 2), np.tile([True, False], len(fills))
+    xs = [synth.step_inputs(w, 0, t) for t in range(L)]
+    m.ring.fill_(255)                                          # stale slots hold NaNs
+    for view, name in zip(m.ring_views(), ("k", "v", "beta", "decay")):
+        for t in range(L):
+            held = torch.from_numpy(np.nonzero(fill > t)[0]).to(dev)
+            view[held, :, t] = harness.token_tensors(w, xs[t], dev)[name][held]
+    x = synth.step_inputs(w, 0, 99)
+    tt = harness.token_tensors(w, x, dev)
+    o = m.new_output()
+    m.step_mixed(torch.from_numpy(np.where(flush, -fill - 1, fill).astype(np.int32)).to(dev), *(tt[n] for n in ("q", "k", "v", "beta", "decay")), o)
+    m.check_status()
+    Om64, C64 = Om.astype(np.float64), C.astype(np.float64)
+    S, ref = S0.astype(np.float64), np.empty((w.batch, w.heads, V))
+    for b in range(w.batch):
+        toks = [tuple(y[g][b].astype(np.float64) for g in ("k", "v", "beta", "decay")) for y in xs[:fill[b]] + [x]]
+        q = x["q"][b].astype(np.float64)
+        if flush[b]:
+            S[b], _U, ref[b] = orc.state_update(kind, S[b], toks, Om64, q)
+        else:
+            ref[b] = orc.decode_step(kind, orc.sketch_of(S[b], Om64), C64, toks, q)
+    assert harness.rel_err(o.cpu().numpy(), ref) <= BAR
+    assert harness.rel_err(m.state.cpu().numpy(), S) <= BAR
+    U = orc.sketch_of(S, np.broadcast_to(Om64, (w.batch,) + Om64.shape))
+    assert harness.rel_err(m.sketch.cpu().numpy().transpose(0, 1, 3, 2), U) <= BAR
