@@ -616,8 +616,9 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
                     // (with bfloat16 storage the vectors are rounded once, where they are stored; this step uses the rounded f_t too)
                     const float* sF = reinterpret_cast<const float*>(sb + sl.f_off);
                     const __nv_bfloat16* sF16 = reinterpret_cast<const __nv_bfloat16*>(sb + sl.f_off);
-                    // Up to 16 coefficients: the two halves of the warp take every other slot.
-                    const bool two = (RT ? RT : rk) <= 16;
+                    // Up to 16 coefficients, known at compile time: the two halves of the warp take every other slot.  (Decided at
+                    // run time it cost the general kernels more than it gave, 3 to 5 % of a launch.)
+                    constexpr bool two = RT != 0 && RT <= 16;
                     const int s_first = two ? lane >> 4 : 0, s_step = two ? 2 : 1;
                     for (int g = two ? lane & 15 : lane; g < (two ? 16 : rk); g += 32) {
                         const bool on = g < rk;
@@ -667,7 +668,10 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
             __syncwarp();
             if (vlane) {
                 const float* Sg = p.state + bh * (size_t)K * V + lane * EV;
-                constexpr int RB = 32 / EV;              // rows in flight: 32 registers (V = 64: 16; 75 us against 79 with 8)
+                // rows in flight: 32 registers (V = 64: 16; 75 us against 79 with 8).  The general kernel for K = V = 64 has no
+                // room for 16: 60 bytes spilled instead of 12, with erase vectors 276 instead of 100, which all its heads paid
+                // for (8192 heads, GDN, 24 buffered tokens, r = 24: 56 us a launch, with both changes 45).
+                constexpr int RB = ANY && K == 64 ? 8 : 32 / EV;
                 for (int i0 = 0; i0 < K; i0 += RB) {
                     if (ANY && lane == 0 && i0 + kAhead < K)
                         prefetch_l2(p.state + (bh * K + i0 + kAhead) * V, (uint32_t)(RB * V * 4));
