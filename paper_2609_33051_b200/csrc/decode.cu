@@ -336,10 +336,15 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
         const bool er_h = er && !full;       // this head forms c_t from projected erase vectors
         // A dense-fallback head among sketched ones takes its rows through registers, a few at a time, and would finish long
         // after the others: the rows after those are asked into L2 (the first ones during the sweep, kAhead rows ahead: at
-        // most 57 MB over all resident warps, within the 126 MB of L2).  Where every head reads its state the bytes in
-        // flight suffice without that, and the requests cost time (window of fp32 KDA full reads, 3072 heads: 440 -> 479 us).
+        // most 57 MB over all resident warps, within the 126 MB of L2).  A line per lane: as bulk copies the requests went
+        // through the unit that also brings the next heads' operands (64 heads, 8 of them dense, GDN 128 x 128, three
+        // buffered tokens, state in L2: 7.2 us without requests, 9.6 with bulk ones, 8.2; state not in L2: 0.67 to 0.93 of
+        // the time without).  Where every head reads its state the bytes in flight suffice without that, and the requests cost time
+        // (window of fp32 KDA full reads, 3072 heads: 440 -> 479 us).
         constexpr int kAhead = 32;
-        if (ANY && full && lane == 0) prefetch_l2(p.state + bh * (size_t)K * V, (uint32_t)(kAhead * V * 4));
+        if (ANY && full) {
+            for (int line = lane; line < kAhead * V / 32; line += 32) prefetch_l2_line(p.state + bh * (size_t)K * V + 32 * line);
+        }
 
         if (__any_sync(0xffffffffu, !DEC_WAIT(barA, parA))) {
             if (lane == 0) record_fault(p.status, FULL ? kFaultFullReadWait : kFaultDecodeWait, (int)blockIdx.x);
@@ -673,8 +678,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
                 // for (8192 heads, GDN, 24 buffered tokens, r = 24: 56 us a launch, with both changes 45).
                 constexpr int RB = ANY && K == 64 ? 8 : 32 / EV;
                 for (int i0 = 0; i0 < K; i0 += RB) {
-                    if (ANY && lane == 0 && i0 + kAhead < K)
-                        prefetch_l2(p.state + (bh * K + i0 + kAhead) * V, (uint32_t)(RB * V * 4));
+                    if (ANY && i0 + kAhead < K && lane < RB * V / 32) prefetch_l2_line(p.state + (bh * K + i0 + kAhead) * V + 32 * lane);
                     float rows[RB][EV];
 #pragma unroll
                     for (int r = 0; r < RB; ++r) load_io<EV>(Sg, (i0 + r) * V, rows[r]);

@@ -57,9 +57,9 @@ __device__ __forceinline__ void store_row(T* row, int j, const float (&s)[E]) {
     for (int m = 0; m < E / 4; ++m) st4(row + 4 * (j + LPH * m), &s[4 * m]);
 }
 
-// Ask L2 to fetch a byte range (16-byte aligned, size a multiple of 16) without occupying shared memory.
-__device__ __forceinline__ void prefetch_l2(const void* src, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+// Ask L2 to fetch the 128-byte line of an address.
+__device__ __forceinline__ void prefetch_l2_line(const void* src) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(src));      // (touches nothing that a load could see: none is held back for it)
 }
 
 template <int LPH>
