@@ -787,12 +787,16 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
         regs = fa.numRegs > 0 ? fa.numRegs : 64;
     }
     const int reg_warps = 65536 / (regs * 32);          // warps the register file holds
+    const long long heads = (long long)p.B * p.H;
     int best_nw = 0, best_ctas = 1, best_warps = 0;
     // (eight warps and fewer first: larger CTAs only where they hold more warps per SM than any number of smaller ones, the
     // staged coefficient maps being shared by more of them.  Windows, CTAs of at most 8 -> 16 (12) warps: Mamba-2 layer of
-    // batch 256 624 -> 605 us, 2048 4458 -> 4385, rank 32 with L = 64 4750 -> 4677, state-dependent bfloat16 map 917 -> 890)
+    // batch 256 624 -> 605 us, 2048 4458 -> 4385, rank 32 with L = 64 4750 -> 4677, state-dependent bfloat16 map 917 -> 890.  With
+    // fewer heads than warps fit, larger CTAs only leave more SMs idle: general kernel, 64 heads, 4.2 -> 4.9 us; the lean ones,
+    // whose CTAs stage less per head, did not lose by it)
     for (int i = 0; i < max_nw; ++i) {
         const int nw = i < 8 ? 8 - i : i + 1;
+        if (nw > 8 && variant == 0 && heads <= (long long)ctx->sm_count * best_warps) break;
         if (p.warps_per_cta && nw != p.warps_per_cta) continue;
         const DecodeSmem d = make_decode_smem(K, p.R, nw, p.full_read, p.coef_per_seq, sl.total);
         if (d.total > smem_budget) continue;
