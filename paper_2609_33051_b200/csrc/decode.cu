@@ -797,7 +797,7 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
     for (int i = 0; i < max_nw; ++i) {
         const int nw = i < 8 ? 8 - i : i + 1;
         if (nw > 8 && variant == 0 && heads <= (long long)ctx->sm_count * best_warps) break;
-        if (p.warps_per_cta && nw != p.warps_per_cta) continue;
+        if (p.warps_per_cta && (nw != p.warps_per_cta || nw > 8)) continue;       // (a caller's own choice: 1 to 8)
         const DecodeSmem d = make_decode_smem(K, p.R, nw, p.full_read, p.coef_per_seq, sl.total);
         if (d.total > smem_budget) continue;
         int ctas = (int)((228u * 1024u) / (d.total + 1024u));

@@ -60,3 +60,23 @@ def test_bfloat16_sketch_with_the_fixed_map_at_every_ring_fill(K, V, rank, io):
     errs = run_schedule(w, w.buf_len + 1, max_heads=10**9, sketch="bf16")
     assert errs["out"] <= 2e-3 + 2.0 ** -9, errs
     assert errs["S"] <= 5e-5 and errs["U"] <= 2.0 ** -7, errs
+
+
+@pytest.mark.parametrize("call", ["decode_step", "full_read_decode"])
+def test_a_callers_warp_count_is_taken_up_to_eight_and_refused_above(call):
+    from paper_2609_33051_b200.binding import SketchSSMError
+    w = synth.Workload("t", "mamba2", 4, 2, 128, 64, 16, 8, 0, "bf16", 419, basis="qr")
+    m, *_rest, dev = make_layer(w)
+    m.state_update(0)
+    tt = harness.token_tensors(w, synth.step_inputs(w, 0, 0), dev)
+    args, outs = (tt["q"], tt["k"], tt["v"], tt["beta"], tt["decay"]), []
+    for nw in (1, 8):
+        m.tune("decode_warps_per_cta", nw)
+        outs.append(getattr(m, call)(0, *args, m.new_output()).clone())
+    assert torch.equal(*outs)
+    for nw in (9, 12, 16, 17):
+        m.tune("decode_warps_per_cta", nw)
+        with pytest.raises(SketchSSMError) as e:
+            getattr(m, call)(0, *args, m.new_output())
+        assert e.value.status == -2
+    m.check_status()
