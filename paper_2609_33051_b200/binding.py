@@ -100,6 +100,9 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     return lib
 
 
+_RAW_STREAM, _DEVICE = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
     return None if t is None else t.data_ptr()       # (the declared argument types make the C pointer of it)
 
@@ -182,9 +185,13 @@ class SketchSSM:
 
     @staticmethod
     def _stream(stream) -> int:
-        """The stream's handle; None: the current stream of the current device (read without building a Stream object,
-        which costs as much as the rest of a call's marshalling)."""
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
+        """The stream's handle; None: the current stream of the current device (where torch offers it, read without
+        building a Stream object, which costs as much as the rest of a call's marshalling)."""
+        if stream is not None:
+            return stream.cuda_stream
+        if _RAW_STREAM is None or _DEVICE is None:
+            return torch.cuda.current_stream().cuda_stream
+        return _RAW_STREAM(_DEVICE())
 
     def new_output(self) -> torch.Tensor:
         return torch.empty(self.B, self.H, self.V, dtype=TORCH_DTYPE[self.out], device=self.device)

@@ -99,3 +99,13 @@ def test_logical_layers_map_onto_the_physical_slots_that_fit():
     assert bench.update_kernel_name(w) == "update_tc_ws_mamba2_kernel"
     assert bench.update_kernel_name(synth.CONFIGS["c4_kda"]) == "update_tc_ws_kda_kernel"
     assert bench.update_kernel_name(synth.CONFIGS["c1_gdn_tiny"]) == "update_kernel"
+
+
+def test_current_stream_without_the_raw_stream_functions(monkeypatch):
+    """torch's raw stream functions are private: where a version lacks them the public call gives the handle."""
+    from types import SimpleNamespace
+    from paper_2609_33051_b200 import binding
+    monkeypatch.setattr(binding, "_RAW_STREAM", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=1234))
+    assert binding.SketchSSM._stream(None) == 1234
+    assert binding.SketchSSM._stream(SimpleNamespace(cuda_stream=77)) == 77
