@@ -130,9 +130,8 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
     const int RP = (R + 7) & ~7;
     // c_t from the projected erase vectors of the buffered tokens instead of the swept query (delta-rule kinds)
     constexpr bool ER = (F & kER) != 0;
-    constexpr bool er = ER;
 
-    const StageLayout sl = make_stage_layout(KIND, (int)sizeof(IO), K, V, R, L, n_cap, FULL, per_seq, su, er);
+    const StageLayout sl = make_stage_layout(KIND, (int)sizeof(IO), K, V, R, L, n_cap, FULL, per_seq, su, ER);
     const DecodeSmem ds = make_decode_smem(K, R, nwarps, FULL, per_seq, sl.total);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + ds.bar_off) + warp * 2;
     float* sX = reinterpret_cast<float*>(smem + ds.scratch_off + (size_t)warp * ds.scratch_stride);   // c or q~
@@ -199,7 +198,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
         case 7: cp_base = p.ring + p.rl.decay_off; cp_stride = p.rl.head_bytes; cp_dst = sl.g_off; cp_unit = KIND == SKETCHSSM_KDA ? (uint32_t)(K * sizeof(IO)) : 0u; cp_mode = 1; break;
         case 8: cp_base = reinterpret_cast<const unsigned char*>(p.sketch); cp_stride = (size_t)R * V * su; cp_dst = sl.u_off; cp_unit = (uint32_t)(V * su); cp_mode = 3; break;
         case 9: cp_base = reinterpret_cast<const unsigned char*>(p.coef); cp_stride = (size_t)R * K * su; cp_dst = sl.c_off; cp_unit = per_seq ? (uint32_t)(K * su) : 0u; cp_mode = 3; break;
-        case 10: cp_base = reinterpret_cast<const unsigned char*>(p.erase); cp_stride = (size_t)L * R * su; cp_dst = sl.f_off; cp_unit = er ? (uint32_t)(R * su) : 0u; cp_mode = 1; break;
+        case 10: cp_base = reinterpret_cast<const unsigned char*>(p.erase); cp_stride = (size_t)L * R * su; cp_dst = sl.f_off; cp_unit = ER ? (uint32_t)(R * su) : 0u; cp_mode = 1; break;
         default: break;
     }
     const uint32_t tokA = 2u * sl.tqk_bytes + sl.tv_bytes + sl.tg_bytes;
@@ -211,7 +210,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
     const uint32_t cp_fixed = cp_mode == 0 ? cp_unit : cp_mode == 1 ? cp_unit * (uint32_t)n_cap
                             : cp_mode == 2 ? (n_cap > 0 ? cp_unit : 0u) : cp_unit * (uint32_t)r_uni;
     const uint32_t txA_fixed = tokA + (uint32_t)n_cap * rowA + (n_cap > 0 ? gateA : 0u);
-    const uint32_t txB_fixed = (uint32_t)r_uni * rowB + (er ? (uint32_t)(n_cap * R * su) : 0u);
+    const uint32_t txB_fixed = (uint32_t)r_uni * rowB + (ER ? (uint32_t)(n_cap * R * su) : 0u);
     uint64_t* barA = &bars[0];
     uint64_t* barB = &bars[1];
     auto issue_a = [&](size_t bh, int n_it) {      // whole warp; n_it: ring fill of the head
@@ -229,7 +228,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
     // whole warp; r_it: sketch rank of the head (0: nothing to fetch), n_it: its ring fill (rows of erase vectors)
     auto issue_b = [&](size_t bh, int r_it, int n_it) {
         if constexpr (DYN) {
-            const uint32_t fbytes = er ? (uint32_t)n_it * (uint32_t)(R * su) : 0u;
+            const uint32_t fbytes = ER ? (uint32_t)n_it * (uint32_t)(R * su) : 0u;
             if (lane == 8 && r_it > 0) mbar_expect_tx(barB, (uint32_t)r_it * rowB + fbytes);
             __syncwarp();
             if ((lane == 8 || lane == 9) && cp_unit && r_it > 0)
@@ -333,7 +332,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
             }
         }
         const bool full = ANY ? rk == 0 : FULL;   // exact read of the whole state for this head
-        const bool er_h = er && !full;       // this head forms c_t from projected erase vectors
+        const bool er_h = ER && !full;       // this head forms c_t from projected erase vectors
         // A dense-fallback head among sketched ones takes its rows through registers, a few at a time, and would finish long
         // after the others: the rows after those are asked into L2 (the first ones during the sweep, kAhead rows ahead: at
         // most 57 MB over all resident warps, within the 126 MB of L2).  A line per lane: as bulk copies the requests went

@@ -278,246 +278,245 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
         // kChunk tokens at a time: their rows -> shared memory (fp32), then the replay
 #pragma unroll 1
         for (int c0 = 0; c0 == 0 || c0 < n_tot; c0 += kChunk) {
-        const int n_here = min(n_tot - c0, kChunk), nb = (n_here + kTok - 1) / kTok;
-        const bool last = c0 + kChunk >= n_tot;
-        if (c0 > 0) __syncthreads();                 // the previous tokens' rows have been read
-        if constexpr (DELTA) {
-            // a thread per (eight tokens, channel)
-            for (int idx = tid; idx < nb * K; idx += T) {
-                const int blk = idx / K, i = idx % K;
-                float k[kTok], g[kTok];
-#pragma unroll
-                for (int s = 0; s < kTok; ++s) {
-                    const int t = c0 + blk * kTok + s;
-                    k[s] = 0.f;
-                    g[s] = 1.f;
-                    if (t < n_ring) {
-                        k[s] = static_cast<float>(rk[(size_t)t * K + i]);
-                        g[s] = KDA ? static_cast<float>(reinterpret_cast<const IO*>(rdec)[(size_t)t * K + i]) : rdec[t];
-                    } else if (t < n_tot) {
-                        k[s] = static_cast<float>(tk[i]);
-                        g[s] = KDA ? static_cast<float>(tg[i]) : *tdec;
-                    }
-                }
-                const int at = blk * kTok * KS + PR::at(i);
-                float pre = 1.f, suf = 1.f;
-                if constexpr (KDA) {
+            const int n_here = min(n_tot - c0, kChunk), nb = (n_here + kTok - 1) / kTok;
+            const bool last = c0 + kChunk >= n_tot;
+            if (c0 > 0) __syncthreads();                 // the previous tokens' rows have been read
+            if constexpr (DELTA) {
+                // a thread per (eight tokens, channel)
+                for (int idx = tid; idx < nb * K; idx += T) {
+                    const int blk = idx / K, i = idx % K;
+                    float k[kTok], g[kTok];
 #pragma unroll
                     for (int s = 0; s < kTok; ++s) {
-                        pre *= g[s];
-                        sKh[at + s * KS] = pre * k[s];
+                        const int t = c0 + blk * kTok + s;
+                        k[s] = 0.f;
+                        g[s] = 1.f;
+                        if (t < n_ring) {
+                            k[s] = static_cast<float>(rk[(size_t)t * K + i]);
+                            g[s] = KDA ? static_cast<float>(reinterpret_cast<const IO*>(rdec)[(size_t)t * K + i]) : rdec[t];
+                        } else if (t < n_tot) {
+                            k[s] = static_cast<float>(tk[i]);
+                            g[s] = KDA ? static_cast<float>(tg[i]) : *tdec;
+                        }
                     }
-                    sG[blk * KS + PR::at(i)] = pre;
-#pragma unroll
-                    for (int s = kTok - 1; s >= 0; --s) {
-                        sKt[at + s * KS] = suf * k[s];
-                        suf *= g[s];
-                    }
-                } else {
-#pragma unroll
-                    for (int s = 0; s < kTok; ++s) sKt[at + s * KS] = k[s];
-                    if (i == 0) {                // scalar decays are applied to the dot products and the e instead
+                    const int at = blk * kTok * KS + PR::at(i);
+                    float pre = 1.f, suf = 1.f;
+                    if constexpr (KDA) {
 #pragma unroll
                         for (int s = 0; s < kTok; ++s) {
                             pre *= g[s];
-                            sPre[blk * kTok + s] = pre;
+                            sKh[at + s * KS] = pre * k[s];
                         }
+                        sG[blk * KS + PR::at(i)] = pre;
 #pragma unroll
                         for (int s = kTok - 1; s >= 0; --s) {
-                            sSuf[blk * kTok + s] = suf;
+                            sKt[at + s * KS] = suf * k[s];
                             suf *= g[s];
+                        }
+                    } else {
+#pragma unroll
+                        for (int s = 0; s < kTok; ++s) sKt[at + s * KS] = k[s];
+                        if (i == 0) {                // scalar decays are applied to the dot products and the e instead
+#pragma unroll
+                            for (int s = 0; s < kTok; ++s) {
+                                pre *= g[s];
+                                sPre[blk * kTok + s] = pre;
+                            }
+#pragma unroll
+                            for (int s = kTok - 1; s >= 0; --s) {
+                                sSuf[blk * kTok + s] = suf;
+                                suf *= g[s];
+                            }
+                        }
+                    }
+                    // this channel's term of every A_sj, summed over the warp's 32 channels: lane l ends up with pair l
+                    float w[kTok], pr[kPairs];
+#pragma unroll
+                    for (int s = 0; s < kTok; ++s) {
+#pragma unroll
+                        for (int j = 0; j < s; ++j) {
+                            w[j] *= g[s];
+                            pr[s * (s - 1) / 2 + j] = k[s] * w[j];
+                        }
+                        w[s] = k[s];
+                    }
+#pragma unroll
+                    for (int i2 = kTok * (kTok - 1) / 2; i2 < kPairs; ++i2) pr[i2] = 0.f;
+                    group_reduce_transpose<32, kPairs>(pr, lane);
+                    sGram[(blk * (K / 32) + i / 32) * kPairs + lane] = pr[0];
+                }
+                for (int s = tid; s < nb * kTok; s += T) sBeta[s] = c0 + s < n_ring ? rbeta[c0 + s] : c0 + s < n_tot ? *tbeta : 0.f;
+            } else {
+                for (int idx = tid; idx < n_here * (K / 4); idx += T) {
+                    const int s = idx / (K / 4), i = 4 * (idx % (K / 4));
+                    float k[4];
+                    ld4(c0 + s < n_ring ? rk + (size_t)(c0 + s) * K + i : tk + i, k);
+                    st4(sKt + s * KS + PR::at(i), k);
+                }
+                // w_s = beta_s prod_{j>s} a_j and the total decay, by a warp scan over up to 64 tokens
+                if (warp == 0 && c0 == 0) {
+                    float a[2], bt[2];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int s = lane + 32 * u;
+                        a[u] = s < n_ring ? rdec[s] : s < n_tot ? *tdec : 1.f;
+                        bt[u] = s < n_ring ? rbeta[s] : s < n_tot ? *tbeta : 0.f;
+                    }
+                    float after = 1.f;               // product of the decays behind this half
+#pragma unroll
+                    for (int u = 1; u >= 0; --u) {
+                        float incl = a[u];
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const float other = __shfl_down_sync(0xffffffffu, incl, o);
+                            if (lane + o < 32) incl *= other;
+                        }
+                        float excl = __shfl_down_sync(0xffffffffu, incl, 1);
+                        if (lane == 31) excl = 1.f;
+                        if (lane + 32 * u < n_tot) sBeta[lane + 32 * u] = bt[u] * (excl * after);
+                        after *= __shfl_sync(0xffffffffu, incl, 0);
+                    }
+                    if (lane == 0) sPre[0] = after;
+                }
+            }
+            {
+                constexpr int PV = 16 / (int)sizeof(IO), in_row = V / PV;        // 16-byte units
+                const uint4* ring_v = reinterpret_cast<const uint4*>(rv);
+                const uint4* tok_v = reinterpret_cast<const uint4*>(tv);
+                for (int idx = tid; idx < n_here * in_row; idx += T) {
+                    const int at = c0 * in_row + idx;
+                    reinterpret_cast<uint4*>(sV)[idx] = at < n_ring * in_row ? ring_v[at] : tok_v[at - n_ring * in_row];
+                }
+            }
+            if (p.q != nullptr && c0 == 0) {
+                for (int i = tid; i < K / 4; i += T) {
+                    float q[4];
+                    ld4(tq + 4 * i, q);
+                    st4(sQ + PR::at(4 * i), q);
+                }
+            }
+            if (p.write_sketch && h != h_staged) {
+                const float* og = p.omega + (size_t)h * K * R;
+#pragma unroll 4
+                for (int idx = tid; idx < K * R; idx += T) {
+                    const int i = idx / R, g = idx % R;
+                    sOm[g * OS + PR::at(i)] = og[idx];
+                }
+                for (int idx = tid; idx < (R8 - R) * K; idx += T) sOm[(R + idx / K) * OS + PR::at(idx % K)] = 0.f;
+                h_staged = h;
+            }
+            // (every thread's wait on the stage; a CTA that gives up leaves its heads as they are)
+            if (__syncthreads_or(failed)) {
+                failed = true;
+                return;
+            }
+            if (staged && last && tid == 0 && n_next >= 0) request(b_next, h_next, n_next);
+            if constexpr (DELTA) {
+                // beta_s A_sj
+                for (int idx = tid; idx < nb * kPairs; idx += T) {
+                    const int blk = idx / kPairs, pair = idx % kPairs;
+                    float a = 0.f;
+#pragma unroll
+                    for (int c = 0; c < K / 32; ++c) a += sGram[(blk * (K / 32) + c) * kPairs + pair];
+                    int s = 1;
+                    while (s < kTok && (s + 1) * s / 2 <= pair) ++s;      // the pair's later token
+                    sA[idx] = s < kTok ? sBeta[blk * kTok + s] * a : 0.f;
+                }
+                __syncthreads();
+            }
+
+            if constexpr (!DELTA) {
+                if (n_tot > 0 && c0 == 0) {
+                    const f32x2 d2 = pack2(sPre[0], sPre[0]);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int i = 0; i < RP / 2; ++i) c2[c][i] = mul2(c2[c][i], d2);
+                }
+            }
+            for (int blk = 0; blk < nb; ++blk) {
+                const int s0 = blk * kTok;
+                const int nt = min(kTok, n_here - s0);
+                const int mine = s0 + part;              // this lane's token where a lane stands for one
+                float x[4];
+                if constexpr (DELTA) {
+                    float vals[32];
+                    const float* kh = (KDA ? sKh : sKt) + s0 * KS + row;
+                    dot4<RP>(c2, kh, KS, vals);
+                    if (nt > 4) {
+                        dot4<RP>(c2, kh + 4 * KS, KS, vals + 16);
+                    } else {
+#pragma unroll
+                        for (int i = 16; i < 32; ++i) vals[i] = 0.f;
+                    }
+                    reduce_parts(vals, lane);
+                    float v[4] = {0.f, 0.f, 0.f, 0.f};
+                    if (mine < n_here) ld4(sV + mine * V + j0, v);
+                    const float bt = sBeta[mine], pre = KIND == SKETCHSSM_GDN ? sPre[mine] : 1.f;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        x[c] = mine < n_here ? bt * (v[c] - (KIND == SKETCHSSM_GDN ? pre * vals[c] : vals[c])) : 0.f;
+                } else {
+                    float v[4] = {0.f, 0.f, 0.f, 0.f};
+                    if (mine < n_here) ld4(sV + mine * V + j0, v);
+                    const float w = mine < n_here ? sBeta[c0 + mine] : 0.f;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) x[c] = w * v[c];
+                }
+                __syncwarp();                            // the previous block's e have been read
+                st4(sE + part * 16 + (lane & 3) * 4, x);
+                __syncwarp();
+                if constexpr (DELTA) {
+                    // forward substitution, one column per lane
+                    if (lane < 16) {
+                        float e[kTok], a[kPairs];
+#pragma unroll
+                        for (int s = 0; s < kTok; ++s) e[s] = sE[s * 16 + lane];
+#pragma unroll
+                        for (int i = 0; i < kPairs / 4 - 1; ++i) ld4(sA + blk * kPairs + 4 * i, a + 4 * i);
+#pragma unroll
+                        for (int j = 0; j < kTok - 1; ++j) {
+#pragma unroll
+                            for (int s = j + 1; s < kTok; ++s) e[s] = fmaf(-a[s * (s - 1) / 2 + j], e[j], e[s]);
+                        }
+#pragma unroll
+                        for (int s = 0; s < kTok; ++s) sE[s * 16 + lane] = KIND == SKETCHSSM_GDN ? sSuf[s0 + s] * e[s] : e[s];
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int i4 = 0; i4 < RP / 4; ++i4) {
+                        f32x2 g01, g23;
+                        if constexpr (KDA) {
+                            const float4 g = *reinterpret_cast<const float4*>(sG + blk * KS + row + 4 * i4);
+                            g01 = pack2(g.x, g.y);
+                            g23 = pack2(g.z, g.w);
+                        } else {
+                            g01 = g23 = pack2(sPre[s0 + kTok - 1], sPre[s0 + kTok - 1]);
+                        }
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            c2[c][2 * i4] = mul2(c2[c][2 * i4], g01);
+                            c2[c][2 * i4 + 1] = mul2(c2[c][2 * i4 + 1], g23);
                         }
                     }
                 }
-                // this channel's term of every A_sj, summed over the warp's 32 channels: lane l ends up with pair l
-                float w[kTok], pr[kPairs];
-#pragma unroll
-                for (int s = 0; s < kTok; ++s) {
-#pragma unroll
-                    for (int j = 0; j < s; ++j) {
-                        w[j] *= g[s];
-                        pr[s * (s - 1) / 2 + j] = k[s] * w[j];
-                    }
-                    w[s] = k[s];
-                }
-#pragma unroll
-                for (int i2 = kTok * (kTok - 1) / 2; i2 < kPairs; ++i2) pr[i2] = 0.f;
-                group_reduce_transpose<32, kPairs>(pr, lane);
-                sGram[(blk * (K / 32) + i / 32) * kPairs + lane] = pr[0];
-            }
-            for (int s = tid; s < nb * kTok; s += T) sBeta[s] = c0 + s < n_ring ? rbeta[c0 + s] : c0 + s < n_tot ? *tbeta : 0.f;
-        } else {
-            for (int idx = tid; idx < n_here * (K / 4); idx += T) {
-                const int s = idx / (K / 4), i = 4 * (idx % (K / 4));
-                float k[4];
-                ld4(c0 + s < n_ring ? rk + (size_t)(c0 + s) * K + i : tk + i, k);
-                st4(sKt + s * KS + PR::at(i), k);
-            }
-            // w_s = beta_s prod_{j>s} a_j and the total decay, by a warp scan over up to 64 tokens
-            if (warp == 0 && c0 == 0) {
-                float a[2], bt[2];
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int s = lane + 32 * u;
-                    a[u] = s < n_ring ? rdec[s] : s < n_tot ? *tdec : 1.f;
-                    bt[u] = s < n_ring ? rbeta[s] : s < n_tot ? *tbeta : 0.f;
-                }
-                float after = 1.f;               // product of the decays behind this half
-#pragma unroll
-                for (int u = 1; u >= 0; --u) {
-                    float incl = a[u];
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const float other = __shfl_down_sync(0xffffffffu, incl, o);
-                        if (lane + o < 32) incl *= other;
-                    }
-                    float excl = __shfl_down_sync(0xffffffffu, incl, 1);
-                    if (lane == 31) excl = 1.f;
-                    if (lane + 32 * u < n_tot) sBeta[lane + 32 * u] = bt[u] * (excl * after);
-                    after *= __shfl_sync(0xffffffffu, incl, 0);
-                }
-                if (lane == 0) sPre[0] = after;
-            }
-        }
-        {
-            constexpr int PV = 16 / (int)sizeof(IO), in_row = V / PV;        // 16-byte units
-            const uint4* ring_v = reinterpret_cast<const uint4*>(rv);
-            const uint4* tok_v = reinterpret_cast<const uint4*>(tv);
-            for (int idx = tid; idx < n_here * in_row; idx += T) {
-                const int at = c0 * in_row + idx;
-                reinterpret_cast<uint4*>(sV)[idx] = at < n_ring * in_row ? ring_v[at] : tok_v[at - n_ring * in_row];
-            }
-        }
-        if (p.q != nullptr && c0 == 0) {
-            for (int i = tid; i < K / 4; i += T) {
-                float q[4];
-                ld4(tq + 4 * i, q);
-                st4(sQ + PR::at(4 * i), q);
-            }
-        }
-        if (p.write_sketch && h != h_staged) {
-            const float* og = p.omega + (size_t)h * K * R;
-#pragma unroll 4
-            for (int idx = tid; idx < K * R; idx += T) {
-                const int i = idx / R, g = idx % R;
-                sOm[g * OS + PR::at(i)] = og[idx];
-            }
-            for (int idx = tid; idx < (R8 - R) * K; idx += T) sOm[(R + idx / K) * OS + PR::at(idx % K)] = 0.f;
-            h_staged = h;
-        }
-        // (every thread's wait on the stage; a CTA that gives up leaves its heads as they are)
-        if (__syncthreads_or(failed)) {
-            failed = true;
-            return;
-        }
-        if (staged && last && tid == 0 && n_next >= 0) request(b_next, h_next, n_next);
-        if constexpr (DELTA) {
-            // beta_s A_sj
-            for (int idx = tid; idx < nb * kPairs; idx += T) {
-                const int blk = idx / kPairs, pair = idx % kPairs;
-                float a = 0.f;
-#pragma unroll
-                for (int c = 0; c < K / 32; ++c) a += sGram[(blk * (K / 32) + c) * kPairs + pair];
-                int s = 1;
-                while (s < kTok && (s + 1) * s / 2 <= pair) ++s;      // the pair's later token
-                sA[idx] = s < kTok ? sBeta[blk * kTok + s] * a : 0.f;
-            }
-            __syncthreads();
-        }
-
-        if constexpr (!DELTA) {
-            if (n_tot > 0 && c0 == 0) {
-                const f32x2 d2 = pack2(sPre[0], sPre[0]);
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-#pragma unroll
-                    for (int i = 0; i < RP / 2; ++i) c2[c][i] = mul2(c2[c][i], d2);
-            }
-        }
-        for (int blk = 0; blk < nb; ++blk) {
-            const int s0 = blk * kTok;
-            const int nt = min(kTok, n_here - s0);
-            const int mine = s0 + part;              // this lane's token where a lane stands for one
-            float x[4];
-            if constexpr (DELTA) {
-                float vals[32];
-                const float* kh = (KDA ? sKh : sKt) + s0 * KS + row;
-                dot4<RP>(c2, kh, KS, vals);
-                if (nt > 4) {
-                    dot4<RP>(c2, kh + 4 * KS, KS, vals + 16);
-                } else {
-#pragma unroll
-                    for (int i = 16; i < 32; ++i) vals[i] = 0.f;
-                }
-                reduce_parts(vals, lane);
-                float v[4] = {0.f, 0.f, 0.f, 0.f};
-                if (mine < n_here) ld4(sV + mine * V + j0, v);
-                const float bt = sBeta[mine], pre = KIND == SKETCHSSM_GDN ? sPre[mine] : 1.f;
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    x[c] = mine < n_here ? bt * (v[c] - (KIND == SKETCHSSM_GDN ? pre * vals[c] : vals[c])) : 0.f;
-            } else {
-                float v[4] = {0.f, 0.f, 0.f, 0.f};
-                if (mine < n_here) ld4(sV + mine * V + j0, v);
-                const float w = mine < n_here ? sBeta[c0 + mine] : 0.f;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) x[c] = w * v[c];
-            }
-            __syncwarp();                            // the previous block's e have been read
-            st4(sE + part * 16 + (lane & 3) * 4, x);
-            __syncwarp();
-            if constexpr (DELTA) {
-                // forward substitution, one column per lane
-                if (lane < 16) {
-                    float e[kTok], a[kPairs];
-#pragma unroll
-                    for (int s = 0; s < kTok; ++s) e[s] = sE[s * 16 + lane];
-#pragma unroll
-                    for (int i = 0; i < kPairs / 4 - 1; ++i) ld4(sA + blk * kPairs + 4 * i, a + 4 * i);
-#pragma unroll
-                    for (int j = 0; j < kTok - 1; ++j) {
-#pragma unroll
-                        for (int s = j + 1; s < kTok; ++s) e[s] = fmaf(-a[s * (s - 1) / 2 + j], e[j], e[s]);
-                    }
-#pragma unroll
-                    for (int s = 0; s < kTok; ++s) sE[s * 16 + lane] = KIND == SKETCHSSM_GDN ? sSuf[s0 + s] * e[s] : e[s];
-                }
-                __syncwarp();
-#pragma unroll
-                for (int i4 = 0; i4 < RP / 4; ++i4) {
-                    f32x2 g01, g23;
-                    if constexpr (KDA) {
-                        const float4 g = *reinterpret_cast<const float4*>(sG + blk * KS + row + 4 * i4);
-                        g01 = pack2(g.x, g.y);
-                        g23 = pack2(g.z, g.w);
-                    } else {
-                        g01 = g23 = pack2(sPre[s0 + kTok - 1], sPre[s0 + kTok - 1]);
-                    }
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        c2[c][2 * i4] = mul2(c2[c][2 * i4], g01);
-                        c2[c][2 * i4 + 1] = mul2(c2[c][2 * i4 + 1], g23);
-                    }
-                }
-            }
-            const float* kt = sKt + s0 * KS + row;
+                const float* kt = sKt + s0 * KS + row;
 #pragma unroll 2
-            for (int s = 0; s < nt; ++s) {
-                const float4 e = *reinterpret_cast<const float4*>(sE + s * 16 + (lane & 3) * 4);
-                const f32x2 e2[4] = {pack2(e.x, e.x), pack2(e.y, e.y), pack2(e.z, e.z), pack2(e.w, e.w)};
+                for (int s = 0; s < nt; ++s) {
+                    const float4 e = *reinterpret_cast<const float4*>(sE + s * 16 + (lane & 3) * 4);
+                    const f32x2 e2[4] = {pack2(e.x, e.x), pack2(e.y, e.y), pack2(e.z, e.z), pack2(e.w, e.w)};
 #pragma unroll
-                for (int i4 = 0; i4 < RP / 4; ++i4) {
-                    const float4 kq = *reinterpret_cast<const float4*>(kt + s * KS + 4 * i4);
-                    const f32x2 k01 = pack2(kq.x, kq.y), k23 = pack2(kq.z, kq.w);
+                    for (int i4 = 0; i4 < RP / 4; ++i4) {
+                        const float4 kq = *reinterpret_cast<const float4*>(kt + s * KS + 4 * i4);
+                        const f32x2 k01 = pack2(kq.x, kq.y), k23 = pack2(kq.z, kq.w);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        c2[c][2 * i4] = fma2(k01, e2[c], c2[c][2 * i4]);
-                        c2[c][2 * i4 + 1] = fma2(k23, e2[c], c2[c][2 * i4 + 1]);
+                        for (int c = 0; c < 4; ++c) {
+                            c2[c][2 * i4] = fma2(k01, e2[c], c2[c][2 * i4]);
+                            c2[c][2 * i4 + 1] = fma2(k23, e2[c], c2[c][2 * i4 + 1]);
+                        }
                     }
                 }
             }
-        }
-
         }
 
         // ---- write the updated state back ----
