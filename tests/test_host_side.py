@@ -109,3 +109,24 @@ def test_current_stream_without_the_raw_stream_functions(monkeypatch):
     monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=1234))
     assert binding.SketchSSM._stream(None) == 1234
     assert binding.SketchSSM._stream(SimpleNamespace(cuda_stream=77)) == 77
+
+
+def test_the_benchmark_prints_one_short_line_and_its_records_beside_it(capsys, tmp_path):
+    """Standard output is one JSON line that does not grow with the sweep; the records go to standard error, where the report
+    finds them.  A derived decode time that would beat a copy is shown as the back-to-back one."""
+    import json
+    import bench
+    from paper_2609_33051_b200 import report
+    rec = {"workload": "w: mamba2 B1", "coefficient_map": "fixed", "sketch_storage": "f32", "n_phys": 1, "value": 1e6,
+           "decode_in_window_us": 10.0, "decode_frac_of_measured": 1.04, "decode_frac_of_8TBs_nominal": 0.86,
+           "decode_back_to_back_us": 13.0, "decode_back_to_back_frac_of_measured": 0.8, "update_kernel": "k", "update_us": 5.0,
+           "update_frac_of_measured": 0.9, "sketch_and_map_overhead_on_flush": 0.05, "full_read": {"sketch_speedup": 2.0},
+           "clocks": {"sm_mhz": 1900.0, "reasons": []}, "padding": "x" * 2000}
+    bench.print_result({"metric": "m", "value": 1.0}, [("sweep", [rec] * 38), ("variant", [rec] * 7)])
+    out, err = capsys.readouterr()
+    assert json.loads(out) == {"metric": "m", "value": 1.0} and out.count("\n") == 1
+    assert [json.loads(ln)["record"] for ln in err.splitlines()] == ["sweep"] * 38 + ["variant"] * 7
+    row = report.table([rec])
+    assert "13.0 (back to back) | 0.80" in row and "1.04" not in row
+    rec["decode_frac_of_measured"] = 0.95
+    assert "| 10.0 | 0.95" in report.table([rec])
