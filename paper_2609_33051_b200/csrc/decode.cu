@@ -95,9 +95,9 @@ __host__ __device__ inline DecodeSmem make_decode_smem(int K, int R, int nwarps,
 //   kFull every head reads the full state (no sketch rows, no map)
 //   kAny  general: per-head ranks (rank 0: that head reads the full state), and kSeq / kPS / kUB as the launch says (kER
 //         stays a compile-time fact).
-// Every flag that is decided inside the loops over heads, ranks or slots costs the launches that do not use it: with the
-// full-read branch and the run-time flags out of the lean instantiations none of them spills, and the launches that had
-// to run the general one take (general -> own, r = L = 16, bfloat16 I/O): state-dependent bfloat16 map, Mamba-2 64-head
+// Every flag that is decided inside the loops over heads, ranks or slots costs the launches that do not use it: without the
+// full-read branch and the run-time flags 138 of the 170 instantiations without kAny spill nothing and the others at most
+// 24 bytes (the general ones 4 to 96), and the launches that had to run the general one take (general -> own, r = L = 16, bfloat16 I/O): state-dependent bfloat16 map, Mamba-2 64-head
 // batch of 256, 33 -> 31 us; the same with erase vectors, GDN 32-head batch of 512, 53 -> 45 us; mixed step of that layer
 // 48 -> 46 us; V = 80 layer of 37 x 24 heads with two dense heads (prefetch below) 13 -> 10 us.
 constexpr int kSeq = 1, kPS = 2, kER = 4, kUB = 8, kAny = 16, kFull = 32;
