@@ -671,9 +671,11 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
 //   KDA, the same, V = 64 or K = 64                               0.95 - 1.4, median 1.07  (two full rounds 0.77)
 // Ranks above 32 outweigh the replay again, unless there is no room for the stage (bfloat16 rows read from global memory:
 // 64 tokens, r = 64, V = 80 1520 us against 1256).  Per-sequence phases: how many sequences flush is not known here, so only
-// the first line counts.
+// the first line counts.  A sketch stored in bfloat16 stays with this kernel: the two differ in the last bits of their fp32
+// sums, and what a sequence's stored sketch is rounded to (2^-8 beside a boundary) shall not depend on the size of its batch.
 static bool update_cols_better(const Ctx* ctx, const Params& p, int n_tot, size_t wave) {
     const size_t heads = (size_t)p.B * p.H;
+    if (p.sketch_bf16) return false;
     if (heads * (p.dv == 128 ? 2 : 1) <= (size_t)ctx->sm_count) return true;
     if (p.n_dev != nullptr) return false;
     const bool kda = ctx->cfg.kind == SKETCHSSM_KDA;
@@ -702,10 +704,8 @@ static int launch_update_t(Ctx* ctx, Params p, cudaStream_t stream) {
     int by_smem = (int)((228u * 1024u) / (us.total + 1024u));
     by_smem = by_smem < 1 ? 1 : by_smem < update_ctas<V>() ? by_smem : update_ctas<V>();
     const size_t wave = (size_t)ctx->sm_count * (size_t)by_smem;
-    if (KIND != SKETCHSSM_MAMBA2 && p.update_impl != 4 && (p.update_impl == 5 || update_cols_better(ctx, p, n_tot, wave))) {
-        const int rc = launch_update_cols(ctx, p, stream);
-        if (rc != SKETCHSSM_UNSUPPORTED_SHAPE) return rc;
-    }
+    if (KIND != SKETCHSSM_MAMBA2 && p.update_impl != 4 && (p.update_impl == 5 || update_cols_better(ctx, p, n_tot, wave)))
+        return launch_update_cols(ctx, p, stream);
     auto kern = update_kernel<KIND, IO, K, V>;
     if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     size_t grid = (size_t)p.B * p.H;

@@ -201,15 +201,16 @@ __global__ void __launch_bounds__(kVT * kParts) update_cols_kernel(const Params 
     // ---- exact output o[j] = <S_new[:, j], q> ----
     if (p.out != nullptr) {
         const float4* qp = reinterpret_cast<const float4*>(sQ + part * (RP + 4));
-        float acc = 0.f;
+        float acc = 0.f, odd = 0.f;                 // (two sums of every other row, here and below: half the rounding steps each)
 #pragma unroll
         for (int i4 = 0; i4 < RP / 4; ++i4) {
             const float4 qq = qp[i4];
             acc = fmaf(qq.x, col[4 * i4 + 0], acc);
-            acc = fmaf(qq.y, col[4 * i4 + 1], acc);
+            odd = fmaf(qq.y, col[4 * i4 + 1], odd);
             acc = fmaf(qq.z, col[4 * i4 + 2], acc);
-            acc = fmaf(qq.w, col[4 * i4 + 3], acc);
+            odd = fmaf(qq.w, col[4 * i4 + 3], odd);
         }
+        acc += odd;
         acc += __shfl_xor_sync(0xffffffffu, acc, 8);
         acc += __shfl_xor_sync(0xffffffffu, acc, 16);
         if (part == 0) {
@@ -222,16 +223,17 @@ __global__ void __launch_bounds__(kVT * kParts) update_cols_kernel(const Params 
     if (p.write_sketch) {
         const size_t ug = (size_t)bh * R * V + j;
         for (int g0 = 0; g0 < R4; g0 += 4) {
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+            float a[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
             const float* op = sOm + (size_t)part * (RP * R4 + 4) + g0;
 #pragma unroll
             for (int ii = 0; ii < RP; ++ii) {
                 const float4 w = *reinterpret_cast<const float4*>(op + ii * R4);
-                a0 = fmaf(w.x, col[ii], a0);
-                a1 = fmaf(w.y, col[ii], a1);
-                a2 = fmaf(w.z, col[ii], a2);
-                a3 = fmaf(w.w, col[ii], a3);
+                a[ii & 1][0] = fmaf(w.x, col[ii], a[ii & 1][0]);
+                a[ii & 1][1] = fmaf(w.y, col[ii], a[ii & 1][1]);
+                a[ii & 1][2] = fmaf(w.z, col[ii], a[ii & 1][2]);
+                a[ii & 1][3] = fmaf(w.w, col[ii], a[ii & 1][3]);
             }
+            float a0 = a[0][0] + a[1][0], a1 = a[0][1] + a[1][1], a2 = a[0][2] + a[1][2], a3 = a[0][3] + a[1][3];
             a0 += __shfl_xor_sync(0xffffffffu, a0, 8);  a0 += __shfl_xor_sync(0xffffffffu, a0, 16);
             a1 += __shfl_xor_sync(0xffffffffu, a1, 8);  a1 += __shfl_xor_sync(0xffffffffu, a1, 16);
             a2 += __shfl_xor_sync(0xffffffffu, a2, 8);  a2 += __shfl_xor_sync(0xffffffffu, a2, 16);
@@ -250,7 +252,6 @@ int launch_cols_t(Ctx* ctx, Params p, cudaStream_t stream) {
     if (p.n_dev != nullptr) p.n_cap = n_tot;        // per-sequence phases: n_before is the largest fill any sequence may have
     const ColsSmem us = make_cols_smem<K>(KIND, n_tot, (p.R + 3) & ~3, kVT);
     auto kern = update_cols_kernel<KIND, IO, K, kVT>;
-    if (us.total > 226u * 1024u) return SKETCHSSM_UNSUPPORTED_SHAPE;
     if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     const dim3 grid((unsigned)((size_t)p.B * p.H * (ctx->cfg.dv / kVT)));
     if ((ctx->last_cuda_error = launch_kernel(kern, grid, dim3(kVT * kParts), us.total, stream, p, p.pdl != 0)) != cudaSuccess)

@@ -156,3 +156,20 @@ def test_mixed_step_with_fills_around_the_chunks(kind, K, V, L, io, impl):
     assert harness.rel_err(m.state.cpu().numpy(), S) <= BAR
     U = orc.sketch_of(S, np.broadcast_to(Om64, (w.batch,) + Om64.shape))
     assert harness.rel_err(m.sketch.cpu().numpy().transpose(0, 1, 3, 2), U) <= BAR
+
+
+@pytest.mark.parametrize("kind,V,L", [("gdn", 128, 8), ("gdn", 80, 36), ("kda", 64, 8)])
+def test_a_bfloat16_sketch_does_not_depend_on_the_batch(kind, V, L):
+    """The rounded sketch (and the state) of a sequence is the same, bit for bit, in a batch of 3 and in one of 301."""
+    got = []
+    for B in (3, 301):
+        w = synth.Workload("t", kind, 301, 2, 128, V, 16, L, 0, "f32", 241, basis="qr")
+        m, S0, Om, *_ = make_layer(w.replace(batch=B), sketch="bf16")
+        m.state.copy_(torch.from_numpy(S0 if len(S0) == B else synth.initial_state(w)[:B]))
+        for t in range(L):
+            tt = {n: x[:B].contiguous() for n, x in harness.token_tensors(w, synth.step_inputs(w, 0, t), m.device).items()}
+            args = (tt["q"], tt["k"], tt["v"], tt["beta"], tt["decay"], m.new_output())
+            (m.decode_step if t < L - 1 else m.state_update)(t, *args)
+        m.check_status()
+        got.append((m.sketch[:3].clone(), m.state[:3].clone()))
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
