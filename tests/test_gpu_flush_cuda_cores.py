@@ -164,8 +164,9 @@ def test_a_bfloat16_sketch_does_not_depend_on_the_batch(kind, V, L):
     got = []
     for B in (3, 301):
         w = synth.Workload("t", kind, 301, 2, 128, V, 16, L, 0, "f32", 241, basis="qr")
-        m, S0, Om, *_ = make_layer(w.replace(batch=B), sketch="bf16")
-        m.state.copy_(torch.from_numpy(S0 if len(S0) == B else synth.initial_state(w)[:B]))
+        m, *_ = make_layer(w.replace(batch=B), sketch="bf16")
+        m.state.copy_(torch.from_numpy(synth.initial_state(w)[:B]))
+        m.state_update(0)
         for t in range(L):
             tt = {n: x[:B].contiguous() for n, x in harness.token_tensors(w, synth.step_inputs(w, 0, t), m.device).items()}
             args = (tt["q"], tt["k"], tt["v"], tt["beta"], tt["decay"], m.new_output())
