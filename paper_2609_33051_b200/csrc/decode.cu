@@ -97,9 +97,10 @@ __host__ __device__ inline DecodeSmem make_decode_smem(int K, int R, int nwarps,
 //         stays a compile-time fact).
 // Every flag that is decided inside the loops over heads, ranks or slots costs the launches that do not use it: without the
 // full-read branch and the run-time flags 138 of the 170 instantiations without kAny spill nothing and the others at most
-// 24 bytes (the general ones 4 to 96), and the launches that had to run the general one take (general -> own, r = L = 16, bfloat16 I/O): state-dependent bfloat16 map, Mamba-2 64-head
-// batch of 256, 33 -> 31 us; the same with erase vectors, GDN 32-head batch of 512, 53 -> 45 us; mixed step of that layer
-// 48 -> 46 us; V = 80 layer of 37 x 24 heads with two dense heads (prefetch below) 13 -> 10 us.
+// 24 bytes (the general ones 4 to 96), and the launches that had to run the general one take (general -> own, r = L = 16,
+// bfloat16 I/O): state-dependent bfloat16 map, Mamba-2 64-head batch of 256, 33 -> 31 us; the same with erase vectors, GDN
+// 32-head batch of 512, 53 -> 45 us; mixed step of that layer 48 -> 46 us.  (How much of it is the unrolled rank has not been
+// measured apart.)  V = 80 layer of 37 x 24 heads with two dense heads (prefetch below): 13 -> 10 us.
 constexpr int kSeq = 1, kPS = 2, kER = 4, kUB = 8, kAny = 16, kFull = 32;
 
 // Warps of the largest CTA; two such CTAs per SM set the register budget: 64 registers for the lean Mamba-2 kernels (32
