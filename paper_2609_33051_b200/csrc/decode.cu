@@ -73,7 +73,7 @@ struct DecodeSmem {
 };
 
 __host__ __device__ inline DecodeSmem make_decode_smem(int K, int R, int nwarps, int full_read, int coef_per_seq,
-                                                       uint32_t stage_bytes) {
+                                                       uint32_t stage_bytes, int team) {
     DecodeSmem d;
     const int RP = (R + 7) & ~7;                       // coefficient rows padded to the reduction width
     d.coef_slot_bytes = (full_read || coef_per_seq) ? 0u : (uint32_t)(RP * K * 4);
@@ -82,8 +82,15 @@ __host__ __device__ inline DecodeSmem make_decode_smem(int K, int R, int nwarps,
     d.scratch_stride = (uint32_t)((K + 80) * 4);       // per warp: q~ (full read) or c (K floats), then 64+ dot products
     d.scratch_off = off; off += (uint32_t)nwarps * d.scratch_stride;
     d.stage_off = off;
-    d.total = off + (uint32_t)nwarps * stage_bytes;
+    d.total = off + (uint32_t)(nwarps / team) * stage_bytes;
     return d;
+}
+
+// state rows, read once: no lines of L1 for them
+template <int N>
+__device__ __forceinline__ void load_stream(const float* src, float (&d)[N]) {
+    if constexpr (N == 4) asm("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(d[0]), "=f"(d[1]), "=f"(d[N - 2]), "=f"(d[N - 1]) : "l"(src));
+    else asm("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(d[0]), "=f"(d[1]) : "l"(src));
 }
 
 }  // namespace
@@ -105,12 +112,15 @@ constexpr int kSeq = 1, kPS = 2, kER = 4, kUB = 8, kAny = 16, kFull = 32;
 
 // Warps of the largest CTA; two such CTAs per SM set the register budget: 64 registers for the lean Mamba-2 kernels (32
 // warps), 80 for the others (24 warps).
-__host__ __device__ constexpr int decode_max_warps(int kind, int F) {
-    return (F & ~(kUB | kFull)) != 0 || kind != SKETCHSSM_MAMBA2 ? 12 : 16;
+__host__ __device__ constexpr int decode_max_warps(int kind, int F, int W) {
+    return ((F & ~(kUB | kFull)) != 0 || kind != SKETCHSSM_MAMBA2 ? 12 : 16) * (W > 1 ? 2 : 1);
 }
 
-template <int KIND, typename IO, int K, int V, int RT, int F>
-__global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kernel(const Params p) {
+// W: warps that share a head (a team).
+template <int KIND, typename IO, int K, int V, int RT, int F, int W>
+__global__ void __launch_bounds__(decode_max_warps(KIND, F, W) * 32, W > 1 ? 1 : 2) decode_kernel(const Params p) {
+    static_assert(W == 1 || F == kFull || F == kAny || (F == 0 && KIND == SKETCHSSM_MAMBA2), "no team for this instantiation");
+    constexpr bool TEAM = W > 1;
     constexpr bool ANY = (F & kAny) != 0, DYN = ANY || (F & kSeq) != 0, FULL = (F & kFull) != 0;
     constexpr int EK = K / 32;
     constexpr int EV = V % 32 == 0 ? V / 32 : 4;        // value elements per lane ...
@@ -120,7 +130,8 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const int nwarps = blockDim.x >> 5;
+    const int nwarps = blockDim.x >> 5, nteams = nwarps / W;
+    const int team = warp / W, sub = TEAM ? warp % W : 0;        // (W divides the warps of a CTA)
     const int R = RT ? RT : p.R;
     const int L = p.L, H = p.H, B = p.B;
     const int n_cap = p.n_before;                       // ring rows the stage has room for (per-sequence phases: the largest fill)
@@ -133,11 +144,28 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
     constexpr bool ER = (F & kER) != 0;
 
     const StageLayout sl = make_stage_layout(KIND, (int)sizeof(IO), K, V, R, L, n_cap, FULL, per_seq, su, ER);
-    const DecodeSmem ds = make_decode_smem(K, R, nwarps, FULL, per_seq, sl.total);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + ds.bar_off) + warp * 2;
+    const DecodeSmem ds = make_decode_smem(K, R, nwarps, FULL, per_seq, sl.total, W);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + ds.bar_off) + team * 2;
     float* sX = reinterpret_cast<float*>(smem + ds.scratch_off + (size_t)warp * ds.scratch_stride);   // c or q~
     float* sP = sX + K;                                                                               // dot products
-    unsigned char* my_stage = smem + ds.stage_off + (size_t)warp * sl.total;
+    unsigned char* my_stage = smem + ds.stage_off + (size_t)team * sl.total;
+
+    // Named barrier of the team; the vote of its waits (so that its warps leave the loop together).
+    auto team_sync = [&]() { if constexpr (TEAM) asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(32 * W) : "memory"); };
+    auto any_of_team = [&](bool bad) -> bool {
+        if constexpr (TEAM) {
+            uint32_t r;
+            asm volatile(
+                "{\n\t.reg .pred p, q;\n\t"
+                "setp.ne.b32 q, %1, 0;\n\t"
+                "bar.red.or.pred p, %2, %3, q;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(r) : "r"(bad ? 1u : 0u), "r"(1 + team), "r"(32 * W) : "memory");
+            return r != 0;
+        } else {
+            return __any_sync(0xffffffffu, bad);
+        }
+    };
 
     // contiguous range of items for this CTA; item = h * B + b
     const long long total = (long long)H * B;
@@ -248,7 +276,9 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
     const int n_items = item1 - item0;
     int* item_ctr = reinterpret_cast<int*>(smem + ds.bar_off + (size_t)nwarps * 16);
     const int second_h_start = (h_first + 1) * B;      // first item of the range's second head index
-    auto claim = [&]() -> int {            // whole warp; returns an item number, or item1 when none is left
+    // (A team of several warps walks its items in a fixed stride instead: its heads are short.)
+    auto claim = [&](int cur) -> int {     // whole warp; returns an item number, or item1 when none is left
+        if constexpr (TEAM) return min(cur + nteams, item1);
         int v = 0;
         if (lane == 0) v = atomicAdd(item_ctr, 1);
         v = __shfl_sync(0xffffffffu, v, 0);
@@ -273,7 +303,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
         return p.n_dev == nullptr ? n_cap : p.n_dev[bb];
     };
 
-    int item = warp < n_items ? item0 + warp : item1;      // the first head of every warp is fixed (the counter starts at nwarps)
+    int item = team < n_items ? item0 + team : item1;      // the first head of every warp is fixed (the counter starts at nwarps)
     int h = 0, b = 0, hn = 0, bn = 0;
     if (item < item1) head_of(item, h, b);
     int rk = item < item1 ? rank_of(h) : 0, rk_next = 0;
@@ -290,7 +320,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
     // head's sketch rows are requested before the predecessor in the stream is waited for, so they travel during its tail.
     // (Not with per-sequence phases: whether the head takes part at all is only known after the wait.)
     const bool early_u = p.early_sketch != 0 && p.n_dev == nullptr;
-    if (item < item1 && early_u) issue_b((size_t)b * H + h, rk, 0);
+    if (item < item1 && early_u && sub == 0) issue_b((size_t)b * H + h, rk, 0);
     grid_dep_wait();                 // from here on the ring and the token tensors (and otherwise the sketch) are read
     // Dependents are released only now: a successor that reads its sketch early must not start before this kernel has
     // seen its own predecessor (possibly a state update) complete.
@@ -299,8 +329,10 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
         const size_t bh0 = (size_t)b * H + h;
         n = fill_of(b);
         if (!DYN || n >= 0) {
-            issue_a(bh0, n);
-            if (!early_u) issue_b(bh0, rk, n);
+            if (sub == 0) {
+                issue_a(bh0, n);
+                if (!early_u) issue_b(bh0, rk, n);
+            }
             scalar_gates(bh0, bt_next, dsc_next);
         }
     }
@@ -313,7 +345,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
         if constexpr (!DYN) { n = n_cap; n_next = n_cap; }      // launch constants
         if constexpr (!ANY) { rk = r_uni; rk_next = r_uni; }
         const size_t bh = (size_t)b * H + h;
-        const int item_next = claim();
+        const int item_next = claim(item);
         const bool has_next = item_next < item1;
         if (has_next) {
             head_of(item_next, hn, bn);
@@ -327,7 +359,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
 
         if constexpr (DYN) {
             if (n < 0) {             // this sequence takes the flush step in this call: nothing to do here
-                if (go_next) { issue_a(bh_next, n_next); issue_b(bh_next, rk_next, n_next); }
+                if (go_next && sub == 0) { issue_a(bh_next, n_next); issue_b(bh_next, rk_next, n_next); }
                 item = item_next; h = hn; b = bn; n = n_next; rk = rk_next;
                 continue;
             }
@@ -343,10 +375,10 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
         // (window of fp32 KDA full reads, 3072 heads: 440 -> 479 us).
         constexpr int kAhead = 32;
         if (ANY && full) {
-            for (int line = lane; line < kAhead * V / 32; line += 32) prefetch_l2_line(p.state + bh * (size_t)K * V + 32 * line);
+            for (int line = lane; line < kAhead * V / 32; line += 32) prefetch_l2_line(p.state + (bh * K + sub * (K / W)) * (size_t)V + 32 * line);
         }
 
-        if (__any_sync(0xffffffffu, !DEC_WAIT(barA, parA))) {
+        if (any_of_team(!DEC_WAIT(barA, parA))) {
             if (lane == 0) record_fault(p.status, FULL ? kFaultFullReadWait : kFaultDecodeWait, (int)blockIdx.x);
             pendA = (int)parA;
             pendB = full ? -1 : (int)(ANY ? parB : parA);
@@ -368,7 +400,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
         if (vlane) load_io<EV>(reinterpret_cast<const IO*>(sb + sl.tv_off), lane * EV, vv);
         if constexpr (KIND == SKETCHSSM_KDA) load_io<EK>(reinterpret_cast<const IO*>(sb + sl.tg_off), lane * EK, gg);
 
-        if (p.append) {
+        if (p.append && sub == 0) {
             unsigned char* rh = p.ring + bh * p.rl.head_bytes;
             store_io<EK>(reinterpret_cast<IO*>(rh) + (size_t)n * K, lane * EK, kk);
             if (vlane) store_io<EV>(reinterpret_cast<IO*>(rh + p.rl.v_off) + (size_t)n * V, lane * EV, vv);
@@ -391,7 +423,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
             kq_t = warp_sum(part);
             const float a = bt * kq_t;
 #pragma unroll
-            for (int e = 0; e < EV; ++e) o[e] = a * vv[e];
+            for (int e = 0; e < EV; ++e) o[e] = sub == 0 ? a * vv[e] : 0.f;        // (a team: the first warp's part of the sum)
             if constexpr (KIND == SKETCHSSM_MAMBA2) {
                 dsuf = dsc;
             } else if constexpr (KIND == SKETCHSSM_GDN) {
@@ -405,14 +437,17 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
 
         // ---- buffered tokens ----
         if constexpr (KIND == SKETCHSSM_MAMBA2) {
-            // independent dot products <k_s, q_t>, eight per transposing reduction; lane l ends up with slot s0 + l/4
-            int s0 = 0;
-            for (; s0 + 4 < n; s0 += NB) {      // blocks of eight while more than four slots remain
+            // independent dot products <k_s, q_t>, eight per transposing reduction; lane l ends up with slot s0 + l/4.  A team
+            // splits the slots: the first warp, which also has the current token, takes the newest.
+            const int per = TEAM ? min(n, ((n + W - 1) / W + 3) & ~3) : n;
+            const int lo = TEAM ? min(n, (W - 1 - sub) * per) : 0, hi = TEAM && sub ? min(n, (W - sub) * per) : n;
+            int s0 = lo;
+            for (; s0 + 4 < hi; s0 += NB) {      // blocks of eight while more than four slots remain
                 float part[NB];
 #pragma unroll
                 for (int i = 0; i < NB; ++i) {
                     float kr[EK];
-                    load_io<EK>(sK, min(s0 + i, n - 1) * K + lane * EK, kr);
+                    load_io<EK>(sK, min(s0 + i, hi - 1) * K + lane * EK, kr);
                     float acc = 0.f;
 #pragma unroll
                     for (int e = 0; e < EK; ++e) acc = fmaf(kr[e], q0[e], acc);
@@ -421,12 +456,12 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
                 group_reduce_transpose<32, NB>(part, lane);
                 if ((lane & 3) == 0) sP[s0 + (lane >> 2)] = part[0];
             }
-            if (s0 < n) {                       // one to four slots left: lane l ends up with slot s0 + l/8
+            if (s0 < hi) {                      // one to four slots left: lane l ends up with slot s0 + l/8
                 float part[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     float kr[EK];
-                    load_io<EK>(sK, min(s0 + i, n - 1) * K + lane * EK, kr);
+                    load_io<EK>(sK, min(s0 + i, hi - 1) * K + lane * EK, kr);
                     float acc = 0.f;
 #pragma unroll
                     for (int e = 0; e < EK; ++e) acc = fmaf(kr[e], q0[e], acc);
@@ -435,9 +470,13 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
                 group_reduce_transpose<32, 4>(part, lane);
                 if ((lane & 7) == 0) sP[s0 + (lane >> 3)] = part[0];
             }
+            if constexpr (TEAM) {               // the decays behind this warp's slots
+#pragma unroll 4
+                for (int s = n - 1; s >= hi; --s) dsuf *= sDec[s];
+            }
             __syncwarp();
 #pragma unroll 4
-            for (int s = n - 1; s >= 0; --s) {
+            for (int s = hi - 1; s >= lo; --s) {
                 const float a = sBeta[s] * dsuf * sP[s];
                 dsuf *= sDec[s];
                 if (vlane) {
@@ -446,6 +485,10 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
 #pragma unroll
                     for (int e = 0; e < EV; ++e) o[e] = fmaf(a, vr[e], o[e]);
                 }
+            }
+            if constexpr (TEAM) {
+#pragma unroll 4
+                for (int s = lo - 1; s >= 0; --s) dsuf *= sDec[s];
             }
 #pragma unroll
             for (int e = 0; e < EK; ++e) x[e] = dsuf * q0[e];
@@ -534,6 +577,10 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
 #pragma unroll
                 for (int e = 0; e < EV; ++e) o[e] = fmaf(a, vr[e], o[e]);
             }
+            if constexpr (TEAM) {        // (the sweep is a chain: every warp of a team runs it, one keeps the buffered values)
+#pragma unroll
+                for (int e = 0; e < EV; ++e) o[e] = sub == 0 ? o[e] : 0.f;
+            }
             if constexpr (ER) {
                 if (er_h) {      // x <- d_[t] * q_t; kk <- d_[t] * k_t (the token's key has been stored and swept by now)
 #pragma unroll
@@ -547,20 +594,28 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
         }
 
         // the sweep is done with the ring part of the stage: the next head's group A may come in
+        // (a team: once all its warps are; with the vote of the wait for the sketch where there is one)
         __syncwarp();
-        if (go_next) issue_a(bh_next, n_next);
+        if (!TEAM && go_next) issue_a(bh_next, n_next);
+        if constexpr (TEAM) {
+            if (full) {
+                team_sync();
+                if (go_next && sub == 0) issue_a(bh_next, n_next);
+            }
+        }
         if (!full) {
             // c = C x, eight coefficients per transposing reduction, handed to all lanes through the scratch
             const float* sC = per_seq ? reinterpret_cast<const float*>(sb + sl.c_off)
                                              : reinterpret_cast<const float*>(smem + (size_t)(h - h_first) * ds.coef_slot_bytes);
             __syncwarp();
             if (per_seq) {        // the head's own map arrives with its sketch rows
-                if (__any_sync(0xffffffffu, !DEC_WAIT(barB, PARB))) {
+                if (any_of_team(!DEC_WAIT(barB, PARB))) {
                     if (lane == 0) record_fault(p.status, kFaultDecodeWait, (int)blockIdx.x);
                     pendB = (int)PARB;
-                    pendA = go_next ? (int)parA : -1;
+                    pendA = go_next && !TEAM ? (int)parA : -1;
                     break;
                 }
+                if (TEAM && go_next && sub == 0) issue_a(bh_next, n_next);
             }
             const bool c16 = per_seq && u_bf16;       // the head's own map travels as bfloat16 (the shared map was widened when staged)
             const int rp_it = RT ? ((RT + 7) & ~7) : ((rk + 7) & ~7);
@@ -568,7 +623,7 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
             if constexpr (ER) both = er_h;
             if (!both) {
 #pragma unroll
-            for (int g0 = 0; g0 < (RT ? ((RT + 7) & ~7) : rp_it); g0 += NB) {
+            for (int g0 = NB * sub; g0 < (RT ? ((RT + 7) & ~7) : rp_it); g0 += NB * W) {      // (a team's warps: every W-th block of ranks)
                 float part[NB];
 #pragma unroll
                 for (int i = 0; i < NB; ++i) {
@@ -606,12 +661,13 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
             }
             __syncwarp();
             if (!per_seq) {
-                if (__any_sync(0xffffffffu, !DEC_WAIT(barB, PARB))) {
+                if (any_of_team(!DEC_WAIT(barB, PARB))) {
                     if (lane == 0) record_fault(p.status, kFaultDecodeWait, (int)blockIdx.x);
                     pendB = (int)PARB;
-                    pendA = go_next ? (int)parA : -1;
+                    pendA = go_next && !TEAM ? (int)parA : -1;
                     break;
                 }
+                if (TEAM && go_next && sub == 0) issue_a(bh_next, n_next);
             }
             if constexpr (ANY) parB ^= 1u;
             if constexpr (ER) {
@@ -655,18 +711,27 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
             }
             const float* sU = reinterpret_cast<const float*>(sb + sl.u_off);
             if (vlane) {
-#pragma unroll (RT ? RT : 4)
-                for (int g = 0; g < (RT ? RT : rk); ++g) {
+                auto rank_row = [&](int g) {
                     const float cg = sX[g];
                     float uu[EV];
                     if (u_bf16) load_io<EV>(reinterpret_cast<const __nv_bfloat16*>(sU), g * V + lane * EV, uu);
                     else load_io<EV>(sU, g * V + lane * EV, uu);
 #pragma unroll
                     for (int e = 0; e < EV; ++e) o[e] = fmaf(cg, uu[e], o[e]);
+                };
+                if constexpr (TEAM) {
+                    for (int g0 = NB * sub; g0 < (RT ? RT : rk); g0 += NB * W) {
+#pragma unroll
+                        for (int i = 0; i < NB; ++i)
+                            if (RT % NB == 0 && RT ? true : g0 + i < (RT ? RT : rk)) rank_row(g0 + i);
+                    }
+                } else {
+#pragma unroll (RT ? RT : 4)
+                    for (int g = 0; g < (RT ? RT : rk); ++g) rank_row(g);
                 }
             }
             __syncwarp();
-            if (go_next) issue_b(bh_next, rk_next, n_next);
+            if (!TEAM && go_next) issue_b(bh_next, rk_next, n_next);
         } else {
             __syncwarp();
             store_io<EK>(sX, lane * EK, x);
@@ -677,11 +742,16 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
                 // room for 16: 60 bytes spilled instead of 12, with erase vectors 276 instead of 100, which all its heads paid
                 // for (8192 heads, GDN, 24 buffered tokens, r = 24: 56 us a launch, with both changes 45).
                 constexpr int RB = ANY && K == 64 ? 8 : 32 / EV;
-                for (int i0 = 0; i0 < K; i0 += RB) {
-                    if (ANY && i0 + kAhead < K && lane < RB * V / 32) prefetch_l2_line(p.state + (bh * K + i0 + kAhead) * V + 32 * lane);
+                for (int i0 = sub * (K / W); i0 < (sub + 1) * (K / W); i0 += RB) {        // (a team's warps: K / W rows each)
+                    if (ANY && i0 + kAhead < (sub + 1) * (K / W) && lane < RB * V / 32) prefetch_l2_line(p.state + (bh * K + i0 + kAhead) * V + 32 * lane);
                     float rows[RB][EV];
+                    if (TEAM && FULL && p.stream_state) {
 #pragma unroll
-                    for (int r = 0; r < RB; ++r) load_io<EV>(Sg, (i0 + r) * V, rows[r]);
+                        for (int r = 0; r < RB; ++r) load_stream<EV>(Sg + (i0 + r) * V, rows[r]);
+                    } else {
+#pragma unroll
+                        for (int r = 0; r < RB; ++r) load_io<EV>(Sg, (i0 + r) * V, rows[r]);
+                    }
 #pragma unroll
                     for (int r = 0; r < RB; ++r) {
                         const float xi = sX[i0 + r];
@@ -691,10 +761,27 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
                 }
             }
             // a head that reads the full state fetched no sketch rows; the next head's are requested here
-            if (go_next) issue_b(bh_next, rk_next, n_next);
+            if (!TEAM && go_next) issue_b(bh_next, rk_next, n_next);
         }
 
-        if (vlane) {
+        if constexpr (TEAM) {        // the parts of the sum, added by the first warp in a fixed order
+            __syncwarp();
+            if (sub && vlane) store_io<EV>(sX, lane * EV, o);
+            team_sync();
+            if (sub == 0) {
+                if (go_next) issue_b(bh_next, rk_next, n_next);
+#pragma unroll
+                for (int w = 1; w < W; ++w) {
+                    if (vlane) {
+                        float part[EV];
+                        load_io<EV>(sX + w * (ds.scratch_stride / 4), lane * EV, part);
+#pragma unroll
+                        for (int e = 0; e < EV; ++e) o[e] += part[e];
+                    }
+                }
+            }
+        }
+        if (vlane && sub == 0) {
             if (p.out_bf16) {
                 store_io<EV>(reinterpret_cast<__nv_bfloat16*>(p.out) + bh * V, lane * EV, o);
             } else {
@@ -713,6 +800,31 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F) * 32, 2) decode_kern
     // they do not land in shared memory that has meanwhile been handed to another CTA.
     if (pendA >= 0) mbar_wait_bounded(barA, (uint32_t)pendA, 1u << 14);
     if (pendB >= 0) mbar_wait_bounded(barB, (uint32_t)pendB, 1u << 14);
+}
+
+// How many warps share a head.  One warp per head keeps the most heads in flight and needs no barrier; a team shortens the
+// time of a head, which is what counts where the heads are few, where their stages leave room for few warps, and for full
+// reads, whose rows (registers, through L1) are then read by warps of which fewer wait for a sweep.  1 / 2 / 4 warps per head,
+// us a launch, `slots` heads' stages per SM:
+//   full read, KDA V = 128, 6 fp32 tokens: 128 heads 6.3 / 5.0 / 4.0; 576 6.8 / 5.4 / 6.7; 1184 (in L2) 14.9 / 15.7 / 12.4; 3072 47 / 34 /
+//     38; 7104 95 / 79 / 84.  GDN, 14 tokens: 576 7.6 / 6.8 / 8.0 (a team repeats the sweep), 2368 33 / 34 / 35, 4736 77 / 54 / 60.
+//     Mamba-2 V = 64: 576 6.1 / 4.4 / 4.0, 2368 11.5 / 10.4 / 12.3, 9472 64 / 50 / 53; 62 tokens, eight slots, 9472 127 / 100 / 86
+//   dense heads among sketched ones (Mamba-2, V = 80, one head of six dense): 288 heads 7.4 / 6.0 / 4.5, 888 7.6 / 6.6 / 5.8, 1776 9.2 / 7.3 / 9.0,
+//     2376 9.1 / 12 / 13
+//   sketch, Mamba-2, rank 32, 16384 heads: 48 tokens (6 slots) 87 / 82 / 82, 56 95 / 90 / 94, 62 (5 slots) 117 / 108 / 99; 32 tokens (10
+//     slots) 59 / 61 / 64
+// Full reads of a state that does not stay in L2 leave L1 to the rows in flight: no lines allocated (50 against 56 us for
+// the 9472 Mamba-2 heads, 34.5 against 36 for the 3072 of KDA; within L2 10 % slower), and the stages of teams
+// of two in at most 200 KB.
+constexpr long long kStreamBytes = 96ll << 20;
+static int team_size(int kind, int need, int n, long long heads, int sms, int slots, long long full_bytes, bool ranks) {
+    if (need == kFull) {
+        if (heads <= 2ll * sms || (heads <= 4ll * sms && (kind == SKETCHSSM_MAMBA2 || n <= 8))) return 4;
+        return slots < 10 ? 4 : full_bytes > kStreamBytes ? 2 : 1;
+    }
+    if (ranks) return heads <= 6ll * sms ? 4 : heads <= 12ll * sms ? 2 : 1;
+    if (need == 0 && kind == SKETCHSSM_MAMBA2) return slots <= 5 ? 4 : slots <= 6 ? 2 : 1;
+    return 1;
 }
 
 template <int N>
@@ -743,13 +855,29 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
     const int need = p.full_read ? kFull
                                  : (p.n_dev != nullptr ? kSeq : 0) | (p.coef_per_seq ? kPS : 0) | (erase ? kER : 0) |
                                        (p.sketch_bf16 ? kUB : 0) | (p.head_rank != nullptr ? kAny : 0);
+    // Warps per head (the rule and its figures: team_size).
+    const long long heads = (long long)p.B * p.H;
+    const int slots = (int)((smem_budget - make_decode_smem(K, p.R, 1, p.full_read, p.coef_per_seq, 0u, 1).stage_off) /
+                            (sl.total + (uint32_t)((K + 80) * 4)));
+    int W = team_size(KIND, need, p.n_before, heads, ctx->sm_count, slots, p.full_read ? heads * K * V * 4 : 0, p.head_rank != nullptr);
+    // (a caller's own choice of warps is one of warps with a head each)
+    if (p.warps_per_cta || p.max_warps_per_sm > 0 || make_decode_smem(K, p.R, W, p.full_read, p.coef_per_seq, sl.total, W).total > smem_budget) W = 1;
+    p.stream_state = heads * K * V * 4 > kStreamBytes ? 1 : 0;
     void (*kern)(const Params) = nullptr;
     int variant = 0, max_nw = 0;
     auto use = [&](int number, auto rt, auto f) {        // (the CTA size follows the instantiation that runs: its launch bound)
         constexpr int RT = decltype(rt)::value, F = decltype(f)::value;
-        kern = decode_kernel<KIND, IO, K, V, RT, F>;
+        kern = decode_kernel<KIND, IO, K, V, RT, F, 1>;
         variant = number;
-        max_nw = decode_max_warps(KIND, F);
+        max_nw = decode_max_warps(KIND, F, 1);
+        if constexpr (F == kFull || F == kAny || (F == 0 && KIND == SKETCHSSM_MAMBA2)) {
+            if (W == 2) kern = decode_kernel<KIND, IO, K, V, RT, F, 2>;
+            if (W == 4) kern = decode_kernel<KIND, IO, K, V, RT, F, 4>;
+            if (W > 1) {
+                variant = number + 13 * (W / 2);
+                max_nw = decode_max_warps(KIND, F, W);
+            }
+        }
     };
     use(0, Int<0>(), Int<kAny>());
     if (need == 0) {
@@ -779,7 +907,7 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
         }
     }
     // registers per thread of the instantiation (queried once): they bound the resident warps like shared memory does
-    static int regs_per_thread[13] = {0};
+    static int regs_per_thread[39] = {0};
     int& regs = regs_per_thread[variant];
     if (regs == 0) {
         cudaFuncAttributes fa;
@@ -787,32 +915,35 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
         regs = fa.numRegs > 0 ? fa.numRegs : 64;
     }
     const int reg_warps = 65536 / (regs * 32);          // warps the register file holds
-    const long long heads = (long long)p.B * p.H;
     int best_nw = 0, best_ctas = 1, best_warps = 0;
     // (eight warps and fewer first: larger CTAs only where they hold more warps per SM than any number of smaller ones, the
     // staged coefficient maps being shared by more of them.  Windows, CTAs of at most 8 -> 16 (12) warps: Mamba-2 layer of
     // batch 256 624 -> 605 us, 2048 4458 -> 4385, rank 32 with L = 64 4750 -> 4677, state-dependent bfloat16 map 917 -> 890.  With
     // fewer heads than warps fit, larger CTAs only leave more SMs idle: general kernel, 64 heads, 4.2 -> 4.9 us; the lean ones,
     // whose CTAs stage less per head, did not lose by it)
+    if (variant < 13) W = 1;
     for (int i = 0; i < max_nw; ++i) {
         const int nw = i < 8 ? 8 - i : i + 1;
+        if (nw % W || nw / W > 15) continue;
         if (nw > 8 && variant == 0 && heads <= (long long)ctx->sm_count * best_warps) break;
         if (p.warps_per_cta && (nw != p.warps_per_cta || nw > 8)) continue;       // (a caller's own choice: 1 to 8)
-        const DecodeSmem d = make_decode_smem(K, p.R, nw, p.full_read, p.coef_per_seq, sl.total);
-        if (d.total > smem_budget) continue;
-        int ctas = (int)((228u * 1024u) / (d.total + 1024u));
+        const DecodeSmem d = make_decode_smem(K, p.R, nw, p.full_read, p.coef_per_seq, sl.total, W);
+        const uint32_t per_sm = (W == 2 && p.full_read && p.stream_state ? 200u : 228u) * 1024u;
+        if (d.total > smem_budget || d.total + 1024u > per_sm) continue;
+        int ctas = (int)(per_sm / (d.total + 1024u));
         if (ctas * nw > cap) ctas = cap / nw;
         if (ctas * nw > reg_warps) ctas = reg_warps / nw;
         if (ctas < 1) continue;
         if (ctas * nw > best_warps) { best_warps = ctas * nw; best_nw = nw; best_ctas = ctas; }
     }
     if (best_nw == 0) return SKETCHSSM_UNSUPPORTED_SHAPE;
-    const DecodeSmem d = make_decode_smem(K, p.R, best_nw, p.full_read, p.coef_per_seq, sl.total);
+    const DecodeSmem d = make_decode_smem(K, p.R, best_nw, p.full_read, p.coef_per_seq, sl.total, W);
     if ((ctx->last_cuda_error = unlock_smem(ctx, kern)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     long long grid = (long long)ctx->sm_count * best_ctas;
     const long long total = (long long)p.B * p.H;
     if (p.batches_per_cta > 0) grid = (total + p.batches_per_cta - 1) / p.batches_per_cta;   // explicit items per CTA
-    if (grid > (total + best_nw - 1) / best_nw) grid = (total + best_nw - 1) / best_nw;      // at least one head per warp
+    const int teams = best_nw / W;
+    if (grid > (total + teams - 1) / teams) grid = (total + teams - 1) / teams;      // at least one head per team
     if (grid < p.H) grid = p.H;                                  // a CTA's range then spans at most two head indices
     if (grid > total) grid = total;
     if ((ctx->last_cuda_error = launch_kernel(kern, dim3((unsigned)grid), dim3(best_nw * 32), d.total, stream, p, p.pdl != 0)) != cudaSuccess)

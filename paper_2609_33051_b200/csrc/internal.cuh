@@ -89,6 +89,7 @@ struct Params {
     int n_cap;            // update (CUDA cores) with per-sequence phases: ring rows the shared-memory layout has room for
     int sketch_bf16;      // U (and the fixed C) are stored as bfloat16
     float* erase;         // projected erase vectors f_s [B][H][L][R] (Eq. 44-45), or nullptr: c_t = C q~_t from the swept query
+    int stream_state;     // decode, full reads: the state is larger than what stays in L2
     int tok_base;         // update (GDN tensor-core kernel): first ring row of this pass when a flush is replayed in blocks of 16 tokens
 };
 

@@ -62,6 +62,45 @@ def test_bfloat16_sketch_with_the_fixed_map_at_every_ring_fill(K, V, rank, io):
     assert errs["S"] <= 5e-5 and errs["U"] <= 2.0 ** -7, errs
 
 
+@pytest.mark.parametrize("kind,batch,heads,K,V,rank,L,io,full,ranks", [
+    # full reads: four warps a head (few heads; long rings), two (the state larger than what stays in L2), odd head counts
+    ("kda", 5, 7, 128, 128, 8, 8, "f32", True, False), ("gdn", 45, 37, 128, 128, 8, 12, "bf16", True, False),
+    ("mamba2", 3, 1, 64, 64, 8, 20, "bf16", True, False), ("mamba2", 99, 37, 128, 64, 8, 8, "f32", True, False),
+    ("mamba2", 67, 7, 128, 80, 8, 64, "bf16", True, False), ("kda", 53, 9, 64, 128, 8, 32, "bf16", True, False),
+    # a dense head among sketched ones: four warps a head, two
+    ("mamba2", 11, 6, 128, 80, 13, 12, "bf16", False, True), ("mamba2", 151, 7, 128, 64, 24, 8, "f32", False, True),
+    ("gdn", 9, 5, 128, 128, 16, 8, "bf16", False, True), ("kda", 171, 6, 64, 64, 9, 12, "bf16", False, True),
+    # long rings and large ranks: two warps a head, then four as the ring fills
+    ("mamba2", 37, 9, 128, 64, 32, 64, "bf16", False, False), ("mamba2", 37, 9, 128, 128, 16, 64, "bf16", False, False),
+    ("mamba2", 31, 9, 128, 80, 21, 64, "f32", False, False), ("mamba2", 31, 9, 64, 128, 45, 64, "f32", False, False)])
+def test_teams_of_warps_and_single_warps_agree(kind, batch, heads, K, V, rank, L, io, full, ranks):
+    """Several warps per head against one (a caller's limit on the warps selects that): the same windows, the rings bit for bit."""
+    w = synth.Workload("t", kind, batch, heads, K, V, rank, L, 0, io, 421, basis="qr")
+    outs, rings = [], []
+    for single in (False, True):
+        m, *_rest, dev = make_layer(w)
+        if ranks:
+            m.head_rank = torch.tensor([[rank, 0, 1, (rank + 1) // 2, rank][h % 5] for h in range(heads)], dtype=torch.int32, device=dev)
+            m.bind()
+        m.ring.zero_()
+        m.bind()
+        m.state_update(0)
+        if single:
+            m.tune("decode_max_warps_per_sm", 32)
+        got = []
+        for t in range(L - 1):
+            tt = harness.token_tensors(w, synth.step_inputs(w, 0, t), dev)
+            call = m.full_read_decode if full else m.decode_step
+            got.append(call(t, tt["q"], tt["k"], tt["v"], tt["beta"], tt["decay"], m.new_output()).cpu().numpy())
+        m.check_status()
+        outs.append(np.stack(got))
+        rings.append(m.ring.cpu().numpy().copy())
+    assert np.all(np.isfinite(outs[1]))
+    for a, b in zip(*outs):
+        assert harness.rel_err(a, b.astype(np.float64)) <= 2e-5
+    assert np.array_equal(*rings)
+
+
 @pytest.mark.parametrize("call", ["decode_step", "full_read_decode"])
 def test_a_callers_warp_count_is_taken_up_to_eight_and_refused_above(call):
     from paper_2609_33051_b200.binding import SketchSSMError
