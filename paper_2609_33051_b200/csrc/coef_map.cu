@@ -846,6 +846,10 @@ static int launch_coef_kv(Ctx* ctx, const Params& p, cudaStream_t stream) {
 // Rebuild the per-(batch, head) coefficient maps from the state and sketch the preceding flush kernel left in memory.
 int launch_coef_map(Ctx* ctx, const Params& p, cudaStream_t stream) {
     if (p.pivots > kMaxPivots) return SKETCHSSM_UNSUPPORTED_SHAPE;
+    if (p.pivots > 0) {        // a warp per head where that is the faster one
+        const int rc = launch_pivot_map(ctx, p, stream);
+        if (rc != SKETCHSSM_UNSUPPORTED_SHAPE) return rc;
+    }
     const int K = ctx->cfg.dk, V = ctx->cfg.dv;
     if (K == 128 && V == 128) return launch_coef_kv<128, 128>(ctx, p, stream);
     if (K == 128 && V == 64) return launch_coef_kv<128, 64>(ctx, p, stream);

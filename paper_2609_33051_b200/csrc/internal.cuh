@@ -108,6 +108,7 @@ int launch_decode_split_kda_bf16(Ctx* ctx, const Params& p, cudaStream_t stream)
 int launch_update(Ctx* ctx, const Params& p, cudaStream_t stream);       // CUDA cores, every configuration
 int launch_update_cols(Ctx* ctx, const Params& p, cudaStream_t stream);  // CUDA cores, delta-rule kinds, a thread per quarter column (launch_update chooses)
 int launch_coef_map(Ctx* ctx, const Params& p, cudaStream_t stream);     // state-dependent coefficient maps from S_new and U (after a flush)
+int launch_pivot_map(Ctx* ctx, const Params& p, cudaStream_t stream);    // the same, up to four pivots, a warp per head; UNSUPPORTED_SHAPE otherwise
 int launch_wait_probe(Ctx* ctx, int poll_limit, int where, cudaStream_t stream);   // self-test: a bounded wait that runs out
 int launch_update_tc(Ctx* ctx, const Params& p, cudaStream_t stream);    // tcgen05 tensor cores, Mamba-2; UNSUPPORTED_SHAPE outside its domain
 int launch_update_tc_ws(Ctx* ctx, const Params& p, cudaStream_t stream); // same, two warp groups per CTA (operand building overlaps the state stream)
