@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(kWsThreads, 2) update_tc_ws_mamba2_kernel(cons
     volatile int* seq_ring = reinterpret_cast<volatile int*>(smem + sm.misc + 16);
     volatile int* seq_pub = reinterpret_cast<volatile int*>(smem + sm.misc + 32);
     auto seq_get = [&](int k) -> int {          // -2: the wait ran out
+#pragma unroll 1
         for (uint32_t it = 0; it < (1u << 22); ++it) {
             if (*seq_pub > k) {
                 __threadfence_block();
@@ -290,7 +291,7 @@ __global__ void __launch_bounds__(kWsThreads, 2) update_tc_ws_mamba2_kernel(cons
                 }
                 const int b = k & 1;
                 const uint32_t tmem_t = tmem_base + (uint32_t)b * 128u;
-#pragma unroll
+#pragma unroll 2
                 for (int c = 0; c < NCH; ++c) {
                     if (!mbar_wait_bounded(&bars[kBarA2Rdy + (c & 1)], (phR >> (c & 1)) & 1u)) { bad = true; break; }
                     phR ^= 1u << (c & 1);
@@ -501,8 +502,8 @@ __global__ void __launch_bounds__(kWsThreads, 2) update_tc_ws_mamba2_kernel(cons
         };
 
         if (gt == 0) claim_issue();
-        stage_next();
-        if (stg_bufs > 1 && n_stage_blocks > 1) stage_next();
+#pragma unroll 1
+        for (int i = stg_bufs > 1 && n_stage_blocks > 1 ? 2 : 1; i > 0; --i) stage_next();
         // W (padding columns, lo halves of the query columns) and the MMA-1 operands (off-diagonal head blocks) hold
         // zeros that no tile ever overwrites: written once
         for (uint32_t o = (uint32_t)gt * 16u; o < 2u * (uint32_t)NP * kK * 2u; o += kGroup * 16u)

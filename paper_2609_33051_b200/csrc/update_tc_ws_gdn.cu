@@ -184,6 +184,7 @@ __global__ void __launch_bounds__(kGThreads, 2) update_tc_ws_gdn_kernel(const Pa
     volatile int* seq_ring = reinterpret_cast<volatile int*>(smem + sm.misc + 16);
     volatile int* seq_pub = reinterpret_cast<volatile int*>(smem + sm.misc + 32);
     auto seq_get = [&](int k) -> int {          // -2: the wait ran out
+#pragma unroll 1
         for (uint32_t it = 0; it < (1u << 22); ++it) {
             if (*seq_pub > k) {
                 __threadfence_block();
@@ -303,25 +304,18 @@ __global__ void __launch_bounds__(kGThreads, 2) update_tc_ws_gdn_kernel(const Pa
             phPro ^= 1u << b;
         };
 
-        int cur = seq_get(0);
-        if (cur >= 0) {
-            wait_pro(0);
-            pass_a(0, false);
-            do_e(0);
-            for (int k = 0; !bad; ++k) {
-                const int b = k & 1;
-                const int raw = seq_get(k + 1);
-                if (raw < -1) { bad = true; break; }
-                if (raw < 0) break;
-                wait_pro(b ^ 1);
-                pass_a(b ^ 1, true);
-                // the E' operand buffer is read by K^T E' of tile k: that must be complete before it is rewritten
-                bad |= !mbar_wait_bounded(&bars[gTfull + b], (phT >> b) & 1u);
-                phT ^= 1u << b;
-                do_e(b ^ 1);
+        // (one call site each, here and in the other roles: the bodies are inlined, and the kernel's code has to stay small)
+        for (int k = 0; !bad; ++k) {
+            const int b = k & 1;
+            const int raw = seq_get(k);
+            if (raw < 0) { bad = raw < -1; break; }
+            wait_pro(b);
+            pass_a(b, k > 0);
+            if (k > 0) {     // the E' operand buffer is read by K^T E' of the tile before: that must be complete before it is rewritten
+                bad |= !mbar_wait_bounded(&bars[gTfull + (b ^ 1)], (phT >> (b ^ 1)) & 1u);
+                phT ^= 1u << (b ^ 1);
             }
-        } else if (cur < -1) {
-            bad = true;
+            do_e(b);
         }
         if (bad && lane == 0) record_fault(p.status, kFaultUpdateWait, 3);
     } else if (warp >= 10) {
@@ -462,19 +456,11 @@ __global__ void __launch_bounds__(kGThreads, 2) update_tc_ws_gdn_kernel(const Pa
                 tc_mma_bf16(tmem_c, ehi, bclo, idescU, 1u);
                 tc_commit(&bars[gTfull + b]);
             };
-            int cur = seq_get(0);
-            if (cur >= 0) {
-                pass_a(0);
-                if (!bad) step_e(0);
-                for (int k = 0; !bad; ++k) {
-                    const int raw = seq_get(k + 1);
-                    if (raw < -1) { bad = true; break; }
-                    if (raw >= 0) pass_a(k + 1);
-                    if (raw < 0 || bad) break;
-                    step_e(k + 1);       // the pass-A group forms E'(k + 1) right after pass A of tile k + 1
-                }
-            } else if (cur < -1) {
-                bad = true;
+            for (int k = 0; !bad; ++k) {
+                const int raw = seq_get(k);
+                if (raw < 0) { bad = raw < -1; break; }
+                pass_a(k);
+                if (!bad) step_e(k);       // the pass-A group forms E'(k) right after pass A of the tile
             }
             if (bad) record_fault(p.status, kFaultUpdateWait, where);
         }
@@ -497,17 +483,10 @@ __global__ void __launch_bounds__(kGThreads, 2) update_tc_ws_gdn_kernel(const Pa
                 if (++stage == NS) { stage = 0; ++round; }
             }
         };
-        int cur = seq_get(0);
-        if (cur >= 0) {
-            load_tile(cur);
-            for (int k = 0; !bad; ++k) {
-                const int raw = seq_get(k + 1);
-                if (raw < -1) { bad = true; break; }
-                if (raw < 0) break;
-                load_tile(raw);
-            }
-        } else if (cur < -1) {
-            bad = true;
+        for (int k = 0; !bad; ++k) {
+            const int raw = seq_get(k);
+            if (raw < 0) { bad = raw < -1; break; }
+            load_tile(raw);
         }
         if (bad && lane == 0) record_fault(p.status, kFaultUpdateWait, 7);
     } else {

@@ -195,6 +195,7 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
     volatile int* seq_ring = reinterpret_cast<volatile int*>(smem + sm.misc + 16);
     volatile int* seq_pub = reinterpret_cast<volatile int*>(smem + sm.misc + 32);
     auto seq_get = [&](int k) -> int {          // -2: the wait ran out
+#pragma unroll 1
         for (uint32_t it = 0; it < (1u << 22); ++it) {
             if (*seq_pub > k) {
                 __threadfence_block();
