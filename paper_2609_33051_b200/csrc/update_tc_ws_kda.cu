@@ -21,15 +21,21 @@
 // [P | U0] and two 128-column accumulators for alternating tiles, so pass A of tile k + 1 (issued before the E step of
 // tile k) never waits for the write-back of tile k.
 //
-// Front group, 256 threads, thread = (token block, channel i): reads column i of its block's staged key and decay rows
-// into registers, forms the running products and writes its rows of Khat / Ktil / G_n * W in the operand layouts.  The
-// 32 x 32 system is handled as two blocks of 16 tokens: the 120 pair sums inside a block are per-channel products of
-// that block's threads reduced over the 128 channels by transposing butterflies (per-warp partials summed in a fixed
-// order: results are bitwise reproducible); the 16 x 16 block that couples the two blocks is an mma.sync product of
-// rescaled keys (the decay product splits at the block boundary without a quotient); T_11 and T_22 by forward
-// substitution (one column per thread, one warp each) while six warps form Ktil [Omega | q] with mma.sync.  The E step
-// (E_1 = T_11 x_1, E_2 = T_22 (x_2 - A_21 E_1), 528 multiply-adds per lane) runs on the pass-B group, between the
-// write-back of one tile and the next, so that the pass-A group only streams.
+// Front group, 256 threads, thread = (block of eight tokens, channel pair): reads its columns of the staged key and decay rows
+// into registers, forms the running products in packed pairs and writes its rows of Khat / Ktil / G_n * W in the operand layouts,
+// four bytes at a time.  The pair sums of A inside a block of eight (28) are per-channel products reduced over the channels by one
+// transposing butterfly (per-warp partials summed in a fixed order: results are bitwise reproducible); the 8 x 8 and 16 x 16
+// blocks that couple them are mma.sync products of rescaled keys (the decay product splits at a block boundary without a
+// quotient).  T_11 and T_22 of the two blocks of 16 by forward substitution (one column per thread, one warp each) while six warps
+// form Ktil [Omega | q] with mma.sync.  The E step (E_1 = T_11 x_1, E_2 = T_22 (x_2 - A_21 E_1), 264 packed multiply-adds per lane)
+// runs on the pass-B group, between the write-back of one tile and the next, so that the pass-A group only streams.
+//
+// What bounds it: the chain of the front group (some 10 k cycles a tile; the state of a tile takes 6.6 k at the rate of a copy),
+// most of it instruction supply and latency of eight warps: pair sums and Z rows 2.4 k, coupling 1.2 k, operand rows 1.4 k,
+// Ktil W and T 2.3 k.  Flush of 16384 heads, 32 tokens: 1030 us with a channel per thread, blocks of 16 tokens (120 pair sums) and
+// 190 KB of code; 740 now (0.56 of a copy's rate).  Not kept: E of the next tile before the write-back (the accumulator is freed
+// late: +60 us), T before the wait for the operand set (+40), the coupling products of a level on one warp with its fragments a
+// step ahead (spills: +100).
 //
 // Domain: KDA, bf16 I/O, K = V = 128, rank <= 16; 1..32 tokens per pass, up to 64 tokens per flush in blocks of 32.
 #include <type_traits>
@@ -47,10 +53,10 @@ constexpr int kKThreads = 576;       // pass-A group (4 warps), front group part
 constexpr int kKFront = 256;         // threads of the front group
 constexpr int kNT = 32;              // tokens per pass
 constexpr int kKStages = 8;          // upper bound on the shared-memory stages of state rows
-constexpr int kAS = 36;              // (sizes the work area of A: 32 rows of 36 floats)
 constexpr int kAS2 = 20;             // row stride (floats) of the two 16 x 16 triangles of A
 constexpr uint32_t kZPitch = 272u;   // bytes between the rows of the rescaled keys Z[token][channel]: 256 + 16, so that the 8 rows of an ldmatrix fall in different banks
-constexpr uint32_t kZHalf = 32u * kZPitch;   // hi rows, then lo rows
+constexpr uint32_t kZHalf = 64u * kZPitch;   // hi rows, then lo rows: tokens 0..31 for the boundary at token 16, again for those at 8 and 24
+constexpr int kOP = 132;             // floats between the columns of Omega in shared memory [16][128]
 // Pass-A window [Khat 32 | G_n * W 32]: 64 rows of 16 bytes per group of 8 channels, the groups 16 bytes further apart than
 // they need to be, so that the per-channel threads of a warp (4 groups) store to different banks
 constexpr uint32_t kLboW = 64u * 16u + 16u;
@@ -62,7 +68,7 @@ constexpr int kKA2 = 2;              // chunk buffers between the pass-A group a
 constexpr int kNPk = 32;             // columns of [Omega | q]: Omega in 0..R-1, q at column QA = round_up(R, 8) <= 16
 
 struct KSmem {
-    uint32_t a2, e, w, w_stride, w_lo, set, set_stride, set_bt, set_bt_lo, set_vv, set_t1, set_bc, set_gn, stg, stg_g, stg_v,
+    uint32_t a2, e, w, w_stride, w_lo, set, set_stride, set_bt, set_bt_lo, set_vv, set_t1, set_bc, set_gn, stg, stg_g,
         stg_beta, stg_q, mats, om, bars, misc, sst, sst_bytes, total;
 };
 
@@ -76,16 +82,17 @@ __host__ __device__ inline KSmem make_ksmem(int stages) {
     // per-tile operand set, double-buffered: Ktil as B operand of Ktil^T E (MN-major, hi | lo), raw value rows, T,
     // Ktil [Omega | q] hi | lo (B operand of the sketch correction), G_n
     s.set = off;
-    s.set_bt = 0u; s.set_bt_lo = kKtHalf; s.set_vv = 2u * kKtHalf; s.set_t1 = s.set_vv + 8192u; s.set_bc = s.set_t1 + 4096u;
+    s.set_bt = 0u; s.set_bt_lo = kKtHalf; s.set_vv = 2u * kKtHalf; s.set_t1 = s.set_vv + 8192u; s.set_bc = s.set_t1 + 3072u;
     s.set_gn = s.set_bc + 4096u;
     s.set_stride = s.set_gn + 512u;
     off += 2u * s.set_stride;
-    // staging of the next tile's raw rows: keys [32][256 B], decays [32][256 B], values [32][256 B], beta [L] floats, query row.
-    // Once a tile's rows are in registers the key / decay area is re-used (A partials, then Ktil in fp32).
-    s.stg_g = 8192u; s.stg_v = 16384u; s.stg_beta = 24576u; s.stg_q = 24832u;
-    s.stg = off; off += 25088u;
-    s.mats = off; off += (uint32_t)kNT * kAS * 4u + 256u;         // A (beta_s A_sj), beta
-    s.om = off; off += (uint32_t)kK * 16u * 4u;                   // Omega of the current head index, fp32 [K][16] (zero beyond the rank)
+    // staging of the next tile's raw rows: keys [32][256 B], decays [32][256 B]; beta [L] floats, query row (double-buffered: it is
+    // read until the tile is finished).  (Value rows go straight into the set.)  Once a tile's rows are in registers the key / decay
+    // area is re-used for the rescaled keys Z.
+    s.stg_g = 8192u; s.stg_beta = 2u * kZHalf; s.stg_q = s.stg_beta + 256u;
+    s.stg = off; off += s.stg_q + 512u;
+    s.mats = off; off += 2u * 16u * kAS2 * 4u + 128u + 8u * 32u * 4u + 4u * 128u * 4u;    // A (beta_s A_sj), beta, partial pair sums, products of the decays of eight tokens
+    s.om = off; off += 16u * kOP * 4u;                            // Omega of the current head index, fp32 (zero beyond the rank)
     s.bars = off; off += 512u;
     s.misc = off; off += 128u;
     off = (off + 127u) & ~127u;
@@ -97,7 +104,7 @@ __host__ __device__ inline KSmem make_ksmem(int stages) {
 
 enum { kPro = 0, kPfull = 2, kTfull = 4, kBdone = 6, kBufFree = 8, kA2free = 10, kA2rdy = 10 + kKA2, kErdy = 10 + 2 * kKA2,
        kStg = 11 + 2 * kKA2, kStDone = 12 + 2 * kKA2, kFull = 14 + 2 * kKA2, kEmpty = 14 + 2 * kKA2 + kKStages,
-       kTfree = 14 + 2 * kKA2 + 2 * kKStages, kNumBars = 16 + 2 * kKA2 + 2 * kKStages };
+       kTfree = 14 + 2 * kKA2 + 2 * kKStages, kVals = 16 + 2 * kKA2 + 2 * kKStages, kNumBars = 18 + 2 * kKA2 + 2 * kKStages };
 
 __device__ __forceinline__ void k_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -123,17 +130,10 @@ __device__ __forceinline__ void k_ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
-__device__ __forceinline__ void k_ldmatrix_x2(uint32_t addr, uint32_t (&r)[2]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
-}
-__device__ __forceinline__ void k_mma_16816(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+__device__ __forceinline__ void k_mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-__device__ __forceinline__ float bf16_at(const unsigned char* base, uint32_t elem) {
-    return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(base)[elem]);
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
 }  // namespace
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
         *reinterpret_cast<volatile int*>(smem + sm.misc + 32) = 0;
         for (int i = 0; i < kNumBars; ++i) {
             // one arrival per warp of a stream group: chunk ready, E ready, stage empty, accumulator halves, pass-B done, slot free
-            const bool per_warp = (i >= kA2rdy && i <= kErdy) || i == kStDone || i == kStDone + 1 || i >= kEmpty || (i >= kBdone && i < kBdone + 4);
+            const bool per_warp = (i >= kA2rdy && i <= kErdy) || i == kStDone || i == kStDone + 1 || (i >= kEmpty && i < kVals) || (i >= kBdone && i < kBdone + 4);
             mbar_init(&bars[i], per_warp ? 4 : 1);
         }
         mbar_fence_init();
@@ -279,25 +279,17 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
             phPro ^= 1u << b;
         };
 
-        int cur = seq_get(0);
-        if (cur >= 0) {
-            wait_pro(0);
-            pass_a(0, 0);
-            for (int k = 0; !bad; ++k) {
-                const int b = k & 1;
-                const int raw = seq_get(k + 1);
-                if (raw < -1) { bad = true; break; }
-                if (raw < 0) break;
-                wait_pro(b ^ 1);
-                pass_a(b ^ 1, k + 1);
-            }
-        } else if (cur < -1) {
-            bad = true;
+        // (one call site each, here and in the other roles: the bodies are inlined, and the kernel's code has to stay small)
+        for (int k = 0; !bad; ++k) {
+            const int raw = seq_get(k);
+            if (raw < 0) { bad = raw < -1; break; }
+            wait_pro(k & 1);
+            pass_a(k & 1, k);
         }
         if (bad && lane == 0) record_fault(p.status, kFaultUpdateWait, 103);
     } else if (warp >= 10 && warp < 14) {
         // =========================== pass-B group: S_new written back, then the sketch rows ===========================
-        uint32_t phT = 0, phP = 0;
+        uint32_t phT = 0, phP = 0, phV = 0;
         bool bad = false;
         // E = T (V - P) with T = (I + Bd A)^{-1} Bd solved in two blocks of 16 tokens -> hi + lo A operand of Ktil^T E
         // (chunk-buffer layout, 32 tokens)
@@ -308,7 +300,9 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
             const unsigned char* set = set_ptr(b);
             const __nv_bfloat16* sV = reinterpret_cast<const __nv_bfloat16*>(set + sm.set_vv);
             const float* sT1 = reinterpret_cast<const float*>(set + sm.set_t1);
-            float x[kNT];
+            if (!mbar_wait_bounded(&bars[kVals + b], (phV >> b) & 1u)) bad = true;      // the value rows
+            phV ^= 1u << b;
+            f32x2 x[kNT / 2];                       // pairs of tokens
             {
                 float x0[16], x1[16];
                 if (!bad) {
@@ -319,55 +313,45 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                     for (int t = 0; t < 16; ++t) { x0[t] = 0.f; x1[t] = 0.f; }
                 }
 #pragma unroll
-                for (int t = 0; t < 16; ++t) {
-                    x[t] = __bfloat162float(sV[t * V + j]) - x0[t];
-                    x[16 + t] = __bfloat162float(sV[(16 + t) * V + j]) - x1[t];
+                for (int t = 0; t < 16; t += 2) {
+                    x[t / 2] = pack2(__bfloat162float(sV[t * V + j]) - x0[t], __bfloat162float(sV[(t + 1) * V + j]) - x0[t + 1]);
+                    x[8 + t / 2] = pack2(__bfloat162float(sV[(16 + t) * V + j]) - x1[t], __bfloat162float(sV[(17 + t) * V + j]) - x1[t + 1]);
                 }
             }
             // The 32 x 32 system in two blocks of 16 tokens:  E_1 = T_11 x_1,  E_2 = T_22 (x_2 - A_21 E_1)
             const float* sT11 = sT1;
             const float* sT22 = sT1 + 256;
             const float* sA21 = sT1 + 512;
-            float e1[16], e2[16];
-#pragma unroll
-            for (int s = 0; s < 16; ++s) {
-                float acc = 0.f;
-#pragma unroll
-                for (int t4 = 0; t4 <= s / 4; ++t4) {      // T_11 is lower triangular
-                    const float4 tt = *reinterpret_cast<const float4*>(sT11 + s * 16 + t4 * 4);
-                    acc = fmaf(tt.x, x[t4 * 4], acc);
-                    acc = fmaf(tt.y, x[t4 * 4 + 1], acc);
-                    acc = fmaf(tt.z, x[t4 * 4 + 2], acc);
-                    acc = fmaf(tt.w, x[t4 * 4 + 3], acc);
-                }
-                e1[s] = acc;
-            }
-#pragma unroll
-            for (int s = 0; s < 16; ++s) {
-                float acc = x[16 + s];
+            // the first 4 n4 columns of a row times 2 n4 pairs
+            auto row_dot = [&](const float* row, const f32x2* v, int n4) {
+                f32x2 a0 = pack2(0.f, 0.f), a1 = a0;
 #pragma unroll
                 for (int t4 = 0; t4 < 4; ++t4) {
-                    const float4 aa = *reinterpret_cast<const float4*>(sA21 + s * 16 + t4 * 4);
-                    acc = fmaf(-aa.x, e1[t4 * 4], acc);
-                    acc = fmaf(-aa.y, e1[t4 * 4 + 1], acc);
-                    acc = fmaf(-aa.z, e1[t4 * 4 + 2], acc);
-                    acc = fmaf(-aa.w, e1[t4 * 4 + 3], acc);
+                    if (t4 < n4) {
+                        const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(row + t4 * 4);
+                        a0 = fma2(m.x, v[2 * t4], a0);
+                        a1 = fma2(m.y, v[2 * t4 + 1], a1);
+                    }
                 }
-                x[16 + s] = acc;
+                float p, q, r, u;
+                unpack2(a0, p, q);
+                unpack2(a1, r, u);
+                return (p + q) + (r + u);
+            };
+            float e1[16], e2[16];
+            f32x2 e1p[8];
+#pragma unroll
+            for (int s = 0; s < 16; ++s) e1[s] = row_dot(sT11 + s * 16, x, s / 4 + 1);          // T_11 is lower triangular
+#pragma unroll
+            for (int s = 0; s < 8; ++s) e1p[s] = pack2(e1[2 * s], e1[2 * s + 1]);
+#pragma unroll
+            for (int s = 0; s < 8; ++s) {
+                float u, v;
+                unpack2(x[8 + s], u, v);
+                x[8 + s] = pack2(u - row_dot(sA21 + (2 * s) * 16, e1p, 4), v - row_dot(sA21 + (2 * s + 1) * 16, e1p, 4));
             }
 #pragma unroll
-            for (int s = 0; s < 16; ++s) {
-                float acc = 0.f;
-#pragma unroll
-                for (int t4 = 0; t4 <= s / 4; ++t4) {      // T_22 is lower triangular
-                    const float4 tt = *reinterpret_cast<const float4*>(sT22 + s * 16 + t4 * 4);
-                    acc = fmaf(tt.x, x[16 + t4 * 4], acc);
-                    acc = fmaf(tt.y, x[16 + t4 * 4 + 1], acc);
-                    acc = fmaf(tt.z, x[16 + t4 * 4 + 2], acc);
-                    acc = fmaf(tt.w, x[16 + t4 * 4 + 3], acc);
-                }
-                e2[s] = acc;
-            }
+            for (int s = 0; s < 16; ++s) e2[s] = row_dot(sT22 + s * 16, x + 8, s / 4 + 1);
             unsigned char* ehi = smem + sm.e;
             unsigned char* elo = ehi + 128u * (uint32_t)kNT * 2u;
 #pragma unroll
@@ -388,12 +372,13 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
             bad = __any_sync(0xffffffffu, bad);
             if (lane == 0 && !bad) k_arrive(&bars[kErdy]);
         };
-        int raw = seq_get(0);
-        if (raw >= 0) do_e(0);
-        else bad = raw < -1;
-        for (int k = 0; !bad && raw >= 0; ++k) {
-            const int tile = raw;
+        for (int k = 0; !bad; ++k) {
+            const int tile = seq_get(k);
+            if (tile < 0) { bad = tile < -1; break; }
             const int b = k & 1;
+            // the E step: the tile's P is complete once its pass A is, and the E operand buffer is free because Ktil^T E of the
+            // tile before has completed (waited for below)
+            do_e(b);
             const int h = tile / tiles_per_h, bb = tile - h * tiles_per_h;
             const size_t bh = (size_t)bb * H + h;
             float* So = p.state + bh * (size_t)K * V + j;
@@ -449,11 +434,6 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                 __syncwarp();
                 if (lane == 0) k_arrive(&bars[kBufFree + b]);       // the slot is free for pass A of tile k + 2
             }
-            // the E step of the next tile: its P is complete once pass A of that tile is, and the E operand buffer is free
-            // because Ktil^T E of this tile has completed (waited for above)
-            raw = seq_get(k + 1);
-            if (raw < 0) { bad |= raw < -1; break; }
-            if (!bad) do_e(b ^ 1);
         }
         if (bad && lane == 0) record_fault(p.status, kFaultUpdateWait, 111);
     } else if (warp == 8) {
@@ -492,66 +472,60 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                 }
                 tc_commit(&bars[kTfull + b]);
             };
-            // The E step of a tile is issued as soon as its E operand is ready, also in the middle of the next tile's pass A:
-            // every wait of pass A polls for it in turn (pend_e: the tile whose E step is still to be issued, or -1).
+            // The E step of a tile is issued as soon as its E operand is ready, also in the middle of the next tile's pass A
+            // (pend_e: the tile whose E step is still to be issued, or -1).
             int pend_e = -1;
-            auto wait_or_e = [&](uint64_t* bar, uint32_t phase) -> bool {
-                for (uint32_t it = 0; it < (1u << 22); ++it) {
-                    if (mbar_test_wait(bar, phase)) return true;
-                    if (pend_e >= 0 && mbar_test_wait(&bars[kErdy], phE)) {
-                        const int ke = pend_e;
-                        pend_e = -1;
-                        step_e(ke);
-                        if (bad) return false;
-                    }
-                }
-                return false;
-            };
-            // [P | U0](b) = S_0^T [Khat^T | G_n * W] chunk by chunk: one 64-row window per tile
-            auto pass_a = [&](int k) {
+            // [P | U0](b) = S_0^T [Khat^T | G_n * W] chunk by chunk: one 64-row window per tile.  Pass A of tile k + 1 starts before the
+            // E step of tile k: the stream of S_0 chunks does not wait for the pass-B group (two accumulators).
+            for (int k = 0; !bad; ++k) {
+                const int raw = seq_get(k);
+                if (raw < -1) { bad = true; break; }
                 const int b = k & 1;
-                if (k >= 2) {                   // the slot still holds the sketch data of tile k - 2 until they are stored
-                    if (!wait_or_e(&bars[kBufFree + b], (phBuf >> b) & 1u)) { bad = true; where = 141; return; }
-                    phBuf ^= 1u << b;
-                    tc_fence_after();
-                }
                 const uint32_t slot = tmem_base + (uint32_t)b * 64u;
                 const uint32_t whi0 = smem_u32(w_ptr(b));
                 const uint32_t wlo0 = whi0 + sm.w_lo;
-#pragma unroll 2
-                for (int c = 0; c < NCH; ++c) {
-                    const int ab = c & (kKA2 - 1);
-                    if (!wait_or_e(&bars[kA2rdy + ab], (phR >> ab) & 1u)) { bad = true; where = 142; return; }
-                    phR ^= 1u << ab;
-                    tc_fence_after();
-                    const uint32_t a2 = a2base + (uint32_t)ab * (2u * 128u * CH * 2u);
-                    const uint64_t ahi = make_desc(a2, LBO_M, SBO);
-                    const uint64_t alo = make_desc(a2 + 128u * CH * 2u, LBO_M, SBO);
-                    const uint64_t whi = make_desc(whi0 + (uint32_t)(c * (CH / 8)) * LBO_W, LBO_W, SBO);
-                    const uint64_t wlo = make_desc(wlo0 + (uint32_t)(c * (CH / 8)) * LBO_W, LBO_W, SBO);
-                    tc_mma_bf16(slot, ahi, whi, idescA, c ? 1u : 0u);
-                    tc_mma_bf16(slot, alo, whi, idescA, 1u);
-                    tc_mma_bf16(slot, ahi, wlo, idescA, 1u);
-                    tc_commit(&bars[kA2free + ab]);
-                    if (c == NCH - 1) tc_commit(&bars[kPfull + b]);
+                // Steps of the tile: -1 the slot's sketch data of tile k - 2 are stored (k >= 2), 0 .. NCH - 1 its chunks; beside them the
+                // E step of the tile before, which is all that is left behind the last tile.
+                int c = raw < 0 ? NCH : k >= 2 ? -1 : 0;
+#pragma unroll 1
+                for (uint32_t it = 0; c < NCH || pend_e >= 0; ++it) {
+                    if (it >= (1u << 22)) {
+                        bad = true;
+                        where = c >= NCH ? 143 : c < 0 ? 141 : 142;
+                        break;
+                    }
+                    if (c < NCH) {
+                        const int ab = c & (kKA2 - 1);
+                        if (mbar_test_wait(c < 0 ? &bars[kBufFree + b] : &bars[kA2rdy + ab], (c < 0 ? phBuf >> b : phR >> ab) & 1u)) {
+                            tc_fence_after();
+                            it = 0;
+                            if (c < 0) {
+                                phBuf ^= 1u << b;
+                            } else {
+                                phR ^= 1u << ab;
+                                const uint32_t a2 = a2base + (uint32_t)ab * (2u * 128u * CH * 2u);
+                                const uint64_t ahi = make_desc(a2, LBO_M, SBO);
+                                const uint64_t alo = make_desc(a2 + 128u * CH * 2u, LBO_M, SBO);
+                                const uint64_t whi = make_desc(whi0 + (uint32_t)(c * (CH / 8)) * LBO_W, LBO_W, SBO);
+                                const uint64_t wlo = make_desc(wlo0 + (uint32_t)(c * (CH / 8)) * LBO_W, LBO_W, SBO);
+                                tc_mma_bf16(slot, ahi, whi, idescA, c ? 1u : 0u);
+                                tc_mma_bf16(slot, alo, whi, idescA, 1u);
+                                tc_mma_bf16(slot, ahi, wlo, idescA, 1u);
+                                tc_commit(&bars[kA2free + ab]);
+                                if (c == NCH - 1) tc_commit(&bars[kPfull + b]);
+                            }
+                            ++c;
+                        }
+                    }
+                    if (pend_e >= 0 && mbar_test_wait(&bars[kErdy], phE)) {
+                        step_e(pend_e);
+                        pend_e = -1;
+                        it = 0;
+                        if (bad) break;
+                    }
                 }
-            };
-            int cur = seq_get(0);
-            if (cur >= 0) {
-                // pass A of tile k + 1 starts before the E step of tile k: the stream of S_0 chunks does not wait for the
-                // pass-B group (two accumulators); the E step goes out as soon as that group has formed E
-                pass_a(0);
-                for (int k = 0; !bad; ++k) {
-                    pend_e = k;
-                    const int raw = seq_get(k + 1);
-                    if (raw < -1) { bad = true; break; }
-                    if (raw >= 0) pass_a(k + 1);
-                    if (bad) break;
-                    if (pend_e >= 0) { pend_e = -1; step_e(k); }
-                    if (raw < 0) break;
-                }
-            } else if (cur < -1) {
-                bad = true;
+                if (bad || raw < 0) break;
+                pend_e = k;
             }
             if (bad) record_fault(p.status, kFaultUpdateWait, where);
         }
@@ -562,6 +536,8 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
         auto load_tile = [&](int tile) {
             const int h = tile / tiles_per_h, bb = tile - h * tiles_per_h;
             const float* src = p.state + ((size_t)bb * H + h) * (size_t)K * V;
+            if (lane == 0)          // (two stages do not cover the latency of memory)
+                asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(K * V * 4) : "memory");
             for (int c = 0; c < NCH; ++c) {
                 if (round > 0) {     // the stage was released by all four stream warps
                     if (!mbar_wait_bounded(&bars[kEmpty + stage], (uint32_t)(round - 1) & 1u)) { bad = true; return; }
@@ -574,35 +550,28 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                 if (++stage == NS) { stage = 0; ++round; }
             }
         };
-        int cur = seq_get(0);
-        if (cur >= 0) {
-            load_tile(cur);
-            for (int k = 0; !bad; ++k) {
-                const int raw = seq_get(k + 1);
-                if (raw < -1) { bad = true; break; }
-                if (raw < 0) break;
-                load_tile(raw);
-            }
-        } else if (cur < -1) {
-            bad = true;
+        for (int k = 0; !bad; ++k) {
+            const int raw = seq_get(k);
+            if (raw < 0) { bad = raw < -1; break; }
+            load_tile(raw);
         }
         if (bad && lane == 0) record_fault(p.status, kFaultUpdateWait, 107);
     } else {
         // =========================== front group: ring-only operands, tile claiming ===========================
-        // 256 threads: thread = (token block fg, channel i).  Block fg holds tokens 16 fg .. 16 fg + 15 of the pass: its
-        // threads build that block's triangle of A, its rows of Khat / Ktil and its rescaled keys, so that the two
-        // halves of a tile's ring-only work run side by side.
+        // 256 threads: thread = (block tb of eight tokens, channel pair cp): its threads build that block's triangle of A, its rows of
+        // Khat / Ktil and its rescaled keys.
         const int ft = warp < 8 ? tid - 128 : tid - (kKThreads - 128) + 128;      // 0..255 (warps 4-7, then the last four warps)
-        const int fg = ft >> 7;               // token block
-        const int i = ft & 127;               // this thread's channel
+        const int tb = ft >> 6;               // token block: tokens 8 tb .. 8 tb + 7 of the pass
+        const int cp = ft & 63;               // channels 2 cp, 2 cp + 1
         const int fw = ft >> 5;               // warp of the group, 0..7
         uint32_t phS = 0;
         bool dead = false;
         float* sA = reinterpret_cast<float*>(smem + sm.mats);
-        float* sBeta = sA + kNT * kAS;
+        float* sBeta = sA + 2 * 16 * kAS2;
+        float* sPart = sBeta + kNT;           // [8 warps][32] pair sums over a warp's 64 channels
+        float* sProd = sPart + 8 * 32;        // [4 blocks][128 channels] product of a block's decays
         float* sOm = reinterpret_cast<float*>(smem + sm.om);
         int cur_h = -1;
-        float* sPart = reinterpret_cast<float*>(sStg + 2u * kZHalf);   // [8 warps][4 batches][32] partial pair sums (over the value rows, copied out by then)
 
         // ---- tile claiming (thread 0 of the group): per-head-index counters behind the status words ----
         int* sched = p.status + kStatusInts;
@@ -635,7 +604,7 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
         // One bulk copy per thread from per-thread constants, spread over the first four warps of the group: copy number c
         // belongs to lane c / 4 of warp c % 4.  0..3: ring keys, decays, values, gates; 4..7: the token's key, decay, value, the query.
         const uint32_t stg_beta_bytes = n_ring > 0 ? (uint32_t)(p.L * 4) : 0u;
-        const uint32_t stg_bytes = (uint32_t)n_ring * 768u + stg_beta_bytes + (p.has_token ? 768u : 0u) + (p.q != nullptr ? 256u : 0u);
+        const uint32_t stg_bytes = (uint32_t)n_ring * 512u + stg_beta_bytes + (p.has_token ? 512u : 0u) + (p.q != nullptr ? 256u : 0u);
         const int cp_c = (ft < 128 && (ft & 31) < 2) ? (ft & 31) * 4 + (ft >> 5) : 32;
         const unsigned char* cp_base = nullptr;
         size_t cp_stride = 0;
@@ -643,20 +612,26 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
         switch (cp_c) {
             case 0: cp_base = p.ring + (size_t)p.tok_base * 256u; cp_stride = p.rl.head_bytes; cp_dst = 0u; cp_bytes = (uint32_t)n_ring * 256u; break;
             case 1: cp_base = p.ring + p.rl.decay_off + (size_t)p.tok_base * 256u; cp_stride = p.rl.head_bytes; cp_dst = sm.stg_g; cp_bytes = (uint32_t)n_ring * 256u; break;
-            case 2: cp_base = p.ring + p.rl.v_off + (size_t)p.tok_base * 256u; cp_stride = p.rl.head_bytes; cp_dst = sm.stg_v; cp_bytes = (uint32_t)n_ring * 256u; break;
+            case 2: cp_base = p.ring + p.rl.v_off + (size_t)p.tok_base * 256u; cp_stride = p.rl.head_bytes; cp_dst = sm.set_vv; cp_bytes = (uint32_t)n_ring * 256u; break;
             case 3: cp_base = p.ring + p.rl.beta_off; cp_stride = p.rl.head_bytes; cp_dst = sm.stg_beta; cp_bytes = stg_beta_bytes; break;
             case 4: cp_base = reinterpret_cast<const unsigned char*>(p.k); cp_stride = (size_t)K * 2; cp_dst = (uint32_t)n_ring * 256u; cp_bytes = p.has_token ? 256u : 0u; break;
             case 5: cp_base = reinterpret_cast<const unsigned char*>(p.decay); cp_stride = (size_t)K * 2; cp_dst = sm.stg_g + (uint32_t)n_ring * 256u; cp_bytes = p.has_token ? 256u : 0u; break;
-            case 6: cp_base = reinterpret_cast<const unsigned char*>(p.v); cp_stride = (size_t)V * 2; cp_dst = sm.stg_v + (uint32_t)n_ring * 256u; cp_bytes = p.has_token ? 256u : 0u; break;
+            case 6: cp_base = reinterpret_cast<const unsigned char*>(p.v); cp_stride = (size_t)V * 2; cp_dst = sm.set_vv + (uint32_t)n_ring * 256u; cp_bytes = p.has_token ? 256u : 0u; break;
             case 7: cp_base = reinterpret_cast<const unsigned char*>(p.q); cp_stride = (size_t)K * 2; cp_dst = sm.stg_q; cp_bytes = p.q != nullptr ? 256u : 0u; break;
             default: break;
         }
-        auto stage_tile = [&](int tile) {       // whole group
+        const bool cp_val = cp_c == 2 || cp_c == 6;
+        auto stage_tile = [&](int tile, int kt) {       // whole group: keys, decays, gates and the query of tile number kt
             const int h = tile / tiles_per_h, bb = tile - h * tiles_per_h;
             const size_t bw = (size_t)bb * H + h;
             if (ft == 0) mbar_expect_tx(&bars[kStg], stg_bytes);      // (the phase cannot complete before this arrival, whatever the order of the copies)
             __syncwarp();
-            if (cp_bytes) bulk_g2s(sStg + cp_dst, cp_base + bw * cp_stride, cp_bytes, &bars[kStg]);
+            if (cp_bytes && !cp_val) bulk_g2s(sStg + cp_dst + (cp_c == 7 ? 256u * (uint32_t)(kt & 1) : 0u), cp_base + bw * cp_stride, cp_bytes, &bars[kStg]);
+        };
+        auto stage_values = [&](size_t bw, int b) {     // whole group: value rows into the operand set (rows behind the last token stay zero)
+            if (ft == 0) mbar_expect_tx(&bars[kVals + b], (uint32_t)n_tot * 256u);
+            __syncwarp();
+            if (cp_bytes && cp_val) bulk_g2s(set_ptr(b) + cp_dst, cp_base + bw * cp_stride, cp_bytes, &bars[kVals + b]);
         };
         auto next_tile = [&](int k) {          // whole group
             if (ft == 0) {
@@ -666,20 +641,22 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
             }
             f_sync();                          // the published entry is the hand-off to the other threads
             const int nxt = seq_ring[k & 3];
-            if (nxt >= 0) stage_tile(nxt);
+            if (nxt >= 0) stage_tile(nxt, k);
         };
-        // the first tile: claimed, published and its rows requested before anything else
-        if (ft == 0) claim_issue();
-        next_tile(0);
         // operand rows that no tile overwrites hold zeros: the padding columns of [Omega | q] in both windows, and the
-        // padding columns of Ktil W in both sets
+        // padding columns of Ktil W in both sets; so do the value rows behind the last token
         for (uint32_t o = (uint32_t)ft * 16u; o < 2u * sm.w_stride; o += kKFront * 16u)
             *reinterpret_cast<uint4*>(smem + sm.w + o) = make_uint4(0, 0, 0, 0);
         for (int sb = 0; sb < 2; ++sb)
-            for (uint32_t o = (uint32_t)ft * 16u; o < 4096u; o += kKFront * 16u)
-                *reinterpret_cast<uint4*>(set_ptr(sb) + sm.set_bc + o) = make_uint4(0, 0, 0, 0);
+            for (uint32_t o = (uint32_t)ft * 16u; o < 8192u; o += kKFront * 16u) {
+                *reinterpret_cast<uint4*>(set_ptr(sb) + sm.set_vv + o) = make_uint4(0, 0, 0, 0);
+                if (o < 4096u) *reinterpret_cast<uint4*>(set_ptr(sb) + sm.set_bc + o) = make_uint4(0, 0, 0, 0);
+            }
+        proxy_fence();
         f_sync();
 
+        if (ft == 0) claim_issue();
+        next_tile(0);
         for (int k = 0; !dead; ++k) {
             const int raw_tile = seq_get(k);
             if (raw_tile < 0) {
@@ -704,11 +681,10 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                 const float* omg = p.omega + (size_t)h * K * R;
                 for (int idx = ft; idx < K * 16; idx += kKFront) {
                     const int kk2 = idx >> 4, g = idx & 15;
-                    sOm[idx] = (g < R && p.write_sketch) ? __ldg(omg + (size_t)kk2 * R + g) : 0.f;
+                    sOm[g * kOP + kk2] = (g < R && p.write_sketch) ? __ldg(omg + (size_t)kk2 * R + g) : 0.f;
                 }
                 cur_h = h;            // (visible to the group after the barrier below)
             }
-            const float* og = sOm + i * 16;
             // the staged rows, gates and query row of this tile must have landed
             if (!f_wait(ft, &bars[kStg], phS)) {
                 if (ft == 0) record_fault(p.status, kFaultUpdateWait, 106);
@@ -717,30 +693,22 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
             }
             phS ^= 1;
 
-            // ---- column i of this block's key and decay rows into registers, the product of the other block's decays;
-            // value rows into the set; gates ----
-            const int t0 = 16 * fg;
-            float kk[16], gg[16];
+            // ---- this thread's channel pair of its block's eight key and decay rows into registers (raw bfloat16 pairs), the
+            // product of the block's decays for the other blocks; gates ----
+            const int t0 = 8 * tb;
+            uint32_t kw[8], gw[8];
 #pragma unroll
-            for (int s = 0; s < 16; ++s) {
+            for (int s = 0; s < 8; ++s) {
                 const bool on = t0 + s < n_tot;
-                kk[s] = on ? bf16_at(sStg, (uint32_t)((t0 + s) * K + i)) : 0.f;
-                gg[s] = on ? bf16_at(sStg + sm.stg_g, (uint32_t)((t0 + s) * K + i)) : 1.f;
+                kw[s] = on ? *reinterpret_cast<const uint32_t*>(sStg + (uint32_t)(t0 + s) * 256u + 4u * (uint32_t)cp) : 0u;
+                gw[s] = on ? *reinterpret_cast<const uint32_t*>(sStg + sm.stg_g + (uint32_t)(t0 + s) * 256u + 4u * (uint32_t)cp) : 0x3f803f80u;
             }
-            float gother = 1.f;
+            auto pair_of = [](uint32_t w) { return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)); };
+            f32x2 own = pair_of(gw[0]);
 #pragma unroll
-            for (int s = 0; s < 16; ++s) {
-                const int t = 16 * (1 - fg) + s;
-                if (t < n_tot) gother *= bf16_at(sStg + sm.stg_g, (uint32_t)(t * K + i));
-            }
-            uint4 vrow[2];            // 512 vectors of 16 bytes: 32 value rows, parked in registers until the set is free
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                const int idx = ft + r * kKFront;
-                vrow[r] = make_uint4(0, 0, 0, 0);
-                if ((idx >> 4) < n_tot) vrow[r] = *reinterpret_cast<const uint4*>(sStg + sm.stg_v + (size_t)idx * 16);
-            }
-            const float q_i = p.q != nullptr ? bf16_at(sStg + sm.stg_q, (uint32_t)i) : 0.f;
+            for (int s = 1; s < 8; ++s) own = mul2(own, pair_of(gw[s]));
+            *reinterpret_cast<f32x2*>(sProd + tb * 128 + 2 * cp) = own;
+            const uint32_t qw = p.q != nullptr ? *reinterpret_cast<const uint32_t*>(sStg + sm.stg_q + 256u * (uint32_t)b + 4u * (uint32_t)cp) : 0u;
             if (ft < kNT) {
                 const int s = ft;
                 float bt = 0.f;
@@ -748,43 +716,119 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                 else if (s < n_tot) bt = tok_beta;
                 sBeta[s] = bt;
             }
-            f_sync();                  // every thread holds its column: the key / decay rows of the staging area are free
+            f_sync();                  // every thread holds its columns: the key / decay rows of the staging area are free
 
-            // ---- pair sums inside this block of 16 tokens (its triangle of A): A_sj = sum_i k_s[i] k_j[i]
-            // prod_{j<m<=s} g_m[i] as per-channel products, reduced over the 32 channels of a warp by a transposing
-            // butterfly, 32 pairs at a time: rows sa and 16 - sa in entries 0..15, rows sa + 1 and 15 - sa in 16..31 ----
+            f32x2 blk[4];              // products of the decays of all blocks
+#pragma unroll
+            for (int u = 0; u < 4; ++u) blk[u] = *reinterpret_cast<const f32x2*>(sProd + u * 128 + 2 * cp);
+            const f32x2 one2 = pack2(1.f, 1.f);
+            const f32x2 g_before = tb == 0 ? one2 : tb == 1 ? blk[0] : tb == 2 ? mul2(blk[0], blk[1]) : mul2(mul2(blk[0], blk[1]), blk[2]);
+            const f32x2 g_after = tb == 3 ? one2 : tb == 2 ? blk[3] : tb == 1 ? mul2(blk[2], blk[3]) : mul2(blk[1], mul2(blk[2], blk[3]));
+            const f32x2 g_all = mul2(mul2(blk[0], blk[1]), mul2(blk[2], blk[3]));
+
+            auto put2 = [](unsigned char* hi, unsigned char* lo, f32x2 x) {       // a pair as bf16 hi + lo
+                float a, c;
+                unpack2(x, a, c);
+                split_bf16x2(a, c, *reinterpret_cast<uint32_t*>(hi), *reinterpret_cast<uint32_t*>(lo));
+            };
+            // ---- A_sj = sum_i k_s[i] k_j[i] prod_{j<m<=s} g_m[i].  Inside a block of eight tokens: 28 pair sums as per-channel
+            // products, reduced over the warp's 64 channels by a transposing butterfly.  Between blocks the decay product splits at a
+            // block boundary without a quotient: X_s = k_s prod_{boundary<=m<=s} g_m against Y_j = k_j prod_{j<m<boundary} g_m, for the
+            // boundary at 16 (rows 0..31 of Z) and those at 8 and 24 (rows 32..63), as bf16 hi + lo rows Z[token][channel] ----
             {
-                float* part = sPart + (size_t)fw * 128;
+                f32x2 k2[8], g2[8];
 #pragma unroll
-                for (int bi = 0; bi < 4; ++bi) {
-                    float vals[32];
+                for (int s = 0; s < 8; ++s) { k2[s] = pair_of(kw[s]); g2[s] = pair_of(gw[s]); }
+                float vals[32];
 #pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        const int sa = 2 * bi + 1 + hh, o = 16 * hh;
-                        {
-                            float r = kk[sa];
+                for (int s = 1; s < 8; ++s) {
+                    f32x2 r = k2[s];
 #pragma unroll
-                            for (int jj = 7; jj >= 0; --jj)
-                                if (jj < sa) { r *= gg[jj + 1]; vals[o + jj] = r * kk[jj]; }
-                        }
-                        if (sa < 8) {
-                            const int sb2 = 16 - sa;
-                            float r = kk[sb2];
-#pragma unroll
-                            for (int jj = 14; jj >= 0; --jj)
-                                if (jj < sb2) { r *= gg[jj + 1]; vals[o + sa + jj] = r * kk[jj]; }
-                        } else {
-#pragma unroll
-                            for (int jj = 8; jj < 16; ++jj) vals[o + jj] = 0.f;
+                    for (int jj = 6; jj >= 0; --jj) {
+                        if (jj < s) {
+                            r = mul2(r, g2[jj + 1]);
+                            float a, c;
+                            unpack2(mul2(r, k2[jj]), a, c);
+                            vals[s * (s - 1) / 2 + jj] = a + c;
                         }
                     }
-                    group_reduce_transpose<32, 32>(vals, lane);      // lane l now holds entry l of the batch
-                    part[bi * 32 + lane] = vals[0];
+                }
+#pragma unroll
+                for (int e = 28; e < 32; ++e) vals[e] = 0.f;
+                group_reduce_transpose<32, 32>(vals, lane);      // lane l now holds pair l
+                sPart[fw * 32 + lane] = vals[0];
+
+                unsigned char* z16 = sStg + (uint32_t)t0 * kZPitch + 4u * (uint32_t)cp;
+                unsigned char* z8 = z16 + 32u * kZPitch;
+                // (blocks 0, 1 lie before the boundary at 16 and take Y there, blocks 2, 3 take X; blocks 0, 2 take Y at 8 / 24)
+                const f32x2 s16 = tb == 0 ? blk[1] : tb == 3 ? blk[2] : one2;
+                if (tb != 0) {
+                    f32x2 r = one2;
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) {
+                        r = mul2(r, g2[s]);
+                        const f32x2 x = mul2(r, k2[s]);
+                        if (tb >= 2) put2(z16 + s * kZPitch, z16 + kZHalf + s * kZPitch, mul2(s16, x));
+                        if (tb & 1) put2(z8 + s * kZPitch, z8 + kZHalf + s * kZPitch, x);
+                    }
+                }
+                if (tb != 3) {
+                    f32x2 r = one2;
+#pragma unroll
+                    for (int s = 7; s >= 0; --s) {
+                        const f32x2 y = mul2(r, k2[s]);
+                        r = mul2(r, g2[s]);
+                        if (tb < 2) put2(z16 + s * kZPitch, z16 + kZHalf + s * kZPitch, mul2(s16, y));
+                        if (!(tb & 1)) put2(z8 + s * kZPitch, z8 + kZHalf + s * kZPitch, y);
+                    }
                 }
             }
+            f_sync();                  // partial pair sums and Z rows are complete
+
+            float cross[4] = {0.f, 0.f, 0.f, 0.f};
+            if (fw >= 4) {
+                // ---- mma.sync products of the Z rows, hi * hi + lo * hi + hi * lo, 16 x 8 per warp.  Warps 6, 7: A_21 = X Y^T (tokens
+                // 16..31 against 0..7, 8..15), kept in registers until the operand set is free.  Warps 4, 5: rows 0..7 X of tokens
+                // 8..15, rows 8..15 X of tokens 24..31, against Y of tokens 0..7 (the upper half counts), 16..23 (the lower half).
+                // One warp per scheduler: a step waits for its fragments and for the accumulators of the step before ----
+                const uint32_t zb = smem_u32(sStg);
+                const int r = lane & 15, nt = fw & 1;
+                const uint32_t arow = fw >= 6 ? 16u + (uint32_t)r : 32u + (uint32_t)(r < 8 ? 8 + r : 16 + r);
+                const uint32_t brow = (uint32_t)(lane & 7) + (fw >= 6 ? (uint32_t)nt * 8u : 32u + (uint32_t)nt * 16u);
+                const uint32_t abase = zb + arow * kZPitch + (uint32_t)(lane >> 4) * 16u;
+                const uint32_t bbase = zb + brow * kZPitch + (uint32_t)((lane >> 3) & 1) * 16u + (uint32_t)(lane >> 4) * kZHalf;     // hi, then lo
+                float c1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+                for (int ks = 0; ks < K / 16; ++ks) {
+                    uint32_t ahi[4], alo[4], y[4];
+                    k_ldmatrix_x4(abase + ks * 32, ahi);
+                    k_ldmatrix_x4(bbase + ks * 32, y);
+                    k_ldmatrix_x4(abase + kZHalf + ks * 32, alo);
+                    k_mma_16816(cross, ahi, y[0], y[1]);
+                    k_mma_16816(c1, ahi, y[2], y[3]);
+                    k_mma_16816(c1, alo, y[0], y[1]);
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) cross[e] += c1[e];
+                if (fw < 6) {
+                    const int r0 = 8 + 16 * nt + (lane >> 2), c0 = (lane & 3) * 2;
+                    sA[r0 * kAS2 + c0] = sBeta[r0] * (nt ? cross[2] : cross[0]);
+                    sA[r0 * kAS2 + c0 + 1] = sBeta[r0] * (nt ? cross[3] : cross[1]);
+                }
+            } else {
+                // ---- beta_s A_sj of the pairs inside the blocks of eight (only entries below the diagonal are read) ----
+                int s = 1;
+                while (s < 8 && (s + 1) * s / 2 <= lane) ++s;        // the pair's later token
+                if (lane < 28) {
+                    const int jj = lane - s * (s - 1) / 2, s32 = 8 * fw + s;
+                    sA[s32 * kAS2 + 8 * (fw & 1) + jj] = sBeta[s32] * (sPart[2 * fw * 32 + lane] + sPart[(2 * fw + 1) * 32 + lane]);
+                }
+            }
+            proxy_fence();             // (the next tile's rows come in by bulk copies over Z)
+            next_tile(k + 1);          // (its barrier:) A is complete and Z has been read: the next tile's rows may come in
 
             // Up to here nothing of the operand set and window b was touched: they are free once Ktil^T E of tile k - 2 has
-            // completed, so the loads and pair sums above overlap the tail of that tile.
+            // completed, so everything above overlaps the tail of that tile.
             if (k >= 2) {
                 if (!f_wait(ft, &bars[kTfull + b], (uint32_t)((k - 2) >> 1) & 1u)) {
                     if (ft == 0) record_fault(p.status, kFaultUpdateWait, 109);
@@ -792,127 +836,47 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                     break;
                 }
             }
-#pragma unroll
-            for (int r = 0; r < 2; ++r)
-                *reinterpret_cast<uint4*>(set + sm.set_vv + (size_t)(ft + r * kKFront) * 16) = vrow[r];
-
-            // ---- running products of this block.  Khat -> window rows 0..31; Ktil -> set (MN-major); G_n * W -> window
-            // rows 32..; and for the 16 x 16 block of A that couples the two token blocks, whose decay product splits at
-            // the block boundary without a quotient (prod_{j<m<=s} = prod_{16<=m<=s} * prod_{j<m<=15}), the rescaled keys
-            // X_s = k_s prod_{16<=m<=s} g_m (s >= 16, by block 1) and Y_j = k_j prod_{j<m<=15} g_m (j < 16, by block 0)
-            // as bf16 hi + lo rows Z[token][channel] over the (now free) key / decay rows of the staging area ----
+            stage_values(bh, b);
+            // ---- running products of this block.  Khat -> window rows 0..31; Ktil -> set (MN-major); G_n * W -> window rows 32.. ----
             {
-                __nv_bfloat16* whi = reinterpret_cast<__nv_bfloat16*>(wb);
-                __nv_bfloat16* wlo = reinterpret_cast<__nv_bfloat16*>(wb + sm.w_lo);
-                __nv_bfloat16* bthi = reinterpret_cast<__nv_bfloat16*>(set + sm.set_bt);
-                __nv_bfloat16* btlo = reinterpret_cast<__nv_bfloat16*>(set + sm.set_bt_lo);
-                __nv_bfloat16* zhi = reinterpret_cast<__nv_bfloat16*>(sStg);
-                __nv_bfloat16* zlo = reinterpret_cast<__nv_bfloat16*>(sStg + kZHalf);
-                const uint32_t wcol = ((uint32_t)(i >> 3) * LBO_W + (uint32_t)(i & 7) * 2u) >> 1;        // K-major: k = channel
-                const uint32_t bcol = ((uint32_t)(i & 7) * 2u + (uint32_t)(i >> 3) * kSboT) >> 1;        // MN-major: mn = channel
-                float G = fg ? gother : 1.f, X = 1.f;
+                unsigned char* wcol = wb + (uint32_t)(cp >> 2) * LBO_W + (uint32_t)(cp & 3) * 4u;              // K-major: k = channel
+                unsigned char* bcol = set + sm.set_bt + (uint32_t)(cp & 3) * 4u + (uint32_t)(cp >> 2) * kSboT;   // MN-major: mn = channel
+                unsigned char* wrow = wcol + (uint32_t)tb * SBO;
+                unsigned char* brow = bcol + (uint32_t)tb * kLboT;
+                f32x2 G = g_before;
 #pragma unroll
-                for (int s = 0; s < 16; ++s) {
-                    G *= gg[s];
-                    __nv_bfloat16 hi, lo;
-                    split_bf16(G * kk[s], hi, lo);
-                    const uint32_t o = wcol + (((uint32_t)(s & 7) * 16u + (uint32_t)((s >> 3) + 2 * fg) * SBO) >> 1);
-                    whi[o] = hi;
-                    wlo[o] = lo;
-                    if (fg) {
-                        X *= gg[s];
-                        split_bf16(X * kk[s], hi, lo);
-                        zhi[(16 + s) * (kZPitch / 2) + i] = hi;
-                        zlo[(16 + s) * (kZPitch / 2) + i] = lo;
-                    }
+                for (int s = 0; s < 8; ++s) {
+                    G = mul2(G, pair_of(gw[s]));
+                    put2(wrow + s * 16, wrow + sm.w_lo + s * 16, mul2(G, pair_of(kw[s])));
                 }
-                const float Gn = fg ? G : G * gother;       // decay of the whole pass
-                float Dn = fg ? 1.f : gother, Yd = 1.f;
+                f32x2 D = g_after;
 #pragma unroll
-                for (int s = 15; s >= 0; --s) {
-                    const float kt = Dn * kk[s];
-                    Dn *= gg[s];
-                    __nv_bfloat16 hi, lo;
-                    split_bf16(kt, hi, lo);
-                    const uint32_t o = bcol + (((uint32_t)(s & 7) * 16u + (uint32_t)((s >> 3) + 2 * fg) * kLboT) >> 1);
-                    bthi[o] = hi;
-                    btlo[o] = lo;
-                    if (!fg) {
-                        split_bf16(Yd * kk[s], hi, lo);
-                        zhi[s * (kZPitch / 2) + i] = hi;
-                        zlo[s * (kZPitch / 2) + i] = lo;
-                        Yd *= gg[s];
-                    }
+                for (int s = 7; s >= 0; --s) {
+                    put2(brow + s * 16, brow + sm.set_bt_lo + s * 16, mul2(D, pair_of(kw[s])));
+                    D = mul2(D, pair_of(gw[s]));
                 }
-                if (!fg) reinterpret_cast<float*>(set + sm.set_gn)[i] = Gn;
-                // G_n * [Omega | q]: block 0 takes the first half of the sketch columns, block 1 the rest and the query
-                const int Rh = (R + 1) >> 1;
+                if (tb == 0) *reinterpret_cast<f32x2*>(set + sm.set_gn + 8 * cp) = g_all;
+                // G_n * [Omega | q]: block tb takes every fourth sketch column, the last one the query
                 if (p.write_sketch) {
-                    const int g_lo = fg ? Rh : 0, g_hi = fg ? R : Rh;
-                    for (int g = g_lo; g < g_hi; ++g) {
-                        __nv_bfloat16 hi, lo;
-                        split_bf16(Gn * og[g], hi, lo);
-                        const uint32_t o = wcol + (((uint32_t)(g & 7) * 16u + (uint32_t)((g >> 3) + 4) * SBO) >> 1);
-                        whi[o] = hi;
-                        wlo[o] = lo;
+                    for (int g = tb; g < R; g += 4) {
+                        unsigned char* at = wcol + (uint32_t)(g & 7) * 16u + (uint32_t)((g >> 3) + 4) * SBO;
+                        put2(at, at + sm.w_lo, mul2(g_all, *reinterpret_cast<const f32x2*>(sOm + g * kOP + 2 * cp)));
                     }
                 }
-                if (fg && p.q != nullptr) {
-                    __nv_bfloat16 hi, lo;
-                    split_bf16(Gn * q_i, hi, lo);
-                    const uint32_t o = wcol + (((uint32_t)(QA & 7) * 16u + (uint32_t)((QA >> 3) + 4) * SBO) >> 1);
-                    whi[o] = hi;
-                    wlo[o] = lo;
+                if (tb == 3 && p.q != nullptr) {
+                    unsigned char* at = wcol + (uint32_t)(QA & 7) * 16u + (uint32_t)((QA >> 3) + 4) * SBO;
+                    put2(at, at + sm.w_lo, mul2(g_all, pair_of(qw)));
+                }
+                if (fw >= 6) {
+                    float* sA21 = reinterpret_cast<float*>(set + sm.set_t1) + 512;
+                    const int r0 = lane >> 2, c0 = (fw & 1) * 8 + (lane & 3) * 2;
+                    sA21[r0 * 16 + c0] = cross[0];
+                    sA21[r0 * 16 + c0 + 1] = cross[1];
+                    sA21[(r0 + 8) * 16 + c0] = cross[2];
+                    sA21[(r0 + 8) * 16 + c0 + 1] = cross[3];
                 }
             }
-            f_sync();                  // partial pair sums, Z rows and Ktil are complete
-
-            if (fw == 7) {
-                // ---- A_21 = X Y^T (16 x 16, tokens 16..31 against tokens 0..15) as mma.sync products of the Z rows,
-                // hi * hi + lo * hi + hi * lo ----
-                float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-                const uint32_t zb = smem_u32(sStg);
-                const uint32_t abase = zb + (uint32_t)(16 + (lane & 15)) * kZPitch + (uint32_t)(lane >> 4) * 16u;
-                const uint32_t bbase = zb + (uint32_t)(lane & 7) * kZPitch + (uint32_t)((lane >> 3) & 1) * 16u;
-#pragma unroll
-                for (int ks = 0; ks < K / 16; ++ks) {
-                    uint32_t ahi[4], alo[4];
-                    k_ldmatrix_x4(abase + ks * 32, ahi);
-                    k_ldmatrix_x4(abase + kZHalf + ks * 32, alo);
-#pragma unroll
-                    for (int nt = 0; nt < 2; ++nt) {
-                        uint32_t bhi[2], blo[2];
-                        k_ldmatrix_x2(bbase + (uint32_t)(nt * 8) * kZPitch + ks * 32, bhi);
-                        k_ldmatrix_x2(bbase + (uint32_t)(nt * 8) * kZPitch + kZHalf + ks * 32, blo);
-                        k_mma_16816(acc[nt], ahi, bhi);
-                        k_mma_16816(acc[nt], alo, bhi);
-                        k_mma_16816(acc[nt], ahi, blo);
-                    }
-                }
-                float* sA21 = reinterpret_cast<float*>(set + sm.set_t1) + 512;
-#pragma unroll
-                for (int nt = 0; nt < 2; ++nt) {
-                    const int r0 = lane >> 2, c0 = nt * 8 + (lane & 3) * 2;
-                    sA21[r0 * 16 + c0] = acc[nt][0];
-                    sA21[r0 * 16 + c0 + 1] = acc[nt][1];
-                    sA21[(r0 + 8) * 16 + c0] = acc[nt][2];
-                    sA21[(r0 + 8) * 16 + c0 + 1] = acc[nt][3];
-                }
-            } else {
-                // ---- beta_s A_sj of the two triangles: the partials of a block's four warps summed in a fixed order ----
-                for (int idx = ft; idx < 2 * 16 * 16; idx += 224) {
-                    const int blk = idx >> 8, s = (idx >> 4) & 15, jj = idx & 15;
-                    float a = 0.f;
-                    if (jj < s) {
-                        const int sa = s <= 8 ? s : 16 - s;
-                        const int e = ((sa - 1) >> 1) * 32 + ((sa - 1) & 1) * 16 + (s <= 8 ? jj : sa + jj);
-                        const float* pp = sPart + blk * 512 + e;
-                        a = ((pp[0] + pp[128]) + pp[256]) + pp[384];
-                    }
-                    sA[blk * (16 * kAS2) + s * kAS2 + jj] = sBeta[16 * blk + s] * a;
-                }
-            }
-            f_sync();                  // A is complete
+            f_sync();                  // Ktil is complete
 
             if ((fw & 3) == 0) {
                 // ---- T_bb = (I + Bd A_bb)^{-1} Bd of block fw / 4 by forward substitution: one column per thread, in registers ----
@@ -945,39 +909,36 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                 // mma.sync products.  A: the Ktil operand just written (its 8 x 8 core matrices are the row-major fragments
                 // ldmatrix wants), hi + lo; B: Omega and q from shared memory into fragments, split into hi + lo in registers ----
                 const int mt = fw >> 2, nt = (fw & 3) - 1;
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+                float acc[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f}, c2[4] = {0.f, 0.f, 0.f, 0.f};
                 const uint32_t btb = smem_u32(set + sm.set_bt);
                 const uint32_t a_row = btb + (uint32_t)(2 * mt + ((lane >> 3) & 1)) * kLboT + (uint32_t)(lane >> 4) * kSboT + (uint32_t)(lane & 7) * 16u;
-                const __nv_bfloat16* sq = reinterpret_cast<const __nv_bfloat16*>(sStg + sm.stg_q);
+                const __nv_bfloat16* sq = reinterpret_cast<const __nv_bfloat16*>(sStg + sm.stg_q + 256u * (uint32_t)b);
                 const int ncol = p.write_sketch ? R : 0;
                 const bool has_q = p.q != nullptr;
                 const int g = nt * 8 + (lane >> 2);
                 const int src = g < ncol ? 0 : (g == QA && has_q) ? 1 : 2;       // Omega column, query, padding
-#pragma unroll 4
+#pragma unroll 2
                 for (int ks = 0; ks < K / 16; ++ks) {
-                    uint32_t ahi[4], alo[4];
+                    uint32_t ahi[4], alo[4], bhi[2], blo[2];
                     k_ldmatrix_x4(a_row + (uint32_t)(2 * ks) * kSboT, ahi);
                     k_ldmatrix_x4(a_row + sm.set_bt_lo + (uint32_t)(2 * ks) * kSboT, alo);
                     const int i0 = ks * 16 + (lane & 3) * 2;
-                    float w[4] = {0.f, 0.f, 0.f, 0.f};
+                    float2 w0 = make_float2(0.f, 0.f), w1 = w0;
                     if (src == 0) {
-                        w[0] = sOm[i0 * 16 + g];
-                        w[1] = sOm[(i0 + 1) * 16 + g];
-                        w[2] = sOm[(i0 + 8) * 16 + g];
-                        w[3] = sOm[(i0 + 9) * 16 + g];
+                        w0 = *reinterpret_cast<const float2*>(sOm + g * kOP + i0);
+                        w1 = *reinterpret_cast<const float2*>(sOm + g * kOP + i0 + 8);
                     } else if (src == 1) {
-                        w[0] = __bfloat162float(sq[i0]);
-                        w[1] = __bfloat162float(sq[i0 + 1]);
-                        w[2] = __bfloat162float(sq[i0 + 8]);
-                        w[3] = __bfloat162float(sq[i0 + 9]);
+                        w0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(sq + i0));
+                        w1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(sq + i0 + 8));
                     }
-                    uint32_t bhi[2], blo[2];
-                    split_bf16x2(w[0], w[1], bhi[0], blo[0]);
-                    split_bf16x2(w[2], w[3], bhi[1], blo[1]);
-                    k_mma_16816(acc, ahi, bhi);
-                    k_mma_16816(acc, alo, bhi);
-                    k_mma_16816(acc, ahi, blo);
+                    split_bf16x2(w0.x, w0.y, bhi[0], blo[0]);
+                    split_bf16x2(w1.x, w1.y, bhi[1], blo[1]);
+                    k_mma_16816(acc, ahi, bhi[0], bhi[1]);
+                    k_mma_16816(c1, alo, bhi[0], bhi[1]);
+                    k_mma_16816(c2, ahi, blo[0], blo[1]);
                 }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[e] += c1[e] + c2[e];
                 __nv_bfloat16* bchi = reinterpret_cast<__nv_bfloat16*>(set + sm.set_bc);
                 __nv_bfloat16* bclo = bchi + 1024;
                 auto put = [&](int s, int gc, float x) {
@@ -996,7 +957,10 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
             proxy_fence();         // operand sets and windows are read by MMAs (async proxy)
             f_sync();
             if (ft == 0) k_arrive(&bars[kPro + b]);
-            next_tile(k + 1);      // the staging area has been read: the next tile's rows may come in
+        }
+        if (dead && ft < 32) {     // copies that may still be in flight get a short, bounded grace period
+            mbar_wait_bounded(&bars[kStg], phS, 1u << 14);
+            for (int sb = 0; sb < 2; ++sb) mbar_wait_bounded(&bars[kVals + sb], 0u, 1u << 12);
         }
         if (ft == 0) {     // scheduler counters back to zero once every CTA is done claiming
             __threadfence();
