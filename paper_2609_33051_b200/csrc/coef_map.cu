@@ -13,7 +13,8 @@
 // Both follow from the paper's basis-aligned statement by carrying the orthogonal change of coordinates R through
 // (J^T R = Omega^T, J^T H R = U^T S^T / mu, J^T H J = U^T U / mu); R itself is never needed.
 //
-// One CTA of 128 threads per (batch, head); the sketch rows sit in shared memory.  Pivot form: one warp orthogonalises
+// One CTA of 128 threads per (batch, head); the sketch rows sit in shared memory.  Pivot form (five to eight pivots and large ranks;
+// the others run coef_map_pivot.cu): one warp orthogonalises
 // the pivot rows in registers and leaves them as tf32 high parts and remainders; RU = U Q^T, ||U_g||^2 and
 // Y[k][j] = <S[k,:], Q_j> run as mma.sync tiles (three tf32 products per tile, ~2^-21 relative), the stream of S with
 // every quarter warp loading one whole 128-byte line of a row (the state is requested into L2 when the CTA starts);
