@@ -33,7 +33,7 @@
 // What bounds it: the chain of the front group (some 10 k cycles a tile; the state of a tile takes 6.6 k at the rate of a copy),
 // most of it instruction supply and latency of eight warps: pair sums and Z rows 2.4 k, coupling 1.2 k, operand rows 1.4 k,
 // Ktil W and T 2.3 k.  Flush of 16384 heads, 32 tokens: 1030 us with a channel per thread, blocks of 16 tokens (120 pair sums) and
-// 190 KB of code; 740 now (0.56 of a copy's rate).  Not kept: E of the next tile before the write-back (the accumulator is freed
+// 190 KB of code; 740 to 850 now, by box (0.49 to 0.56 of a copy's rate).  Not kept: E of the next tile before the write-back (the accumulator is freed
 // late: +60 us), T before the wait for the operand set (+40), the coupling products of a level on one warp with its fragments a
 // step ahead (spills: +100).
 //
