@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kWsThreads, 2) update_tc_ws_mamba2_kernel(cons
         const int fwarp = gt >> 5;
         int cur_h = -1;                       // head index whose Omega sits in W
         int ops_built = 0;                    // MMA-1 operand sets written so far (single buffer)
-        int prev_tile = -1, last_b = 0;       // the tile whose sketch rows are still to be stored (-1: none) and its buffer
+        int prev_tile = -1;       // the tile whose sketch rows are still to be stored (-1: none)
         uint32_t phU = 0, phB = 0;
         bool dead = false;
 
@@ -514,231 +514,233 @@ __global__ void __launch_bounds__(kWsThreads, 2) update_tc_ws_mamba2_kernel(cons
 
         for (int k = 0; !dead; ++k) {
             const int tile = seq_get(k);
-            if (tile < 0) {
-                if (tile < -1) {
-                    if (gt == 0) record_fault(p.status, kFaultUpdateWait, 8);
-                    dead = true;
-                }
+            if (tile < -1) {
+                if (gt == 0) record_fault(p.status, kFaultUpdateWait, 8);
+                dead = true;
                 break;
             }
             const int b = k & 1;
-            const int h = tile / tiles_per_h;
-            const int b0 = (tile - h * tiles_per_h) * NH;
-            __nv_bfloat16* sB2hi = reinterpret_cast<__nv_bfloat16*>(smem + sm.b2);
-            __nv_bfloat16* sB2lo = sB2hi + (size_t)NP * kK;
-            float* sW = reinterpret_cast<float*>(smem + sm.w + (uint32_t)b * sm.w_stride);
-            unsigned char* sA1hi = smem + sm.op;
-            unsigned char* sA1lo = sA1hi + OPB;
-            unsigned char* sB1 = sA1lo + OPB;
+            if (tile >= 0) {
+                const int h = tile / tiles_per_h;
+                const int b0 = (tile - h * tiles_per_h) * NH;
+                __nv_bfloat16* sB2hi = reinterpret_cast<__nv_bfloat16*>(smem + sm.b2);
+                __nv_bfloat16* sB2lo = sB2hi + (size_t)NP * kK;
+                float* sW = reinterpret_cast<float*>(smem + sm.w + (uint32_t)b * sm.w_stride);
+                unsigned char* sA1hi = smem + sm.op;
+                unsigned char* sA1lo = sA1hi + OPB;
+                unsigned char* sB1 = sA1lo + OPB;
 
-            // gates of the current token (one warp per head needs them for the weight scan): requested early
-            float tok_beta = 0.f, tok_a = 1.f;
-            if (fwarp < NH && p.has_token) {
-                const size_t bw = (size_t)(b0 + fwarp) * H + h;
-                tok_beta = p.beta[bw];
-                tok_a = reinterpret_cast<const float*>(p.decay)[bw];
-            }
-            // ---- W = [Omega | q | q'] hi/lo, K-major; the Omega part once per head index.  MMA 2 of the previous tile
-            // still reads W, so that tile is finished (and its sketch rows stored) first. ----
-            if (h != cur_h) {
-                if (prev_tile >= 0) {
-                    if (!store_ut(prev_tile, b ^ 1)) {
-                        if (gt == 0) record_fault(p.status, kFaultUpdateWait, 5);
-                        dead = true;
-                        break;
-                    }
-                    prev_tile = -1;
-                    group_sync(2);
+                // gates of the current token (one warp per head needs them for the weight scan): requested early
+                float tok_beta = 0.f, tok_a = 1.f;
+                if (fwarp < NH && p.has_token) {
+                    const size_t bw = (size_t)(b0 + fwarp) * H + h;
+                    tok_beta = p.beta[bw];
+                    tok_a = reinterpret_cast<const float*>(p.decay)[bw];
                 }
-                const float* og = p.omega + (size_t)h * K * R;
-                if (!p.write_sketch) {
-                    // no sketch: the Omega columns stay zero (written once before the tile loop)
-                } else if ((R & 3) == 0) {
-                    // four ranks of one state row per step; all loads of a thread are in flight together
-                    const int per_row = R >> 2, items = K * per_row;
-                    for (int base = 0; base < items; base += 4 * kGroup) {
-                        float4 x[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int idx = base + u * kGroup + gt;
-                            x[u] = idx < items ? *reinterpret_cast<const float4*>(og + (size_t)idx * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const int idx = base + u * kGroup + gt;
-                            if (idx < items) {
-                                const int i = idx / per_row, g4 = (idx - i * per_row) * 4;
-                                const float xv[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    const int g = g4 + e;
-                                    __nv_bfloat16 hi, lo;
-                                    split_bf16(xv[e], hi, lo);
-                                    const uint32_t o2 = ((g & 7) * 16 + (g >> 3) * SBO + (i >> 3) * LBO2B + (i & 7) * 2) >> 1;
-                                    sB2hi[o2] = hi;
-                                    sB2lo[o2] = lo;
-                                }
-                            }
-                        }
-                    }
-                } else {
-                    for (int idx = gt; idx < K * R; idx += kGroup) {
-                        const int i = idx / R, g = idx % R;
-                        __nv_bfloat16 hi, lo;
-                        split_bf16(og[idx], hi, lo);
-                        const uint32_t o2 = ((g & 7) * 16 + (g >> 3) * SBO + (i >> 3) * LBO2B + (i & 7) * 2) >> 1;
-                        sB2hi[o2] = hi;
-                        sB2lo[o2] = lo;
-                    }
-                }
-                cur_h = h;
-            }
-            // the first block of this tile (with its gates and query rows) must have landed
-            if (staging) {
-                if (!group_wait(2, gt, &bars[kBarStg + cq_idx % stg_bufs], (uint32_t)(cq_idx / stg_bufs) & 1u)) {
-                    if (gt == 0) record_fault(p.status, kFaultUpdateWait, 6);
-                    dead = true;
-                    break;
-                }
-            }
-            if (p.q != nullptr) {       // query columns of this tile's group (bf16-exact: lo = 0)
-                for (int idx = gt; idx < K * NH; idx += kGroup) {
-                    const int i = idx % K, hd = idx / K, g = QA + 8 * b + hd;
-                    const uint32_t o2 = ((g & 7) * 16 + (g >> 3) * SBO + (i >> 3) * LBO2B + (i & 7) * 2) >> 1;
-                    sB2hi[o2] = reinterpret_cast<const __nv_bfloat16*>(sStg + (size_t)hd * sm.stg_tile_head + sm.stg_q)[i];
-                }
-            }
-            // ---- token weights w_s = beta_s prod_{j>s} a_j and the total decay: one warp per head, suffix scan ----
-            if (fwarp < NH) {
-                const int hd = fwarp, lane = gt & 31;
-                const float* sg = reinterpret_cast<const float*>(sStg + (size_t)hd * sm.stg_tile_head);
-                float suf = 1.f;          // product of the decays of all later tokens
-                for (int base = ((n_tot + 31) & ~31) - 32; base >= 0; base -= 32) {
-                    const int s = base + lane;
-                    float beta = 0.f, a = 1.f;
-                    if (s < n_ring) { beta = sg[s]; a = sg[p.L + s]; }
-                    else if (s < n_tot) { beta = tok_beta; a = tok_a; }
-                    // inclusive suffix product of a over lanes >= lane
-                    float incl = a;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const float other = __shfl_down_sync(0xffffffffu, incl, o);
-                        if (lane + o < 32) incl *= other;
-                    }
-                    float excl = __shfl_down_sync(0xffffffffu, incl, 1);
-                    if (lane == 31) excl = 1.f;
-                    if (s < n_tot) sW[hd * 208 + s] = beta * excl * suf;
-                    suf *= __shfl_sync(0xffffffffu, incl, 0);
-                }
-                if (lane == 0) sW[hd * 208 + 64] = suf;
-            }
-            proxy_fence();         // W is read by MMA 2 (async proxy)
-            group_sync(2);
-
-            // ---- MMA 1 over blocks of kTokBlock tokens per head ----
-            for (int blk = 0; blk < n_blocks; ++blk) {
-                if (ops_built > 0) {      // the previous MMA-1 block (of this or the previous tile) must have read the operand buffers
-                    if (!group_wait(2, gt, &bars[kBarBlk], phB)) {
-                        if (gt == 0) record_fault(p.status, kFaultUpdateWait, 1);
-                        dead = true;
-                        break;
-                    }
-                    phB ^= 1;
-                    tc_fence_after();
-                }
-                // Operand rows are moved 16 bytes per thread.  The 8 lanes of a quarter warp take the 8 token rows of a core
-                // matrix, each at a different 8-element vector (a diagonal), so that neither the reads of the staged rows
-                // (row pitch 256 or 128 bytes) nor the writes of the core matrices meet in a bank.
-                {
-                    // rows come from the block's staging buffer; only the diagonal head blocks of A are written
-                    if (blk > 0 && staging) {      // (the first block was waited for above)
-                        if (!group_wait(2, gt, &bars[kBarStg + cq_idx % stg_bufs], (uint32_t)(cq_idx / stg_bufs) & 1u)) {
-                            if (gt == 0) record_fault(p.status, kFaultUpdateWait, 6);
+                // ---- W = [Omega | q | q'] hi/lo, K-major; the Omega part once per head index.  MMA 2 of the previous tile
+                // still reads W, so that tile is finished (and its sketch rows stored) first. ----
+                if (h != cur_h) {
+                    if (prev_tile >= 0) {
+                        if (!store_ut(prev_tile, b ^ 1)) {
+                            if (gt == 0) record_fault(p.status, kFaultUpdateWait, 5);
                             dead = true;
                             break;
                         }
+                        prev_tile = -1;
+                        group_sync(2);
                     }
-                    const unsigned char* sBlk = smem + sm.stg_blk + (size_t)(cq_idx % stg_bufs) * sm.stg_blk_stride;
-                    const int s_base = blk * kTokBlock;
-                    constexpr int NB = KD1 * (K / 8) / kGroup;          // B-operand vectors per thread
-                    uint4 kv[NB];
+                    const float* og = p.omega + (size_t)h * K * R;
+                    if (!p.write_sketch) {
+                        // no sketch: the Omega columns stay zero (written once before the tile loop)
+                    } else if ((R & 3) == 0) {
+                        // four ranks of one state row per step; all loads of a thread are in flight together
+                        const int per_row = R >> 2, items = K * per_row;
+                        for (int base = 0; base < items; base += 4 * kGroup) {
+                            float4 x[4];
 #pragma unroll
-                    for (int r = 0; r < NB; ++r) {
-                        const int idx = gt + r * kGroup;
-                        const int a = ((idx >> 3) + (idx & 7)) % (K / 8), sp = (idx & 7) + 8 * (idx / (8 * (K / 8)));
-                        const int hd = sp / kTokBlock, s = sp % kTokBlock;
-                        kv[r] = s_base + s < n_tot ? *reinterpret_cast<const uint4*>(sBlk + (size_t)hd * sm.stg_blk_head + (size_t)s * 256 + a * 16)
-                                                   : make_uint4(0, 0, 0, 0);
-                    }
-                    constexpr int NA = NH * kTokBlock * (V / 8) / kGroup;      // diagonal A-operand vectors per thread
-                    uint4 vv[NA];
-                    float wv[NA];
+                            for (int u = 0; u < 4; ++u) {
+                                const int idx = base + u * kGroup + gt;
+                                x[u] = idx < items ? *reinterpret_cast<const float4*>(og + (size_t)idx * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                            }
 #pragma unroll
-                    for (int r = 0; r < NA; ++r) {
-                        const int it = gt + r * kGroup;
-                        const int t8 = it & 7, a = ((it >> 3) + t8) % (V / 8), rest = it / V;
-                        const int hd = rest >> 1, s = (rest & 1) * 8 + t8;
-                        const bool live = s_base + s < n_tot;
-                        vv[r] = live ? *reinterpret_cast<const uint4*>(sBlk + (size_t)hd * sm.stg_blk_head + 4096 + (size_t)s * V * 2 + a * 16)
-                                     : make_uint4(0, 0, 0, 0);
-                        wv[r] = live ? sW[hd * 208 + s_base + s] : 0.f;
-                    }
+                            for (int u = 0; u < 4; ++u) {
+                                const int idx = base + u * kGroup + gt;
+                                if (idx < items) {
+                                    const int i = idx / per_row, g4 = (idx - i * per_row) * 4;
+                                    const float xv[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
 #pragma unroll
-                    for (int r = 0; r < NB; ++r) {
-                        const int idx = gt + r * kGroup;
-                        const int a = ((idx >> 3) + (idx & 7)) % (K / 8), sp = (idx & 7) + 8 * (idx / (8 * (K / 8)));
-                        *reinterpret_cast<uint4*>(sB1 + (sp & 7) * 16 + a * SBO + (sp >> 3) * LBO1) = kv[r];
-                    }
-#pragma unroll
-                    for (int r = 0; r < NA; ++r) {
-                        const int it = gt + r * kGroup;
-                        const int t8 = it & 7, a = ((it >> 3) + t8) % (V / 8), rest = it / V;
-                        const int hd = rest >> 1, sp = hd * kTokBlock + (rest & 1) * 8 + t8;
-                        const int a128 = hd * (V / 8) + a;
-                        const uint32_t vin[4] = {vv[r].x, vv[r].y, vv[r].z, vv[r].w};
-                        uint32_t ohi[4], olo[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float f0 = wv[r] * __uint_as_float(vin[e] << 16), f1 = wv[r] * __uint_as_float(vin[e] & 0xffff0000u);
-                            split_bf16x2(f0, f1, ohi[e], olo[e]);
+                                    for (int e = 0; e < 4; ++e) {
+                                        const int g = g4 + e;
+                                        __nv_bfloat16 hi, lo;
+                                        split_bf16(xv[e], hi, lo);
+                                        const uint32_t o2 = ((g & 7) * 16 + (g >> 3) * SBO + (i >> 3) * LBO2B + (i & 7) * 2) >> 1;
+                                        sB2hi[o2] = hi;
+                                        sB2lo[o2] = lo;
+                                    }
+                                }
+                            }
                         }
-                        const uint32_t off = (sp & 7) * 16 + a128 * SBO + (sp >> 3) * LBO1;
-                        *reinterpret_cast<uint4*>(sA1hi + off) = make_uint4(ohi[0], ohi[1], ohi[2], ohi[3]);
-                        *reinterpret_cast<uint4*>(sA1lo + off) = make_uint4(olo[0], olo[1], olo[2], olo[3]);
+                    } else {
+                        for (int idx = gt; idx < K * R; idx += kGroup) {
+                            const int i = idx / R, g = idx % R;
+                            __nv_bfloat16 hi, lo;
+                            split_bf16(og[idx], hi, lo);
+                            const uint32_t o2 = ((g & 7) * 16 + (g >> 3) * SBO + (i >> 3) * LBO2B + (i & 7) * 2) >> 1;
+                            sB2hi[o2] = hi;
+                            sB2lo[o2] = lo;
+                        }
                     }
-                    ++cq_idx;
+                    cur_h = h;
                 }
-                proxy_fence();
-                tc_fence_before();
-                group_sync(2);
-                ++ops_built;
-                if (gt == mma_thread) {
-                    tc_fence_after();
-                    const uint32_t tmem_t = tmem_base + (uint32_t)b * 128u;
+                // the first block of this tile (with its gates and query rows) must have landed
+                if (staging) {
+                    if (!group_wait(2, gt, &bars[kBarStg + cq_idx % stg_bufs], (uint32_t)(cq_idx / stg_bufs) & 1u)) {
+                        if (gt == 0) record_fault(p.status, kFaultUpdateWait, 6);
+                        dead = true;
+                        break;
+                    }
+                }
+                if (p.q != nullptr) {       // query columns of this tile's group (bf16-exact: lo = 0)
+                    for (int idx = gt; idx < K * NH; idx += kGroup) {
+                        const int i = idx % K, hd = idx / K, g = QA + 8 * b + hd;
+                        const uint32_t o2 = ((g & 7) * 16 + (g >> 3) * SBO + (i >> 3) * LBO2B + (i & 7) * 2) >> 1;
+                        sB2hi[o2] = reinterpret_cast<const __nv_bfloat16*>(sStg + (size_t)hd * sm.stg_tile_head + sm.stg_q)[i];
+                    }
+                }
+                // ---- token weights w_s = beta_s prod_{j>s} a_j and the total decay: one warp per head, suffix scan ----
+                if (fwarp < NH) {
+                    const int hd = fwarp, lane = gt & 31;
+                    const float* sg = reinterpret_cast<const float*>(sStg + (size_t)hd * sm.stg_tile_head);
+                    float suf = 1.f;          // product of the decays of all later tokens
+                    for (int base = ((n_tot + 31) & ~31) - 32; base >= 0; base -= 32) {
+                        const int s = base + lane;
+                        float beta = 0.f, a = 1.f;
+                        if (s < n_ring) { beta = sg[s]; a = sg[p.L + s]; }
+                        else if (s < n_tot) { beta = tok_beta; a = tok_a; }
+                        // inclusive suffix product of a over lanes >= lane
+                        float incl = a;
 #pragma unroll
-                    for (int ks = 0; ks < KD1 / 16; ++ks) {
-                        const uint64_t bd = make_desc(smem_u32(sB1) + ks * 2 * LBO1, LBO1, SBO);
-                        tc_mma_bf16(tmem_t, make_desc(smem_u32(sA1hi) + ks * 2 * LBO1, LBO1, SBO), bd, idesc1, (blk | ks) ? 1u : 0u);
-                        tc_mma_bf16(tmem_t, make_desc(smem_u32(sA1lo) + ks * 2 * LBO1, LBO1, SBO), bd, idesc1, 1u);
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const float other = __shfl_down_sync(0xffffffffu, incl, o);
+                            if (lane + o < 32) incl *= other;
+                        }
+                        float excl = __shfl_down_sync(0xffffffffu, incl, 1);
+                        if (lane == 31) excl = 1.f;
+                        if (s < n_tot) sW[hd * 208 + s] = beta * excl * suf;
+                        suf *= __shfl_sync(0xffffffffu, incl, 0);
                     }
-                    tc_commit(&bars[kBarBlk]);
-                    if (blk + 1 == n_blocks) {
-                        tc_commit(&bars[kBarT + b]);
-                        mbar_arrive(&bars[kBarPro + b]);      // after the group barrier: W, weights and decay are written
-                    }
+                    if (lane == 0) sW[hd * 208 + 64] = suf;
                 }
-                stage_next();        // the block buffer just read is free again
-            }
-            if (dead) break;
-            if (n_blocks == 0) {
-                // no token to replay: nothing reads the staging buffer after the query columns; T counts as zero
-                ++cq_idx;
+                proxy_fence();         // W is read by MMA 2 (async proxy)
                 group_sync(2);
-                if (gt == 0) {
-                    mbar_arrive(&bars[kBarT + b]);
-                    mbar_arrive(&bars[kBarPro + b]);
+
+                // ---- MMA 1 over blocks of kTokBlock tokens per head ----
+                // (without a token to replay: one step that only passes the staging buffer on.  stage_next and store_ut are inlined, so they
+                // have as few call sites as the order allows: the code of this kernel has to stay small)
+                for (int blk = 0; blk < (n_blocks > 0 ? n_blocks : 1); ++blk) {
+                    if (n_blocks > 0) {
+                        if (ops_built > 0) {      // the previous MMA-1 block (of this or the previous tile) must have read the operand buffers
+                            if (!group_wait(2, gt, &bars[kBarBlk], phB)) {
+                                if (gt == 0) record_fault(p.status, kFaultUpdateWait, 1);
+                                dead = true;
+                                break;
+                            }
+                            phB ^= 1;
+                            tc_fence_after();
+                        }
+                        // Operand rows are moved 16 bytes per thread.  The 8 lanes of a quarter warp take the 8 token rows of a core
+                        // matrix, each at a different 8-element vector (a diagonal), so that neither the reads of the staged rows
+                        // (row pitch 256 or 128 bytes) nor the writes of the core matrices meet in a bank.
+                        {
+                            // rows come from the block's staging buffer; only the diagonal head blocks of A are written
+                            if (blk > 0 && staging) {      // (the first block was waited for above)
+                                if (!group_wait(2, gt, &bars[kBarStg + cq_idx % stg_bufs], (uint32_t)(cq_idx / stg_bufs) & 1u)) {
+                                    if (gt == 0) record_fault(p.status, kFaultUpdateWait, 6);
+                                    dead = true;
+                                    break;
+                                }
+                            }
+                            const unsigned char* sBlk = smem + sm.stg_blk + (size_t)(cq_idx % stg_bufs) * sm.stg_blk_stride;
+                            const int s_base = blk * kTokBlock;
+                            constexpr int NB = KD1 * (K / 8) / kGroup;          // B-operand vectors per thread
+                            uint4 kv[NB];
+#pragma unroll
+                            for (int r = 0; r < NB; ++r) {
+                                const int idx = gt + r * kGroup;
+                                const int a = ((idx >> 3) + (idx & 7)) % (K / 8), sp = (idx & 7) + 8 * (idx / (8 * (K / 8)));
+                                const int hd = sp / kTokBlock, s = sp % kTokBlock;
+                                kv[r] = s_base + s < n_tot ? *reinterpret_cast<const uint4*>(sBlk + (size_t)hd * sm.stg_blk_head + (size_t)s * 256 + a * 16)
+                                                           : make_uint4(0, 0, 0, 0);
+                            }
+                            constexpr int NA = NH * kTokBlock * (V / 8) / kGroup;      // diagonal A-operand vectors per thread
+                            uint4 vv[NA];
+                            float wv[NA];
+#pragma unroll
+                            for (int r = 0; r < NA; ++r) {
+                                const int it = gt + r * kGroup;
+                                const int t8 = it & 7, a = ((it >> 3) + t8) % (V / 8), rest = it / V;
+                                const int hd = rest >> 1, s = (rest & 1) * 8 + t8;
+                                const bool live = s_base + s < n_tot;
+                                vv[r] = live ? *reinterpret_cast<const uint4*>(sBlk + (size_t)hd * sm.stg_blk_head + 4096 + (size_t)s * V * 2 + a * 16)
+                                             : make_uint4(0, 0, 0, 0);
+                                wv[r] = live ? sW[hd * 208 + s_base + s] : 0.f;
+                            }
+#pragma unroll
+                            for (int r = 0; r < NB; ++r) {
+                                const int idx = gt + r * kGroup;
+                                const int a = ((idx >> 3) + (idx & 7)) % (K / 8), sp = (idx & 7) + 8 * (idx / (8 * (K / 8)));
+                                *reinterpret_cast<uint4*>(sB1 + (sp & 7) * 16 + a * SBO + (sp >> 3) * LBO1) = kv[r];
+                            }
+#pragma unroll
+                            for (int r = 0; r < NA; ++r) {
+                                const int it = gt + r * kGroup;
+                                const int t8 = it & 7, a = ((it >> 3) + t8) % (V / 8), rest = it / V;
+                                const int hd = rest >> 1, sp = hd * kTokBlock + (rest & 1) * 8 + t8;
+                                const int a128 = hd * (V / 8) + a;
+                                const uint32_t vin[4] = {vv[r].x, vv[r].y, vv[r].z, vv[r].w};
+                                uint32_t ohi[4], olo[4];
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    const float f0 = wv[r] * __uint_as_float(vin[e] << 16), f1 = wv[r] * __uint_as_float(vin[e] & 0xffff0000u);
+                                    split_bf16x2(f0, f1, ohi[e], olo[e]);
+                                }
+                                const uint32_t off = (sp & 7) * 16 + a128 * SBO + (sp >> 3) * LBO1;
+                                *reinterpret_cast<uint4*>(sA1hi + off) = make_uint4(ohi[0], ohi[1], ohi[2], ohi[3]);
+                                *reinterpret_cast<uint4*>(sA1lo + off) = make_uint4(olo[0], olo[1], olo[2], olo[3]);
+                            }
+                            ++cq_idx;
+                        }
+                        proxy_fence();
+                        tc_fence_before();
+                        group_sync(2);
+                        ++ops_built;
+                        if (gt == mma_thread) {
+                            tc_fence_after();
+                            const uint32_t tmem_t = tmem_base + (uint32_t)b * 128u;
+#pragma unroll
+                            for (int ks = 0; ks < KD1 / 16; ++ks) {
+                                const uint64_t bd = make_desc(smem_u32(sB1) + ks * 2 * LBO1, LBO1, SBO);
+                                tc_mma_bf16(tmem_t, make_desc(smem_u32(sA1hi) + ks * 2 * LBO1, LBO1, SBO), bd, idesc1, (blk | ks) ? 1u : 0u);
+                                tc_mma_bf16(tmem_t, make_desc(smem_u32(sA1lo) + ks * 2 * LBO1, LBO1, SBO), bd, idesc1, 1u);
+                            }
+                            tc_commit(&bars[kBarBlk]);
+                            if (blk + 1 == n_blocks) {
+                                tc_commit(&bars[kBarT + b]);
+                                mbar_arrive(&bars[kBarPro + b]);      // after the group barrier: W, weights and decay are written
+                            }
+                        }
+                    } else {
+                        // nothing reads the staging buffer after the query columns; T counts as zero
+                        ++cq_idx;
+                        group_sync(2);
+                        if (gt == 0) {
+                            mbar_arrive(&bars[kBarT + b]);
+                            mbar_arrive(&bars[kBarPro + b]);
+                        }
+                    }
+                    stage_next();        // the block buffer just read is free again
                 }
-                stage_next();
+                if (dead) break;
             }
 
             // ---- sketch rows and exact output of the previous tile, once the stream group has finished it ----
@@ -748,12 +750,8 @@ __global__ void __launch_bounds__(kWsThreads, 2) update_tc_ws_mamba2_kernel(cons
                     dead = true;
                 }
             }
+            if (tile < 0) break;          // (that was the last tile)
             prev_tile = tile;
-            last_b = b;
-        }
-        if (!dead && prev_tile >= 0) {
-            // the last tile used buffer (number of tiles - 1) & 1; phU tells which buffer has an odd number of stores
-            if (!store_ut(prev_tile, last_b) && gt == 0) record_fault(p.status, kFaultUpdateWait, 5);
         }
         if (gt == 0) {     // scheduler counters back to zero once every CTA is done claiming
             __threadfence();
