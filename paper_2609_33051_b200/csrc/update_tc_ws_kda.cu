@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
         // until the pass-B group has read it
         auto pass_a = [&](int b, int kt) {
             const float* sGn = reinterpret_cast<const float*>(set_ptr(b) + sm.set_gn);
-#pragma unroll 2
+#pragma unroll 1
             for (int c = 0; c < NCH; ++c) {
                 if (c == 0 && kt >= 2) {
                     bad |= !mbar_wait_bounded(&bars[kTfree + b], (phTf >> b) & 1u);
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
             bad |= !mbar_wait_bounded(&bars[kTfull + b], (phT >> b) & 1u);      // Ktil^T E and the sketch correction are complete
             phT ^= 1u << b;
             tc_fence_after();
-#pragma unroll 2
+#pragma unroll 1
             for (int c = 0; c < NCH; ++c) {
                 if (!bad) {
                     float t[CH];
