@@ -19,6 +19,7 @@
 // per buffered token.
 #include "internal.cuh"
 #include "lanegroup.cuh"
+#include "state_rows.h"
 
 namespace sketchssm {
 
@@ -373,9 +374,9 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F, W) * 32, W > 1 ? 1 :
         // buffered tokens, state in L2: 7.2 us without requests, 9.6 with bulk ones, 8.2; state not in L2: 0.67 to 0.93 of
         // the time without).  Where every head reads its state the bytes in flight suffice without that, and the requests cost time
         // (window of fp32 KDA full reads, 3072 heads: 440 -> 479 us).
-        constexpr int kAhead = 32;
         if (ANY && full) {
-            for (int line = lane; line < kAhead * V / 32; line += 32) prefetch_l2_line(p.state + (bh * K + sub * (K / W)) * (size_t)V + 32 * line);
+            const float* mine = p.state + (bh * K + first_row(K, W, sub)) * (size_t)V;
+            for (int line = lane; line < rows_asked_first(K, W) * V / 32; line += 32) prefetch_l2_line(mine + 32 * line);
         }
 
         if (any_of_team(!DEC_WAIT(barA, parA))) {
@@ -742,8 +743,9 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, F, W) * 32, W > 1 ? 1 :
                 // room for 16: 60 bytes spilled instead of 12, with erase vectors 276 instead of 100, which all its heads paid
                 // for (8192 heads, GDN, 24 buffered tokens, r = 24: 56 us a launch, with both changes 45).
                 constexpr int RB = ANY && K == 64 ? 8 : 32 / EV;
-                for (int i0 = sub * (K / W); i0 < (sub + 1) * (K / W); i0 += RB) {        // (a team's warps: K / W rows each)
-                    if (ANY && i0 + kAhead < (sub + 1) * (K / W) && lane < RB * V / 32) prefetch_l2_line(p.state + (bh * K + i0 + kAhead) * V + 32 * lane);
+                static_assert((K / W) % RB == 0 && kAhead % RB == 0, "whole blocks of rows for every warp");
+                for (int i0 = first_row(K, W, sub); i0 < end_row(K, W, sub); i0 += RB) {        // (a team's warps: K / W rows each)
+                    if (ANY && asks_ahead(K, W, sub, i0) && lane < RB * V / 32) prefetch_l2_line(p.state + (bh * K + i0 + kAhead) * V + 32 * lane);
                     float rows[RB][EV];
                     if (TEAM && FULL && p.stream_state) {
 #pragma unroll

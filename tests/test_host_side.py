@@ -130,3 +130,38 @@ def test_the_benchmark_prints_one_short_line_and_its_records_beside_it(capsys, t
     assert "13.0 (back to back) | 0.80" in row and "1.04" not in row
     rec["decode_frac_of_measured"] = 0.95
     assert "| 10.0 | 0.95" in report.table([rec])
+
+
+_ROWS = r"""
+#include <cstdio>
+#include <initializer_list>
+#include "state_rows.h"
+using namespace sketchssm;
+int main() {
+    for (int K : {64, 128}) for (int W : {1, 2, 4}) for (int RB : {8, 16}) for (int sub = 0; sub < W; ++sub) {
+        if ((K / W) % RB) continue;
+        const int a = first_row(K, W, sub);
+        std::printf("%d %d %d 0 %d %d\n", K, W, sub, a, a + rows_asked_first(K, W));
+        for (int i0 = a; i0 < end_row(K, W, sub); i0 += RB) {
+            std::printf("%d %d %d 1 %d %d\n", K, W, sub, i0, i0 + RB);
+            if (asks_ahead(K, W, sub, i0)) std::printf("%d %d %d 0 %d %d\n", K, W, sub, i0 + kAhead, i0 + kAhead + RB);
+        }
+    }
+}
+"""
+
+
+def test_a_dense_heads_warps_read_each_row_once_and_ask_only_for_their_own(tmp_path):
+    """A request for a row that another warp owns is made twice, and one behind the last head's state may not be mapped."""
+    (tmp_path / "rows.cpp").write_text(_ROWS)
+    exe = str(tmp_path / "rows")
+    subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "paper_2609_33051_b200", "csrc"), str(tmp_path / "rows.cpp"),
+                    "-o", exe], check=True)
+    read, asked = {}, {}
+    for ln in subprocess.run([exe], check=True, capture_output=True, text=True).stdout.splitlines():
+        K, W, sub, is_read, a, b = map(int, ln.split())
+        (read if is_read else asked).setdefault((K, W, sub), set()).update(range(a, b))
+    for (K, W, sub), rows in read.items():
+        assert rows == set(range(sub * K // W, (sub + 1) * K // W)), (K, W, sub)
+        assert asked[K, W, sub] <= rows, (K, W, sub)
+    assert len(read) == 2 * (1 + 2 + 4)
