@@ -24,9 +24,9 @@
 // Front group, 256 threads, thread = (block of eight tokens, channel pair): reads its columns of the staged key and decay rows
 // into registers, forms the running products in packed pairs and writes its rows of Khat / Ktil / G_n * W in the operand layouts,
 // four bytes at a time.  The pair sums of A inside a block of eight (28) are per-channel products reduced over the channels by one
-// transposing butterfly (per-warp partials summed in a fixed order: results are bitwise reproducible); the 8 x 8 and 16 x 16
-// blocks that couple them are mma.sync products of rescaled keys (the decay product splits at a block boundary without a
-// quotient).  T_11 and T_22 of the two blocks of 16 by forward substitution (one column per thread, one warp each) while six warps
+// transposing butterfly (per-warp partials summed in a fixed order: results are bitwise reproducible); the 8 x 8 blocks that
+// couple them are dot products of rescaled keys (the decay product splits at a block boundary without a quotient), all of it in
+// fp32; the 16 x 16 block of tokens 16..31 against 0..15 is an mma.sync product of rescaled keys as bf16 hi + lo.  T_11 and T_22 of the two blocks of 16 by forward substitution (one column per thread, one warp each) while six warps
 // form Ktil [Omega | q] with mma.sync.  The E step (E_1 = T_11 x_1, E_2 = T_22 (x_2 - A_21 E_1), 264 packed multiply-adds per lane)
 // runs on the pass-B group, between the write-back of one tile and the next, so that the pass-A group only streams.
 //
@@ -55,7 +55,9 @@ constexpr int kNT = 32;              // tokens per pass
 constexpr int kKStages = 8;          // upper bound on the shared-memory stages of state rows
 constexpr int kAS2 = 20;             // row stride (floats) of the two 16 x 16 triangles of A
 constexpr uint32_t kZPitch = 272u;   // bytes between the rows of the rescaled keys Z[token][channel]: 256 + 16, so that the 8 rows of an ldmatrix fall in different banks
-constexpr uint32_t kZHalf = 64u * kZPitch;   // hi rows, then lo rows: tokens 0..31 for the boundary at token 16, again for those at 8 and 24
+constexpr uint32_t kZHalf = 32u * kZPitch;   // hi rows, then lo rows, for the boundary at token 16 ...
+constexpr uint32_t kZ8 = 2u * kZHalf;        // ... then fp32 rows for those at 8 and 24,
+constexpr uint32_t kZ8Pitch = 528u;          // 512 + 16 bytes apart: rows that differ by less than eight fall in different banks
 constexpr int kOP = 132;             // floats between the columns of Omega in shared memory [16][128]
 // Pass-A window [Khat 32 | G_n * W 32]: 64 rows of 16 bytes per group of 8 channels, the groups 16 bytes further apart than
 // they need to be, so that the per-channel threads of a warp (4 groups) store to different banks
@@ -89,7 +91,7 @@ __host__ __device__ inline KSmem make_ksmem(int stages) {
     // staging of the next tile's raw rows: keys [32][256 B], decays [32][256 B]; beta [L] floats, query row (double-buffered: it is
     // read until the tile is finished).  (Value rows go straight into the set.)  Once a tile's rows are in registers the key / decay
     // area is re-used for the rescaled keys Z.
-    s.stg_g = 8192u; s.stg_beta = 2u * kZHalf; s.stg_q = s.stg_beta + 256u;
+    s.stg_g = 8192u; s.stg_beta = kZ8 + 32u * kZ8Pitch; s.stg_q = s.stg_beta + 256u;
     s.stg = off; off += s.stg_q + 512u;
     s.mats = off; off += 2u * 16u * kAS2 * 4u + 128u + 8u * 32u * 4u + 4u * 128u * 4u;    // A (beta_s A_sj), beta, partial pair sums, products of the decays of eight tokens
     s.om = off; off += 16u * kOP * 4u;                            // Omega of the current head index, fp32 (zero beyond the rank)
@@ -734,7 +736,10 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
             // ---- A_sj = sum_i k_s[i] k_j[i] prod_{j<m<=s} g_m[i].  Inside a block of eight tokens: 28 pair sums as per-channel
             // products, reduced over the warp's 64 channels by a transposing butterfly.  Between blocks the decay product splits at a
             // block boundary without a quotient: X_s = k_s prod_{boundary<=m<=s} g_m against Y_j = k_j prod_{j<m<boundary} g_m, for the
-            // boundary at 16 (rows 0..31 of Z) and those at 8 and 24 (rows 32..63), as bf16 hi + lo rows Z[token][channel] ----
+            // boundary at 16 as bf16 hi + lo rows Z[token][channel], for those at 8 and 24 as fp32 rows: inside 16 tokens A is a sum of
+            // fp32 products.  (As hi + lo rows and mma.sync products A lost bits there that keys of few large channels show: 2-norm error
+            // of S_new after 12 tokens of one channel 2.4e-5 instead of 1.9e-5, of two 1.29e-5 instead of 1.15e-5.  No faster: window of
+            // 16384 heads, 32 tokens, 2854 us with those, 2863 with these, runs 0.3 % apart.) ----
             {
                 f32x2 k2[8], g2[8];
 #pragma unroll
@@ -759,7 +764,7 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                 sPart[fw * 32 + lane] = vals[0];
 
                 unsigned char* z16 = sStg + (uint32_t)t0 * kZPitch + 4u * (uint32_t)cp;
-                unsigned char* z8 = z16 + 32u * kZPitch;
+                unsigned char* z8 = sStg + kZ8 + (uint32_t)t0 * kZ8Pitch + 8u * (uint32_t)cp;
                 // (blocks 0, 1 lie before the boundary at 16 and take Y there, blocks 2, 3 take X; blocks 0, 2 take Y at 8 / 24)
                 const f32x2 s16 = tb == 0 ? blk[1] : tb == 3 ? blk[2] : one2;
                 if (tb != 0) {
@@ -769,7 +774,7 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                         r = mul2(r, g2[s]);
                         const f32x2 x = mul2(r, k2[s]);
                         if (tb >= 2) put2(z16 + s * kZPitch, z16 + kZHalf + s * kZPitch, mul2(s16, x));
-                        if (tb & 1) put2(z8 + s * kZPitch, z8 + kZHalf + s * kZPitch, x);
+                        if (tb & 1) *reinterpret_cast<f32x2*>(z8 + s * kZ8Pitch) = x;
                     }
                 }
                 if (tb != 3) {
@@ -779,22 +784,20 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                         const f32x2 y = mul2(r, k2[s]);
                         r = mul2(r, g2[s]);
                         if (tb < 2) put2(z16 + s * kZPitch, z16 + kZHalf + s * kZPitch, mul2(s16, y));
-                        if (!(tb & 1)) put2(z8 + s * kZPitch, z8 + kZHalf + s * kZPitch, y);
+                        if (!(tb & 1)) *reinterpret_cast<f32x2*>(z8 + s * kZ8Pitch) = y;
                     }
                 }
             }
             f_sync();                  // partial pair sums and Z rows are complete
 
             float cross[4] = {0.f, 0.f, 0.f, 0.f};
-            if (fw >= 4) {
-                // ---- mma.sync products of the Z rows, hi * hi + lo * hi + hi * lo, 16 x 8 per warp.  Warps 6, 7: A_21 = X Y^T (tokens
-                // 16..31 against 0..7, 8..15), kept in registers until the operand set is free.  Warps 4, 5: rows 0..7 X of tokens
-                // 8..15, rows 8..15 X of tokens 24..31, against Y of tokens 0..7 (the upper half counts), 16..23 (the lower half).
-                // One warp per scheduler: a step waits for its fragments and for the accumulators of the step before ----
+            if (fw >= 6) {
+                // ---- A_21 = X Y^T (tokens 16..31 against 0..7, 8..15) as mma.sync products of the Z rows, hi * hi + lo * hi + hi * lo, 16 x 8
+                // per warp, kept in registers until the operand set is free.  One warp per scheduler (with those of the 8 x 8 blocks): a
+                // step waits for its fragments and for the accumulators of the step before ----
                 const uint32_t zb = smem_u32(sStg);
-                const int r = lane & 15, nt = fw & 1;
-                const uint32_t arow = fw >= 6 ? 16u + (uint32_t)r : 32u + (uint32_t)(r < 8 ? 8 + r : 16 + r);
-                const uint32_t brow = (uint32_t)(lane & 7) + (fw >= 6 ? (uint32_t)nt * 8u : 32u + (uint32_t)nt * 16u);
+                const uint32_t arow = 16u + (uint32_t)(lane & 15);
+                const uint32_t brow = (uint32_t)(lane & 7) + (uint32_t)(fw & 1) * 8u;
                 const uint32_t abase = zb + arow * kZPitch + (uint32_t)(lane >> 4) * 16u;
                 const uint32_t bbase = zb + brow * kZPitch + (uint32_t)((lane >> 3) & 1) * 16u + (uint32_t)(lane >> 4) * kZHalf;     // hi, then lo
                 float c1[4] = {0.f, 0.f, 0.f, 0.f};
@@ -810,18 +813,53 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                 }
 #pragma unroll
                 for (int e = 0; e < 4; ++e) cross[e] += c1[e];
-                if (fw < 6) {
-                    const int r0 = 8 + 16 * nt + (lane >> 2), c0 = (lane & 3) * 2;
-                    sA[r0 * kAS2 + c0] = sBeta[r0] * (nt ? cross[2] : cross[0]);
-                    sA[r0 * kAS2 + c0 + 1] = sBeta[r0] * (nt ? cross[3] : cross[1]);
+            } else if (fw >= 2) {
+                // ---- the 8 x 8 blocks of tokens t1 .. t1 + 7 against the eight before them (t1 = 8, 24), half of the columns per warp: a lane
+                // takes rows u, u + 4, columns w, w + 2 and a quarter of the channels ----
+                const int t1 = 8 + 16 * (fw & 1), u = (lane >> 1) & 3, w = (fw >= 4 ? 4 : 0) + (lane & 1);
+                const unsigned char* zx = sStg + kZ8 + (uint32_t)(t1 + u) * kZ8Pitch + (uint32_t)(lane >> 3) * 128u;
+                const unsigned char* zy = sStg + kZ8 + (uint32_t)(t1 - 8 + w) * kZ8Pitch + (uint32_t)(lane >> 3) * 128u;
+                f32x2 acc[2][2];
+#pragma unroll
+                for (int a = 0; a < 2; ++a)
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) acc[a][c] = pack2(0.f, 0.f);
+#pragma unroll 4
+                for (int i = 0; i < K / 4; i += 4) {
+                    ulonglong2 x[2], y[2];
+#pragma unroll
+                    for (int a = 0; a < 2; ++a) {
+                        x[a] = *reinterpret_cast<const ulonglong2*>(zx + 4 * a * kZ8Pitch + 4 * i);
+                        y[a] = *reinterpret_cast<const ulonglong2*>(zy + 2 * a * kZ8Pitch + 4 * i);
+                    }
+#pragma unroll
+                    for (int a = 0; a < 2; ++a)
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) acc[a][c] = fma2(x[a].y, y[c].y, fma2(x[a].x, y[c].x, acc[a][c]));
                 }
+#pragma unroll
+                for (int a = 0; a < 2; ++a)
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        float lo, hi;
+                        unpack2(acc[a][c], lo, hi);
+                        lo += hi;
+                        lo += __shfl_xor_sync(0xffffffffu, lo, 8);
+                        lo += __shfl_xor_sync(0xffffffffu, lo, 16);
+                        const int r0 = t1 + u + 4 * a;
+                        if (lane < 8) sA[r0 * kAS2 + w + 2 * c] = sBeta[r0] * lo;
+                    }
             } else {
-                // ---- beta_s A_sj of the pairs inside the blocks of eight (only entries below the diagonal are read) ----
+                // ---- beta_s A_sj of the pairs inside the blocks of eight, two blocks per warp (only entries below the diagonal are read) ----
                 int s = 1;
                 while (s < 8 && (s + 1) * s / 2 <= lane) ++s;        // the pair's later token
                 if (lane < 28) {
-                    const int jj = lane - s * (s - 1) / 2, s32 = 8 * fw + s;
-                    sA[s32 * kAS2 + 8 * (fw & 1) + jj] = sBeta[s32] * (sPart[2 * fw * 32 + lane] + sPart[(2 * fw + 1) * 32 + lane]);
+                    const int jj = lane - s * (s - 1) / 2;
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const int s32 = 16 * fw + 8 * u + s;
+                        sA[s32 * kAS2 + 8 * u + jj] = sBeta[s32] * (sPart[(4 * fw + 2 * u) * 32 + lane] + sPart[(4 * fw + 2 * u + 1) * 32 + lane]);
+                    }
                 }
             }
             proxy_fence();             // (the next tile's rows come in by bulk copies over Z)

@@ -54,3 +54,91 @@ def test_ctas_with_several_tiles(batch, heads):
     m, S0, Om, _C, _ = make_layer(w)
     for n, token in [(31, True), (9, True), (20, False)]:
         _flush(m, w, S0, Om, n, token)
+
+
+def _given_tokens(w, S0, Om, toks, q, dev_layer):
+    """A flush of the given tokens [n][B, H, ..] (float64 arrays of stored values), the last one as the current token: S, U, o."""
+    m, n = dev_layer, len(toks)
+    m.state.copy_(torch.from_numpy(S0))
+    dt = (torch.bfloat16, torch.bfloat16, torch.float32, torch.bfloat16)
+    on = [[torch.from_numpy(x).to(m.device, d).contiguous() for x, d in zip(t, dt)] for t in toks]
+    for t in range(n - 1):
+        for view, x in zip(m.ring_views(), on[t]):
+            view[:, :, t] = x
+    o = m.new_output()
+    m.state_update(n - 1, torch.from_numpy(q).to(m.device, torch.bfloat16), *on[-1], o)
+    m.check_status()
+    S, U, ref = orc.state_update(w.kind, S0.astype(np.float64), toks, np.broadcast_to(Om.astype(np.float64), (w.batch,) + Om.shape), q)
+    return (m.state.cpu().numpy(), S), (m.sketch.cpu().numpy().transpose(0, 1, 3, 2), U), (o.cpu().numpy(), ref)
+
+
+def _bf16(x):
+    return torch.from_numpy(x).bfloat16().double().numpy()
+
+
+def _norm_err(got, ref):
+    return np.linalg.norm(got - ref) / np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n", [8, 16, 24, 32, 64])
+@pytest.mark.parametrize("spread", [0.1, 0.0])
+def test_keys_of_one_direction_and_slow_decays(n, spread):
+    """Nearly equal (equal) keys, beta and decays near one: the system I + Bd A is as far from the identity as unit keys make it.
+    2-norm, bar as above: each operand 2^-16, three products in a row."""
+    w = synth.Workload("t", "kda", 6, 3, 128, 128, 16, 64, 0, "bf16", 613, basis="qr")
+    m, S0, Om, _C, _ = make_layer(w)
+    rng = np.random.default_rng(n)
+    base = rng.standard_normal((w.batch, w.heads, 128))
+    toks = []
+    for _ in range(n):
+        k = base + spread * rng.standard_normal(base.shape)
+        toks.append((_bf16(k / np.linalg.norm(k, axis=-1, keepdims=True)), _bf16(rng.standard_normal(base.shape)),
+                     (1 - 0.01 * rng.random(base.shape[:2])).astype(np.float32).astype(np.float64),
+                     _bf16(1 - 2.0 ** -(4 + 4 * rng.random(base.shape)))))
+    q = _bf16(base / np.linalg.norm(base, axis=-1, keepdims=True))
+    for got, ref in _given_tokens(w, S0, Om, toks, q, m):
+        assert _norm_err(got, ref) <= FP32_GUARD, n
+
+
+def test_pair_sums_inside_sixteen_tokens_are_fp32():
+    """Keys of one channel: a pair sum is a single product, so what its operands are held in shows in S_new.  From a zero state
+    S_new = K~^T E with both factors as two bfloat16 halves (lo lo left out) and E = T V from an exact A is what the kernel may
+    lose; with the pair sums of tokens 8..11 against 0..7 from halves as well the error would be 1.25 times that.  Bar: 1.1 times
+    (fp32 sums: 2^-24 of 2^-17)."""
+    w = synth.Workload("t", "kda", 64, 4, 128, 128, 16, 16, 0, "bf16", 617, basis="qr")
+    m, S0, Om, _C, _ = make_layer(w)
+    S0 = np.zeros_like(S0)
+    rng, n, shape = np.random.default_rng(3), 12, (w.batch, w.heads, 128)
+    ch, toks = 37, []
+    for _ in range(n):
+        k = np.zeros(shape)
+        k[..., ch] = 0.5 + rng.random(shape[:2])
+        toks.append((_bf16(k), _bf16(rng.standard_normal(shape)), (1 - 0.01 * rng.random(shape[:2])).astype(np.float32).astype(np.float64),
+                     _bf16(1 - 2.0 ** -(4 + 4 * rng.random(shape)))))
+    k, g = (np.stack([t[i][..., ch] for t in toks], -1) for i in (0, 3))
+    v, beta = np.stack([t[1] for t in toks], -2), np.stack([t[2] for t in toks], -1)
+
+    def halves(x):
+        hi = _bf16(np.ascontiguousarray(x))
+        return hi, _bf16(x - hi)
+
+    def expected(split_pairs):
+        prod = lambda a, b: np.prod(g[..., a:b], axis=-1)
+        A = np.zeros(k.shape[:2] + (n, n))
+        for s in range(n):
+            for j in range(s):
+                if split_pairs and s >= 8 > j:
+                    (xh, xl), (yh, yl) = halves(k[..., s] * prod(8, s + 1)), halves(k[..., j] * prod(j + 1, 8))
+                    A[..., s, j] = xh * yh + xl * yh + xh * yl
+                else:
+                    A[..., s, j] = k[..., s] * k[..., j] * prod(j + 1, s + 1)
+        E = np.linalg.solve(np.eye(n) + beta[..., None] * A, beta[..., None] * v)
+        (th, tl), (eh, el) = halves(np.stack([k[..., s] * prod(s + 1, n) for s in range(n)], -1)), halves(E)
+        row = lambda t, e: np.einsum("bhs,bhsv->bhv", t, e)
+        return row(th, eh) + row(tl, eh) + row(th, el)
+
+    (S, ref), _, _ = _given_tokens(w, S0, Om, toks, np.zeros(shape), m)
+    exact = ref[:, :, ch]
+    kept = _norm_err(expected(False), exact)
+    assert _norm_err(expected(True), exact) >= 1.2 * kept
+    assert _norm_err(S[:, :, ch].astype(np.float64), exact) <= 1.1 * kept
