@@ -22,12 +22,12 @@ namespace sketchssm {
 
 namespace {
 
+constexpr int kBuffers = 2;            // chunks on their way
 // Lanes that share a row (16 or 20 columns each); a chunk is two rows per lane, 4 KB (V = 80: 5 KB).
 template <int V>
 __host__ __device__ constexpr int pivot_parts() { return V == 128 ? 8 : 4; }
 template <int V>
 __host__ __device__ constexpr int pivot_rows() { return 2 * 32 / pivot_parts<V>(); }
-constexpr int kBuffers = 2;
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -62,18 +62,23 @@ __host__ __device__ inline PivotSmem make_pivot_smem(int R, int su) {
 
 }  // namespace
 
-constexpr int kPivotWarps = 4;         // of a CTA
+// Warps of an SM (the registers hold no more), each a CTA: few heads spread over the SMs, and large ranks leave room for as many warps
+// as shared memory holds.  In CTAs of four 64 heads ran on 16 SMs.  Sketch and map from a prefilled state, K = 128, us: CTA per head
+// (coef_map.cu) / CTAs of four / of one, and rows of Omega asked for ahead of their use above 16 ranks:
+//   V = 128, rank 16, fp32: 64 heads 22.2 / 22.5 / 21.7, 888 43.6 / 38.3 / 37.5;  rank 24: 64 heads 24.5 / 28.4 / 23.7, 888 46.9 / 45.0 / 40.7
+//   V = 64,  rank 16, fp32: 4 heads 14.1 / 15.2 / 13.9, 256 21.0 / 20.9 / 20.2;  rank 24: 4 heads 16.4 / 17.9 / 16.2, 888 33.5 / 34.0 / 30.5
+constexpr int kPivotWarps = 12;
 
 template <int K, int V, bool BF>
-__global__ void __launch_bounds__(kPivotWarps * 32, 3) pivot_map_kernel(const Params p) {
+__global__ void __launch_bounds__(32, kPivotWarps) pivot_map_kernel(const Params p) {
     constexpr int kRows = pivot_rows<V>(), PARTS = pivot_parts<V>(), RS = 32 / PARTS, VP = V / PARTS, NB = kBuffers, NC = K / kRows, SU = BF ? 2 : 4;
     constexpr uint32_t kRowBytes = (V + 4) * 4, kChunkBytes = kRows * kRowBytes;
     static_assert(NC >= NB, "the next head's first chunks are requested from this head's last ones");
     extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int lane = threadIdx.x;
     const int R = p.R, H = p.H;
     const PivotSmem sm = make_pivot_smem<K, V>(R, SU);
-    unsigned char* base = smem + (size_t)warp * sm.total;
+    unsigned char* base = smem;
     const uint32_t sbase = smem_u32(base);
     float* sQ = reinterpret_cast<float*>(base + sm.q);
     float* sY = reinterpret_cast<float*>(base + sm.y);
@@ -87,7 +92,7 @@ __global__ void __launch_bounds__(kPivotWarps * 32, 3) pivot_map_kernel(const Pa
     // Heads in descending order, the warps of the grid side by side: what the flush wrote last is still in L2.  A head's rank:
     // the configured one or the caller's (0: it reads its full state and has no map); with per-sequence phases only the
     // sequences that were just flushed get a new map.
-    const int heads = p.B * H, stride = (int)gridDim.x * nwarps;        // (at most 2^24 heads)
+    const int heads = p.B * H, stride = (int)gridDim.x;        // (at most 2^24 heads)
     auto rank_of = [&](int bh) -> int {
         if (p.head_rank == nullptr) return R;
         const int r = p.head_rank[bh % H];
@@ -117,7 +122,7 @@ __global__ void __launch_bounds__(kPivotWarps * 32, 3) pivot_map_kernel(const Pa
         if (++fill == NB) fill = 0;
     };
 
-    int bh = settle(heads - 1 - ((int)blockIdx.x * nwarps + warp));
+    int bh = settle(heads - 1 - (int)blockIdx.x);
     if (bh < 0) return;
 #pragma unroll
     for (int c = 0; c < NB; ++c) {
@@ -428,19 +433,28 @@ __global__ void __launch_bounds__(kPivotWarps * 32, 3) pivot_map_kernel(const Pa
                 for (int c = 0; c < 4; ++c)
                     if (4 * c < G4) pass2(4 * c, o[c]);
             } else {
-                for (int g0 = 0; g0 < G4; g0 += 4) {
-                    float o[2][4];
-                    om4(0, g0, o[0]);
-                    om4(1, g0, o[1]);
-                    pass1(g0, o);
-                }
+                // (more: read twice, four ranks ahead of their use)
+                auto walk = [&](auto pass) {
+                    float a[2][4], b[2][4];
+                    om4(0, 0, a[0]);
+                    om4(1, 0, a[1]);
+                    for (int g0 = 0; g0 < G4; g0 += 8) {
+                        const bool more = g0 + 4 < G4;
+                        if (more) {
+                            om4(0, g0 + 4, b[0]);
+                            om4(1, g0 + 4, b[1]);
+                        }
+                        pass(g0, a);
+                        if (g0 + 8 < G4) {
+                            om4(0, g0 + 8, a[0]);
+                            om4(1, g0 + 8, a[1]);
+                        }
+                        if (more) pass(g0 + 4, b);
+                    }
+                };
+                walk(pass1);
                 solve();
-                for (int g0 = 0; g0 < G4; g0 += 4) {
-                    float o[2][4];
-                    om4(0, g0, o[0]);
-                    om4(1, g0, o[1]);
-                    pass2(g0, o);
-                }
+                walk(pass2);
             }
         }
         __syncwarp();                                    // the tables are written again for the next head
@@ -451,29 +465,21 @@ __global__ void __launch_bounds__(kPivotWarps * 32, 3) pivot_map_kernel(const Pa
 template <int K, int V>
 static int launch_pivot_kv(Ctx* ctx, const Params& p, cudaStream_t stream) {
     const PivotSmem sm = make_pivot_smem<K, V>(p.R, p.sketch_bf16 ? 2 : 4);
-    const uint32_t budget = 227u * 1024u;
-    if (sm.total > budget) return SKETCHSSM_UNSUPPORTED_SHAPE;
+    if (sm.total > 227u * 1024u) return SKETCHSSM_UNSUPPORTED_SHAPE;
     if (ctx->sm_count == 0) {
         int sms = 0;
         if ((ctx->last_cuda_error = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->cfg.device)) != cudaSuccess)
             return SKETCHSSM_CUDA_ERROR;
         ctx->sm_count = sms;
     }
-    // one head per warp: CTAs of four warps, smaller ones where the sketch rows of large ranks leave room for fewer
-    int nw = 1, ctas = 1;
-    for (int w = kPivotWarps; w >= 1; --w) {
-        if ((uint32_t)w * sm.total > budget) continue;
-        int n = (int)(228u * 1024u / ((uint32_t)w * sm.total + 1024u));
-        if (n * w > 12) n = 12 / w;
-        if (n < 1) n = 1;
-        if (n * w > nw * ctas || (nw == 1 && ctas == 1)) { nw = w; ctas = n; }
-    }
+    int ctas = (int)(228u * 1024u / (sm.total + 1024u));
+    if (ctas > kPivotWarps) ctas = kPivotWarps;
     const long long heads = (long long)p.B * p.H;
     long long grid = (long long)ctx->sm_count * ctas;
-    if (grid > (heads + nw - 1) / nw) grid = (heads + nw - 1) / nw;
+    if (grid > heads) grid = heads;
     auto kern = p.sketch_bf16 ? pivot_map_kernel<K, V, true> : pivot_map_kernel<K, V, false>;
     if ((ctx->last_cuda_error = unlock_smem(ctx, kern, true)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
-    kern<<<dim3((unsigned)grid), dim3((unsigned)(32 * nw)), (uint32_t)nw * sm.total, stream>>>(p);
+    kern<<<dim3((unsigned)grid), dim3(32), sm.total, stream>>>(p);
     if ((ctx->last_cuda_error = cudaGetLastError()) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     ctx->last_launches += 1;
     return SKETCHSSM_OK;

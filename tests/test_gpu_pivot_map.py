@@ -12,7 +12,7 @@ from tests.test_gpu_parity import make_layer, run_schedule
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("rank,pivots", [(1, 4), (2, 4), (3, 2), (5, 1), (8, 4), (13, 3), (15, 4), (17, 4), (24, 4)])
+@pytest.mark.parametrize("rank,pivots", [(1, 4), (2, 4), (3, 2), (5, 1), (8, 4), (13, 3), (15, 4), (17, 4), (20, 4), (21, 3), (24, 4)])
 @pytest.mark.parametrize("K,V", [(128, 64), (128, 80), (128, 128), (64, 64), (64, 128)])
 def test_ranks_pivots_and_shapes(rank, pivots, K, V):
     w = synth.Workload("t", "mamba2", 3, 2, K, V, rank, 4, 0, "f32", 503, basis="qr")
