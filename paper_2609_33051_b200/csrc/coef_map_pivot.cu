@@ -488,10 +488,12 @@ static int launch_pivot_kv(Ctx* ctx, const Params& p, cudaStream_t stream) {
 int launch_pivot_map(Ctx* ctx, const Params& p, cudaStream_t stream) {
     const int K = ctx->cfg.dk, V = ctx->cfg.dv;
     if (p.pivots < 1 || (p.pivots > 4 && p.R > 4)) return SKETCHSSM_UNSUPPORTED_SHAPE;
-    // Large ranks stay with the CTA per head (coef_map.cu): the sketch rows and two reads of Omega weigh as much as the state, and the warp has
-    // them to itself.  Flush + map, that kernel -> this one, fp32: rank 32, V = 64, 128 heads 27.5 -> 30.3 us, 4736 187 -> 190; V = 128,
-    // 288 heads 45.3 -> 43.9, 4736 554 -> 536; rank 64, V = 64, 288 heads 42.6 -> 47.5.
-    if (p.R > 32 || (p.R > 24 && (V == 64 || (long long)p.B * p.H <= 256))) return SKETCHSSM_UNSUPPORTED_SHAPE;
+    // By the rank and the state's shape alone: the two kernels differ in the last bits, and what a stored element is rounded to shall not
+    // depend on the size of the batch.  Above 24 ranks the sketch rows and two reads of Omega weigh as much as the state of 64 columns,
+    // and a warp has them to itself.  Sketch and map from a prefilled state, fp32, CTA per head -> warp per head, us: rank 32, V = 64, 64
+    // heads 22.6 -> 22.7, 888 39.2 -> 35.0;  V = 128, 4 heads 24.1 -> 24.6, 64 25.9 -> 25.8, 888 51.5 -> 45.4, 4736 231 -> 200;  V = 80, 4 heads
+    // 21.7 -> 22.9, 256 27.0 -> 27.2, 888 50.4 -> 45.7.
+    if (p.R > 32 || (p.R > 24 && V == 64)) return SKETCHSSM_UNSUPPORTED_SHAPE;
     if (K == 128 && V == 128) return launch_pivot_kv<128, 128>(ctx, p, stream);
     if (K == 128 && V == 64) return launch_pivot_kv<128, 64>(ctx, p, stream);
     if (K == 128 && V == 80) return launch_pivot_kv<128, 80>(ctx, p, stream);

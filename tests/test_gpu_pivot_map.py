@@ -65,3 +65,18 @@ def test_zero_state_gives_a_zero_map():
     m.state_update(0)
     m.check_status()
     assert torch.equal(m.coef, torch.zeros_like(m.coef))
+
+
+@pytest.mark.parametrize("V,rank", [(128, 16), (128, 25), (128, 32), (80, 28), (64, 24), (64, 28), (128, 33)])
+def test_a_stored_map_does_not_depend_on_the_batch(V, rank):
+    """The same sequences alone and among many: their maps bit for bit."""
+    maps = []
+    for batch in (2, 130):
+        w = synth.Workload("t", "mamba2", batch, 3, 128, V, rank, 4, 0, "bf16", 523, basis="qr")
+        m, _S0, _Om, _C, dev = make_layer(w, coef="pivot")
+        gen = torch.Generator().manual_seed(7)
+        m.state.copy_(torch.randn(130, 3, 128, V, generator=gen)[:batch] * 0.02)
+        m.state_update(0)
+        m.check_status()
+        maps.append((m.sketch[:2].clone(), m.coef[:2].clone()))
+    assert torch.equal(maps[0][0], maps[1][0]) and torch.equal(maps[0][1], maps[1][1])
