@@ -2,10 +2,12 @@
 // constants (no CUDA), so that a test can walk them.
 #pragma once
 
+#ifndef SKETCHSSM_BOTH
 #ifdef __CUDACC__
 #define SKETCHSSM_BOTH __host__ __device__
 #else
 #define SKETCHSSM_BOTH
+#endif
 #endif
 
 namespace sketchssm {

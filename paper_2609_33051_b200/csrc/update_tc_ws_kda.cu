@@ -41,6 +41,7 @@
 #include <type_traits>
 #include "internal.cuh"
 #include "lanegroup.cuh"
+#include "operand_sets.h"
 #include "tc_common.cuh"
 
 namespace sketchssm {
@@ -567,6 +568,7 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
         const int cp = ft & 63;               // channels 2 cp, 2 cp + 1
         const int fw = ft >> 5;               // warp of the group, 0..7
         uint32_t phS = 0;
+        int filled = 0;                       // tiles whose value rows were requested
         bool dead = false;
         float* sA = reinterpret_cast<float*>(smem + sm.mats);
         float* sBeta = sA + 2 * 16 * kAS2;
@@ -875,6 +877,7 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
                 }
             }
             stage_values(bh, b);
+            ++filled;
             // ---- running products of this block.  Khat -> window rows 0..31; Ktil -> set (MN-major); G_n * W -> window rows 32.. ----
             {
                 unsigned char* wcol = wb + (uint32_t)(cp >> 2) * LBO_W + (uint32_t)(cp & 3) * 4u;              // K-major: k = channel
@@ -998,7 +1001,7 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
         }
         if (dead && ft < 32) {     // copies that may still be in flight get a short, bounded grace period
             mbar_wait_bounded(&bars[kStg], phS, 1u << 14);
-            for (int sb = 0; sb < 2; ++sb) mbar_wait_bounded(&bars[kVals + sb], 0u, 1u << 12);
+            for (int t = first_unfinished(filled); t < filled; ++t) mbar_wait_bounded(&bars[kVals + set_of_tile(t)], parity_of_tile(t), 1u << 12);
         }
         if (ft == 0) {     // scheduler counters back to zero once every CTA is done claiming
             __threadfence();

@@ -165,3 +165,35 @@ def test_a_dense_heads_warps_read_each_row_once_and_ask_only_for_their_own(tmp_p
         assert rows == set(range(sub * K // W, (sub + 1) * K // W)), (K, W, sub)
         assert asked[K, W, sub] <= rows, (K, W, sub)
     assert len(read) == 2 * (1 + 2 + 4)
+
+
+_SETS = r"""
+#include <cstdio>
+#include "operand_sets.h"
+using namespace sketchssm;
+int main() {
+    for (int tiles = 0; tiles < 12; ++tiles) {
+        std::printf("%d", tiles);
+        for (int t = first_unfinished(tiles); t < tiles; ++t) std::printf(" %d %u", set_of_tile(t), parity_of_tile(t));
+        std::printf("\n");
+    }
+}
+"""
+
+
+def test_a_flush_that_gives_up_waits_for_the_last_fill_of_each_operand_set(tmp_path):
+    """A barrier answers a wait for parity p at once unless its current phase has that parity: a wait for another phase than the one
+    in flight gives the copies no time."""
+    (tmp_path / "sets.cpp").write_text(_SETS)
+    exe = str(tmp_path / "sets")
+    csrc = os.path.join(ROOT, "paper_2609_33051_b200", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-I", csrc, str(tmp_path / "sets.cpp"), "-o", exe], check=True)
+    for ln in subprocess.run([exe], check=True, capture_output=True, text=True).stdout.splitlines():
+        tiles, *waits = map(int, ln.split())
+        waits = set(zip(waits[::2], waits[1::2]))
+        fills = [[t for t in range(tiles) if t % 2 == s] for s in (0, 1)]
+        # the last fill of a set is not complete: its barrier is in phase len(fills) - 1
+        assert waits == {(s, (len(f) - 1) % 2) for s, f in enumerate(fills) if f}, tiles
+    src = open(os.path.join(csrc, "update_tc_ws_kda.cu")).read()
+    grace = src[src.index("if (dead && ft < 32)"):]
+    assert "kVals + set_of_tile(t)], parity_of_tile(t)" in grace[:600]
