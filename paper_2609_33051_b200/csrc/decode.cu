@@ -87,11 +87,13 @@ __host__ __device__ inline DecodeSmem make_decode_smem(int K, int R, int nwarps,
     return d;
 }
 
-// state rows, read once: no lines of L1 for them
+// state rows, read once: no lines of L1 for them.  (A flush that runs before this kernel writes them: never ahead of the wait for it.)
 template <int N>
 __device__ __forceinline__ void load_stream(const float* src, float (&d)[N]) {
-    if constexpr (N == 4) asm("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(d[0]), "=f"(d[1]), "=f"(d[N - 2]), "=f"(d[N - 1]) : "l"(src));
-    else asm("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(d[0]), "=f"(d[1]) : "l"(src));
+    if constexpr (N == 4)
+        asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(d[0]), "=f"(d[1]), "=f"(d[N - 2]), "=f"(d[N - 1]) : "l"(src) : "memory");
+    else
+        asm volatile("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(d[0]), "=f"(d[1]) : "l"(src) : "memory");
 }
 
 }  // namespace

@@ -197,3 +197,23 @@ def test_a_flush_that_gives_up_waits_for_the_last_fill_of_each_operand_set(tmp_p
     src = open(os.path.join(csrc, "update_tc_ws_kda.cu")).read()
     grace = src[src.index("if (dead && ft < 32)"):]
     assert "kVals + set_of_tile(t)], parity_of_tile(t)" in grace[:600]
+
+
+def test_inline_loads_are_ordered_with_the_waits_before_them():
+    """A load in inline assembly that is not volatile is to the compiler a function of its address, which it may move ahead of the
+    wait for the kernel that writes the memory; one of global memory has to name memory as well, as plain loads and stores do not
+    keep their order with it otherwise."""
+    import glob
+    import re
+    csrc, seen = os.path.join(ROOT, "paper_2609_33051_b200", "csrc"), 0
+    for path in sorted(glob.glob(os.path.join(csrc, "*.cu*"))):
+        src = open(path).read()
+        for m in re.finditer(r"\basm\b(\s+volatile)?\s*\((.*?)\)\s*;\s*(?:\n|\})", src, re.S):
+            stmt = m.group(2)
+            where = (os.path.basename(path), src[:m.start()].count("\n") + 1)
+            if re.search(r"\b(ld\.|ldmatrix|tcgen05\.ld)", stmt):
+                seen += 1
+                assert m.group(1), where
+            if re.search(r"\bld\.(global|acquire|relaxed|volatile)", stmt):
+                assert '"memory"' in stmt, where
+    assert seen >= 6
