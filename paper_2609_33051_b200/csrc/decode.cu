@@ -106,22 +106,24 @@ __device__ __forceinline__ void load_stream(const float* src, float (&d)[N]) {
 //   kAny  general: per-head ranks (rank 0: that head reads the full state), and kSeq / kPS / kUB as the launch says (kER
 //         stays a compile-time fact).
 // Every flag that is decided inside the loops over heads, ranks or slots costs the launches that do not use it: without the
-// full-read branch and the run-time flags 138 of the 170 instantiations without kAny spill nothing and the others at most
-// 24 bytes (the general ones 4 to 96), and the launches that had to run the general one take (general -> own, r = L = 16,
+// full-read branch and the run-time flags 223 of the 282 instantiations without kAny spill nothing and the others at most
+// 24 bytes (the fp32 full reads of K = V = 64 with two warps a head 72), the 110 general ones up to 96, and the launches that had to run the general one take (general -> own, r = L = 16,
 // bfloat16 I/O): state-dependent bfloat16 map, Mamba-2 64-head batch of 256, 33 -> 31 us; the same with erase vectors, GDN
 // 32-head batch of 512, 53 -> 45 us; mixed step of that layer 48 -> 46 us.  (How much of it is the unrolled rank has not been
 // measured apart.)  V = 80 layer of 37 x 24 heads with two dense heads (prefetch below): 13 -> 10 us.
 constexpr int kSeq = 1, kPS = 2, kER = 4, kUB = 8, kAny = 16, kFull = 32;
 
-// Warps of the largest CTA; two such CTAs per SM set the register budget: 64 registers for the lean Mamba-2 kernels (32
-// warps), 80 for the others (24 warps).
-__host__ __device__ constexpr int decode_max_warps(int kind, int F, int W) {
-    return ((F & ~(kUB | kFull)) != 0 || kind != SKETCHSSM_MAMBA2 ? 12 : 16) * (W > 1 ? 2 : 1);
+// Warps of the largest CTA; two such CTAs per SM (one of a team kernel's, which are twice as large) set the register budget: 64 registers
+// for the lean Mamba-2 kernels (32 warps), 80 for the others (24 warps), the full reads of Mamba-2 teams among them: their rows in flight
+// spilled 152 to 372 bytes at 64 (nothing at 80; 0.91 of the time with two warps a head on average; with K = V = 64 64 is faster: 9472 heads 26.8 against 28.7 us).
+__host__ __device__ constexpr int decode_max_warps(int kind, int K, int V, int F, int W) {
+    const bool lean = kind == SKETCHSSM_MAMBA2 && (F & ~(kUB | kFull)) == 0 && !(W > 1 && F == kFull && K * V > 64 * 64);
+    return (lean ? 16 : 12) * (W > 1 ? 2 : 1);
 }
 
 // W: warps that share a head (a team).
 template <int KIND, typename IO, int K, int V, int RT, int F, int W>
-__global__ void __launch_bounds__(decode_max_warps(KIND, F, W) * 32, W > 1 ? 1 : 2) decode_kernel(const Params p) {
+__global__ void __launch_bounds__(decode_max_warps(KIND, K, V, F, W) * 32, W > 1 ? 1 : 2) decode_kernel(const Params p) {
     static_assert(W == 1 || F == kFull || F == kAny || (F == 0 && KIND == SKETCHSSM_MAMBA2), "no team for this instantiation");
     constexpr bool TEAM = W > 1;
     constexpr bool ANY = (F & kAny) != 0, DYN = ANY || (F & kSeq) != 0, FULL = (F & kFull) != 0;
@@ -873,13 +875,13 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
         constexpr int RT = decltype(rt)::value, F = decltype(f)::value;
         kern = decode_kernel<KIND, IO, K, V, RT, F, 1>;
         variant = number;
-        max_nw = decode_max_warps(KIND, F, 1);
+        max_nw = decode_max_warps(KIND, K, V, F, 1);
         if constexpr (F == kFull || F == kAny || (F == 0 && KIND == SKETCHSSM_MAMBA2)) {
             if (W == 2) kern = decode_kernel<KIND, IO, K, V, RT, F, 2>;
             if (W == 4) kern = decode_kernel<KIND, IO, K, V, RT, F, 4>;
             if (W > 1) {
                 variant = number + 13 * (W / 2);
-                max_nw = decode_max_warps(KIND, F, W);
+                max_nw = decode_max_warps(KIND, K, V, F, W);
             }
         }
     };
