@@ -16,7 +16,7 @@ UNITS = [("api.cu", "", []), ("update.cu", "", []), ("update_cols.cu", "", []), 
          *[(src, f"_k{k}_io{io}", [f"-DSKETCHSSM_GROUP_KIND={k}", f"-DSKETCHSSM_GROUP_IO={io}"])
            for src in ("decode.cu", "decode_split.cu") for k in range(3) for io in range(2)]]
 HEADERS = [os.path.join(CSRC, "internal.cuh"), os.path.join(CSRC, "lanegroup.cuh"), os.path.join(CSRC, "tc_common.cuh"),
-           os.path.join(CSRC, "state_rows.h"), os.path.join(CSRC, "operand_sets.h"),
+           os.path.join(CSRC, "state_rows.h"), os.path.join(CSRC, "operand_sets.h"), os.path.join(CSRC, "team_size.h"),
            os.path.join(ROOT, "include", "sketchssm.h")]
 
 

@@ -20,6 +20,7 @@
 #include "internal.cuh"
 #include "lanegroup.cuh"
 #include "state_rows.h"
+#include "team_size.h"
 
 namespace sketchssm {
 
@@ -928,9 +929,15 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
     // fewer heads than warps fit, larger CTAs only leave more SMs idle: general kernel, 64 heads, 4.2 -> 4.9 us; the lean ones,
     // whose CTAs stage less per head, did not lose by it)
     if (variant < 13) W = 1;
+    // A team's CTA holds no more heads than an SM has, and warps that no head would take do not count: with all warps that fit, 60 heads
+    // of a rank table sat on five SMs (GDN 128 x 128, 12 tokens, 300 heads 12.2 -> 6.5 us a launch with one dense head in twelve), and CTAs of
+    // single teams, each with its copy of the maps, won by a warp (GDN 64 x 64, teams of two, 876 heads 8.3 -> 3.6).  With a rank table up to
+    // eight warps, which fetch the maps sooner than four (Mamba-2 128 x 80, 144 heads 4.1 -> 3.6).
+    const int least = need != kFull && p.head_rank != nullptr ? 8 : W;
+    const int useful = W > 1 ? useful_team_warps(W, heads, ctx->sm_count) : 1 << 20;
     for (int i = 0; i < max_nw; ++i) {
         const int nw = i < 8 ? 8 - i : i + 1;
-        if (nw % W || nw / W > 15) continue;
+        if (nw % W || nw / W > 15 || (W > 1 && team_cta_too_large(nw, W, least, heads, ctx->sm_count))) continue;
         if (nw > 8 && variant == 0 && heads <= (long long)ctx->sm_count * best_warps) break;
         if (p.warps_per_cta && (nw != p.warps_per_cta || nw > 8)) continue;       // (a caller's own choice: 1 to 8)
         const DecodeSmem d = make_decode_smem(K, p.R, nw, p.full_read, p.coef_per_seq, sl.total, W);
@@ -940,7 +947,8 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
         if (ctas * nw > cap) ctas = cap / nw;
         if (ctas * nw > reg_warps) ctas = reg_warps / nw;
         if (ctas < 1) continue;
-        if (ctas * nw > best_warps) { best_warps = ctas * nw; best_nw = nw; best_ctas = ctas; }
+        const int warps = ctas * nw < useful ? ctas * nw : useful;
+        if (warps > best_warps) { best_warps = warps; best_nw = nw; best_ctas = ctas; }
     }
     if (best_nw == 0) return SKETCHSSM_UNSUPPORTED_SHAPE;
     const DecodeSmem d = make_decode_smem(K, p.R, best_nw, p.full_read, p.coef_per_seq, sl.total, W);
