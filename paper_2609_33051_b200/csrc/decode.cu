@@ -116,7 +116,7 @@ constexpr int kSeq = 1, kPS = 2, kER = 4, kUB = 8, kAny = 16, kFull = 32;
 
 // Warps of the largest CTA; two such CTAs per SM (one of a team kernel's, which are twice as large) set the register budget: 64 registers
 // for the lean Mamba-2 kernels (32 warps), 80 for the others (24 warps), the full reads of Mamba-2 teams among them: their rows in flight
-// spilled 152 to 372 bytes at 64 (nothing at 80; 0.91 of the time with two warps a head on average; with K = V = 64 64 is faster: 9472 heads 26.8 against 28.7 us).
+// spilled 152 to 372 bytes at 64 (nothing at 80; 0.91 of the time with two warps a head on average; with K = V = 64 64 is faster: team_size.h).
 __host__ __device__ constexpr int decode_max_warps(int kind, int K, int V, int F, int W) {
     const bool lean = kind == SKETCHSSM_MAMBA2 && (F & ~(kUB | kFull)) == 0 && !(W > 1 && F == kFull && K * V > 64 * 64);
     return (lean ? 16 : 12) * (W > 1 ? 2 : 1);
@@ -809,30 +809,10 @@ __global__ void __launch_bounds__(decode_max_warps(KIND, K, V, F, W) * 32, W > 1
     if (pendB >= 0) mbar_wait_bounded(barB, (uint32_t)pendB, 1u << 14);
 }
 
-// How many warps share a head.  One warp per head keeps the most heads in flight and needs no barrier; a team shortens the
-// time of a head, which is what counts where the heads are few, where their stages leave room for few warps, and for full
-// reads, whose rows (registers, through L1) are then read by warps of which fewer wait for a sweep.  1 / 2 / 4 warps per head,
-// us a launch, `slots` heads' stages per SM:
-//   full read, KDA V = 128, 6 fp32 tokens: 128 heads 6.3 / 5.0 / 4.0; 576 6.8 / 5.4 / 6.7; 1184 (in L2) 14.9 / 15.7 / 12.4; 3072 47 / 34 /
-//     38; 7104 95 / 79 / 84.  GDN, 14 tokens: 576 7.6 / 6.8 / 8.0 (a team repeats the sweep), 2368 33 / 34 / 35, 4736 77 / 54 / 60.
-//     Mamba-2 V = 64: 576 6.1 / 4.4 / 4.0, 2368 11.5 / 10.4 / 12.3, 9472 64 / 50 / 53; 62 tokens, eight slots, 9472 127 / 100 / 86
-//   dense heads among sketched ones (Mamba-2, V = 80, one head of six dense): 288 heads 7.4 / 6.0 / 4.5, 888 7.6 / 6.6 / 5.8, 1776 9.2 / 7.3 / 9.0,
-//     2376 9.1 / 12 / 13
-//   sketch, Mamba-2, rank 32, 16384 heads: 48 tokens (6 slots) 87 / 82 / 82, 56 95 / 90 / 94, 62 (5 slots) 117 / 108 / 99; 32 tokens (10
-//     slots) 59 / 61 / 64
 // Full reads of a state that does not stay in L2 leave L1 to the rows in flight: no lines allocated (50 against 56 us for
-// the 9472 Mamba-2 heads, 34.5 against 36 for the 3072 of KDA; within L2 10 % slower), and the stages of teams
+// the 9472 Mamba-2 heads of 128 x 64, 34.5 against 36 for 3072 of KDA; within L2 10 % slower), and the stages of teams
 // of two in at most 200 KB.
 constexpr long long kStreamBytes = 96ll << 20;
-static int team_size(int kind, int need, int n, long long heads, int sms, int slots, long long full_bytes, bool ranks) {
-    if (need == kFull) {
-        if (heads <= 2ll * sms || (heads <= 4ll * sms && (kind == SKETCHSSM_MAMBA2 || n <= 8))) return 4;
-        return slots < 10 ? 4 : full_bytes > kStreamBytes ? 2 : 1;
-    }
-    if (ranks) return heads <= 6ll * sms ? 4 : heads <= 12ll * sms ? 2 : 1;
-    if (need == 0 && kind == SKETCHSSM_MAMBA2) return slots <= 5 ? 4 : slots <= 6 ? 2 : 1;
-    return 1;
-}
 
 template <int N>
 struct Int {
@@ -862,11 +842,15 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
     const int need = p.full_read ? kFull
                                  : (p.n_dev != nullptr ? kSeq : 0) | (p.coef_per_seq ? kPS : 0) | (erase ? kER : 0) |
                                        (p.sketch_bf16 ? kUB : 0) | (p.head_rank != nullptr ? kAny : 0);
-    // Warps per head (the rule and its figures: team_size).
+    // Warps per head (the rules and their figures: team_size.h).
     const long long heads = (long long)p.B * p.H;
     const int slots = (int)((smem_budget - make_decode_smem(K, p.R, 1, p.full_read, p.coef_per_seq, 0u, 1).stage_off) /
                             (sl.total + (uint32_t)((K + 80) * 4)));
-    int W = team_size(KIND, need, p.n_before, heads, ctx->sm_count, slots, p.full_read ? heads * K * V * 4 : 0, p.head_rank != nullptr);
+    constexpr bool kMamba2 = KIND == SKETCHSSM_MAMBA2;
+    int W = need == kFull           ? full_read_team(kMamba2, p.n_before, heads, ctx->sm_count, slots, K, V, kStreamBytes)
+            : p.head_rank != nullptr ? rank_table_team(kMamba2, p.n_before, heads, ctx->sm_count, slots, K, V)
+            : need == 0 && kMamba2   ? sketch_team(slots)
+                                     : 1;
     // (a caller's own choice of warps is one of warps with a head each)
     if (p.warps_per_cta || p.max_warps_per_sm > 0 || make_decode_smem(K, p.R, W, p.full_read, p.coef_per_seq, sl.total, W).total > smem_budget) W = 1;
     p.stream_state = heads * K * V * 4 > kStreamBytes ? 1 : 0;
