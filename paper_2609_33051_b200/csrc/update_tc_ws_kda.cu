@@ -26,8 +26,8 @@
 // four bytes at a time.  The pair sums of A inside a block of eight (28) are per-channel products reduced over the channels by one
 // transposing butterfly (per-warp partials summed in a fixed order: results are bitwise reproducible); the 8 x 8 blocks that
 // couple them are dot products of rescaled keys (the decay product splits at a block boundary without a quotient), all of it in
-// fp32; the 16 x 16 block of tokens 16..31 against 0..15 is an mma.sync product of rescaled keys as bf16 hi + lo.  T_11 and T_22 of the two blocks of 16 by forward substitution (one column per thread, one warp each) while six warps
-// form Ktil [Omega | q] with mma.sync.  The E step (E_1 = T_11 x_1, E_2 = T_22 (x_2 - A_21 E_1), 264 packed multiply-adds per lane)
+// fp32; the 16 x 16 block of tokens 16..31 against 0..15 is an mma.sync product of rescaled keys as bf16 hi + lo.  T_11 and T_22 of
+// the two blocks of 16 by forward substitution (one column per thread, one warp each) while six warps form Ktil [Omega | q] with mma.sync.  The E step (E_1 = T_11 x_1, E_2 = T_22 (x_2 - A_21 E_1), 288 packed multiply-adds per lane)
 // runs on the pass-B group, between the write-back of one tile and the next, so that the pass-A group only streams.
 //
 // What bounds it: the chain of the front group (some 10 k cycles a tile; the state of a tile takes 6.6 k at the rate of a copy),
@@ -105,9 +105,9 @@ __host__ __device__ inline KSmem make_ksmem(int stages) {
     return s;
 }
 
-enum { kPro = 0, kPfull = 2, kTfull = 4, kBdone = 6, kBufFree = 8, kA2free = 10, kA2rdy = 10 + kKA2, kErdy = 10 + 2 * kKA2,
-       kStg = 11 + 2 * kKA2, kStDone = 12 + 2 * kKA2, kFull = 14 + 2 * kKA2, kEmpty = 14 + 2 * kKA2 + kKStages,
-       kTfree = 14 + 2 * kKA2 + 2 * kKStages, kVals = 16 + 2 * kKA2 + 2 * kKStages, kNumBars = 18 + 2 * kKA2 + 2 * kKStages };
+enum { kPro = 0, kPfull = 2, kTfull = 4, kBufFree = 6, kA2free = 8, kA2rdy = 8 + kKA2, kErdy = 8 + 2 * kKA2,
+       kStg = 9 + 2 * kKA2, kStDone = 10 + 2 * kKA2, kFull = 12 + 2 * kKA2, kEmpty = 12 + 2 * kKA2 + kKStages,
+       kTfree = 12 + 2 * kKA2 + 2 * kKStages, kVals = 14 + 2 * kKA2 + 2 * kKStages, kNumBars = 16 + 2 * kKA2 + 2 * kKStages };
 
 __device__ __forceinline__ void k_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kKThreads, 1) update_tc_ws_kda_kernel(const Pa
         *reinterpret_cast<volatile int*>(smem + sm.misc + 32) = 0;
         for (int i = 0; i < kNumBars; ++i) {
             // one arrival per warp of a stream group: chunk ready, E ready, stage empty, accumulator halves, pass-B done, slot free
-            const bool per_warp = (i >= kA2rdy && i <= kErdy) || i == kStDone || i == kStDone + 1 || (i >= kEmpty && i < kVals) || (i >= kBdone && i < kBdone + 4);
+            const bool per_warp = (i >= kA2rdy && i <= kErdy) || i == kStDone || i == kStDone + 1 || (i >= kEmpty && i < kVals) || i == kBufFree || i == kBufFree + 1;
             mbar_init(&bars[i], per_warp ? 4 : 1);
         }
         mbar_fence_init();
