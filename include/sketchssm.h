@@ -227,7 +227,7 @@ int sketchssm_step_mixed(sketchssm_ctx* ctx, const int32_t* phase, const void* q
 
 /* Exact decode step that reads the whole state: o = S_0^T q~_t + sum_s a_s v_s (Eq. 4).
  * Same arguments and ring behaviour as sketchssm_decode_step; U and C are not read.
- * By default both decode calls run as one kernel with a warp per (batch, head) and leave `work` alone; with the
+ * By default both decode calls run as one kernel with one, two or four warps per (batch, head) and leave `work` alone; with the
  * tune key "decode_impl" = 0 they run as two kernels, the first of which forms the buffer weights a_s and the
  * coefficients (c_t, or q~_t for the full read) into `work` and the second the weighted sum of rows. */
 int sketchssm_full_read_decode(sketchssm_ctx* ctx, int n_before, const void* q, const void* k,
@@ -299,13 +299,17 @@ int sketchssm_last_launch_count(const sketchssm_ctx* ctx);
  * the two-kernel decode serves for its head; 0 = library default), "decode_stages" (1 or 2 shared-memory
  * stages per lane group of the two-kernel decode; for the warp-specialised update kernels an upper
  * bound >= 2 on their shared-memory stages of state rows; 0 = library default), "decode_warps_per_cta",
- * "decode_max_warps_per_sm" (also caps the update kernels' CTAs per SM), "update_impl" (0 = warp-specialised
+ * "decode_max_warps_per_sm" (0 = library default, the most that fit up to 32; also caps the update kernels' CTAs per SM; a value above 0
+ * for this or the key before it also selects one warp per head), "update_impl" (0 = warp-specialised
  * tensor-core kernels where their shape limits allow and CUDA cores otherwise, the default; 1 = CUDA cores
  * only; 3 = as 0 but the single-group tensor-core kernel for Mamba-2 and CUDA cores for the delta-rule kinds;
  * 4, 5 = as 1 but always the kernel that replays eight tokens together, or (delta-rule kinds) the one that replays them singly),
- * "decode_impl" (0 = two kernels; 1 = one fused kernel with a warp per head, the default), "pdl"
+ * "decode_impl" (0 = two kernels; 1 = one fused kernel, the default), "pdl"
  * (1 = programmatic dependent launch, the default).
- * Results depend on these only through floating-point summation order. */
+ * Results depend on these only through floating-point summation order.  By default the decode calls choose by the number of heads,
+ * the ring fill and the shape how many warps share a head, and add their parts of an output in another order: the last bits of
+ * a decode step's output may therefore differ between batch sizes.  So may those of an fp32 state and sketch of the delta-rule kinds where
+ * the flush runs on CUDA cores (two kernels, chosen by the number of heads); nothing that is stored in bfloat16 does. */
 int sketchssm_tune(sketchssm_ctx* ctx, const char* key, int value);
 
 const char* sketchssm_status_string(int status);

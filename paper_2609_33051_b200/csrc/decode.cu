@@ -1,14 +1,17 @@
-// Decode-step kernel, one warp per (batch, head) (sm_100a): the default for decode_step and full_read_decode.
+// Decode-step kernel, one warp per (batch, head) or a team of two or four (sm_100a): the default for decode_step and full_read_decode.
 //
 // CTAs are persistent: each walks a contiguous range of (head index, batch) items, so a single wave of CTAs
 // covers the launch, the coefficient map C of at most two head indices is staged in shared memory once per CTA,
-// and no per-CTA start-up cost is paid more than once per SM slot.  A warp owns one head at a time.  All of the
-// head's operands -- the sketch U, the buffered keys / values / gates of the ring and the current token's
-// q, k, v rows -- arrive in the warp's private shared-memory stage by 1-D bulk asynchronous copies (TMA, no
+// and no per-CTA start-up cost is paid more than once per SM slot.  A warp owns one head at a time and claims the next from a
+// counter of its CTA (its first one is fixed).  All of the head's operands -- the sketch U, the buffered keys / values / gates of the
+// ring and the current token's q, k, v rows -- arrive in the warp's private shared-memory stage by 1-D bulk asynchronous copies (TMA, no
 // multicast).  The stage is filled in two groups with an mbarrier each: what the ring sweep reads, and the sketch.
 // The next head's first group is issued right after the current head's sweep and its sketch right after the current
 // sketch has been used, each copy by its own lane, and the token's scalar gates are fetched one head ahead: the
 // loads of a head overlap the arithmetic of the one before it without a second stage.
+// A team (how many warps: team_size.h) shares a stage, which its first warp fills, and takes items in a fixed stride.  Its warps wait for a
+// group through the vote of a named barrier, so that they leave together if a wait runs out; that vote, or the barrier before the
+// parts of the output are added, is also what lets the first warp refill the stage and the others write their scratch again.
 //
 // Arithmetic per head (Algorithm 1, non-flush step; Eq. 4):
 //   x <- q_t;  for s = t .. 1:  a_s = beta_s <k_s, x>;  x <- D_s (x - a_s k_s)   [Mamba-2: a_s = beta_s (prod_{j>s} a_j) <k_s, q_t>]
