@@ -933,6 +933,7 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
         int ctas = (int)(per_sm / (d.total + 1024u));
         if (ctas * nw > cap) ctas = cap / nw;
         if (ctas * nw > reg_warps) ctas = reg_warps / nw;
+        if (W > 1 && ctas > kTeamCtas) ctas = kTeamCtas;
         if (ctas < 1) continue;
         const int warps = ctas * nw < useful ? ctas * nw : useful;
         if (warps > best_warps) { best_warps = warps; best_nw = nw; best_ctas = ctas; }

@@ -15,13 +15,15 @@ inline long long heads_per_sm(long long heads, int sms) { return (heads + sms - 
 inline bool team_cta_too_large(int warps, int W, int least, long long heads, int sms) { return warps > least && warps / W > heads_per_sm(heads, sms); }
 // ... and of the warps that fit an SM only those count that a head would take.
 inline int useful_team_warps(int W, long long heads, int sms) { return heads_per_sm(heads, sms) < 64 ? W * (int)heads_per_sm(heads, sms) : 1 << 20; }
+// The kernels name their barriers by the team's number, so each CTA holds all 16 that a CTA can have, of an SM's 64.
+constexpr int kTeamCtas = 64 / 16;
 
 // Every head reads its state.  h = heads per SM.  Over 396 points (14 kinds, shapes and types, 64 to 9472 heads, 3 to 62 tokens) the rule
 // is at worst 1.02 times one warp per head (GDN 128 x 80 beyond L2 1.12), 0.82 of it in the mean:
 //   h <= 2: 4.  128 heads: KDA, 128 x 128, 6 fp32 tokens 6.6 / 5.3 / 4.2, GDN, 14 tokens 7.7 / 6.2 / 5.0, Mamba-2, 128 x 64, 62 tokens 10.0 / 6.0 / 4.5
 //   h <= 4 (Mamba-2 6, delta rule 5 up to 16 tokens: a team repeats the sweep, a chain): 2.  592 heads: KDA fp32 7.0 / 5.9 / 7.3, GDN 8.0 / 6.7 / 7.9, Mamba-2
 //     128 x 64 6.0 / 4.4 / 4.8; 888 heads: Mamba-2 6.0 / 4.9 / 5.4, KDA fp32 7.7 / 8.2 / 8.1
-//   few slots: 4 (delta rule from as many heads per SM as there are slots).  Mamba-2, 62 tokens, 8 slots: 1776 heads 30 / 20 / 16, 9472 130 / 135 / 91; KDA, 20
+//   few slots: 4 (delta rule with 128 rows, from as many heads per SM as there are slots; else 2: 64 x 128, 30 fp32 tokens, GDN 4736 heads 57 / 56 / 68, KDA 69 / 68 / 75).  Mamba-2, 62 tokens, 8 slots: 1776 heads 30 / 20 / 16, 9472 130 / 135 / 91; KDA, 20
 //     fp32 tokens, 6 slots: 888 heads 16 / 13 / 15, 2368 57 / 66 / 44; 128 x 128, 13 slots: Mamba-2, 30 tokens 2368 heads 49 / 32 / 28, GDN, 30 tokens 1776 32 / 35 / 28,
 //     4736 79 / 70 / 74
 //   a state beyond L2: 2.  GDN 4736 heads 69 / 51 / 56, KDA fp32 3552 54 / 38 / 40, Mamba-2 128 x 64 9472 55 / 51 / 51
@@ -32,7 +34,7 @@ inline int full_read_team(bool mamba2, int n, long long heads, int sms, int slot
     auto up_to = [&](int h) { return heads <= (long long)h * sms; };
     if (up_to(2) || (up_to(3) && (mamba2 || (n <= 16 && K == 128)))) return 4;
     if (up_to(4) || (mamba2 ? up_to(6) && slots >= 10 : up_to(5) && n <= 16)) return 2;
-    if (slots < 10) return mamba2 || !up_to(slots) ? 4 : 2;
+    if (slots < 10) return mamba2 || (K == 128 && !up_to(slots)) ? 4 : 2;
     if (slots < 16 && wide && (mamba2 || (n > 16 && !up_to(6) && up_to(24)))) return 4;
     if (heads * K * V * 4 > stream_bytes) return 2;
     if (mamba2 && wide && up_to(8) && slots < 32) return 4;

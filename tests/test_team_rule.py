@@ -18,7 +18,7 @@ FULL = """
     mamba2 62 888 8 128 64 11.2 8.4 7.7; mamba2 8 1184 37 128 128 11.2 14.0 10.5; mamba2 8 1184 65 64 64 4.1 4.1 5.2; mamba2 8 2368 42 128 80 21.5 22.3 24.9
     mamba2 8 2368 45 128 64 11.6 11.8 11.8; mamba2 8 2368 65 64 64 5.4 6.3 8.0; mamba2 8 296 37 128 128 7.4 4.6 4.0; mamba2 8 296 42 128 80 7.8 5.0 4.5
     mamba2 8 296 65 64 64 3.8 3.0 2.9; mamba2 8 4736 42 128 80 36.8 34.8 44.3; mamba2 8 592 45 128 64 6.0 4.3 4.8; mamba2 8 888 37 128 128 8.3 6.8 6.9
-    mamba2 8 888 42 128 80 8.2 6.4 6.6; mamba2 8 888 45 128 64 6.0 4.9 5.3
+    mamba2 8 888 42 128 80 8.2 6.4 6.6; mamba2 8 888 45 128 64 6.0 4.9 5.3; gdn 30 4736 9 64 128 57.0 56.2 67.5; kda 30 9472 6 64 128 136.8 127.3 142.2
 """
 
 # the same: us a launch of a decode step with a rank table, 1, 2, 4 warps per head; without a dense
@@ -92,6 +92,7 @@ _CTA = r"""
 #include <cstdio>
 #include <initializer_list>
 #include "team_size.h"
+static_assert(sketchssm::kTeamCtas * 16 <= 64, "an SM has 64 named barriers, each CTA of a team kernel holds 16");
 int main() {
     for (int W : {2, 4}) for (int least : {W, 8}) for (long long heads : {1, 12, 60, 148, 300, 588, 876, 1200, 4736, 20000}) {
         int largest = 0;
