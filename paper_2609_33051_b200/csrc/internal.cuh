@@ -205,11 +205,19 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
 // Bounded wait: returns false if the barrier phase did not complete within the iteration limit.  (Sleeping between
 // polls was measured too: neutral for the kernels with many warps, up to 1.7x slower for those with few.)
 // The loop is not unrolled: with four copies at every wait the warp-specialised kernels were 120 to 190 KB of code, and their
-// roles, each a long body that a few warps run once per tile, waited for instructions.
+// roles, each a long body that a few warps run once per tile, waited for instructions (CUDA-core Mamba-2 flushes gained 5 % too).
+// ROLLED = false leaves it to the compiler: KDA's CUDA-core flush comes out faster that way (update.cu).
+template <bool ROLLED = true>
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, uint32_t limit = (1u << 22)) {
+    if constexpr (ROLLED) {
 #pragma unroll 1
-    for (uint32_t it = 0; it < limit; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
+        for (uint32_t it = 0; it < limit; ++it) {
+            if (mbar_try_wait(bar, parity)) return true;
+        }
+    } else {
+        for (uint32_t it = 0; it < limit; ++it) {
+            if (mbar_try_wait(bar, parity)) return true;
+        }
     }
     return false;
 }

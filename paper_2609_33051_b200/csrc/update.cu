@@ -253,8 +253,10 @@ __global__ void __launch_bounds__(2 * V, update_ctas<V>()) update_kernel(const P
             tg = reinterpret_cast<const IO*>(smem + us.st_tg);
             tbeta = sTok;
             tdec = sTok + 1;
-            failed = !mbar_wait_bounded(bar, parity);
-            if (failed) mbar_wait_bounded(bar, parity, 1u << 14);    // a last chance for copies in flight before the CTA leaves
+            // (KDA at 128 registers spills 24 to 32 bytes with the wait rolled or in four copies by pragma, none as the compiler has it: sketch of
+            // 8192 heads of 128 x 128 177 -> 160 us, flush of four fp32 tokens 344 -> 313; Mamba-2, V = 80 is 5 % faster rolled)
+            failed = !mbar_wait_bounded<!KDA>(bar, parity);
+            if (failed) mbar_wait_bounded<!KDA>(bar, parity, 1u << 14);    // a last chance for copies in flight before the CTA leaves
             parity ^= 1u;
             const float* Ss = reinterpret_cast<const float*>(smem + us.st_off) + (part * RP) * V + j0;
 #pragma unroll
