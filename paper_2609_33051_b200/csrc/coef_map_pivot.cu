@@ -475,8 +475,11 @@ static int launch_pivot_kv(Ctx* ctx, const Params& p, cudaStream_t stream) {
     int ctas = (int)(228u * 1024u / (sm.total + 1024u));
     if (ctas > kPivotWarps) ctas = kPivotWarps;
     const long long heads = (long long)p.B * p.H;
+    // With per-sequence phases a CTA for every head: which sequences flush is known to the device alone, and in a fixed stride some warps
+    // have three heads of those while others have none.  Mixed step of 4096 heads, CTA per head (coef_map.cu) / in a stride / so:
+    // Mamba-2 128 x 64, a quarter flushing, bfloat16 maps 60 / 67 / 55 us, 128 x 128, rank 32, a sixteenth 83 / 98 / 79; GDN 128 x 128, a quarter 115 / 123 / 106.
     long long grid = (long long)ctx->sm_count * ctas;
-    if (grid > heads) grid = heads;
+    if (grid > heads || p.n_dev != nullptr) grid = heads;
     auto kern = p.sketch_bf16 ? pivot_map_kernel<K, V, true> : pivot_map_kernel<K, V, false>;
     if ((ctx->last_cuda_error = unlock_smem(ctx, kern, true)) != cudaSuccess) return SKETCHSSM_CUDA_ERROR;
     kern<<<dim3((unsigned)grid), dim3(32), sm.total, stream>>>(p);

@@ -6,6 +6,7 @@ import torch
 
 from oracle import sketchssm_oracle as orc
 from paper_2609_33051_b200 import synth
+from tests import harness
 from tests.test_gpu_coef_map import COEF_GUARD, check_coef
 from tests.test_gpu_parity import make_layer, run_schedule
 
@@ -80,3 +81,25 @@ def test_a_stored_map_does_not_depend_on_the_batch(V, rank):
         m.check_status()
         maps.append((m.sketch[:2].clone(), m.coef[:2].clone()))
     assert torch.equal(maps[0][0], maps[1][0]) and torch.equal(maps[0][1], maps[1][1])
+
+
+@pytest.mark.parametrize("share", [1, 3, 16])
+def test_mixed_steps_map_the_sequences_that_flush_and_no_others(share):
+    """More heads than warps of the grid: a map for every head of the flushing sequences, the one its new state gives; the others stay."""
+    w = synth.Workload("t", "mamba2", 331, 7, 128, 64, 16, 8, 0, "f32", 541, basis="qr")
+    m, _S0, _Om, _C, dev = make_layer(w, coef="pivot")
+    m.ring.zero_()
+    m.state_update(0)
+    before = torch.full_like(m.coef, 7.0)
+    m.coef.copy_(before)
+    phase = torch.full((331,), 2, dtype=torch.int32, device=dev)
+    phase[::share] = -8
+    tt = harness.token_tensors(w, synth.step_inputs(w, 0, 0), dev)
+    m.step_mixed(phase, tt["q"], tt["k"], tt["v"], tt["beta"], tt["decay"], m.new_output())
+    m.check_status()
+    flushed = phase < 0
+    got = m.coef.clone()
+    assert torch.equal(got[~flushed], before[~flushed])
+    m.state_update(0)                                   # sketch and maps from the states as they are
+    m.check_status()
+    assert harness.rel_err(got[flushed].cpu().numpy(), m.coef[flushed].cpu().numpy().astype(np.float64)) <= COEF_GUARD
