@@ -11,8 +11,9 @@
 // banks.  Everything is fp32.
 //
 // Bound by memory: the state's second reading beside the flush's dirty lines leaving L2.  A CTA per head with the products as mma.sync tiles
-// on tf32 parts issued 7.0 k (V = 128: 10.2 k) warp instructions per head in stages between block barriers; this takes 4.4 k (6.4 k).
-// The map of 16384 heads, bfloat16 storage, rank 16: 183 -> 141 us (128 x 64), 306 -> 218 us (128 x 128).  Without the products
+// on tf32 parts issued 7.0 k (V = 128: 10.2 k) warp instructions per head in stages between block barriers; this takes 4.4 k (6.4 k; fp32
+// maps 3.9 k).  The map of 16384 heads, bfloat16 storage, rank 16, in CTAs of four warps: 183 -> 141 us (128 x 64), 306 -> 218 us (128 x 128); as it is
+// now, fp32, under ncu 190 -> 135 us (128 x 64; DRAM 65 %, issue slots 47 %).  Without the products
 // of the stream it takes 5 us less, without Gram-Schmidt's sweeps 12, without the columns 29; with the next chunks asked into L2 as
 // well, or probe rows read from shared memory by lanes that own half a row (14 warps instead of 12), the same.
 #include "internal.cuh"

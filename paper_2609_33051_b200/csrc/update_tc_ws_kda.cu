@@ -27,13 +27,14 @@
 // transposing butterfly (per-warp partials summed in a fixed order: results are bitwise reproducible); the 8 x 8 blocks that
 // couple them are dot products of rescaled keys (the decay product splits at a block boundary without a quotient), all of it in
 // fp32; the 16 x 16 block of tokens 16..31 against 0..15 is an mma.sync product of rescaled keys as bf16 hi + lo.  T_11 and T_22 of
-// the two blocks of 16 by forward substitution (one column per thread, one warp each) while six warps form Ktil [Omega | q] with mma.sync.  The E step (E_1 = T_11 x_1, E_2 = T_22 (x_2 - A_21 E_1), 288 packed multiply-adds per lane)
-// runs on the pass-B group, between the write-back of one tile and the next, so that the pass-A group only streams.
+// the two blocks of 16 by forward substitution (one column per thread, one warp each) while six warps form Ktil [Omega | q] with mma.sync.
+// The E step (E_1 = T_11 x_1, E_2 = T_22 (x_2 - A_21 E_1), 288 packed multiply-adds per lane) runs on the pass-B group, between the
+// write-back of one tile and the next, so that the pass-A group only streams.
 //
 // What bounds it: the chain of the front group (some 10 k cycles a tile; the state of a tile takes 6.6 k at the rate of a copy),
 // most of it instruction supply and latency of eight warps: pair sums and Z rows 2.4 k, coupling 1.2 k, operand rows 1.4 k,
 // Ktil W and T 2.3 k.  Flush of 16384 heads, 32 tokens: 1030 us with a channel per thread, blocks of 16 tokens (120 pair sums) and
-// 190 KB of code; 740 to 850 now, by box (0.49 to 0.56 of a copy's rate).  Not kept: E of the next tile before the write-back (the accumulator is freed
+// 190 KB of code; 775 now (0.53 of a copy's rate; 740 to 850 by box).  Not kept: E of the next tile before the write-back (the accumulator is freed
 // late: +60 us), T before the wait for the operand set (+40), the coupling products of a level on one warp with its fragments a
 // step ahead (spills: +100).
 //
