@@ -851,7 +851,7 @@ static int launch_decode_t(Ctx* ctx, Params p, cudaStream_t stream) {
                             (sl.total + (uint32_t)((K + 80) * 4)));
     constexpr bool kMamba2 = KIND == SKETCHSSM_MAMBA2;
     int W = need == kFull           ? full_read_team(kMamba2, p.n_before, heads, ctx->sm_count, slots, K, V, kStreamBytes)
-            : p.head_rank != nullptr ? rank_table_team(kMamba2, p.n_before, heads, ctx->sm_count, slots, K, V)
+            : p.head_rank != nullptr ? rank_table_team(kMamba2, p.n_dev != nullptr, p.n_before, heads, ctx->sm_count, slots, K, V)
             : need == 0 && kMamba2   ? sketch_team(slots)
                                      : 1;
     // (a caller's own choice of warps is one of warps with a head each)

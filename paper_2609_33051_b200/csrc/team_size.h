@@ -54,8 +54,12 @@ inline int full_read_team(bool mamba2, int n, long long heads, int sms, int slot
 //     8.0 / 6.0 / 6.2, 28 tokens 8.2 / 8.7 / 10.6 | 11.1 / 9.1 / 11.0; 1776, 4 tokens 5.8 / 6.5 / 9.1 | 11.8 / 7.7 / 10.1, 12 tokens 8.0 / 10.3 / 12.3 | 10.3 / 12.3 / 12.8
 //   smaller states: 128 x 64 2 to 6 (Mamba-2 4 to 3, 2 to 11, to 9 above 16 tokens): 876 heads of Mamba-2 4.1 / 4.2 / 5.4 | 5.8 / 4.7 / 5.4, 1488, 12 tokens 5.8 / 5.8 / 8.3 |
 //     7.2 / 6.3 / 8.6, 1776 4.7 / 6.0 / 8.0 | 6.5 / 6.1 / 8.0; 64 x 64 2 to 4: 444 heads of GDN 3.2 / 3.3 / 3.5 | 3.7 / 3.4 / 3.5, 876 3.4 / 3.6 / 5.3 | 3.9 / 3.8 / 5.3
-inline int rank_table_team(bool mamba2, int n, long long heads, int sms, int slots, int K, int V) {
+//   a mixed step between three quarters of a head and one and a half per SM: 1.  The flush of the same call starts on the SMs that the decode leaves; spread over
+//     all of them by teams it makes the flush's CTAs share SMs.  128 x 128, one sequence in 16 flushing: 108 heads of GDN 14.2 / 14.2 / 14.2, 144 14.2 / 14.3 / 21.1, 192
+//     15.0 / 21.3 / 17.4, Mamba-2 144 11.7 / 11.7 / 16.4, 192 12.3 / 16.4 / 13.2, 288 16.2 / 15.0 / 15.7 (without a flush 144 heads 8.5 / 6.4 / 5.3)
+inline int rank_table_team(bool mamba2, bool mixed, int n, long long heads, int sms, int slots, int K, int V) {
     auto up_to = [&](int h) { return heads <= (long long)h * sms; };
+    if (mixed && 4 * heads > 3ll * sms && 2 * heads <= 3ll * sms) return 1;
     if (up_to(1)) return 4;
     if (K * V < 128 * 64) return up_to(4) ? 2 : 1;
     if (K * V < 128 * 80) return mamba2 && up_to(3) ? 4 : up_to(!mamba2 ? 6 : n > 16 ? 9 : 11) ? 2 : 1;

@@ -42,6 +42,13 @@ TABLE = """
     mamba2 30 1776 9 128 80 14.0 12.8 11.8 18.8 15.3 11.8
 """
 
+# the same: us a mixed step, one head of twelve dense and one sequence in 16 flushing
+MIXED = """
+    gdn 15 108 13 128 128 14.2 14.2 14.2; gdn 15 144 13 128 128 14.2 14.3 21.1; gdn 15 192 13 128 128 15.0 21.3 17.4; gdn 15 432 13 128 128 23.2 22.5 19.9
+    mamba2 15 108 13 128 128 11.6 11.7 11.6; mamba2 15 144 13 128 128 11.7 11.7 16.4; mamba2 15 192 13 128 128 12.3 16.4 13.2
+    mamba2 15 288 13 128 128 16.2 15.0 15.7; mamba2 15 144 19 128 80 11.8 11.5 12.4; mamba2 15 720 19 128 80 18.6 17.8 16.3
+"""
+
 _MAIN = r"""
 #include <cstdio>
 #include "team_size.h"
@@ -49,7 +56,7 @@ int main() {
     int table, mamba2, n, slots, K, V;
     long long heads;
     while (std::scanf("%d %d %d %lld %d %d %d", &table, &mamba2, &n, &heads, &slots, &K, &V) == 7)
-        std::printf("%d\n", table ? sketchssm::rank_table_team(mamba2, n, heads, 148, slots, K, V)
+        std::printf("%d\n", table ? sketchssm::rank_table_team(mamba2, table == 2, n, heads, 148, slots, K, V)
                                   : sketchssm::full_read_team(mamba2, n, heads, 148, slots, K, V, 96ll << 20));
 }
 """
@@ -76,6 +83,15 @@ def test_full_reads_are_no_slower_than_with_a_warp_per_head(tmp_path):
     for p, t, w in zip(pts, times, chosen):
         assert t[w] <= 1.05 * t[0], p
     assert sum(t[w] / min(t) for t, w in zip(times, chosen)) <= 1.05 * len(pts)
+
+
+def test_mixed_steps_are_no_slower_than_with_a_warp_per_head(tmp_path):
+    pts = _points(MIXED)
+    chosen = _chosen(tmp_path, [(2, int(p[0] == "mamba2"), *p[1:6]) for p in pts])
+    assert len(chosen) == len(pts)
+    for p, w in zip(pts, chosen):
+        t = list(map(float, p[6:]))
+        assert t[w] <= 1.05 * t[0], p
 
 
 def test_rank_tables_gain_with_a_dense_head_what_they_lose_without(tmp_path):
