@@ -70,9 +70,6 @@ def test_bfloat16_sketch_with_the_fixed_map_at_every_ring_fill(K, V, rank, io):
     # a dense head among sketched ones: four warps a head, two
     ("mamba2", 11, 6, 128, 80, 13, 12, "bf16", False, True), ("mamba2", 151, 7, 128, 64, 24, 8, "f32", False, True),
     ("gdn", 9, 5, 128, 128, 16, 8, "bf16", False, True), ("kda", 171, 6, 64, 64, 9, 12, "bf16", False, True),
-    # (the last head dense, its rows the last of the state: four warps with sixteen rows each)
-    ("mamba2", 5, 7, 64, 64, 9, 12, "bf16", False, True), ("kda", 4, 7, 64, 128, 16, 16, "f32", False, True),
-    ("gdn", 11, 2, 64, 64, 24, 8, "f32", False, True),
     # long rings and large ranks: two warps a head, then four as the ring fills
     ("mamba2", 37, 9, 128, 64, 32, 64, "bf16", False, False), ("mamba2", 37, 9, 128, 128, 16, 64, "bf16", False, False),
     ("mamba2", 31, 9, 128, 80, 21, 64, "f32", False, False), ("mamba2", 31, 9, 64, 128, 45, 64, "f32", False, False)])
@@ -122,3 +119,10 @@ def test_a_callers_warp_count_is_taken_up_to_eight_and_refused_above(call):
             getattr(m, call)(0, *args, m.new_output())
         assert e.value.status == -2
     m.check_status()
+
+
+@pytest.mark.parametrize("case", [("mamba2", 5, 7, 64, 64, 9, 12, "bf16", False, True), ("kda", 4, 7, 64, 128, 16, 16, "f32", False, True),
+                                  ("gdn", 11, 2, 64, 64, 24, 8, "f32", False, True)])
+def test_the_last_head_dense_with_sixteen_rows_per_warp(case):
+    """Its rows are the last of the state: four warps a head, K = 64."""
+    test_teams_of_warps_and_single_warps_agree(*case)
